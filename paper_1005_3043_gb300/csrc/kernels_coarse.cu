@@ -583,11 +583,27 @@ void prolongator_to_boundary(double2* out, const double2* P, int nv, const Geom&
 // partials in the same order, so all CTAs take identical decisions.
 namespace wmg {
 
-// One CG phase on the aggregates of this CTA, `xpb` at a time: stage the
-// operand on X and its 8 neighbours in shared memory, then apply the coarse
-// stencil.  Thread (x, d, row group) accumulates R consecutive rows a of block
-// A[X][d] (one 16-byte load carries rows a, a+1 of column b) with U
-// independent loads in flight; shared memory sums the 9 directions.
+// How the rows are dealt out (host: cgnr_split).  The rows of every aggregate
+// are cut into rsp parts of equal size; unit u = X * rsp + part.  A CTA works on
+// upb consecutive units at a time, tpu = 9 * bs * (row groups of a part) threads
+// each: thread (unit, d, column part, row group).
+// FP32 and FP16 operators (bound by the operator's bytes): rsp = bs = 1, whole
+// aggregates, as many as fit the CTA.  FP64 (bound by the FP64 pipe, two FMAs
+// per clock and SM): every SM has to have an equal share of the rows.  With
+// whole aggregates an 8^4 lattice (16 aggregates) ran on 4 SMs and 12^3 x 24
+// (162 aggregates) on 54; cut into parts, one CTA per SM (its partial sums are
+// re-added in FP64 by every CTA, so no more CTAs than SMs).  Measured with the
+// FP64 operator's CTAs above: an 8^4 solve (Nv = 8) 321 -> 169 ms, 12^3 x 24
+// (Nv = 12) 285 -> 193 ms.
+struct CgnrSplit {
+    int upb, rsp, bs;
+};
+
+// One CG phase on the units of this CTA, upb at a time: stage the operand on
+// their aggregates and the 8 neighbours in shared memory, then apply the coarse
+// stencil.  A thread accumulates R consecutive rows a of block A[X][d] (one
+// 16-byte load carries rows a, a+1 of column b) with U independent loads in
+// flight; shared memory sums the 9 directions and the column parts.
 // The operand is formed while staging (STAGE):
 //   ST_P: pn = s + beta * p_old   (first iteration: pn = s); own entries -> p_new
 //         output q = D_c pn;          partial sums: n0 = ||q||^2
@@ -640,18 +656,25 @@ template <typename T> struct PhaseArgs {
 
 template <typename T, bool DAG, int STAGE, bool H16>
 __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, const __half2* __restrict__ A16,
-                         const float* __restrict__ s16, int nc, int xpb, const Geom& g, v2<T>* xs, cx<T>* part,
-                         const int* __restrict__ nbr, T& n0, T& n1) {
+                         const float* __restrict__ s16, int nc, const CgnrSplit& sp, const Geom& g, v2<T>* xs,
+                         cx<T>* part, const int* __restrict__ nbr, T& n0, T& n1) {
     constexpr int R = RowsPerThread<T, H16>::value;
-    const int nvh = nc >> 1, nrow = 9 * nc, ngrp = nc / R, nthr = 9 * ngrp, nall = xpb * nrow;
-    const int xl = threadIdx.x / nthr, rem = threadIdx.x - xl * nthr;
-    const int d = rem / ngrp, a0 = (rem - d * ngrp) * R;
-    for (int Xb = blockIdx.x * xpb; Xb < g.Vc; Xb += gridDim.x * xpb) {
+    const int nvh = nc >> 1, nrow = 9 * nc, ngl = nc / R / sp.rsp, rows = ngl * R, nsum = 9 * sp.bs;
+    const int tpu = nsum * ngl, nunit = g.Vc * sp.rsp;
+    const int ul = threadIdx.x / tpu, rem = threadIdx.x - ul * tpu;
+    const int db = rem / ngl, a0 = (rem - db * ngl) * R;   // a0: row within the part
+    const int d = db / sp.bs, bp = db - d * sp.bs;
+    const int bc = (nc + sp.bs - 1) / sp.bs, b_lo = bp * bc, b_hi = min(nc, b_lo + bc);
+    for (int Ub = blockIdx.x * sp.upb; Ub < nunit; Ub += gridDim.x * sp.upb) {
+        const int Ue = min(Ub + sp.upb, nunit), Xb = Ub / sp.rsp, nall = ((Ue - 1) / sp.rsp - Xb + 1) * nrow;
         for (int i = threadIdx.x; i < nall; i += blockDim.x) {
             int xi = i / nrow, ri = i - xi * nrow;
             int di = ri / nc, b = ri - di * nc;
             int X = Xb + xi;
-            if (X < g.Vc) {
+            {
+                // the CTA that owns row b of X does that entry's vector updates
+                const int u = X * sp.rsp + b / rows;
+                const bool own = di == 0 && u >= Ub && u < Ue;
                 int Y = __ldg(nbr + (size_t)X * 9 + di);
                 size_t o = (size_t)Y * nc + b;
                 cx<T> v;
@@ -660,10 +683,10 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
                 } else if (STAGE == ST_P) {
                     v = ld<T>(ph.s + o);
                     if (!ph.first) v = v + ph.coef * ld<T>(ph.p_old + o);
-                    if (di == 0) st<T>(ph.p_new + o, v);
+                    if (own) st<T>(ph.p_new + o, v);
                 } else {
                     v = ld<T>(ph.r_old + o) - ph.coef * ld<T>(ph.q + o);
-                    if (di == 0) {
+                    if (own) {
                         st<T>(ph.r_new + o, v);
                         st<T>(ph.y + o, ld<T>(ph.y + o) + ph.coef * ld<T>(ph.p_new + o));
                         n1 += norm2(v);
@@ -674,23 +697,24 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
             }
         }
         __syncthreads();
-        const int X = Xb + xl;
-        if (threadIdx.x < xpb * nthr && X < g.Vc) {
-            const v2<T>* xd = xs + xl * nrow + d * nc;
+        const int U0 = Ub + ul, X = U0 / sp.rsp, ar = (U0 - X * sp.rsp) * rows + a0;   // ar: row within the block
+        if (ul < sp.upb && U0 < nunit) {
+            const v2<T>* xd = xs + (X - Xb) * nrow + d * nc;
+            cx<T>* pd = part + (size_t)(ul * nsum + db) * rows + a0;
             cx<T> acc[R][2];
 #pragma unroll
             for (int r = 0; r < R; ++r) { acc[r][0] = cx<T>(0, 0); acc[r][1] = cx<T>(0, 0); }
             constexpr int U = 4;
             if constexpr (H16) {
-                const __half2* Ad = A16 + ((size_t)X * 9 + d) * nc * nc + a0;
-                for (int b0 = 0; b0 < nc; b0 += U) {
+                const __half2* Ad = A16 + ((size_t)X * 9 + d) * nc * nc + ar;
+                for (int b0 = b_lo; b0 < b_hi; b0 += U) {
                     uint4 raw[U];
 #pragma unroll
                     for (int j = 0; j < U; ++j)
-                        if (b0 + j < nc) raw[j] = __ldg(reinterpret_cast<const uint4*>(Ad + (size_t)(b0 + j) * nc));
+                        if (b0 + j < b_hi) raw[j] = __ldg(reinterpret_cast<const uint4*>(Ad + (size_t)(b0 + j) * nc));
 #pragma unroll
                     for (int j = 0; j < U; ++j)
-                        if (b0 + j < nc) {
+                        if (b0 + j < b_hi) {
                             cx<T> xb = ld<T>(xd + b0 + j);
                             const __half2* h = reinterpret_cast<const __half2*>(&raw[j]);
 #pragma unroll
@@ -702,34 +726,34 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
                 }
                 const T sc = (T)s16[(size_t)X * 9 + d];
 #pragma unroll
-                for (int r = 0; r < R; ++r) part[xl * nrow + d * nc + a0 + r] = sc * (acc[r][0] + acc[r][1]);
+                for (int r = 0; r < R; ++r) pd[r] = sc * (acc[r][0] + acc[r][1]);
             } else {
-                const v2<T>* Ad = A + ((size_t)X * 9 + d) * nc * nc + a0;
-                for (int b0 = 0; b0 < nc; b0 += U) {
+                const v2<T>* Ad = A + ((size_t)X * 9 + d) * nc * nc + ar;
+                for (int b0 = b_lo; b0 < b_hi; b0 += U) {
                     cx<T> av[U][R];
 #pragma unroll
                     for (int j = 0; j < U; ++j)
-                        if (b0 + j < nc) RowLoad<T, R>::load(Ad + (size_t)(b0 + j) * nc, av[j]);
+                        if (b0 + j < b_hi) RowLoad<T, R>::load(Ad + (size_t)(b0 + j) * nc, av[j]);
 #pragma unroll
                     for (int j = 0; j < U; ++j)
-                        if (b0 + j < nc) {
+                        if (b0 + j < b_hi) {
                             cx<T> xb = ld<T>(xd + b0 + j);
 #pragma unroll
                             for (int r = 0; r < R; ++r) cmad(acc[r][j & 1], av[j][r], xb);
                         }
                 }
 #pragma unroll
-                for (int r = 0; r < R; ++r) part[xl * nrow + d * nc + a0 + r] = acc[r][0] + acc[r][1];
+                for (int r = 0; r < R; ++r) pd[r] = acc[r][0] + acc[r][1];
             }
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < xpb * nc; t += blockDim.x) {
-            int x2 = t / nc, a2 = t - x2 * nc;
-            int X2 = Xb + x2;
-            if (X2 < g.Vc) {
-                cx<T> sum = part[x2 * nrow + a2];
-#pragma unroll
-                for (int dd = 1; dd < 9; ++dd) sum = sum + part[x2 * nrow + dd * nc + a2];
+        for (int t = threadIdx.x; t < sp.upb * rows; t += blockDim.x) {
+            const int u2 = t / rows, U2 = Ub + u2, X2 = U2 / sp.rsp, a2 = (U2 - X2 * sp.rsp) * rows + (t - u2 * rows);
+            if (U2 < nunit) {
+                const cx<T>* ps = part + (size_t)u2 * nsum * rows + (t - u2 * rows);
+                cx<T> sum = ps[0];
+#pragma unroll 8
+                for (int dd = 1; dd < nsum; ++dd) sum = sum + ps[dd * rows];
                 if (DAG && a2 >= nvh) sum = cx<T>(-sum.r, -sum.i);
                 st<T>(ph.out + (size_t)X2 * nc + a2, sum);
                 n0 += norm2(sum);
@@ -745,14 +769,16 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
 // with two grid barriers per iteration: the elementwise updates of p and r are
 // done while staging the neighbour operands of the next stencil (p and r
 // double-buffered so that no CTA overwrites what another still reads).
-template <typename T> struct CgnrMaxThreads { static constexpr int value = 384; };
+// FP64: one CTA per SM, registers for all columns of a thread's loads in flight
+template <typename T> struct CgnrMaxThreads { static constexpr int value = 384, blocks = sizeof(T) == 8 ? 1 : 2; };
 
 template <typename T, bool H16>
-__global__ void __launch_bounds__(CgnrMaxThreads<T>::value, 2) k_cgnr_persistent(CgnrArgs<T> a) {
+__global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::blocks) k_cgnr_persistent(CgnrArgs<T> a) {
     extern __shared__ unsigned char smem_raw[];
-    const int nc = a.nc, xpb = a.xpb;
+    const int nc = a.nc;
+    const CgnrSplit sp{a.upb, a.rsp, a.bs};
     v2<T>* xs = reinterpret_cast<v2<T>*>(smem_raw);
-    cx<T>* part = reinterpret_cast<cx<T>*>(smem_raw + sizeof(v2<T>) * 9 * nc * xpb);
+    cx<T>* part = reinterpret_cast<cx<T>*>(smem_raw + sizeof(v2<T>) * 9 * nc * ((sp.upb + 2 * sp.rsp - 2) / sp.rsp));
     __shared__ T shr[33];
     const unsigned int G = gridDim.x;
     unsigned int* cnt = a.bar;
@@ -761,11 +787,11 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, 2) k_cgnr_persistent
     v2<T>* pbuf[2] = {a.p, a.p1};
     // y = 0, r = rc on the aggregates of this CTA; ||rc||^2
     T loc = 0;
-    for (int Xb = blockIdx.x * xpb; Xb < a.g.Vc; Xb += G * xpb)
-        for (int t = threadIdx.x; t < xpb * nc; t += blockDim.x) {
-            int X = Xb + t / nc;
-            if (X < a.g.Vc) {
-                size_t o = (size_t)X * nc + (t % nc);
+    const int rows = nc / sp.rsp;   // rows of a unit: unit u holds entries u * rows ..
+    for (int Ub = blockIdx.x * sp.upb; Ub < a.g.Vc * sp.rsp; Ub += G * sp.upb)
+        for (int t = threadIdx.x; t < sp.upb * rows; t += blockDim.x) {
+            if (Ub + t / rows < a.g.Vc * sp.rsp) {
+                size_t o = (size_t)Ub * rows + t;
                 v2<T> v = a.rc[o];
                 a.r[o] = v;
                 v2<T> z; z.x = 0; z.y = 0;
@@ -784,7 +810,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, 2) k_cgnr_persistent
         // s = D_c^dag r, gamma = ||s||^2
         ph.in = a.r;
         ph.out = a.s;
-        cg_phase<T, true, ST_PLAIN, H16>(ph, a.A, a.A16, a.s16, nc, xpb, a.g, xs, part, a.nbr, n0, n1);
+        cg_phase<T, true, ST_PLAIN, H16>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
         write_partial<T>(n0, a.partials, 1, shr);
         if (!grid_sync(cnt, gen, G, a.err)) return;
         T gamma = sum_partials<T>(a.partials, 1, G, shr);
@@ -796,7 +822,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, 2) k_cgnr_persistent
             ph.s = a.s; ph.p_old = pbuf[b ^ 1]; ph.p_new = pbuf[b]; ph.out = a.q;
             ph.coef = beta; ph.first = (it == 0);
             n0 = 0; n1 = 0;
-            cg_phase<T, false, ST_P, H16>(ph, a.A, a.A16, a.s16, nc, xpb, a.g, xs, part, a.nbr, n0, n1);
+            cg_phase<T, false, ST_P, H16>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
             write_partial<T>(n0, a.partials, 0, shr);
             if (!grid_sync(cnt, gen, G, a.err)) return;
             T qq = sum_partials<T>(a.partials, 0, G, shr);
@@ -807,7 +833,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, 2) k_cgnr_persistent
             ph.r_old = rbuf[b]; ph.q = a.q; ph.r_new = rbuf[b ^ 1]; ph.y = a.y; ph.p_new = pbuf[b];
             ph.out = a.s; ph.coef = alpha;
             n0 = 0; n1 = 0;
-            cg_phase<T, true, ST_R, H16>(ph, a.A, a.A16, a.s16, nc, xpb, a.g, xs, part, a.nbr, n0, n1);
+            cg_phase<T, true, ST_R, H16>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
             write_partial<T>(n0, a.partials, 1, shr);
             write_partial<T>(n1, a.partials, 2, shr);
             if (!grid_sync(cnt, gen, G, a.err)) return;
@@ -828,54 +854,59 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, 2) k_cgnr_persistent
     }
 }
 
-// aggregates per CTA: as many 9*nc-thread groups as fit in the thread limit
-template <typename T, bool H16> int cgnr_threads_per_x(int nc) { return 9 * (nc / RowsPerThread<T, H16>::value); }
-template <typename T, bool H16> int cgnr_xpb(int nc) {
-    int x = CgnrMaxThreads<T>::value / cgnr_threads_per_x<T, H16>(nc);
-    return x > 0 ? x : 1;
+// Split of the rows (see CgnrSplit) and its shared memory.
+template <typename T, bool H16> size_t cgnr_smem(int nc, const CgnrSplit& s) {
+    const size_t xmax = (s.upb + 2 * s.rsp - 2) / s.rsp;   // aggregates that upb consecutive units can touch
+    return sizeof(v2<T>) * 9 * nc * xmax + sizeof(cx<T>) * 9 * s.bs * (nc / s.rsp) * s.upb;
 }
-template <typename T, bool H16> int cgnr_block_threads(int nc) {
-    return ((cgnr_xpb<T, H16>(nc) * cgnr_threads_per_x<T, H16>(nc) + 31) / 32) * 32;
+template <typename T, bool H16> int cgnr_block_threads(int nc, const CgnrSplit& s) {
+    const int tpu = 9 * s.bs * (nc / RowsPerThread<T, H16>::value / s.rsp);
+    return (s.upb * tpu + 31) / 32 * 32;
 }
-template <typename T, bool H16> size_t cgnr_smem(int nc) {
-    return (sizeof(v2<T>) + sizeof(cx<T>)) * 9 * (size_t)nc * cgnr_xpb<T, H16>(nc);
-}
-
-// co-resident CTAs for this nc, then the smallest balanced grid covering all aggregates
-template <typename T, bool H16> int cgnr_grid(int nc, int Vc) {
-    // per device (SM count and occupancy may differ between devices); slots are
-    // atomic so host threads calling at once see either 0 or the final value
-    constexpr int kDevs = 16;
-    static std::atomic<int> cached[kDevs][2][128];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs) return 0;
-    int key = nc < 128 ? nc : 127;
-    std::atomic<int>& slot = cached[dev][H16 ? 1 : 0][key];
-    int gmax = slot.load(std::memory_order_acquire);
-    if (gmax == 0) {
-        int sms = 0, per = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        size_t sm = cgnr_smem<T, H16>(nc);   // < 48 KB: no attribute needed
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cgnr_persistent<T, H16>, cgnr_block_threads<T, H16>(nc), sm);
-        gmax = per * sms;
-        slot.store(gmax, std::memory_order_release);
+template <typename T, bool H16> CgnrSplit cgnr_split(int nc, int Vc, int sms) {
+    constexpr int most = CgnrMaxThreads<T>::value;
+    const int ngrp = nc / RowsPerThread<T, H16>::value;
+    if (sizeof(T) == 4) return CgnrSplit{std::max(1, most / (9 * ngrp)), 1, 1};
+    // FP64: the parts per aggregate that give the busiest SM the fewest rows
+    // (2 % per part for the operand staged once per CTA that shares an aggregate)
+    int rsp = 1;
+    double best = 1e30;
+    for (int r = 1; r <= ngrp; ++r) {
+        if (ngrp % r) continue;
+        const double cost = (double)((Vc * r + sms - 1) / sms) / r * (1.0 + 0.02 * r);
+        if (cost < best) { best = cost; rsp = r; }
     }
-    if (gmax <= 0) return 0;
-    int xpb = cgnr_xpb<T, H16>(nc);
-    int batches = (Vc + xpb - 1) / xpb;               // CTA-sized pieces of work
-    int rounds = (batches + gmax - 1) / gmax;         // pieces per CTA
-    return (batches + rounds - 1) / rounds;
+    // columns in bs parts while the busiest CTA's units leave threads idle
+    const int ngl = ngrp / rsp, per = std::max(1, std::min((Vc * rsp + sms - 1) / sms, most / (9 * ngl)));
+    int bs = 1;
+    while (bs < 8 && 2 * bs * 4 <= nc && 9 * ngl * 2 * bs * per <= most) bs *= 2;
+    return CgnrSplit{per, rsp, bs};
 }
 
+// grid: co-resident CTAs for this split (FP64: one per SM), then the smallest
+// balanced grid covering all units
 template <typename T, bool H16> cudaError_t cgnr_launch(const CgnrArgs<T>& args, cudaStream_t st) {
-    int G = cgnr_grid<T, H16>(args.nc, args.g.Vc);
-    if (G <= 0) return cudaErrorCooperativeLaunchTooLarge;
+    const int sms = device_sm_count();
+    const CgnrSplit sp = cgnr_split<T, H16>(args.nc, args.g.Vc, sms);
+    const int thr = cgnr_block_threads<T, H16>(args.nc, sp);
+    const size_t sm = cgnr_smem<T, H16>(args.nc, sp);
+    const void* fn = (const void*)k_cgnr_persistent<T, H16>;
+    if (sm > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+    }
+    int per = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, thr, sm);
+    if (e != cudaSuccess) return e;
+    const int gmax = (sizeof(T) == 8 ? std::min(per, 1) : per) * sms;
+    if (gmax <= 0) return cudaErrorCooperativeLaunchTooLarge;
+    const int batches = (args.g.Vc * sp.rsp + sp.upb - 1) / sp.upb;   // CTA-sized pieces of work
+    const int rounds = (batches + gmax - 1) / gmax;                    // pieces per CTA
     CgnrArgs<T> a = args;
-    a.xpb = cgnr_xpb<T, H16>(a.nc);
+    a.upb = sp.upb; a.rsp = sp.rsp; a.bs = sp.bs;
     void* params[] = {&a};
     note_launch();
-    return cudaLaunchCooperativeKernel((const void*)k_cgnr_persistent<T, H16>, dim3(G),
-                                       dim3(cgnr_block_threads<T, H16>(a.nc)), params, cgnr_smem<T, H16>(a.nc), st);
+    return cudaLaunchCooperativeKernel(fn, dim3((batches + rounds - 1) / rounds), dim3(thr), params, sm, st);
 }
 template <> cudaError_t cgnr_persistent<float>(const CgnrArgs<float>& a, cudaStream_t st) {
     if (a.A16) {

@@ -190,7 +190,7 @@ int device_sm_count() {
 // measured on 24^3x64, 99.8 -> 92.2 us with L2 flushed, 93.9 -> 85.8 us back to
 // back; 6 gave the same, 8 (64 registers, spills) 111 us.  FP64: 256 x 2.
 template <typename T, int MINB> struct DslashShape { static constexpr int threads = 128, blocks = MINB; };
-template <int MINB> struct DslashShape<double, MINB> { static constexpr int threads = 256, blocks = 2; };
+template <int MINB> struct DslashShape<double, MINB> { static constexpr int threads = 64, blocks = 6; };
 constexpr int kDslashOneWave = 7, kDslashMultiWave = 5;
 
 template <typename T, int MODE, int MINB>
@@ -253,7 +253,12 @@ __global__ void __launch_bounds__(DslashShape<T, MINB>::threads, DslashShape<T, 
 template <typename T, int MINB>
 static void dslash_launch(int mode, v2<T>* out, const v2<T>* in, const v2<T>* U, const v2<T>* src, const Geom& g,
                           T diag, double omega, int slot, const Reduce& R, cudaStream_t st) {
-    constexpr int thr = DslashShape<T, MINB>::threads;
+    // FP64 in CTAs of one or two warps: the pipe issues two FMAs per clock and SM,
+    // so every SM has to have its share of the sites.  With 256 threads 8^4 ran on
+    // 16 SMs (74 us) and 12^3 x 24 left half of the SMs with twice the sites of the
+    // others (121 us); FP32 waits on memory, and its reductions on the CTA count,
+    // so it keeps its shape on every lattice.
+    const int thr = sizeof(T) == 8 && g.V <= 256LL * device_sm_count() ? 32 : DslashShape<T, MINB>::threads;
     const int grid = grid_for(g.V, thr);
     note_launch();
     switch (mode) {

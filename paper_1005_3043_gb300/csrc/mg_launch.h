@@ -135,7 +135,7 @@ template <typename T> struct CgnrArgs {
     const int* nbr;        // coarse neighbour table [Vc][9]
     const v2<T>* rc;
     int nc;
-    int xpb;               // aggregates per CTA (set by the launcher)
+    int upb, rsp, bs;      // split of the rows over CTAs and threads (set by the launcher)
     Geom g;
     double tol2;
     int maxit;
