@@ -597,6 +597,10 @@ namespace wmg {
 // (Nv = 12) 285 -> 193 ms.
 struct CgnrSplit {
     int upb, rsp, bs;
+    // the FP32 / FP16 split with its constants known to the compiler (index
+    // arithmetic by run-time divisors cost 5-8 % of an iteration)
+    template <typename T> __device__ int parts() const { return sizeof(T) == 4 ? 1 : rsp; }
+    template <typename T> __device__ int cols() const { return sizeof(T) == 4 ? 1 : bs; }
 };
 
 // One CG phase on the units of this CTA, upb at a time: stage the operand on
@@ -659,22 +663,23 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
                          const float* __restrict__ s16, int nc, const CgnrSplit& sp, const Geom& g, v2<T>* xs,
                          cx<T>* part, const int* __restrict__ nbr, T& n0, T& n1) {
     constexpr int R = RowsPerThread<T, H16>::value;
-    const int nvh = nc >> 1, nrow = 9 * nc, ngl = nc / R / sp.rsp, rows = ngl * R, nsum = 9 * sp.bs;
-    const int tpu = nsum * ngl, nunit = g.Vc * sp.rsp;
+    const int rsp = sp.template parts<T>(), bs = sp.template cols<T>();
+    const int nvh = nc >> 1, nrow = 9 * nc, ngl = nc / R / rsp, rows = sizeof(T) == 4 ? nc : ngl * R, nsum = 9 * bs;
+    const int tpu = nsum * ngl, nunit = g.Vc * rsp;
     const int ul = threadIdx.x / tpu, rem = threadIdx.x - ul * tpu;
     const int db = rem / ngl, a0 = (rem - db * ngl) * R;   // a0: row within the part
-    const int d = db / sp.bs, bp = db - d * sp.bs;
-    const int bc = (nc + sp.bs - 1) / sp.bs, b_lo = bp * bc, b_hi = min(nc, b_lo + bc);
+    const int d = db / bs, bp = db - d * bs;
+    const int bc = (nc + bs - 1) / bs, b_lo = bp * bc, b_hi = min(nc, b_lo + bc);
     for (int Ub = blockIdx.x * sp.upb; Ub < nunit; Ub += gridDim.x * sp.upb) {
-        const int Ue = min(Ub + sp.upb, nunit), Xb = Ub / sp.rsp, nall = ((Ue - 1) / sp.rsp - Xb + 1) * nrow;
+        const int Ue = min(Ub + sp.upb, nunit), Xb = Ub / rsp, nall = ((Ue - 1) / rsp - Xb + 1) * nrow;
         for (int i = threadIdx.x; i < nall; i += blockDim.x) {
             int xi = i / nrow, ri = i - xi * nrow;
             int di = ri / nc, b = ri - di * nc;
             int X = Xb + xi;
             {
                 // the CTA that owns row b of X does that entry's vector updates
-                const int u = X * sp.rsp + b / rows;
-                const bool own = di == 0 && u >= Ub && u < Ue;
+                const int u = X * rsp + b / rows;
+                const bool own = di == 0 && (sizeof(T) == 4 || (u >= Ub && u < Ue));
                 int Y = __ldg(nbr + (size_t)X * 9 + di);
                 size_t o = (size_t)Y * nc + b;
                 cx<T> v;
@@ -697,7 +702,7 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
             }
         }
         __syncthreads();
-        const int U0 = Ub + ul, X = U0 / sp.rsp, ar = (U0 - X * sp.rsp) * rows + a0;   // ar: row within the block
+        const int U0 = Ub + ul, X = U0 / rsp, ar = (U0 - X * rsp) * rows + a0;   // ar: row within the block
         if (ul < sp.upb && U0 < nunit) {
             const v2<T>* xd = xs + (X - Xb) * nrow + d * nc;
             cx<T>* pd = part + (size_t)(ul * nsum + db) * rows + a0;
@@ -748,7 +753,7 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
         }
         __syncthreads();
         for (int t = threadIdx.x; t < sp.upb * rows; t += blockDim.x) {
-            const int u2 = t / rows, U2 = Ub + u2, X2 = U2 / sp.rsp, a2 = (U2 - X2 * sp.rsp) * rows + (t - u2 * rows);
+            const int u2 = t / rows, U2 = Ub + u2, X2 = U2 / rsp, a2 = (U2 - X2 * rsp) * rows + (t - u2 * rows);
             if (U2 < nunit) {
                 const cx<T>* ps = part + (size_t)u2 * nsum * rows + (t - u2 * rows);
                 cx<T> sum = ps[0];
