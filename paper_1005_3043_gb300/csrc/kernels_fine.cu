@@ -379,51 +379,114 @@ template <typename T> void normalize_dev(v2<T>* x, size_t n, int slot, const Red
 // ================================================================ GCR
 __device__ __forceinline__ int rslot(int j, int k) { return S_GCR_R + 2 * (k * K_MAX + j); }
 
-template <typename T, int NJ>
-__global__ void k_gcr_multidot(const v2<T>* __restrict__ basis, size_t n, int k, Reduce R) {
+// Entries per thread and step of the basis passes: 16 bytes of one vector (FP32:
+// two complex entries; fine and coarse vectors have an even number of entries).
+template <typename T> struct BasisVec {
+    static constexpr int E = sizeof(T) == 4 ? 2 : 1;
+    cx<T> c[E];
+    __device__ __forceinline__ void load(const v2<T>* p) {
+        if constexpr (E == 2) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+            c[0] = cx<T>(q.x, q.y);
+            c[1] = cx<T>(q.z, q.w);
+        } else {
+            c[0] = ldg<T>(p);
+        }
+    }
+    __device__ __forceinline__ void store(v2<T>* p) const {
+        if constexpr (E == 2) *reinterpret_cast<float4*>(p) = make_float4(c[0].r, c[0].i, c[1].r, c[1].i);
+        else st<T>(p, c[0]);
+    }
+};
+
+// Projections <basis_j, basis_k>, j < k, in one pass.  GM (the GMRES smoother):
+// basis vector j stands for f_j basis_j, f_j = 1 / |basis_j| in scal[S_GMRES_F + j],
+// and basis_k for f_{k-1} times itself (D applied to the stored basis_{k-1}), so
+// that no pass normalises a vector: the factors join the projections here and
+// the coefficients in k_gcr_orth_norm.  (16^3x32, FP32, GMRES(12): 13 passes of
+// 20 us per cycle.)  Bound by the bytes of the basis: all k + 1 loads of a step
+// are independent, the grid is what an SM holds (a few hundred partial sums).
+// Measured with the reductions of mg_common.cuh: the Krylov kernels of one solve
+// 35.6 -> 20.1 ms on 16^3x32 (FP32, GMRES(12)), 67 -> 39 ms on 12^3x24 (FP64).
+template <typename T, int NJ, bool GM>
+__global__ void __launch_bounds__(kThreads) k_gcr_multidot(const v2<T>* __restrict__ basis, size_t n, int k, Reduce R) {
+    constexpr int E = BasisVec<T>::E;
     T a[2 * NJ];
 #pragma unroll
     for (int j = 0; j < 2 * NJ; ++j) a[j] = 0;
-    const v2<T>* pk = basis + (size_t)k * n;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        cx<T> v = ld<T>(pk + i);
+    for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
+        BasisVec<T> v;
+        v.load(basis + (size_t)k * n + i);
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
             if (j < k) {
-                cx<T> pj = ld<T>(basis + (size_t)j * n + i);
+                BasisVec<T> pj;
+                pj.load(basis + (size_t)j * n + i);
                 cx<T> t(a[2 * j], a[2 * j + 1]);
-                cmadc(t, pj, v);
+#pragma unroll
+                for (int e = 0; e < E; ++e) cmadc(t, pj.c[e], v.c[e]);
                 a[2 * j] = t.r;
                 a[2 * j + 1] = t.i;
             }
         }
     }
     grid_reduce<2 * NJ, T>(a, R.partials, R.ticket, R.partial_bytes, [&](double (&t)[2 * NJ]) {
+        const double fk = GM ? R.scal[S_GMRES_F + k - 1] : 1.0;
         for (int j = 0; j < k && j < NJ; ++j) {
-            R.scal[rslot(j, k)] = t[2 * j];
-            R.scal[rslot(j, k) + 1] = t[2 * j + 1];
+            const double f = GM ? fk * R.scal[S_GMRES_F + j] : 1.0;
+            R.scal[rslot(j, k)] = GM ? f * t[2 * j] : t[2 * j];
+            R.scal[rslot(j, k) + 1] = GM ? f * t[2 * j + 1] : t[2 * j + 1];
         }
     });
 }
-template <typename T>
-__global__ void k_gcr_orth_norm(v2<T>* basis, size_t n, int k, Reduce R) {
-    __shared__ double beta[2 * K_MAX];
-    for (int j = threadIdx.x; j < 2 * k; j += blockDim.x) beta[j] = R.scal[S_GCR_R + 2 * k * K_MAX + j];
+// basis_k -= sum_j h_jk basis_j and its norm.  GM: factors as above, the norm
+// recorded as h_{k,k-1} (k = 0: the norm of the residual, nothing to subtract or
+// store) with its reciprocal f_k (0 for a zero vector: a breakdown ends the space).
+template <typename T, int NJ, bool GM>
+__global__ void __launch_bounds__(kThreads) k_gcr_orth_norm(v2<T>* basis, size_t n, int k, Reduce R) {
+    constexpr int E = BasisVec<T>::E;
+    __shared__ T beta[2 * NJ];
+    for (int j = threadIdx.x; j < k; j += blockDim.x) {
+        const double f = GM ? R.scal[S_GMRES_F + j] : 1.0;
+        beta[2 * j] = (T)(f * R.scal[rslot(j, k)]);
+        beta[2 * j + 1] = (T)(f * R.scal[rslot(j, k) + 1]);
+    }
     __syncthreads();
+    const T fk = GM && k > 0 ? (T)R.scal[S_GMRES_F + k - 1] : T(1);
     v2<T>* pk = basis + (size_t)k * n;
     T a = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        cx<T> v = ld<T>(pk + i);
-        for (int j = 0; j < k; ++j) {
-            cx<T> b((T)beta[2 * j], (T)beta[2 * j + 1]);
-            cx<T> pj = ld<T>(basis + (size_t)j * n + i);
-            v = v - b * pj;
+    for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
+        BasisVec<T> v;
+#pragma unroll
+        for (int e = 0; e < E; ++e) v.c[e] = ld<T>(pk + i + e);
+        if (GM)
+#pragma unroll
+            for (int e = 0; e < E; ++e) v.c[e] = fk * v.c[e];
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            if (j < k) {
+                BasisVec<T> pj;
+                pj.load(basis + (size_t)j * n + i);
+                const cx<T> b(beta[2 * j], beta[2 * j + 1]);
+#pragma unroll
+                for (int e = 0; e < E; ++e) v.c[e] = v.c[e] - b * pj.c[e];
+            }
         }
-        st<T>(pk + i, v);
-        a += norm2(v);
+        if (k > 0) v.store(pk + i);
+#pragma unroll
+        for (int e = 0; e < E; ++e) a += norm2(v.c[e]);
     }
     T acc[1] = {a};
-    grid_reduce<1, T>(acc, R.partials, R.ticket, R.partial_bytes, [&](double (&t)[1]) { R.scal[S_GCR_PN2] = t[0]; });
+    grid_reduce<1, T>(acc, R.partials, R.ticket, R.partial_bytes, [&](double (&t)[1]) {
+        if (GM) {
+            const double nk = sqrt(t[0]);
+            R.scal[rslot(k, k)] = nk;
+            R.scal[rslot(k, k) + 1] = 0.0;
+            R.scal[S_GMRES_F + k] = nk > 0 ? 1.0 / nk : 0.0;
+        } else {
+            R.scal[S_GCR_PN2] = t[0];
+        }
+    });
 }
 template <typename T>
 __global__ void k_gcr_cdot(const v2<T>* __restrict__ basis, const v2<T>* __restrict__ r, size_t n, int k, Reduce R) {
@@ -471,16 +534,39 @@ __global__ void k_gcr_xupdate(double2* x, const v2<T>* __restrict__ Z, size_t n,
     }
 }
 
+// CTAs of the basis passes: what the SMs hold at once (registers: 2 of 256
+// threads in FP64, 3 in FP32), no more than the vector fills
+template <typename T> static int basis_grid(size_t n) {
+    const size_t need = (n / BasisVec<T>::E + kThreads - 1) / kThreads, most = (sizeof(T) == 8 ? 2 : 3) * (size_t)device_sm_count();
+    return (int)std::max<size_t>(1, std::min(need, most));
+}
+template <typename T, bool GM>
+static void multidot_launch(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
+    const int grid = basis_grid<T>(n);
+    note_launch();
+    if (k <= 4) k_gcr_multidot<T, 4, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    else if (k <= 8) k_gcr_multidot<T, 8, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    else if (k <= 16) k_gcr_multidot<T, 16, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    else k_gcr_multidot<T, 32, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+}
+template <typename T, bool GM>
+static void orth_launch(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
+    const int grid = basis_grid<T>(n);
+    note_launch();
+    if (k <= 4) k_gcr_orth_norm<T, 4, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    else if (k <= 8) k_gcr_orth_norm<T, 8, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    else if (k <= 16) k_gcr_orth_norm<T, 16, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    else k_gcr_orth_norm<T, 32, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+}
 template <typename T> void gcr_multidot(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    int grid = reduce_grid(n);
-    if (k <= 4) { note_launch(); k_gcr_multidot<T, 4><<<grid, kThreads, 0, st>>>(basis, n, k, R); }
-    else if (k <= 8) { note_launch(); k_gcr_multidot<T, 8><<<grid, kThreads, 0, st>>>(basis, n, k, R); }
-    else if (k <= 16) { note_launch(); k_gcr_multidot<T, 16><<<grid, kThreads, 0, st>>>(basis, n, k, R); }
-    else { note_launch(); k_gcr_multidot<T, 32><<<grid, kThreads, 0, st>>>(basis, n, k, R); }
+    multidot_launch<T, false>(basis, n, k, R, st);
 }
 template <typename T> void gcr_orth_norm(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    note_launch();
-    k_gcr_orth_norm<T><<<reduce_grid(n), kThreads, 0, st>>>(basis, n, k, R);
+    orth_launch<T, false>(basis, n, k, R, st);
+}
+template <typename T> void gmres_orth(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
+    if (k > 0) multidot_launch<T, true>(basis, n, k, R, st);
+    orth_launch<T, true>(basis, n, k, R, st);
 }
 template <typename T>
 void gcr_cdot(const v2<T>* basis, const v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st) {
@@ -499,22 +585,10 @@ void gcr_xupdate(double2* x, const v2<T>* Z, size_t n, int k, const GcrCoef& y, 
 
 // ================================================================ GMRES(k) smoother
 // One application of GMRES(k) with under-relaxation (Sec. III-IV): Arnoldi
-// vectors basis[0..k] (basis[0] = r / beta), column j of the Hessenberg matrix
-// Hbar in the scalars: h_ij = scal[rslot(i, j+1)] (i <= j) from
-// k_gcr_multidot / k_gcr_orth_norm (one classical Gram-Schmidt pass), and
-// h_{j+1,j} = scal[rslot(j+1, j+1)] written when basis[j+1] is normalised.
-template <typename T> __global__ void k_gmres_normalize(v2<T>* basis, size_t n, int k, const double* __restrict__ in,
-                                                        double* __restrict__ out) {
-    const double nk = sqrt(in[S_GCR_PN2]);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        out[rslot(k, k)] = nk;
-        out[rslot(k, k) + 1] = 0.0;
-    }
-    const T f = (T)(nk > 0 ? 1.0 / nk : 0.0);   // a zero vector stays zero (breakdown: exact in the space)
-    v2<T>* pk = basis + (size_t)k * n;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        st<T>(pk + i, f * ld<T>(pk + i));
-}
+// vectors f_j basis[j] (basis[0] = r, f_j = 1 / |basis[j]|), column j of the
+// Hessenberg matrix Hbar in the scalars: h_ij = scal[rslot(i, j+1)] (i <= j) and
+// h_{j+1,j} = scal[rslot(j+1, j+1)] from one classical Gram-Schmidt pass
+// (gmres_orth).
 // y = argmin || beta e_1 - Hbar y || by Givens rotations (one thread), then
 // scal[S_GCR_C + 2j] = omega y_j.  beta = scal[rslot(0, 0)] (the norm of r,
 // recorded when basis[0] was normalised).  The space ends at the first zero
@@ -523,10 +597,8 @@ constexpr int kGmresMax = 16;   // largest smoother Krylov dimension (mg_params 
 __global__ void k_gmres_ls(double* scal, int k, double omega) {
     // one warp: lane jj owns column jj of the Hessenberg matrix (lane kGmresMax
     // the right-hand side g), so each Givens rotation is applied to all columns at
-    // once with the same arithmetic per column as a serial sweep; the back
-    // substitution runs in lane 0 in the usual order
+    // once with the same arithmetic per column as a serial sweep
     __shared__ double hr[kGmresMax + 1][kGmresMax + 1], hi[kGmresMax + 1][kGmresMax + 1];
-    __shared__ double yr[kGmresMax], yi[kGmresMax];
     __shared__ int s_dim;
     const int lane = threadIdx.x;
     if (blockIdx.x != 0 || lane >= 32 || k > kGmresMax) return;
@@ -557,9 +629,12 @@ __global__ void k_gmres_ls(double* scal, int k, double omega) {
     for (int j = 0; j < dim; ++j) {
         const double ar = hr[j][j], ai = hi[j][j], br = hr[j + 1][j], bi = hi[j + 1][j];
         __syncwarp();
-        const double nrm = sqrt(ar * ar + ai * ai + br * br + bi * bi);
-        if (nrm > 0 && col >= 0 && (col >= j)) {
-            const double cr = ar / nrm, ci = ai / nrm, sr = br / nrm, si = bi / nrm;
+        const double n2 = ar * ar + ai * ai + br * br + bi * bi;
+        if (n2 > 0 && col >= 0 && (col >= j)) {
+            // one reciprocal square root per rotation: FP64 divisions and roots are
+            // long chains on this part's narrow FP64 pipe
+            const double inv = rsqrt(n2);
+            const double cr = ar * inv, ci = ai * inv, sr = br * inv, si = bi * inv;
             // [conj(c) conj(s); -s c] applied to rows j, j+1
             const double x1r = hr[j][col], x1i = hi[j][col], x2r = hr[j + 1][col], x2i = hi[j + 1][col];
             hr[j][col] = cr * x1r + ci * x1i + sr * x2r + si * x2i;
@@ -569,47 +644,70 @@ __global__ void k_gmres_ls(double* scal, int k, double omega) {
         }
         __syncwarp();
     }
-    if (lane == 0) {
-        for (int i = dim - 1; i >= 0; --i) {
-            double ar = hr[i][kGmresMax], ai = hi[i][kGmresMax];
-            for (int jj = i + 1; jj < dim; ++jj) {
-                ar -= hr[i][jj] * yr[jj] - hi[i][jj] * yi[jj];
-                ai -= hr[i][jj] * yi[jj] + hi[i][jj] * yr[jj];
-            }
-            const double dr = hr[i][i], di = hi[i][i], dd = dr * dr + di * di;
-            yr[i] = dd > 0 ? (ar * dr + ai * di) / dd : 0.0;
-            yi[i] = dd > 0 ? (ai * dr - ar * di) / dd : 0.0;
+    // back substitution by columns: lane i keeps row i's right-hand side and the
+    // reciprocal of its diagonal; once y_j is known every row above subtracts it
+    double gr = 0.0, gi = 0.0, dr = 0.0, di = 0.0, yr = 0.0, yi = 0.0;
+    if (lane < dim) {
+        gr = hr[lane][kGmresMax];
+        gi = hi[lane][kGmresMax];
+        dr = hr[lane][lane];
+        di = hi[lane][lane];
+        const double dd = dr * dr + di * di, inv = dd > 0 ? 1.0 / dd : 0.0;
+        dr *= inv;
+        di *= -inv;
+    }
+    for (int j = dim - 1; j >= 0; --j) {
+        if (lane == j) {
+            yr = gr * dr - gi * di;
+            yi = gr * di + gi * dr;
+        }
+        const double tr = __shfl_sync(0xffffffffu, yr, j), ti = __shfl_sync(0xffffffffu, yi, j);
+        if (lane < j) {
+            gr -= hr[lane][j] * tr - hi[lane][j] * ti;
+            gi -= hr[lane][j] * ti + hi[lane][j] * tr;
         }
     }
-    __syncwarp();
-    for (int j = lane; j < k; j += 32) {
-        scal[S_GCR_C + 2 * j] = j < dim ? omega * yr[j] : 0.0;
-        scal[S_GCR_C + 2 * j + 1] = j < dim ? omega * yi[j] : 0.0;
+    if (lane < k) {
+        scal[S_GCR_C + 2 * lane] = lane < dim ? omega * yr : 0.0;
+        scal[S_GCR_C + 2 * lane + 1] = lane < dim ? omega * yi : 0.0;
     }
 }
-// z += sum_{j<k} c_j basis[j], c_j = scal[S_GCR_C + 2j]
-template <typename T>
-__global__ void k_multi_axpy(v2<T>* z, const v2<T>* __restrict__ basis, size_t n, int k, const double* __restrict__ scal) {
-    __shared__ double c[2 * K_MAX];
-    for (int j = threadIdx.x; j < 2 * k; j += blockDim.x) c[j] = scal[S_GCR_C + j];
+// z += sum_{j<k} c_j f_j basis[j], c_j = scal[S_GCR_C + 2j], f_j = scal[S_GMRES_F + j]
+template <typename T, int NJ>
+__global__ void __launch_bounds__(kThreads) k_multi_axpy(v2<T>* z, const v2<T>* __restrict__ basis, size_t n, int k,
+                                                         const double* __restrict__ scal) {
+    constexpr int E = BasisVec<T>::E;
+    __shared__ T c[2 * NJ];
+    for (int j = threadIdx.x; j < k; j += blockDim.x) {
+        const double f = scal[S_GMRES_F + j];
+        c[2 * j] = (T)(f * scal[S_GCR_C + 2 * j]);
+        c[2 * j + 1] = (T)(f * scal[S_GCR_C + 2 * j + 1]);
+    }
     __syncthreads();
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        cx<T> v = ld<T>(z + i);
-        for (int j = 0; j < k; ++j) cmad(v, cx<T>((T)c[2 * j], (T)c[2 * j + 1]), ld<T>(basis + (size_t)j * n + i));
-        st<T>(z + i, v);
+    for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
+        BasisVec<T> v;
+#pragma unroll
+        for (int e = 0; e < E; ++e) v.c[e] = ld<T>(z + i + e);
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+            if (j < k) {
+                BasisVec<T> pj;
+                pj.load(basis + (size_t)j * n + i);
+#pragma unroll
+                for (int e = 0; e < E; ++e) cmad(v.c[e], cx<T>(c[2 * j], c[2 * j + 1]), pj.c[e]);
+            }
+        v.store(z + i);
     }
-}
-template <typename T> void gmres_normalize(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    note_launch();
-    k_gmres_normalize<T><<<stream_grid(n), kThreads, 0, st>>>(basis, n, k, R.scal, R.scal);
 }
 void gmres_ls(const Reduce& R, int k, double omega, cudaStream_t st) {
     note_launch();
     k_gmres_ls<<<1, 32, 0, st>>>(R.scal, k, omega);
 }
 template <typename T> void multi_axpy(v2<T>* z, const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
+    const int grid = basis_grid<T>(n);
     note_launch();
-    k_multi_axpy<T><<<stream_grid(n), kThreads, 0, st>>>(z, basis, n, k, R.scal);
+    if (k <= 8) k_multi_axpy<T, 8><<<grid, kThreads, 0, st>>>(z, basis, n, k, R.scal);
+    else k_multi_axpy<T, kGmresMax><<<grid, kThreads, 0, st>>>(z, basis, n, k, R.scal);
 }
 
 // ================================================================ instantiations
@@ -631,7 +729,7 @@ template <typename T> void multi_axpy(v2<T>* z, const v2<T>* basis, size_t n, in
     template void gcr_cdot<T>(const v2<T>*, const v2<T>*, size_t, int, const Reduce&, cudaStream_t);                \
     template void gcr_update<T>(v2<T>*, v2<T>*, size_t, int, const Reduce&, cudaStream_t);                          \
     template void gcr_xupdate<T>(double2*, const v2<T>*, size_t, int, const GcrCoef&, cudaStream_t);          \
-    template void gmres_normalize<T>(v2<T>*, size_t, int, const Reduce&, cudaStream_t);                        \
+    template void gmres_orth<T>(v2<T>*, size_t, int, const Reduce&, cudaStream_t);                             \
     template void multi_axpy<T>(v2<T>*, const v2<T>*, size_t, int, const Reduce&, cudaStream_t);
 INST(float)
 INST(double)

@@ -253,11 +253,10 @@ __global__ void __launch_bounds__(kHalfThreads) k_h_multidot(const uint2* __rest
     __shared__ float fac[K_MAX];   // basis j < k is normalised through its stored norm
     for (int j = threadIdx.x; j < k && j < K_MAX; j += blockDim.x) fac[j] = inv_norm(R.scal + S_GMRES_F + j);
     __syncthreads();
-    const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     float a[2 * NJ];
 #pragma unroll
     for (int j = 0; j < 2 * NJ; ++j) a[j] = 0.f;
-    if (s < g.V) {
+    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < g.V; s += (long long)gridDim.x * blockDim.x) {
         const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
         const size_t self6 = (size_t)X * 6 * g.Vb + l, V6 = (size_t)6 * g.V;
         cx<float> w[12];
@@ -267,7 +266,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_h_multidot(const uint2* __rest
             if (j < k) {
                 cx<float> v[12];
                 ld_site_h(B + (size_t)j * V6 + self6, S[(size_t)j * g.V + s] * fac[j], g.Vb, v);
-                cx<float> t(0.f, 0.f);
+                cx<float> t(a[2 * j], a[2 * j + 1]);
 #pragma unroll
                 for (int q = 0; q < 12; ++q) cmadc(t, v[q], w[q]);
                 a[2 * j] = t.r;
@@ -382,11 +381,14 @@ void dslash_h_mrdot(HalfSpinor out, ConstHalfSpinor in, const uint2* U16, const 
 }
 void h_multidot(const uint2* B, const float* S, const Geom& g, int k, const Reduce& R, cudaStream_t st) {
     note_launch();
-    // one block per 128 sites, 2 NJ <= 32 float partial sums each: the context
-    // sizes the reduction buffer for V / 128 such blocks (reduce_partial_bytes)
-    if (k <= 4) k_h_multidot<4><<<half_grid(g.V), kHalfThreads, 0, st>>>(B, S, g, k, R);
-    else if (k <= 8) k_h_multidot<8><<<half_grid(g.V), kHalfThreads, 0, st>>>(B, S, g, k, R);
-    else k_h_multidot<16><<<half_grid(g.V), kHalfThreads, 0, st>>>(B, S, g, k, R);
+    // at most the CTAs that the SMs hold at once, with equal numbers of sites: each
+    // ends with a reduction of up to 32 sums, and the last one adds all of them
+    const long long need = half_grid(g.V), most = 4LL * device_sm_count();
+    const int grid = (int)((need + (need + most - 1) / most - 1) / ((need + most - 1) / most));
+    if (k <= 4) k_h_multidot<4><<<grid, kHalfThreads, 0, st>>>(B, S, g, k, R);
+    else if (k <= 8) k_h_multidot<8><<<grid, kHalfThreads, 0, st>>>(B, S, g, k, R);
+    else if (k <= 12) k_h_multidot<12><<<grid, kHalfThreads, 0, st>>>(B, S, g, k, R);
+    else k_h_multidot<16><<<grid, kHalfThreads, 0, st>>>(B, S, g, k, R);
 }
 void h_orth(uint2* B, float* S, const Geom& g, int k, const Reduce& R, cudaStream_t st) {
     note_launch();

@@ -174,30 +174,45 @@ __device__ __forceinline__ void block_reduce(double (&v)[N], double (*sh)[32]) {
     }
 }
 
-template <typename TA> __device__ __forceinline__ TA warp_sum_acc(TA v) {
+__host__ __device__ constexpr int pow2_ceil(int n) { return n <= 1 ? 1 : 2 * pow2_ceil((n + 1) / 2); }
+
+// Sums over the warp of P values per lane (P a power of two, <= 32), all at
+// once: each step exchanges the half of the values that the lane gives up for
+// the half that it keeps, so P values take P - 1 + log2(32 / P) shuffles instead
+// of 5 P.  Lane l returns the sum of value l / (32 / P).
+template <int P, typename TA> __device__ __forceinline__ TA warp_sums(TA (&v)[P]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-// Block-reduce N values of type TA; result valid in thread 0.
-template <int N, typename TA>
-__device__ __forceinline__ void block_reduce_acc(TA (&v)[N], TA (*sh)[32]) {
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int h = P / 2; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
 #pragma unroll
-    for (int k = 0; k < N; ++k) v[k] = warp_sum_acc(v[k]);
-    __syncthreads();
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) sh[k][warp] = v[k];
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            TA x = lane < nw ? sh[k][lane] : TA(0);
-            v[k] = warp_sum_acc(x);
+        for (int i = 0; i < h; ++i) {
+            const TA send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
+    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+// Block sums of N <= 64 values: the result of value t in thread t < N.  sh: one
+// array of 32 per value of the padded count.
+template <int N, typename TA> __device__ __forceinline__ TA block_sums(const TA (&v)[N], TA (*sh)[32]) {
+    constexpr int P = pow2_ceil(N) > 32 ? 32 : pow2_ceil(N);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int k0 = 0; k0 < N; k0 += P) {
+        TA w[P];
+#pragma unroll
+        for (int k = 0; k < P; ++k) w[k] = k0 + k < N ? v[k0 + k] : TA(0);
+        const TA a = warp_sums<P, TA>(w);
+        if ((lane & (32 / P - 1)) == 0) sh[k0 + lane / (32 / P)][warp] = a;
+    }
+    __syncthreads();
+    TA a = TA(0);
+    if ((int)threadIdx.x < N)
+        for (int w = 0; w < nw; ++w) a += sh[threadIdx.x][w];
+    return a;
 }
 
 // Smallest partial-sum buffer of the grid reductions (Reduce::partials); a
@@ -224,32 +239,54 @@ __device__ __forceinline__ void grid_reduce(TA (&v)[N], double* partials, unsign
         }
         return;
     }
-    __shared__ TA sh[N][32];
+    // threads t < N hold the block's sums; the last block reads the partial sums of
+    // all blocks with consecutive threads on consecutive values, 32 / P2 or more
+    // blocks at a time (one thread per value and a strided walk over the blocks
+    // made this tail longer than the pass itself for 26 values and 1216 blocks)
+    constexpr int P2 = pow2_ceil(N);
+    __shared__ TA sh[P2][32];
+    __shared__ double tot[N];
     __shared__ bool is_last;
-    block_reduce_acc<N, TA>(v, sh);
+    const TA mine = block_sums<N, TA>(v, sh);
     TA* part = reinterpret_cast<TA*>(partials);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) part[(size_t)blockIdx.x * N + k] = v[k];
+    if ((int)threadIdx.x < N) {
+        part[(size_t)blockIdx.x * N + threadIdx.x] = mine;
         __threadfence();
+    }
+    if (N > 32) __syncthreads();
+    else __syncwarp();
+    if (threadIdx.x == 0) {
         unsigned int t = atomicAdd(ticket, 1u);
         is_last = (t == gridDim.x - 1);
     }
     __syncthreads();
     if (!is_last) return;
     __threadfence();
-    TA acc[N];
+    const int k = threadIdx.x % P2, nch = max((int)blockDim.x / P2, 1);
+    TA acc[4] = {TA(0), TA(0), TA(0), TA(0)};
+    if (k < N) {
+        int b = threadIdx.x / P2;
+        for (; b + 3 * nch < (int)gridDim.x; b += 4 * nch)
 #pragma unroll
-    for (int k = 0; k < N; ++k) acc[k] = TA(0);
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) acc[k] += __ldcg(part + (size_t)b * N + k);
+            for (int q = 0; q < 4; ++q) acc[q] += __ldcg(part + (size_t)(b + q * nch) * N + k);
+        for (; b < (int)gridDim.x; b += nch) acc[0] += __ldcg(part + (size_t)b * N + k);
     }
-    block_reduce_acc<N, TA>(acc, sh);
+    TA a = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    for (int o = 16; o >= P2; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    // one row of sums per warp, or per P2 threads when a row is wider than a warp
+    const int row = P2 <= 32 ? (int)threadIdx.x >> 5 : (int)threadIdx.x / P2, nrow = P2 <= 32 ? (int)blockDim.x >> 5 : nch;
+    if (P2 > 32 || (int)(threadIdx.x & 31) < P2) sh[k][row] = a;
+    __syncthreads();
+    if ((int)threadIdx.x < N) {
+        TA t = TA(0);
+        for (int w = 0; w < nrow; ++w) t += sh[threadIdx.x][w];
+        tot[threadIdx.x] = (double)t;
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
         double t[N];
 #pragma unroll
-        for (int k = 0; k < N; ++k) t[k] = (double)acc[k];
+        for (int q = 0; q < N; ++q) t[q] = tot[q];
         fin(t);
         *ticket = 0u;
     }

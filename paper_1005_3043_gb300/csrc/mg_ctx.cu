@@ -674,17 +674,14 @@ int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt
         dslash<T>(DS_XMY, V, z, U, r, ctx->g, ctx->mass, 0.0, 0, Rs, ctx->st);
         PROF_END(MG_K_DSLASH);
         PROF_BEGIN(MG_K_KRYLOV);
-        norm2<T>(V, n, S_GCR_PN2, Rs, ctx->st);
-        gmres_normalize<T>(V, n, 0, Rs, ctx->st);
+        gmres_orth<T>(V, n, 0, Rs, ctx->st);
         PROF_END(MG_K_KRYLOV);
         for (int j = 0; j < steps; ++j) {
             PROF_BEGIN(MG_K_DSLASH);
             dslash<T>(DS_PLAIN, V + (size_t)(j + 1) * n, V + (size_t)j * n, U, V, ctx->g, ctx->mass, 0.0, 0, Rs, ctx->st);
             PROF_END(MG_K_DSLASH);
             PROF_BEGIN(MG_K_KRYLOV);
-            gcr_multidot<T>(V, n, j + 1, Rs, ctx->st);
-            gcr_orth_norm<T>(V, n, j + 1, Rs, ctx->st);
-            gmres_normalize<T>(V, n, j + 1, Rs, ctx->st);
+            gmres_orth<T>(V, n, j + 1, Rs, ctx->st);
             PROF_END(MG_K_KRYLOV);
         }
         PROF_BEGIN(MG_K_KRYLOV);
@@ -838,13 +835,10 @@ template <typename T> int smooth_l1(mg_ctx* ctx, const v2<T>* r1, v2<T>* z, int 
     coarse_apply<T>(V, A1, z, ctx->full.nc, false, -1, ctx->g, Rs, ctx->st);   // v_0 = r1 - D_c z
     scale<T>(V, n1, -1.0, ctx->st);
     axpy<T>(V, r1, n1, 1.0, 0.0, ctx->st);
-    norm2<T>(V, n1, S_GCR_PN2, Rs, ctx->st);
-    gmres_normalize<T>(V, n1, 0, Rs, ctx->st);
+    gmres_orth<T>(V, n1, 0, Rs, ctx->st);
     for (int j = 0; j < k; ++j) {
         coarse_apply<T>(V + (size_t)(j + 1) * n1, A1, V + (size_t)j * n1, ctx->full.nc, false, -1, ctx->g, Rs, ctx->st);
-        gcr_multidot<T>(V, n1, j + 1, Rs, ctx->st);
-        gcr_orth_norm<T>(V, n1, j + 1, Rs, ctx->st);
-        gmres_normalize<T>(V, n1, j + 1, Rs, ctx->st);
+        gmres_orth<T>(V, n1, j + 1, Rs, ctx->st);
     }
     gmres_ls(Rs, k, ctx->prm.omega, ctx->st);
     multi_axpy<T>(z, V, n1, k, Rs, ctx->st);
