@@ -185,8 +185,8 @@ def batched_leg(wmg, torch, stream, prec, name="wilson_24x24x24x64_nv24_beta6_76
     """Many right-hand sides on the 24^3 x 64 workload (Nv = 24, 48 coarse dof):
     12 spin-colour point sources at the origin + 64 Gaussian sources in one
     batched solve (lockstep flexible GCR(8), the coarse solve of all sources
-    one CGLS on an RHS panel with the tensor-core stencil, its iterations
-    replayed from a CUDA graph), against n_single of the same sources solved
+    one CG on an RHS panel with the tensor-core stencil, one persistent
+    launch), against n_single of the same sources solved
     one at a time (the single-source path, on-chip or persistent coarse CG).
     Setup once at the workload's mass; both timed with CUDA events."""
     import synth
@@ -246,13 +246,13 @@ def batched_leg(wmg, torch, stream, prec, name="wilson_24x24x24x64_nv24_beta6_76
     except Exception:
         pass
     hbm, bf16 = peaks.get("hbm_gbs", 6800.0), peaks.get("bf16_tflops", 1900.0)
-    out["tc_stencil"] = {"kernel": "k_coarse_apply_tc", "columns": n, "us": 1e3 * tc_ms,
+    out["tc_stencil"] = {"kernel": "k_bcg (one stencil)", "columns": n, "us": 1e3 * tc_ms,
                          "bytes": tc_bytes, "GB/s": tc_bytes / (tc_ms * 1e-3) / 1e9,
                          "hbm_frac": tc_bytes / (tc_ms * 1e-3) / 1e9 / hbm,
                          "useful_TFLOP/s": tc_flops / (tc_ms * 1e-3) / 1e12,
                          "tensor_frac": tc_flops / (tc_ms * 1e-3) / 1e12 / bf16,
-                         "note": "bound by streaming the FP16 embedded operator (9 x (2Nv x 2)^2 halves per aggregate, "
-                                 "larger than L2); useful flops exclude the padding of M to 128 and the hi/lo "
+                         "note": "bound by streaming the FP16 operator (9 x (2Nv)^2 complex halves per aggregate) "
+                                 "and the panel, which the launch first turns into FP16 tiles; useful flops exclude the padding of M to 128 and the hi/lo "
                                  "split; peaks of MEASURED_PEAKS.json (HBM copy, bf16 burst)"}
     return out
 
@@ -271,7 +271,7 @@ def coarse_tc_probe(nrhs=64, reps=20):
     mg.setup(V0)
     ms, nb, fl = mg.time_coarse_batched(nrhs, reps)
     mg.close()
-    print(json.dumps({"kernel": "k_coarse_apply_tc", "workload": w.name, "columns": nrhs, "us": 1e3 * ms,
+    print(json.dumps({"kernel": "k_bcg (one stencil)", "workload": w.name, "columns": nrhs, "us": 1e3 * ms,
                       "GB/s": nb / (ms * 1e-3) / 1e9, "useful_TFLOP/s": fl / (ms * 1e-3) / 1e12}), flush=True)
 
 

@@ -281,8 +281,8 @@ int mg_solve_device(mg_ctx* ctx, const double* b_dev, double* x_dev, mg_solve_in
  * with its own Krylov space and scalars, the fine-level steps per source and
  * the coarse solve of all sources as one batched CGNR on an RHS panel, its
  * stencil a dense contraction on the tensor cores (FP16 operator, FP16 hi+lo
- * panel, FP32 accumulation), its iterations replayed from a captured CUDA
- * graph.  b, x: nrhs consecutive host fine spinors; info: nrhs entries.
+ * panel, FP32 accumulation), the whole CG one persistent launch.
+ * b, x: nrhs consecutive host fine spinors; info: nrhs entries.
  * Needs prec_inner MG_FP32 or MG_FP16 (the smoother then follows the FP16
  * storage rules of mg_params.smoother_fp16) and 2*nvec a multiple of 16
  * (<= 128), nrhs <= 256; with MG_FP64 the sources are solved one after
@@ -319,9 +319,9 @@ int mg_solve_eo_cg_device(mg_ctx* ctx, const double* b_dev, double* x_dev, doubl
 
 /* Timing of the tensor-core batched coarse stencil (measurement hook, no
  * counterpart in the paper): `reps` launches of y = D_c x on a device panel of
- * nrhs columns (the chunk width from the autotuner), CUDA events on the
+ * nrhs columns, CUDA events on the
  * context stream; *ms_per_launch, and per launch the algorithmic bytes (the
- * FP16 embedded operator once, the FP32 panel read and written once) and the
+ * FP16 operator once, the FP32 panel read and written once) and the
  * useful flops (8 per complex multiply-add of D_c x_n).  Allocates and frees
  * two panels.  Same shape limits as mg_apply_coarse_batched with impl 0. */
 int mg_time_coarse_batched(mg_ctx* ctx, int nrhs, int reps, double* ms_per_launch, double* bytes_per_launch,

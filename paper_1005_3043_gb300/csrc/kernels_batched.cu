@@ -1,326 +1,831 @@
-// Batched (multi right-hand side) coarse level: the coarse stencil applied to
-// an RHS panel on the 5th-generation tensor cores, and the per-RHS CGNR steps.
+// Batched (multi right-hand side) coarse level: CG on the normal equations of
+// D_c for a panel of right-hand sides, whole solve in one persistent cooperative
+// launch, the stencil a dense contraction on the 5th-generation tensor cores.
 //
-// Panel layout: xB[X][b][n] complex FP32, n < npad (RHS index fastest, npad a
-// multiple of 16).  For one aggregate X the stencil is a dense contraction
-//   y[X][a][n] = sum_d sum_b A[X][d][a][b] x[X+d][b][n],
-// written as a real GEMM through the embedding
-//   [Re y]   [Re A  -Im A] [Re x]
-//   [Im y] = [Im A   Re A] [Im x]      (M = K = 2 nc per direction d),
-// M padded to 128, K = 9 * 2nc, N = npad.  A is stored once per (X, d) in
-// FP16 in the tensor-core shared-memory layout and copied with the bulk-copy
-// engine; x is split into FP16 hi + lo parts (x = hi + lo to ~22 bits) so two
-// MMAs per K step give an FP32-accurate product against the FP16 operator.
+// Panel layout: xB[X][b][n] complex FP32, n < npad (RHS index fastest).  For one
+// aggregate X the stencil is
+//   y[X][a][n] = sum_d sum_b A[X][d][a][b] x[X+d][b][n].
+// As a real GEMM the rows are the real parts of A followed by the imaginary
+// parts (M = 2 nc <= 96 of the MMA's 128), K = b, and a right-hand side is four
+// columns: Re x and Im x, each split into FP16 hi + lo (x = hi + lo to ~22 bits):
+//   D[a] = Re A x, D[nc + a] = Im A x,
+//   Re y = D[a][Re] - D[nc + a][Im],  Im y = D[a][Im] + D[nc + a][Re].
+// So neither the operator nor the operand is stored twice (the embedding
+// [[Re, -Im], [Im, Re]] doubles the operator's bytes and its MMAs): at 16^3x32
+// (Nv = 20) an aggregate's stencil reads 58 KB of operator and takes 27 MMAs of
+// 128 x 64 x 16 for 16 right-hand sides.
+//
+// The operand is kept in global memory as FP16 tiles in the tensor-core layout,
+// written once by the CTA that owns the aggregate when it computes the entries
+// (scaled by a power of two per right-hand side from the last known norm), so a
+// stencil only moves tiles: per direction one bulk copy of A[X][d] and one of the
+// tile of x[X+d].
+//
+// Iteration: the Chronopoulos-Gear arrangement of CG on D_c^dag D_c (as the
+// single-source solver): phase A u = D_c s, one exchange of (|u|^2, |s|^2, |r|^2)
+// per right-hand side, phase B w = D_c^dag u and, in its epilogue,
+//   p = s + beta p, z = w + beta z, q = u + beta q, y += alpha p, r -= alpha q,
+//   s -= alpha z,
+// two grid barriers per iteration.  Separate kernels for the split, the stencil,
+// the reductions and the updates (ten launches per iteration, replayed from a
+// graph) took 76 us per iteration on 16^3x32 with 12 sources (Nv = 16), 34 us of it
+// in each stencil, and 64 us on 8^3x16 with 21 sources, all latency; this kernel
+// takes 25 and 14 us.  What is left: about 1.2 us per job (copies, 18 MMAs and the
+// epilogue overlap), 3 us per grid barrier.
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <mutex>
-#include <vector>
 
 #include "mg_launch.h"
 #include "mg_ptx.cuh"
 
 namespace wmg {
 
-// half offset of element (row r, k) in a K-major core-matrix tile with K columns
-__host__ __device__ __forceinline__ int core_off(int r, int k, int K) {
-    return (((r >> 3) * (K >> 3) + (k >> 3)) << 6) + ((r & 7) << 3) + (k & 7);
+// ---------------------------------------------------------------- operator tiles
+// At[X][d][kc][rg][8][8]: core matrices (8 rows x 8 K, 128 bytes) of one K group
+// kc adjacent over the row groups rg; row a the real part of row a of A, row
+// nc + a the imaginary part.
+__global__ void k_coarse_tiles(__half* At, const double2* __restrict__ A, int nc, long long nblk) {
+    const long long total = nblk * nc * nc;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+        const long long blk = i / (nc * nc);
+        const int rem = (int)(i - blk * nc * nc), b = rem / nc, a = rem - b * nc;
+        const double2 v = A[i];   // column-major block: A[b][a] = A_ab
+        __half* t = At + blk * 2 * nc * nc + (size_t)(b >> 3) * (nc >> 2) * 64 + (b & 7);
+        const int m = nc + a;
+        t[((a >> 3) << 6) + ((a & 7) << 3)] = __double2half(v.x);
+        t[((m >> 3) << 6) + ((m & 7) << 3)] = __double2half(v.y);
+    }
 }
-
-// ---------------------------------------------------------------- operator embedding
-// Aemb[X][d]: 2nc x 2nc FP16 real embedding of A[X][d] in the core-matrix layout
-// (rows 2nc..127 of the 128-row MMA tile are zero in shared memory only).
-__global__ void k_coarse_embed(__half* Aemb, const double2* __restrict__ A, int nc, long long nblk) {
-    const int K = 2 * nc;
-    long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    long long total = nblk * K * K;
-    if (idx >= total) return;
-    long long blk = idx / (K * K);
-    int rem = (int)(idx - blk * K * K);
-    int m = rem / K, k = rem - m * K;
-    int a = m % nc, b = k % nc;
-    bool imr = m >= nc, imc = k >= nc;
-    double2 v = A[blk * nc * nc + (size_t)b * nc + a];   // column-major block: A[b][a] = A_ab
-    double e = (!imr && !imc) ? v.x : (!imr && imc) ? -v.y : (imr && !imc) ? v.y : v.x;
-    Aemb[blk * K * K + core_off(m, k, K)] = __double2half(e);
-}
-
-void coarse_embed(__half* Aemb, const double2* A, int nc, int Vc, cudaStream_t st) {
-    long long nblk = (long long)Vc * 9;
-    long long total = nblk * 4 * nc * nc;
+void coarse_tiles(__half* At, const double2* A, int nc, int Vc, cudaStream_t st) {
+    const long long total = (long long)Vc * 9 * nc * nc;
     note_launch();
-    k_coarse_embed<<<(int)((total + 255) / 256), 256, 0, st>>>(Aemb, A, nc, nblk);
+    k_coarse_tiles<<<(int)std::min<long long>((total + 255) / 256, 32LL * device_sm_count()), 256, 0, st>>>(
+        At, A, nc, (long long)Vc * 9);
 }
 
-// ---------------------------------------------------------------- tensor-core batched stencil
-constexpr int kTcThreads = 128;
-constexpr int kTcMaxStages = 3;   // pipeline depth when it fits shared memory, else 2
-constexpr long long kTcWaitLimit = 20000000LL;
+// ---------------------------------------------------------------- the persistent kernel
+// Warps: 0 copies the operator's tiles and 1 the operand's, a lane per direction; 2
+// and 3 issue the MMAs of every second job each (lane 0); 4..11 the epilogue.  One
+// thread for all copies and one for all MMAs were the pipeline's rate: 2.5 us per
+// job at 16^3x32, 12 sources.
+constexpr int kEpiWarps = 8, kEpi = 32 * kEpiWarps, kEpi0 = 128, kBcgThreads = kEpi0 + kEpi;
+constexpr int kBcgMaxStages = 16;
+constexpr long long kBcgWait = 20000000LL;    // polls of a wait before it gives up
+constexpr int kBcgStatic = 1024;              // barriers, flags
 
-__host__ __device__ inline int tc_tmem_cols(int npad) {
-    int c = 32;
-    while (c < npad) c <<= 1;
-    return c;
-}
-// one pipeline stage: the (padded) 128-row A tile, the hi and lo B tiles
-__host__ __device__ inline size_t tc_stage_bytes(int nc, int nw) {
-    const size_t K = 2 * nc;
-    return 128 * K * 2 + 2 * (size_t)nw * K * 2;
-}
-constexpr size_t kTcStaticSmem = 256;   // barriers, TMEM address, flag
-__host__ __device__ inline int tc_stages(int nc, int nw) {
-    return kTcMaxStages * tc_stage_bytes(nc, nw) + kTcStaticSmem <= 227 * 1024 ? kTcMaxStages : 2;
-}
-__host__ __device__ inline int tc_stages_of(const TcApplyArgs& a) { return a.stages > 0 ? a.stages : tc_stages(a.nc, a.nw); }
+// shared memory of a shape: stages of (operator, operand) tiles, then T (the
+// products of one job), S2 (entries on their way into the tile), the column
+// sums and the per-column scalars
+struct BcgSmem {
+    int kcp;            // K groups of a stage (nc / 8 rounded up to even, the last one zero)
+    uint32_t a_bytes, b_bytes, stage, a_copy, b_copy;
+    size_t off_t, off_s2, off_acc, off_col, total;
+    int ts, rgs;
+    __host__ __device__ BcgSmem(int nc, int nw, int npad, int stages) {
+        kcp = ((nc >> 3) + 1) & ~1;
+        a_copy = (uint32_t)nc * nc * 4;            // (nc / 8) x (2 nc x 8) halves
+        b_copy = (uint32_t)nc * nw * 8;            // (nc / 8) x (4 nw x 8) halves
+        a_bytes = (uint32_t)kcp * nc * 32;
+        b_bytes = (uint32_t)kcp * nw * 64;
+        if (b_bytes < 2048) b_bytes = 2048;        // the 128-row MMA reads up to 1.8 KB past the operator rows
+        stage = a_bytes + b_bytes;
+        ts = nw + 1;
+        rgs = kEpi / nw;
+        off_t = (size_t)stages * stage;
+        off_s2 = off_t + (size_t)2 * nc * ts * 8;
+        off_acc = off_s2 + (size_t)nc * ts * 8;
+        off_col = off_acc + (size_t)3 * rgs * npad * 8;
+        off_col = (off_col + 15) & ~(size_t)15;
+        total = off_col + (size_t)npad * (3 * 8 + 12 * 4);
+    }
+};
 
-// The operand panel as FP16 hi + lo tiles in the tensor-core shared-memory
-// layout, one tile pair per (aggregate Y, column chunk c):
-//   bt[((Y * nch + c) * 2 + {0 hi, 1 lo}) * nw * K + core_off(n, k, K)],
-// k = b (real part) or nc + b (imaginary part) of x[Y][b][c * nw + n], with the
-// column scale and, for the adjoint, the sigma3 sign of rows b >= nc/2 applied.
-// One thread per (Y, c, n, 8-column group of k): two 16-byte stores.
-__global__ void k_tc_split(__half* __restrict__ bt, const float2* __restrict__ x, int nc, int npad, int nw, int dag,
-                           const double* __restrict__ colscale, long long total) {
-    const int K = 2 * nc, kg8 = K >> 3, nch = npad / nw, nvh = nc >> 1;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int kg = (int)(i % kg8);
-        long long t = i / kg8;
-        const int n = (int)(t % nw);
-        t /= nw;
-        const int c = (int)(t % nch);
-        const long long Y = t / nch;
-        const int col = c * nw + n;
-        const float sc = colscale ? (float)colscale[col] : 1.f;
-        __align__(16) __half hi[8], lo[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int k = kg * 8 + e, b = k < nc ? k : k - nc;
-            const float2 v = x[((size_t)Y * nc + b) * npad + col];
-            float f = (k < nc ? v.x : v.y) * sc;
-            if (dag && b >= nvh) f = -f;
-            const __half h = __float2half_rn(f);
-            hi[e] = h;
-            lo[e] = __float2half_rn(f - __half2float(h));
+__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// barrier of the epilogue warps; the return value is the OR of p over them
+__device__ __forceinline__ bool epi_sync(bool p = false) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(r)
+        : "r"((uint32_t)p), "n"(kEpi)
+        : "memory");
+    return r != 0;
+}
+// 8 consecutive FP32 columns of this thread's TMEM lane; tmem_wait_ld before use
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+// waits for this thread's loads; the registers pass through, so that no use of
+// them moves above the wait
+__device__ __forceinline__ void tmem_wait_ld8(uint32_t (&a)[8], uint32_t (&b)[8], uint32_t (&c)[8], uint32_t (&d)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+                   "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
+                 :
+                 : "memory");
+    asm volatile(""
+                 : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6]), "+r"(c[7]),
+                   "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7])
+                 :
+                 : "memory");
+}
+// wait for a phase of an mbarrier: false when the CTA's fail flag is up or the
+// poll limit is reached (the flag and the launch's error flag are then raised)
+__device__ __forceinline__ bool bcg_wait(uint64_t* bar, uint32_t parity, volatile int* fail, int* err) {
+    for (long long i = 0; i < kBcgWait; ++i) {
+        if (mbar_try_wait(bar, parity)) return true;
+        if ((i & 63) == 63) {
+            if (*fail) return false;
+            __nanosleep(20);
         }
-        __half* base = bt + ((size_t)(Y * nch + c) * 2) * nw * K + core_off(n, kg * 8, K);
-        *reinterpret_cast<uint4*>(base) = *reinterpret_cast<const uint4*>(hi);
-        *reinterpret_cast<uint4*>(base + (size_t)nw * K) = *reinterpret_cast<const uint4*>(lo);
     }
+    *fail = 1;
+    atomicExch(err, 1);
+    return false;
+}
+// sum in two floats (Knuth's two-sum): the column sums run over many aggregates
+// and CTAs, and FP64 adds are two per clock and SM here
+struct Sum2 {
+    float h, l;
+};
+__device__ __forceinline__ void add2(Sum2& s, float x) {
+    const float t = s.h + x, b = t - s.h;
+    s.l += (s.h - (t - b)) + (x - b);
+    s.h = t;
+}
+// power of two near sqrt(rows / s): entries of a column with |x|^2 = s then have
+// rms about 1, far above the FP16 subnormal range, with room for a column
+// concentrated on one site
+__device__ __forceinline__ float col_scale(double s, float rows) {
+    const float x = rows / (float)s;
+    if (!(x > 1e-38f) || !(x < 1e38f)) return 1.f;
+    return __int_as_float((127 + ((((__float_as_int(x) >> 23) & 255) - 127) >> 1)) << 23);
+}
+__device__ __forceinline__ uint32_t half_pair(float a, float b) {
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// One CTA per (aggregate X, column chunk of width nw).  Thread 0 runs a
-// pipeline of 3 (or, where shared memory is short, 2) stages over the 9
-// directions d: the bulk-copy engine brings
-// A_emb[X][d] and the hi/lo tiles of x[X+d] (split beforehand by k_tc_split)
-// into a stage, thread 0 issues the MMAs (hi and lo per K step) into the TMEM
-// accumulator (128 lanes = embedded rows, nw columns = right-hand sides) and
-// commits them to the stage's "empty" barrier; a stage is refilled once its
-// MMAs are done.  Then the four warps read the accumulator back.
-__global__ void __launch_bounds__(kTcThreads, 1) k_coarse_apply_tc(TcApplyArgs a) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    // grid (column chunks, aggregates): the chunks of one aggregate run side by
-    // side and share its operator tiles through L2
-    const int nc = a.nc, npad = a.npad, nw = a.nw, chunk = blockIdx.x, n0 = chunk * nw, K = 2 * nc, nvh = nc / 2;
-    const int nch = npad / nw, S = tc_stages_of(a);
-    const size_t SA = (size_t)128 * K * 2, SB = (size_t)nw * K * 2, SS = SA + 2 * SB;
-    __shared__ __align__(8) uint64_t bar[2 * kTcMaxStages];   // [0, S): stage full, [S, 2S): stage empty
-    __shared__ uint32_t s_taddr;
-    __shared__ int s_ok;
-    const int X = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t ncols = tc_tmem_cols(nw);
-    const uint32_t bytesA = (uint32_t)(K * K * 2), bytesB = (uint32_t)SB;
+// units of a fixed-point grid sum whose last value was s: 2^36 / s to a power of two
+__device__ __forceinline__ float unit_of(float s) {
+    if (!(s > 0.f)) return 0x1p42f;
+    const int e = ((__float_as_int(s) >> 23) & 255) - 127;
+    return __int_as_float((127 + min(36 - e, 120)) << 23);
+}
 
-    if (tid == 0) {
-        for (int i = 0; i < 2 * S; ++i) mbar_init(bar + i, 1);
+struct BcgCta {
+    const BcgArgs& a;
+    const BcgSmem L;
+    int nc, nvh, nw, nch, j0, j1;
+    unsigned char* sm;
+    uint64_t *full, *empty, *acc_full, *acc_empty, *gate;
+    volatile int *fail, *stop;
+
+    __device__ BcgCta(const BcgArgs& args, unsigned char* smem, uint64_t* bars, int* flags)
+        : a(args), L(args.nc, args.nw, args.npad, args.stages), sm(smem) {
+        nc = a.nc; nvh = nc >> 1; nw = a.nw; nch = a.npad / nw;
+        const long long NJ = (long long)a.g.Vc * nch;
+        j0 = (int)(blockIdx.x * NJ / gridDim.x);
+        j1 = (int)((blockIdx.x + 1) * NJ / gridDim.x);
+        full = bars; empty = bars + kBcgMaxStages; acc_full = bars + 2 * kBcgMaxStages; acc_empty = acc_full + 2;
+        gate = acc_empty + 2;
+        fail = flags; stop = flags + 1;
+    }
+
+    // ------------------------------------------------------------ copies (two warps)
+    // Items (job, direction) in order, item i of the launch in stage i % stages, whose
+    // "full" barrier takes one arrival and the bytes of each tile.  Both warps run over
+    // all items, up to `stages` directions at a time (so that no lane waits for what
+    // another lane of its round has yet to copy).  The operator does not depend on the
+    // iteration: its tiles run ahead across the grid barriers, as far as stages are
+    // free; the operand's wait for the gate of each phase.
+    __device__ void copy_operator(unsigned int* b_items) {
+        const int S = a.stages, R = min(S, 9), lane = threadIdx.x & 31;
+        const size_t blk = (size_t)2 * nc * nc;
+        unsigned int next = 0;      // past the last item this lane armed
+        bool ok = true;
+        for (unsigned int job = 0; ok; job += j1 - j0)
+            for (int j = j0; j < j1 && ok; ++j)
+                for (int d0 = 0; d0 < 9 && ok; d0 += R) {
+                    const int d = d0 + lane;
+                    bool mine = true;
+                    if (lane < R && d < 9) {
+                        const unsigned int i = (job + (j - j0)) * 9 + d, k = i / S;
+                        const int st = (int)(i - k * S);
+                        mine = i < (unsigned int)S || wait_stop(empty + st, (k - 1) & 1u);
+                        if (mine) {
+                            mbar_expect_tx(full + st, L.a_copy);
+                            bulk_copy_g2s(sm + (size_t)st * L.stage, a.At + ((size_t)(j / nch) * 9 + d) * blk, L.a_copy,
+                                          full + st);
+                            next = i + 1;
+                        }
+                    }
+                    ok = __all_sync(0xffffffffu, mine);
+                }
+        // drain: the tiles that no operand joined (the arrival that is missing is made
+        // here); after a failure, time enough for any copy to land
+        asm volatile("barrier.cta.sync 2, 64;" ::: "memory");
+        if (*fail) {
+            for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+            return;
+        }
+        const unsigned int b0 = *b_items;
+        for (unsigned int i = b0; i < b0 + S; ++i)
+            if (lane < R && (int)(i % 9) % R == lane && i < next) {
+                const unsigned int k = i / S;
+                const int st = (int)(i - k * S);
+                mbar_arrive(full + st);
+                mbar_wait(full + st, k & 1u, kBcgWait);
+            }
+    }
+    __device__ void copy_operand(int phase, unsigned int* b_items) {   // phase odd: the adjoint's operand (btu)
+        const int S = a.stages, R = min(S, 9), lane = threadIdx.x & 31;
+        const size_t tile = (size_t)4 * nc * nw;
+        unsigned int job = 0;
+        for (uint32_t gate_par = 0;; ++phase, gate_par ^= 1u, job += j1 - j0) {
+            if (!__all_sync(0xffffffffu, bcg_wait(gate, gate_par, fail, a.err)) || *stop) break;
+            fence_proxy_async_all();    // tiles written by other CTAs before the grid barrier
+            const __half* bt = (phase & 1) ? a.btu : a.bts;
+            bool ok = true;
+            for (int j = j0; j < j1 && ok; ++j)
+                for (int d0 = 0; d0 < 9 && ok; d0 += R) {
+                    const int d = d0 + lane;
+                    bool mine = true;
+                    if (lane < R && d < 9) {
+                        const unsigned int i = (job + (j - j0)) * 9 + d, k = i / S;
+                        const int st = (int)(i - k * S), X = j / nch, c = j - X * nch;
+                        const int Y = __ldg(a.nbr + (size_t)X * 9 + d);
+                        mine = i < (unsigned int)S || bcg_wait(empty + st, (k - 1) & 1u, fail, a.err);
+                        if (mine) {
+                            mbar_expect_tx(full + st, L.b_copy);
+                            bulk_copy_g2s(sm + (size_t)st * L.stage + L.a_bytes, bt + ((size_t)Y * nch + c) * tile,
+                                          L.b_copy, full + st);
+                        }
+                    }
+                    ok = __all_sync(0xffffffffu, mine);
+                }
+            if (!ok) break;
+        }
+        if (lane == 0) *b_items = job * 9;
+        asm volatile("barrier.cta.sync 2, 64;" ::: "memory");
+    }
+    // as bcg_wait; false without an error when the launch has ended
+    __device__ bool wait_stop(uint64_t* bar, uint32_t parity) {
+        for (long long i = 0; i < kBcgWait; ++i) {
+            if (mbar_try_wait(bar, parity)) return true;
+            if (*fail || *stop) return false;
+            if (i > 64) __nanosleep(20);
+        }
+        *fail = 1;
+        atomicExch(a.err, 1);
+        return false;
+    }
+
+    // ------------------------------------------------------------ MMAs (one thread of two warps)
+    __device__ void multiply(uint32_t tmem, int which, uint64_t* drain) {
+        const unsigned int S = a.stages, jobs = j1 - j0;
+        const int nks = L.kcp >> 1;
+        const uint32_t idesc = idesc_f16(128, 4 * nw), lbo_a = (uint32_t)nc * 32, lbo_b = (uint32_t)nw * 64;
+        // descriptors of stage 0; the address field counts 16 bytes
+        const uint64_t da0 = smem_desc(smem_u32(sm), lbo_a, 128), db0 = smem_desc(smem_u32(sm) + L.a_bytes, lbo_b, 128);
+        const uint64_t step_a = lbo_a >> 3, step_b = lbo_b >> 3, step_st = L.stage >> 4;
+        const uint32_t acc = tmem + (uint32_t)(which * 4 * nw);
+        uint32_t gate_par = 0, acc_par = 1u;   // a fresh barrier passes a wait for parity 1
+        unsigned int job = 0;
+        for (bool ok = true; ok; job += jobs) {
+            if (!bcg_wait(gate, gate_par, fail, a.err) || *stop) break;
+            gate_par ^= 1u;
+            for (unsigned int j = (job ^ which) & 1u; j < jobs && ok; j += 2) {   // this warp's jobs: (job + j) odd or even
+                if (!bcg_wait(acc_empty + which, acc_par, fail, a.err)) { ok = false; break; }
+                acc_par ^= 1u;
+                tc_fence_after();
+                const unsigned int i0 = (job + j) * 9, k0 = i0 / S;
+                unsigned int st = i0 - k0 * S;
+                uint32_t par = k0 & 1u;
+                uint64_t da = da0 + st * step_st, db = db0 + st * step_st;
+                for (int d = 0; d < 9; ++d) {
+                    if (!bcg_wait(full + st, par, fail, a.err)) { ok = false; break; }
+                    tc_fence_after();
+                    mma_f16(acc, da, db, idesc, d > 0 ? 1u : 0u);
+                    if (nks > 1) mma_f16(acc, da + step_a, db + step_b, idesc, 1u);
+                    if (nks > 2) mma_f16(acc, da + 2 * step_a, db + 2 * step_b, idesc, 1u);
+                    mma_commit(empty + st);
+                    da += step_st;
+                    db += step_st;
+                    if (++st == S) {
+                        st = 0;
+                        par ^= 1u;
+                        da = da0;
+                        db = db0;
+                    }
+                }
+                if (ok) mma_commit(acc_full + which);
+            }
+        }
+        mma_commit(drain);
+        mbar_wait(drain, 0, kBcgWait);
+    }
+
+    // ------------------------------------------------------------ epilogue warps
+    float2 *T, *S2;
+    Sum2* acc;
+    int t, n, rg, rgs;
+    long long job_count = 0;
+    unsigned int arrived = 0;
+
+    // entries staged in S2[row][n] (scaled) -> the four FP16 rows of the tile
+    __device__ void write_tile(__half* bt, int X, int c) {
+        __half* base = bt + ((size_t)X * nch + c) * 4 * nc * nw;
+        for (int i = t; i < (nc >> 3) * nw; i += kEpi) {
+            const int kc = i / nw, m = i - kc * nw;
+            uint32_t w[4][4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float2 v[2];
+                float hr[2], hi[2];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    v[q] = S2[(kc * 8 + 2 * e + q) * L.ts + m];
+                    v[q].x = fminf(fmaxf(v[q].x, -65504.f), 65504.f);
+                    v[q].y = fminf(fmaxf(v[q].y, -65504.f), 65504.f);
+                    hr[q] = __half2float(__float2half_rn(v[q].x));
+                    hi[q] = __half2float(__float2half_rn(v[q].y));
+                }
+                w[0][e] = half_pair(hr[0], hr[1]);
+                w[1][e] = half_pair(hi[0], hi[1]);
+                w[2][e] = half_pair(v[0].x - hr[0], v[1].x - hr[1]);
+                w[3][e] = half_pair(v[0].y - hi[0], v[1].y - hi[1]);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int row = j * nw + m;
+                *reinterpret_cast<uint4*>(base + ((size_t)(kc * (nw >> 1) + (row >> 3)) << 6) + ((row & 7) << 3)) =
+                    make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
+            }
+        }
+    }
+
+    // grid barrier of the epilogue warps (all writes before it visible to all reads
+    // after it, tile writes to the bulk copies too); opens the gate of the next phase
+    __device__ bool grid_barrier(bool open) {
+        fence_proxy_async_all();
+        if (epi_sync(*fail != 0)) return false;
+        if (t == 0) {
+            __threadfence();
+            ++arrived;
+            const unsigned int want = arrived * gridDim.x;
+            atomicAdd(a.bar, 1u);
+            long long spins = 0;
+            unsigned int got;
+            for (;;) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(a.bar) : "memory");
+                if ((int)(got - want) >= 0) break;
+                if (*(volatile int*)a.err) { *fail = 1; break; }
+                if (++spins > kBcgWait) { *fail = 1; atomicExch(a.err, 1); break; }
+                if (spins > 64) __nanosleep(20);
+            }
+            __threadfence();
+            fence_proxy_async_all();
+            if (open && !*fail) mbar_arrive(gate);
+        }
+        return !epi_sync(*fail != 0);
+    }
+    __device__ void open_gate() {
+        if (t == 0) mbar_arrive(gate);
+    }
+
+    // products of the next job into T; false on failure (uniform over the warps)
+    __device__ bool take(uint32_t tmem) {
+        const int buf = (int)(job_count & 1), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int quad = warp & 3, half = (warp - 4) >> 2, m = 32 * quad + lane;
+        const bool ok = __all_sync(0xffffffffu, bcg_wait(acc_full + buf, (uint32_t)((job_count >> 1) & 1), fail, a.err));
+        tc_fence_after();
+        if (ok && 32 * quad < 2 * nc) {
+            const uint32_t base = tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(buf * 4 * nw);
+            for (int c0 = 8 * half; c0 < nw; c0 += 16) {
+                uint32_t rh[8], ih[8], rl[8], il[8];
+                tmem_ld8(base + c0, rh);
+                tmem_ld8(base + nw + c0, ih);
+                tmem_ld8(base + 2 * nw + c0, rl);
+                tmem_ld8(base + 3 * nw + c0, il);
+                tmem_wait_ld8(rh, ih, rl, il);
+                if (m < 2 * nc)
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        T[(size_t)m * L.ts + c0 + e] = make_float2(__uint_as_float(rh[e]) + __uint_as_float(rl[e]),
+                                                                   __uint_as_float(ih[e]) + __uint_as_float(il[e]));
+            }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc_empty + buf);
+        ++job_count;
+        return !epi_sync(!ok);
+    }
+    __device__ __forceinline__ float2 product(int r, float inv, bool dag) const {
+        const float2 x = T[(size_t)r * L.ts + n], w = T[(size_t)(nc + r) * L.ts + n];
+        const float f = dag && r >= nvh ? -inv : inv;
+        return make_float2(f * (x.x - w.y), f * (x.y + w.x));
+    }
+    __device__ __forceinline__ void stage(int r, float2 v, float sc, bool dag) {
+        const float f = dag && r >= nvh ? -sc : sc;
+        S2[r * L.ts + n] = make_float2(f * v.x, f * v.y);
+    }
+    __device__ __forceinline__ Sum2& col_acc(int val, int col) { return acc[((size_t)val * rgs + rg) * a.npad + col]; }
+
+    // Grid sums of the column sums, in 64-bit fixed point: integer adds give the same
+    // sum in any order, so a CTA adds its share with one atomic per value and reads the
+    // sums after the grid barrier.  (Every CTA adding up all CTAs' partial sums in a
+    // fixed order took 5-7 us per iteration at 152 x 48 values.)  The unit of a value
+    // is 2^-36 of its last grid sum (fx; 2^-42 of |r|^2 before the first), so a sum
+    // keeps more bits than its FP32 terms have; a value out of range (it grew 2^19
+    // times in one iteration, or is not finite) ends its column.
+    __device__ void publish(const float* fx, unsigned long long* sums) {
+        epi_sync();
+        for (int i = t; i < 3 * a.npad; i += kEpi) {
+            const int v = i / a.npad, c = i - v * a.npad;
+            Sum2 s{0.f, 0.f};
+            for (int g = 0; g < rgs; ++g) {
+                Sum2& e = acc[((size_t)v * rgs + g) * a.npad + c];
+                add2(s, e.h);
+                s.l += e.l;
+                e = Sum2{0.f, 0.f};
+            }
+            const float h = s.h * fx[i], l = s.l * fx[i];
+            const long long q = fabsf(h) < 0x1p55f ? __float2ll_rn(h) + __float2ll_rn(l) : -(1LL << 54);
+            if (q != 0) atomicAdd(sums + i, (unsigned long long)q);
+        }
+        __threadfence();
+    }
+
+    __device__ void epilogue(uint32_t tmem) {
+        t = threadIdx.x - kEpi0;
+        rgs = L.rgs;
+        n = t % nw;
+        rg = t / nw;
+        const bool act = rg < rgs;
+        T = reinterpret_cast<float2*>(sm + L.off_t);
+        S2 = reinterpret_cast<float2*>(sm + L.off_s2);
+        acc = reinterpret_cast<Sum2*>(sm + L.off_acc);
+        const int np = a.npad, jobs = j1 - j0;
+        double* gam = reinterpret_cast<double*>(sm + L.off_col);   // 1 / gamma, 1 / alpha of the last iteration, |r_0|^2
+        double* alo = gam + np;
+        double* rho0 = alo + np;
+        float* fx = reinterpret_cast<float*>(rho0 + np);           // [3][npad] units of the grid sums (reciprocals)
+        float* al = fx + 3 * np;                                   // alpha, beta of this iteration
+        float* be = al + np;
+        float* iss = be + np;                                      // 1 / scale of the s tile, of the u tile
+        float* isu = iss + np;
+        float* sc_s = isu + np;                                    // scales for the next s and u tiles
+        float* sc_u = sc_s + np;
+        float* fr = sc_u + np;                                     // power of two that brings rc to unit size
+        int* done = reinterpret_cast<int*>(fr + np);               // 1: this column is frozen
+        int* its = done + np;
+        const float rows = (float)((double)a.g.Vc * nc);
+        for (int i = t; i < 3 * rgs * np; i += kEpi) acc[i] = Sum2{0.f, 0.f};
+        epi_sync();
+
+        if (a.mode == BCG_APPLY) {   // y = D_c x (dag: D_c^dag x): tiles of x, one stencil
+            for (int j = 0; j < jobs; ++j) {
+                const int X = (j0 + j) / nch, c = j0 + j - X * nch;
+                if (act)
+                    for (int r = rg; r < nc; r += rgs)
+                        stage(r, a.rc[((size_t)X * nc + r) * np + c * nw + n], 1.f, a.dag != 0);
+                epi_sync();
+                write_tile(a.dag ? a.btu : a.bts, X, c);
+                epi_sync();
+            }
+            if (!grid_barrier(true)) return;
+            for (int j = 0; j < jobs; ++j) {
+                const int X = (j0 + j) / nch, c = j0 + j - X * nch;
+                if (!take(tmem)) return;
+                if (act)
+                    for (int r = rg; r < nc; r += rgs)
+                        a.y[((size_t)X * nc + r) * np + c * nw + n] = product(r, 1.f, a.dag != 0);
+                epi_sync();
+            }
+            if (t == 0) *stop = 1;
+            epi_sync();
+            open_gate();
+            return;
+        }
+
+        // the size of rc per column: the largest CTA's |rc|^2 (float bits order as integers)
+        if (act)
+            for (int j = 0; j < jobs; ++j) {
+                const int X = (j0 + j) / nch, col = (j0 + j - X * nch) * nw + n;
+                float s = 0.f;
+                for (int r = rg; r < nc; r += rgs) {
+                    const float2 v = a.rc[((size_t)X * nc + r) * np + col];
+                    s += v.x * v.x + v.y * v.y;
+                }
+                add2(col_acc(0, col), s);
+            }
+        epi_sync();
+        for (int i = t; i < np; i += kEpi) {
+            float s = 0.f;
+            for (int g = 0; g < rgs; ++g) {
+                Sum2& e = acc[(size_t)g * np + i];
+                s += e.h;
+                e = Sum2{0.f, 0.f};
+            }
+            atomicMax(a.mx + i, __float_as_uint(fabsf(s)));   // fabs: one sign for every NaN
+        }
+        __threadfence();
+        if (!grid_barrier(false)) return;
+        for (int i = t; i < np; i += kEpi) {
+            const unsigned int m = __ldcg(a.mx + i);
+            const bool zero = m < 0x00800000u, finite = m < 0x7f800000u;   // below the normal range counts as zero
+            // rc 2^-e with 2^(2 e) near its largest share: every right-hand side starts near
+            // unit size, exactly; a column that is not finite passes on its NaNs
+            const int e = ((int)(m >> 23) - 127) >> 1;
+            fr[i] = finite ? __int_as_float((127 - e) << 23) : 1.f;
+            done[i] = (i >= a.nrhs || zero || !finite || a.maxit <= 0) ? (finite ? 1 : 2) : 0;
+            its[i] = 0;
+            sc_s[i] = sc_u[i] = col_scale(4.0, rows);
+            iss[i] = isu[i] = 1.f / sc_s[i];
+            fx[i] = fx[np + i] = fx[2 * np + i] = 0x1p42f;
+        }
+        epi_sync();
+        // r = rc 2^-e, y = 0; the tile of r for s = D_c^dag r
+        for (int j = 0; j < jobs; ++j) {
+            const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+            if (act) {
+                float s = 0.f;
+                const float f = done[col] ? 0.f : fr[col], sc = sc_u[col];
+                const bool nan = done[col] == 2;
+                for (int r = rg; r < nc; r += rgs) {
+                    const size_t o = ((size_t)X * nc + r) * np + col;
+                    float2 v = a.rc[o];
+                    const float2 z = nan ? make_float2(0.f * v.x, 0.f * v.y) : make_float2(0.f, 0.f);
+                    v = f != 0.f ? make_float2(f * v.x, f * v.y) : make_float2(0.f, 0.f);
+                    a.r[o] = v;
+                    a.y[o] = z;
+                    s += v.x * v.x + v.y * v.y;
+                    stage(r, v, sc, true);
+                }
+                add2(col_acc(2, col), s);
+            }
+            epi_sync();
+            write_tile(a.btu, X, c);
+            epi_sync();
+        }
+        if (!grid_barrier(true)) return;
+        // s = D_c^dag r, its tile and norm
+        for (int j = 0; j < jobs; ++j) {
+            const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+            if (!take(tmem)) return;
+            if (act) {
+                float s = 0.f;
+                const float inv = isu[col], sc = sc_s[col];
+                for (int r = rg; r < nc; r += rgs) {
+                    const float2 v = product(r, inv, true);
+                    a.s[((size_t)X * nc + r) * np + col] = v;
+                    s += v.x * v.x + v.y * v.y;
+                    stage(r, v, sc, false);
+                }
+                add2(col_acc(1, col), s);
+            }
+            epi_sync();
+            write_tile(a.bts, X, c);
+        }
+        for (int it = 0;; ++it) {
+            if (!grid_barrier(true)) return;
+            // phase A: u = D_c s, its tile and norm
+            for (int j = 0; j < jobs; ++j) {
+                const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+                if (!take(tmem)) return;
+                if (act) {
+                    float s = 0.f;
+                    const float inv = iss[col], sc = sc_u[col];
+                    for (int r = rg; r < nc; r += rgs) {
+                        const float2 v = product(r, inv, false);
+                        a.u[((size_t)X * nc + r) * np + col] = v;
+                        s += v.x * v.x + v.y * v.y;
+                        stage(r, v, sc, true);
+                    }
+                    add2(col_acc(0, col), s);
+                }
+                epi_sync();
+                write_tile(a.btu, X, c);
+            }
+            unsigned long long* sums = a.sums + (size_t)(it & 1) * 3 * np;
+            publish(fx, sums);
+            if (!grid_barrier(true)) return;
+            // the scalars of the iteration, while phase B's copies and MMAs run
+            if (blockIdx.x == 0)   // the other half's readers are all past this barrier, its writers behind the next
+                for (int i = t; i < 3 * np; i += kEpi) a.sums[(size_t)((it + 1) & 1) * 3 * np + i] = 0ull;
+            bool running = false;
+            for (int i = t; i < np; i += kEpi) {
+                isu[i] = 1.f / sc_u[i];
+                if (!done[i]) {
+                    double tot[3];
+#pragma unroll
+                    for (int v = 0; v < 3; ++v) {
+                        const long long q = (long long)__ldcg(sums + v * np + i);
+                        tot[v] = (double)q * (double)(1.f / fx[v * np + i]);
+                        fx[v * np + i] = unit_of((float)tot[v]);
+                    }
+                    const double delta = tot[0], gamma = tot[1], rho = tot[2];
+                    its[i] = it;
+                    double beta = 0.0, den = delta;
+                    if (it > 0) {   // gam, alo: reciprocals of the last gamma and alpha
+                        beta = gamma * gam[i];
+                        den = delta - beta * gamma * alo[i];
+                    } else {
+                        rho0[i] = rho;
+                    }
+                    if ((it > 0 && rho <= a.tol2 * rho0[i]) || it >= a.maxit || !(gamma > 0) || !(den > 0)) {
+                        done[i] = 1;
+                        al[i] = be[i] = 0.f;
+                    } else {
+                        const double alpha = gamma / den;
+                        gam[i] = gamma;   // turned into reciprocals after phase B
+                        alo[i] = alpha;
+                        al[i] = (float)alpha;
+                        be[i] = (float)beta;
+                        running = true;
+                        sc_s[i] = col_scale(gamma, rows);
+                        sc_u[i] = col_scale(delta, rows);
+                    }
+                }
+            }
+            running = epi_sync(running);
+            // phase B: w = D_c^dag u and the updates on the own rows
+            const bool first = it == 0;
+            for (int j = 0; j < jobs; ++j) {
+                const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+                if (!take(tmem)) return;
+                if (!running) continue;   // nothing left to do but to take what was started
+                if (act) {
+                    float sg = 0.f, sr = 0.f;
+                    const bool frozen = done[col] != 0;
+                    const float inv = isu[col], sc = sc_s[col], alpha = al[col], beta = be[col];
+#pragma unroll 3
+                    for (int r = rg; r < nc; r += rgs) {
+                        const size_t o = ((size_t)X * nc + r) * np + col;
+                        float2 s = a.s[o];
+                        if (!frozen) {
+                            const float2 u = a.u[o], w = product(r, inv, true);
+                            float2 p = s, z = w, q = u, y = a.y[o], rr = a.r[o];
+                            if (!first) {
+                                const float2 p0 = a.p[o], z0 = a.z[o], q0 = a.q[o];
+                                p.x += beta * p0.x; p.y += beta * p0.y;
+                                z.x += beta * z0.x; z.y += beta * z0.y;
+                                q.x += beta * q0.x; q.y += beta * q0.y;
+                            }
+                            y.x += alpha * p.x; y.y += alpha * p.y;
+                            rr.x -= alpha * q.x; rr.y -= alpha * q.y;
+                            s.x -= alpha * z.x; s.y -= alpha * z.y;
+                            a.p[o] = p; a.z[o] = z; a.q[o] = q;
+                            a.y[o] = y; a.r[o] = rr; a.s[o] = s;
+                            sg += s.x * s.x + s.y * s.y;
+                            sr += rr.x * rr.x + rr.y * rr.y;
+                        }
+                        stage(r, s, sc, false);
+                    }
+                    if (!frozen) {
+                        add2(col_acc(1, col), sg);
+                        add2(col_acc(2, col), sr);
+                    }
+                }
+                epi_sync();
+                write_tile(a.bts, X, c);
+            }
+            for (int i = t; i < np; i += kEpi) {
+                iss[i] = 1.f / sc_s[i];
+                if (!done[i]) {
+                    gam[i] = 1.0 / gam[i];
+                    alo[i] = 1.0 / alo[i];
+                }
+            }
+            if (!running) break;
+        }
+        // the solution in the units of rc
+        if (act)
+            for (int j = 0; j < jobs; ++j) {
+                const int X = (j0 + j) / nch, col = (j0 + j - X * nch) * nw + n;
+                if (done[col] == 2) continue;
+                const float f = 1.f / fr[col];
+                for (int r = rg; r < nc; r += rgs) {
+                    const size_t o = ((size_t)X * nc + r) * np + col;
+                    const float2 v = a.y[o];
+                    a.y[o] = make_float2(f * v.x, f * v.y);
+                }
+            }
+        if (blockIdx.x == 0)
+            for (int i = t; i < np; i += kEpi) a.iters[i] = (double)its[i];
+        if (t == 0) *stop = 1;
+        epi_sync();
+        open_gate();
+    }
+};
+
+__global__ void __launch_bounds__(kBcgThreads, 1) k_bcg(BcgArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) uint64_t bars[2 * kBcgMaxStages + 7];
+    __shared__ uint32_t s_taddr;
+    __shared__ unsigned int s_items;
+    __shared__ int s_flags[2];
+    BcgCta c(a, smem, bars, s_flags);
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kBcgMaxStages; ++i) { mbar_init(c.full + i, 2); mbar_init(c.empty + i, 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(c.acc_full + i, 1); mbar_init(c.acc_empty + i, kEpiWarps); }
+        for (int i = 0; i < 3; ++i) mbar_init(c.gate + i, 1);   // the gate, the MMA threads' drains
         fence_mbar_init();
+        s_flags[0] = s_flags[1] = 0;
+        s_items = 0;
     }
-    // zero the padding rows (2nc..127) of every stage's A tile once
-    for (int st = 0; st < S; ++st) {
-        __half* As = reinterpret_cast<__half*>(smem + st * SS);
-        for (int i = K * K + tid; i < 128 * K; i += kTcThreads) As[i] = __float2half(0.f);
-    }
-    fence_proxy_async();   // the zeros are read by the MMAs (async proxy)
-    if (warp == 0) {
-        tmem_alloc(&s_taddr, ncols);
+    // zero the stages: the padding K group stays zero, the copies fill the rest
+    for (size_t i = threadIdx.x; i < (size_t)a.stages * c.L.stage / 16; i += kBcgThreads)
+        reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+    fence_proxy_async();
+    if (warp == 2) {
+        tmem_alloc(&s_taddr, a.tmem_cols);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_taddr;
-
-    if (tid == 0) {
-        const uint32_t idesc = idesc_f16(128, nw);
-        const uint32_t lbo = 128, sbo = (uint32_t)(K >> 3) * 128;
-        // stage bookkeeping for the drain: parity of the copy in flight per stage (-1: none)
-        int pending[kTcMaxStages];
-        for (int st = 0; st < kTcMaxStages; ++st) pending[st] = -1;
-        auto issue = [&](int d, int st) {
-            unsigned char* base = smem + st * SS;
-            const int Y = coarse_neighbour(a.g, X, d);
-            mbar_expect_tx(bar + st, bytesA + 2 * bytesB);
-            bulk_copy_g2s(base, a.Aemb + ((size_t)X * 9 + d) * K * K, bytesA, bar + st);
-            const __half* bsrc = a.bt + ((size_t)(Y * nch + chunk) * 2) * nw * K;
-            bulk_copy_g2s(base + SA, bsrc, bytesB, bar + st);
-            bulk_copy_g2s(base + SA + SB, bsrc + (size_t)nw * K, bytesB, bar + st);
-            pending[st] = (d / S) & 1;
-        };
-        bool ok = true;
-        int last = -1;   // stage * 2 + parity of the last commit
-        for (int d = 0; d < S && d < 9; ++d) issue(d, d);
-        for (int d = 0; d < 9 && ok; ++d) {
-            // refill the stage the previous direction's MMAs used, once they are done
-            const int dp = d - 1;
-            if (dp >= 0 && dp + S < 9) {
-                const int sp = dp % S;
-                if (!mbar_wait(bar + S + sp, (uint32_t)((dp / S) & 1), kTcWaitLimit)) { ok = false; break; }
-                issue(dp + S, sp);
-            }
-            const int s = d % S;
-            if (!mbar_wait(bar + s, (uint32_t)((d / S) & 1), kTcWaitLimit)) { ok = false; break; }
-            pending[s] = -1;
-            tc_fence_after();
-            const uint32_t a0 = smem_u32(smem + s * SS), bh0 = a0 + (uint32_t)SA, bl0 = bh0 + (uint32_t)SB;
-            for (int ks = 0; ks < (K >> 4); ++ks) {
-                const uint64_t ad = smem_desc(a0 + ks * 256, lbo, sbo);
-                mma_f16(tmem, ad, smem_desc(bh0 + ks * 256, lbo, sbo), idesc, (d > 0 || ks > 0) ? 1u : 0u);
-                mma_f16(tmem, ad, smem_desc(bl0 + ks * 256, lbo, sbo), idesc, 1u);
-            }
-            mma_commit(bar + S + s);
-            last = s * 2 + ((d / S) & 1);
-        }
-        // drain: the last commit covers every MMA issued; then every copy still in flight
-        if (last >= 0 && !mbar_wait(bar + S + (last >> 1), (uint32_t)(last & 1), kTcWaitLimit)) ok = false;
-        for (int st = 0; st < S; ++st)
-            if (pending[st] >= 0 && !mbar_wait(bar + st, (uint32_t)pending[st], kTcWaitLimit)) ok = false;
-        s_ok = ok ? 1 : 0;
+    if (warp == 0) {
+        c.copy_operator(&s_items);
+    } else if (warp == 1) {
+        c.copy_operand(a.mode == BCG_APPLY ? (a.dag ? 1 : 0) : 1, &s_items);
+    } else if (warp < 4) {
+        if ((threadIdx.x & 31) == 0) c.multiply(tmem, warp - 2, c.gate + warp - 1);
+    } else {
+        c.epilogue(tmem);
     }
-    __syncthreads();
-    const bool ok = s_ok != 0;
-    tc_fence_after();
-    // epilogue: warp w reads TMEM lanes 32w..32w+31 (embedded rows m) into a
-    // row-major tile in the (now idle) stage memory, T[m][n] (stride nw + 1);
-    // then rows a (real part) and nc + a (imaginary part) leave as one complex
-    // column-contiguous row of y, coalesced over the right-hand sides n
-    float* T = reinterpret_cast<float*>(smem);
-    const int ts = nw + 1;
-    const int m = warp * 32 + lane;
-    for (int c0 = 0; c0 < nw; c0 += 16) {
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-        if (m < K)
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                T[m * ts + c0 + j] = a.colscale ? v[j] * (float)(1.0 / a.colscale[n0 + c0 + j]) : v[j];
-    }
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (ok) {
-        float2* y = a.y;
-        for (int i = tid; i < nc * nw; i += kTcThreads) {
-            const int ar = i / nw, n = i - ar * nw;
-            const float sg = (a.dag && ar >= nvh) ? -1.f : 1.f;
-            y[((size_t)X * nc + ar) * npad + n0 + n] = make_float2(sg * T[ar * ts + n], sg * T[(nc + ar) * ts + n]);
-        }
-        if (a.norms)
-            for (int n = tid; n < nw; n += kTcThreads) {
-                float q = 0.f;
-                for (int r = 0; r < K; ++r) q += T[r * ts + n] * T[r * ts + n];
-                a.norms[(size_t)X * npad + n0 + n] = q;
-            }
-    } else if (a.norms) {
-        for (int n = tid; n < nw; n += kTcThreads) a.norms[(size_t)X * npad + n0 + n] = 0.f;
-    }
-    if (!ok && tid == 0) atomicExch(a.err, 1);
-    if (warp == 0) tmem_dealloc(tmem, ncols);
+    tc_fence_after();
+    if (warp == 2) tmem_dealloc(tmem, a.tmem_cols);
 }
 
-// Dynamic shared memory of one CTA: its pipeline stages, padded so that at
-// most 512 / ncols CTAs fit on an SM (their TMEM allocations never exceed the
-// 512 columns of an SM, so no allocation waits).
-static size_t tc_launch_smem(int nc, int nw, int stages) {
-    size_t sm = (size_t)stages * tc_stage_bytes(nc, nw);
-    size_t per_sm = 228 * 1024, cap = 512 / tc_tmem_cols(nw);
-    size_t min_sm = per_sm / (cap + 1) + 1024;
-    return sm > min_sm ? sm : min_sm;
+// ---------------------------------------------------------------- shape and launch
+// Columns per job: the multiple of 8 that divides npad and gives the busiest SM
+// the fewest bytes of tiles (operator per job, operand per column); more jobs
+// than SMs on the small lattices, the operator read once for up to 64 columns
+// on the large ones.
+bool bcg_shape(int nc, int npad, int Vc, int* nw_out, int* stages_out) {
+    // the panel widths the interface takes (Nv = 24: up to 224 columns)
+    if (nc % 8 || nc > 48 || npad % 8 || npad < 8 || npad > 256 || nc * (64 + npad) > 14512) return false;
+    const long long sms = device_sm_count();
+    double best = 1e300;
+    for (int nw = 8; nw <= 64 && nw <= npad; nw += 8) {
+        if (npad % nw) continue;
+        const BcgSmem one(nc, nw, npad, 1);
+        const long long room = 227 * 1024 - kBcgStatic - (long long)(one.total - one.stage);
+        const int stages = (int)std::min<long long>(kBcgMaxStages, room / one.stage);
+        if (stages < 3) continue;
+        const long long jobs = (long long)Vc * (npad / nw), per = (jobs + sms - 1) / sms;
+        // a job of few columns also pays for its barriers: 20 KB of tiles' worth
+        const double cost = (double)per * (9.0 * (one.a_copy + one.b_copy) + 20480.0);
+        if (cost < best) {
+            best = cost;
+            *nw_out = nw;
+            *stages_out = stages;
+        }
+    }
+    return best < 1e300;
 }
-bool coarse_apply_tc_supported(int nc, int npad) {
-    return npad % 16 == 0 && npad >= 16 && npad <= 256 && (2 * nc) % 16 == 0 && 2 * nc <= 128 &&
-           tc_launch_smem(nc, npad, 2) + kTcStaticSmem <= 227 * 1024;
-}
-// attribute for the largest chunk width used with this nc (every nw <= npad fits)
-cudaError_t coarse_apply_tc_prepare(int nc, int npad) {
-    if (!coarse_apply_tc_supported(nc, npad)) return cudaErrorInvalidValue;
-    size_t mx = 0;
-    for (int nw = 16; nw <= npad; nw += 16) mx = std::max(mx, tc_launch_smem(nc, nw, tc_stages(nc, nw)));
-    return cudaFuncSetAttribute(k_coarse_apply_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx);
-}
-// launch only (coarse_apply_tc_prepare must have been called for this shape);
-// args.nw = column chunk per CTA (multiple of 16 dividing npad; 0 = npad)
-cudaError_t coarse_apply_tc(const TcApplyArgs& args, cudaStream_t st) {
-    TcApplyArgs a = args;
-    if (a.nw <= 0) a.nw = a.npad;
-    if (!a.bt || a.g.Vc > 65535) return cudaErrorInvalidValue;   // aggregates index grid.y
-    const long long total = (long long)a.g.Vc * a.npad * (2 * a.nc / 8);
-    note_launch();
-    k_tc_split<<<(int)std::min<long long>((total + 255) / 256, 16LL * device_sm_count()), 256, 0, st>>>(
-        a.bt, a.x, a.nc, a.npad, a.nw, a.dag, a.colscale, total);
+size_t bcg_tile_bytes(int nc, int npad, long long Vc) { return (size_t)Vc * 4 * nc * npad * sizeof(__half); }
+
+cudaError_t bcg_launch(const BcgArgs& args, cudaStream_t st) {
+    BcgArgs a = args;
+    a.mx = a.bar + 4;
+    a.sums = reinterpret_cast<unsigned long long*>(a.bar + 4 + a.npad);
+    if (!bcg_shape(a.nc, a.npad, a.g.Vc, &a.nw, &a.stages)) return cudaErrorInvalidValue;
+    const int sms = device_sm_count();
+    const long long jobs = (long long)a.g.Vc * (a.npad / a.nw);
+    const int grid = (int)std::min<long long>(jobs, sms);
+    // past half an SM, so that one CTA has the SM's tensor memory to itself
+    const size_t sm = std::max<size_t>(BcgSmem(a.nc, a.nw, a.npad, a.stages).total, 116 * 1024);
+    a.tmem_cols = 32;
+    while (a.tmem_cols < 8 * a.nw) a.tmem_cols *= 2;
+    cudaError_t e = cudaFuncSetAttribute(k_bcg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(a.bar, 0, bcg_sync_bytes(a.npad), st);
+    if (e != cudaSuccess) return e;
     TmemOrder order(st);
     if (order.error() != cudaSuccess) return order.error();
+    void* params[] = {&a};
     note_launch();
-    if (a.stages != 0 && (a.stages < 2 || a.stages > tc_stages(a.nc, a.nw))) return cudaErrorInvalidValue;
-    k_coarse_apply_tc<<<dim3(a.npad / a.nw, a.g.Vc), kTcThreads, tc_launch_smem(a.nc, a.nw, tc_stages_of(a)), st>>>(a);
-    cudaError_t e = cudaGetLastError();
+    e = cudaLaunchCooperativeKernel((const void*)k_bcg, dim3(grid), dim3(kBcgThreads), params, sm, st);
     if (e != cudaSuccess) return e;
     return order.launched();
-}
-
-// Chunk width and pipeline depth for (nc, npad): every candidate (multiples of
-// 16 dividing npad; 2 or 3 stages where 3 fit -- 2 can leave room for a second
-// CTA on the SM) is timed with CUDA events on the given stream and the fastest
-// is kept.  The cache is keyed by device as well and guarded for concurrent
-// host threads.
-int coarse_apply_tc_tune(const TcApplyArgs& args, cudaStream_t st, int* stages) {
-    struct Entry { int dev, nc, npad, nw, stages; };
-    static std::vector<Entry> cache;
-    static std::mutex mu;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        for (const Entry& e : cache)
-            if (e.dev == dev && e.nc == args.nc && e.npad == args.npad) {
-                if (stages) *stages = e.stages;
-                return e.nw;
-            }
-    }
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    int best = args.npad, best_s = tc_stages(args.nc, args.npad);
-    float best_ms = 1e30f;
-    for (int cand = 0; cand < 2 * 16; ++cand) {
-        const int nw = 16 * (cand / 2 + 1), S = 2 + cand % 2;
-        if (nw > args.npad || args.npad % nw || S > tc_stages(args.nc, nw)) continue;
-        TcApplyArgs a = args;
-        a.nw = nw;
-        a.stages = S;
-        coarse_apply_tc(a, st);   // warm-up
-        cudaEventRecord(e0, st);
-        for (int r = 0; r < 5; ++r) coarse_apply_tc(a, st);
-        cudaEventRecord(e1, st);
-        cudaEventSynchronize(e1);
-        float ms = 0;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (ms < best_ms) { best_ms = ms; best = nw; best_s = S; }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    std::lock_guard<std::mutex> lock(mu);
-    cache.push_back({dev, args.nc, args.npad, best, best_s});
-    if (stages) *stages = best_s;
-    return best;
 }
 
 // ---------------------------------------------------------------- SIMT reference of the same contraction
@@ -328,8 +833,7 @@ int coarse_apply_tc_tune(const TcApplyArgs& args, cudaStream_t st, int* stages) 
 // path and to cross-check the tensor-core kernel.
 template <typename T>
 __global__ void k_coarse_apply_batched_simt(v2<T>* __restrict__ y, const double2* __restrict__ A,
-                                            const v2<T>* __restrict__ x, int nc, int npad, int dag, Geom g,
-                                            float* norms) {
+                                            const v2<T>* __restrict__ x, int nc, int npad, int dag, Geom g) {
     int X = blockIdx.x, a = blockIdx.y;
     int nvh = nc / 2;
     for (int n = threadIdx.x; n < npad; n += blockDim.x) {
@@ -348,237 +852,17 @@ __global__ void k_coarse_apply_batched_simt(v2<T>* __restrict__ y, const double2
         v2<T> o; o.x = (T)acc.r; o.y = (T)acc.i;
         y[((size_t)X * nc + a) * npad + n] = o;
     }
-    (void)norms;
 }
 template <typename T>
 void coarse_apply_batched_simt(v2<T>* y, const double2* A, const v2<T>* x, int nc, int npad, bool dag, const Geom& g,
                                cudaStream_t st) {
     note_launch();
-    k_coarse_apply_batched_simt<T><<<dim3(g.Vc, nc), 128, 0, st>>>(y, A, x, nc, npad, dag ? 1 : 0, g, nullptr);
+    k_coarse_apply_batched_simt<T><<<dim3(g.Vc, nc), 128, 0, st>>>(y, A, x, nc, npad, dag ? 1 : 0, g);
 }
 template void coarse_apply_batched_simt<float>(v2<float>*, const double2*, const v2<float>*, int, int, bool,
                                                const Geom&, cudaStream_t);
 template void coarse_apply_batched_simt<double>(v2<double>*, const double2*, const v2<double>*, int, int, bool,
                                                 const Geom&, cudaStream_t);
-
-// ---------------------------------------------------------------- per-RHS CGNR steps
-// Per-RHS scalars (double, npad entries each) in BatchScal.  Column sums are
-// reduced in two fixed-order stages: per-block partials part[block][n], then
-// one CTA per column adds the partials.  Columns whose done flag is set are
-// frozen.
-constexpr int kRowChunks = kBatchRowChunks;
-
-// rows [r0, r1) of block b of nb over `rows`; thread (rg, n), rgs row groups
-struct ColTile {
-    int n, rg, rgs;
-    long long r0, r1;
-    __device__ ColTile(int npad, long long rows) {
-        rgs = blockDim.x / npad;
-        if (rgs < 1) rgs = 1;
-        n = threadIdx.x % npad;
-        rg = threadIdx.x / npad;
-        r0 = (long long)blockIdx.x * rows / gridDim.x;
-        r1 = (long long)(blockIdx.x + 1) * rows / gridDim.x;
-    }
-    __device__ bool active() const { return rg < rgs; }
-};
-// per-column sum of v over the row groups of this block (fixed order) -> part[blockIdx][n]
-__device__ __forceinline__ void col_partial(float v, const ColTile& t, int npad, float* sh, float* part) {
-    if (t.active()) sh[t.rg * npad + t.n] = v;
-    __syncthreads();
-    for (int n = threadIdx.x; n < npad; n += blockDim.x) {
-        float s = 0.f;
-        for (int g = 0; g < t.rgs; ++g) s += sh[g * npad + n];
-        part[(size_t)blockIdx.x * npad + n] = s;
-    }
-}
-// one CTA per column: sum of part[c][n] over c < nparts, fixed order
-__device__ __forceinline__ double col_total(const float* part, int nparts, int npad) {
-    __shared__ double sh[33];
-    const int n = blockIdx.x;
-    double a = 0;
-    for (int c = threadIdx.x; c < nparts; c += blockDim.x) a += (double)part[(size_t)c * npad + n];
-    double v[1] = {a};
-    block_reduce<1>(v, (double (*)[32])sh);
-    if (threadIdx.x == 0) sh[32] = v[0];
-    __syncthreads();
-    return sh[32];
-}
-
-__global__ void k_bcol_norm(const float2* __restrict__ v, long long rows, int npad, float* part) {
-    extern __shared__ float shf[];
-    ColTile t(npad, rows);
-    float s = 0.f;
-    if (t.active())
-        for (long long r = t.r0 + t.rg; r < t.r1; r += t.rgs) {
-            float2 a = v[r * npad + t.n];
-            s += a.x * a.x + a.y * a.y;
-        }
-    col_partial(s, t, npad, shf, part);
-}
-// scale_n = ||rc_n||, done = (scale == 0 || n >= nrhs)
-// power of two nearest sqrt(rows / s): entries of a column with |x|^2 = s then sit
-// near 1 in magnitude, far above the FP16 subnormal range, after scaling
-__device__ __forceinline__ double pow2_scale(double s, long long rows) {
-    if (!(s > 0)) return 1.0;
-    const double e = rint(0.5 * log2((double)rows / s));
-    return exp2(fmin(fmax(e, -120.0), 120.0));
-}
-__global__ void k_bcg_scale(BatchScal S, const float* part, int nparts, int npad, int nrhs, int maxit, long long rows) {
-    double s = col_total(part, nparts, npad);
-    if (threadIdx.x != 0) return;
-    int n = blockIdx.x;
-    double sc = sqrt(s);
-    S.scale[n] = sc;
-    S.done[n] = (n >= nrhs || !(sc > 0) || maxit <= 0) ? 1.0 : 0.0;
-    S.iters[n] = 0;
-    S.r2[n] = S.done[n] != 0 ? 0.0 : 1.0;
-    S.csr[n] = pow2_scale(1.0, rows);   // r starts with unit norm
-}
-__global__ void k_bcg_start(float2* __restrict__ y, float2* __restrict__ r, const float2* __restrict__ rc,
-                            long long total, int npad, BatchScal S) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        int n = (int)(i % npad);
-        double sc = S.scale[n];
-        float f = sc > 0 ? (float)(1.0 / sc) : 0.f;
-        float2 v = rc[i];
-        r[i] = make_float2(v.x * f, v.y * f);
-        y[i] = make_float2(0.f, 0.f);
-    }
-}
-// gamma = ||s||^2 (first direction)
-__global__ void k_bcg_gamma0(BatchScal S, const float* xpart, int nx, int npad, long long rows) {
-    double s = col_total(xpart, nx, npad);
-    if (threadIdx.x == 0) {
-        S.gamma[blockIdx.x] = s;
-        S.csp[blockIdx.x] = pow2_scale(s, rows);   // p = s
-    }
-}
-// alpha = gamma / ||q||^2
-__global__ void k_bcg_alpha(BatchScal S, const float* xpart, int nx, int npad) {
-    double s = col_total(xpart, nx, npad);
-    int n = blockIdx.x;
-    if (threadIdx.x != 0 || S.done[n] != 0) return;
-    if (s > 0) S.alpha[n] = S.gamma[n] / s;
-    else { S.alpha[n] = 0; S.done[n] = 1; }
-}
-// y += alpha p, r -= alpha q (active columns), column partials of ||r||^2; zeroes *active
-__global__ void k_bcg_update1(float2* __restrict__ y, float2* __restrict__ r, const float2* __restrict__ p,
-                              const float2* __restrict__ q, long long rows, int npad, BatchScal S, float* part,
-                              int* active) {
-    extern __shared__ float shf[];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *active = 0;
-    ColTile t(npad, rows);
-    float s = 0.f;
-    if (t.active() && S.done[t.n] == 0) {
-        const float al = (float)S.alpha[t.n];
-        for (long long rr = t.r0 + t.rg; rr < t.r1; rr += t.rgs) {
-            long long i = rr * npad + t.n;
-            float2 pv = p[i], qv = q[i], yv = y[i], rv = r[i];
-            y[i] = make_float2(yv.x + al * pv.x, yv.y + al * pv.y);
-            float2 rn = make_float2(rv.x - al * qv.x, rv.y - al * qv.y);
-            r[i] = rn;
-            s += rn.x * rn.x + rn.y * rn.y;
-        }
-    }
-    col_partial(s, t, npad, shf, part);
-}
-// ||r||^2, iteration count, stopping test; *active counts columns still running
-__global__ void k_bcg_check(BatchScal S, const float* part, int nparts, int npad, double tol2, int maxit, int* active,
-                            long long rows) {
-    double s = col_total(part, nparts, npad);
-    int n = blockIdx.x;
-    if (threadIdx.x != 0 || S.done[n] != 0) return;
-    S.r2[n] = s;                         // relative to ||rc_n||^2 = 1 after scaling
-    S.csr[n] = pow2_scale(s, rows);
-    S.iters[n] += 1;
-    if (s <= tol2 || S.iters[n] >= maxit) S.done[n] = 1;
-    else atomicAdd(active, 1);
-}
-// beta = ||s||^2 / gamma, gamma = ||s||^2
-__global__ void k_bcg_beta(BatchScal S, const float* xpart, int nx, int npad, long long rows) {
-    double s = col_total(xpart, nx, npad);
-    int n = blockIdx.x;
-    if (threadIdx.x != 0 || S.done[n] != 0) return;
-    S.beta[n] = S.gamma[n] > 0 ? s / S.gamma[n] : 0.0;
-    S.gamma[n] = s;
-    S.csp[n] = pow2_scale(s, rows);      // p = s + beta p is of the size of s or larger
-}
-__global__ void k_bcg_update2(float2* __restrict__ p, const float2* __restrict__ s, long long total, int npad,
-                              BatchScal S, int first) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        int n = (int)(i % npad);
-        if (!first && S.done[n] != 0) continue;
-        float be = first ? 0.f : (float)S.beta[n];
-        float2 sv = s[i], pv = first ? make_float2(0.f, 0.f) : p[i];
-        p[i] = make_float2(sv.x + be * pv.x, sv.y + be * pv.y);
-    }
-}
-// y *= scale (undo the normalisation)
-__global__ void k_bcg_unscale(float2* __restrict__ y, long long total, int npad, BatchScal S) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        int n = (int)(i % npad);
-        float f = (float)S.scale[n];
-        float2 v = y[i];
-        y[i] = make_float2(v.x * f, v.y * f);
-    }
-}
-
-static inline int ew_grid(long long total) {
-    long long b = (total + 255) / 256;
-    if (b > 8LL * device_sm_count()) b = 8LL * device_sm_count();
-    return (int)(b > 0 ? b : 1);
-}
-static inline int col_threads(int npad) {
-    int rgs = 256 / npad;
-    if (rgs < 1) rgs = 1;
-    return ((rgs * npad + 31) / 32) * 32;
-}
-static inline size_t col_smem(int npad) { return sizeof(float) * (size_t)col_threads(npad) + sizeof(float) * npad; }
-
-// One CGLS iteration on all columns (kernels only: capturable in a CUDA graph).
-void bcg_iteration(const BatchCg& c, cudaStream_t st) {
-    const long long rows = (long long)c.g.Vc * c.nc, total = rows * c.npad;
-    const int ct = col_threads(c.npad);
-    const size_t cs = col_smem(c.npad);
-    TcApplyArgs ap{c.Aemb, c.p, c.q, c.nc, c.npad, c.nw, 0, c.g, c.xpart, c.err, c.S.csp, c.bt, c.stages};
-    coarse_apply_tc(ap, st);                                                               // q = D_c p
-    note_launch();
-    k_bcg_alpha<<<c.npad, 256, 0, st>>>(c.S, c.xpart, c.g.Vc, c.npad);
-    note_launch();
-    k_bcg_update1<<<kRowChunks, ct, cs, st>>>(c.y, c.r, c.p, c.q, rows, c.npad, c.S, c.rpart, c.active);
-    note_launch();
-    k_bcg_check<<<c.npad, 256, 0, st>>>(c.S, c.rpart, kRowChunks, c.npad, c.tol2, c.maxit, c.active, rows);
-    TcApplyArgs as{c.Aemb, c.r, c.s, c.nc, c.npad, c.nw, 1, c.g, c.xpart, c.err, c.S.csr, c.bt, c.stages};
-    coarse_apply_tc(as, st);                                                               // s = D_c^dag r
-    note_launch();
-    k_bcg_beta<<<c.npad, 256, 0, st>>>(c.S, c.xpart, c.g.Vc, c.npad, rows);
-    note_launch();
-    k_bcg_update2<<<ew_grid(total), 256, 0, st>>>(c.p, c.s, total, c.npad, c.S, 0);
-}
-
-// y = 0, r = rc/||rc||, s = D_c^dag r, gamma, p = s
-void bcg_start(const BatchCg& c, cudaStream_t st) {
-    const long long rows = (long long)c.g.Vc * c.nc, total = rows * c.npad;
-    note_launch();
-    k_bcol_norm<<<kRowChunks, col_threads(c.npad), col_smem(c.npad), st>>>(c.rc, rows, c.npad, c.rpart);
-    note_launch();
-    k_bcg_scale<<<c.npad, 256, 0, st>>>(c.S, c.rpart, kRowChunks, c.npad, c.nrhs, c.maxit, rows);
-    note_launch();
-    k_bcg_start<<<ew_grid(total), 256, 0, st>>>(c.y, c.r, c.rc, total, c.npad, c.S);
-    TcApplyArgs as{c.Aemb, c.r, c.s, c.nc, c.npad, c.nw, 1, c.g, c.xpart, c.err, c.S.csr, c.bt, c.stages};
-    coarse_apply_tc(as, st);
-    note_launch();
-    k_bcg_gamma0<<<c.npad, 256, 0, st>>>(c.S, c.xpart, c.g.Vc, c.npad, rows);
-    note_launch();
-    k_bcg_update2<<<ew_grid(total), 256, 0, st>>>(c.p, c.s, total, c.npad, c.S, 1);
-}
-
-void bcg_finish(const BatchCg& c, cudaStream_t st) {
-    const long long total = (long long)c.g.Vc * c.nc * c.npad;
-    note_launch();
-    k_bcg_unscale<<<ew_grid(total), 256, 0, st>>>(c.y, total, c.npad, c.S);
-}
 
 }  // namespace wmg
 

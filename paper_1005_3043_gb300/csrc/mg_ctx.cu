@@ -31,8 +31,8 @@ struct CoarseLevel {
     float2* P32 = nullptr;
     double2* A64 = nullptr;   // [X][9][nc][nc] column-major blocks
     float2* A32 = nullptr;
-    __half* Aemb = nullptr;   // FP16 tensor-core embedding of A64 (batched path), built on demand
-    bool emb_valid = false;
+    __half* At = nullptr;     // FP16 tensor-core tiles of A64 (batched path), built on demand
+    bool at_valid = false;
     __half2* A16 = nullptr;   // FP16 copy with per-block scales s16 (FP16-storage mode), built on demand
     float* s16 = nullptr;
     bool a16_valid = false;
@@ -49,12 +49,12 @@ struct CoarseLevel {
 // Workspace of the batched (multi-RHS) solve, sized for npad panel columns.
 struct BatchWork {
     int npad = 0, nrhs_cap = 0, K = 0, nc = 0;
-    float2 *rcB = nullptr, *yB = nullptr, *rB = nullptr, *sB = nullptr, *pB = nullptr, *qB = nullptr;
-    double* cgs = nullptr;          // 9 x npad per-RHS CG scalars
-    __half* bt = nullptr;           // split operand tiles of the tensor-core stencil
-    float* xpart = nullptr;         // Vc x npad
-    float* rpart = nullptr;         // kBatchRowChunks x npad
-    int* flags = nullptr;           // [0] active columns, [1] error
+    float2 *rcB = nullptr, *yB = nullptr, *rB = nullptr, *sB = nullptr, *pB = nullptr, *qB = nullptr, *uB = nullptr,
+           *zB = nullptr;
+    __half *bts = nullptr, *btu = nullptr;   // operand tiles of the tensor-core stencil
+    unsigned int* sync = nullptr;   // grid barrier and grid sums of the coarse kernel
+    double* iters = nullptr;        // npad
+    int* flags = nullptr;           // [0] error
     int* h_flags = nullptr;         // pinned
     double* h_iters = nullptr;      // pinned, npad
     float2* r32 = nullptr;          // nrhs x n
@@ -64,9 +64,6 @@ struct BatchWork {
     double2* b64 = nullptr;         // nrhs x n
     double* scal = nullptr;         // nrhs x S_COUNT
     double* h_scal = nullptr;       // pinned nrhs x S_COUNT
-    cudaStream_t cap = nullptr;     // capture stream
-    cudaGraphExec_t graph = nullptr;
-    long long graph_key[6] = {0, 0, 0, 0, 0, 0};
 };
 
 // Workspace of the red-black preconditioned CG (checkerboard layout).
@@ -329,14 +326,14 @@ template <typename T> int ensure_work(mg_ctx* ctx) {
 int ensure_level(mg_ctx* ctx, CoarseLevel& L, int nv) {
     if (L.cap < nv) {
         // every buffer sized by the capacity goes, the derived ones (FP16 copy,
-        // tensor-core embedding) are rebuilt at the new size on demand
+        // tensor-core tiles) are rebuilt at the new size on demand
         CK(cudaStreamSynchronize(ctx->st));
-        for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.Aemb, (void*)L.A16,
+        for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.At, (void*)L.A16,
                         (void*)L.s16})
             dfree(ctx, q);
         L.P64 = nullptr; L.P32 = nullptr; L.A64 = nullptr; L.A32 = nullptr;
-        L.Aemb = nullptr; L.A16 = nullptr; L.s16 = nullptr;
-        L.emb_valid = L.a16_valid = L.au_valid = L.valid = false;
+        L.At = nullptr; L.A16 = nullptr; L.s16 = nullptr;
+        L.at_valid = L.a16_valid = L.au_valid = L.valid = false;
         size_t np = (size_t)nv * nfine(ctx);
         size_t na = (size_t)ctx->g.Vc * 9 * (2 * nv) * (2 * nv);
         TRY(dalloc(ctx, &L.P64, sizeof(double2) * np));
@@ -390,7 +387,7 @@ int build_level(mg_ctx* ctx, CoarseLevel& L, const double2* V, int nv) {
     CKL();
     L.mass = ctx->mass;
     L.valid = true;
-    L.emb_valid = false;
+    L.at_valid = false;
     L.a16_valid = false;
     L.au_valid = false;
     return MG_OK;
@@ -769,12 +766,12 @@ int clear_epoch_tags(mg_ctx* ctx) {
 int ensure_level2(mg_ctx* ctx, CoarseLevel& L, int nv2) {
     if (L.cap < nv2) {
         CK(cudaStreamSynchronize(ctx->st));
-        for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.Aemb, (void*)L.A16,
+        for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.At, (void*)L.A16,
                         (void*)L.s16})
             dfree(ctx, q);
         L.P64 = nullptr; L.P32 = nullptr; L.A64 = nullptr; L.A32 = nullptr;
-        L.Aemb = nullptr; L.A16 = nullptr; L.s16 = nullptr;
-        L.emb_valid = L.a16_valid = L.au_valid = L.valid = false;
+        L.At = nullptr; L.A16 = nullptr; L.s16 = nullptr;
+        L.at_valid = L.a16_valid = L.au_valid = L.valid = false;
         const size_t np = (size_t)nv2 * ctx->g.Vc * 2 * ctx->prm.nvec;
         const size_t na = (size_t)ctx->g2.Vc * 9 * (2 * nv2) * (2 * nv2);
         TRY(dalloc(ctx, &L.P64, sizeof(double2) * np));
@@ -813,7 +810,7 @@ int build_level2(mg_ctx* ctx, CoarseLevel& L, const double2* V2, int nv2) {
     CKL();
     L.mass = ctx->mass;
     L.valid = true;
-    L.emb_valid = L.a16_valid = L.au_valid = false;
+    L.at_valid = L.a16_valid = L.au_valid = false;
     return MG_OK;
 }
 
@@ -1452,8 +1449,8 @@ void mg_destroy(mg_ctx* ctx) {
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
-    if (ctx->bw.graph) cudaGraphExecDestroy(ctx->bw.graph);
-    if (ctx->bw.cap) cudaStreamDestroy(ctx->bw.cap);
+    
+    
     if (ctx->bw.h_flags) cudaFreeHost(ctx->bw.h_flags);
     if (ctx->bw.h_iters) cudaFreeHost(ctx->bw.h_iters);
     if (ctx->bw.h_scal) cudaFreeHost(ctx->bw.h_scal);
@@ -1509,7 +1506,7 @@ int mg_set_mass(mg_ctx* ctx, double m) {
         convert<double, float>(ctx->full.A32, ctx->full.A64, (size_t)ctx->g.Vc * 9 * ctx->full.nc * ctx->full.nc, ctx->st);
         CKL();
         ctx->full.mass = m;
-        ctx->full.emb_valid = false;
+        ctx->full.at_valid = false;
         ctx->full.a16_valid = false;
         ctx->full.au_valid = false;
     }
@@ -1519,7 +1516,7 @@ int mg_set_mass(mg_ctx* ctx, double m) {
         convert<double, float>(L.A32, L.A64, (size_t)ctx->g2.Vc * 9 * L.nc * L.nc, ctx->st);
         CKL();
         L.mass = m;
-        L.emb_valid = L.a16_valid = L.au_valid = false;
+        L.at_valid = L.a16_valid = L.au_valid = false;
     }
     ctx->mass = m;
     CK(cudaStreamSynchronize(ctx->st));
@@ -2522,22 +2519,19 @@ extern "C" int mg_solve_eo_cg(mg_ctx* ctx, const double* b, double* x, double to
 // ======================================================================= batched right-hand sides
 // Lockstep flexible GCR over nrhs sources: the fine-level steps of each source
 // use the single-source kernels, the coarse solve of all sources runs as one
-// batched CGNR on an RHS panel (tensor-core stencil, iterations replayed from a
-// captured CUDA graph), each source keeps its own GCR scalars.
+// batched CGNR on an RHS panel (one persistent launch, tensor-core stencil), each
+// source keeps its own GCR scalars.
 namespace {
-
-constexpr int kBatchCheck = 8;   // coarse iterations per graph replay between host checks
 
 int round16(int n) { return ((n + 15) / 16) * 16; }
 
-int ensure_embedding(mg_ctx* ctx, CoarseLevel& L) {
-    if (L.emb_valid) return MG_OK;
-    // per (X, d) block: the (2 nc) x (2 nc) real embedding, nc = 2 nv
-    const size_t kemb = (size_t)4 * L.cap;
-    if (!L.Aemb) TRY(dalloc(ctx, &L.Aemb, sizeof(__half) * (size_t)ctx->g.Vc * 9 * kemb * kemb));
-    coarse_embed(L.Aemb, L.A64, L.nc, ctx->g.Vc, ctx->st);
+int ensure_tiles(mg_ctx* ctx, CoarseLevel& L) {
+    if (L.at_valid) return MG_OK;
+    const size_t nc = (size_t)2 * L.cap;
+    if (!L.At) TRY(dalloc(ctx, &L.At, sizeof(__half) * (size_t)ctx->g.Vc * 9 * 2 * nc * nc));
+    coarse_tiles(L.At, L.A64, L.nc, ctx->g.Vc, ctx->st);
     CKL();
-    L.emb_valid = true;
+    L.at_valid = true;
     return MG_OK;
 }
 
@@ -2549,13 +2543,10 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
     if (b.npad >= npad && b.nrhs_cap >= nrhs && b.nc == nc && b.K >= K) return MG_OK;
     if (b.npad || b.nrhs_cap) {   // grow: release the smaller workspace first
         CK(cudaStreamSynchronize(ctx->st));
-        for (void* q : {(void*)b.rcB, (void*)b.yB, (void*)b.rB, (void*)b.sB, (void*)b.pB, (void*)b.qB, (void*)b.cgs,
-                        (void*)b.bt,
-                        (void*)b.xpart, (void*)b.rpart, (void*)b.flags, (void*)b.r32, (void*)b.Z, (void*)b.Pk,
-                        (void*)b.x64, (void*)b.b64, (void*)b.scal})
+        for (void* q : {(void*)b.rcB, (void*)b.yB, (void*)b.rB, (void*)b.sB, (void*)b.pB, (void*)b.qB, (void*)b.uB,
+                        (void*)b.zB, (void*)b.bts, (void*)b.btu, (void*)b.sync, (void*)b.iters, (void*)b.flags,
+                        (void*)b.r32, (void*)b.Z, (void*)b.Pk, (void*)b.x64, (void*)b.b64, (void*)b.scal})
             dfree(ctx, q);
-        if (b.graph) cudaGraphExecDestroy(b.graph);
-        if (b.cap) cudaStreamDestroy(b.cap);
         cudaFreeHost(b.h_flags);
         cudaFreeHost(b.h_iters);
         cudaFreeHost(b.h_scal);
@@ -2569,10 +2560,12 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
     TRY(dalloc(ctx, &b.sB, sizeof(float2) * pe));
     TRY(dalloc(ctx, &b.pB, sizeof(float2) * pe));
     TRY(dalloc(ctx, &b.qB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.cgs, sizeof(double) * 9 * npad));
-    TRY(dalloc(ctx, &b.bt, tc_split_bytes(nc, npad, ctx->g.Vc)));
-    TRY(dalloc(ctx, &b.xpart, sizeof(float) * (size_t)ctx->g.Vc * npad));
-    TRY(dalloc(ctx, &b.rpart, sizeof(float) * kBatchRowChunks * npad));
+    TRY(dalloc(ctx, &b.uB, sizeof(float2) * pe));
+    TRY(dalloc(ctx, &b.zB, sizeof(float2) * pe));
+    TRY(dalloc(ctx, &b.bts, bcg_tile_bytes(nc, npad, ctx->g.Vc)));
+    TRY(dalloc(ctx, &b.btu, bcg_tile_bytes(nc, npad, ctx->g.Vc)));
+    TRY(dalloc(ctx, &b.sync, bcg_sync_bytes(npad)));
+    TRY(dalloc(ctx, &b.iters, sizeof(double) * npad));
     TRY(dalloc(ctx, &b.flags, sizeof(int) * 4));
     TRY(dalloc(ctx, &b.r32, sizeof(float2) * n * nrhs));
     TRY(dalloc(ctx, &b.Z, sizeof(float2) * n * nrhs * K));
@@ -2583,7 +2576,6 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
     CK(cudaMallocHost(&b.h_flags, sizeof(int) * 4));
     CK(cudaMallocHost(&b.h_iters, sizeof(double) * npad));
     CK(cudaMallocHost(&b.h_scal, sizeof(double) * S_COUNT * nrhs));
-    CK(cudaStreamCreateWithFlags(&b.cap, cudaStreamNonBlocking));
     CK(cudaMemsetAsync(b.scal, 0, sizeof(double) * S_COUNT * nrhs, ctx->st));
     CK(cudaMemsetAsync(b.flags, 0, sizeof(int) * 4, ctx->st));
     b.npad = npad;
@@ -2593,70 +2585,27 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
     return MG_OK;
 }
 
-BatchCg batch_cg(mg_ctx* ctx, double tol, int maxit, int nrhs) {
-    BatchWork& b = ctx->bw;
-    BatchCg c;
-    c.Aemb = ctx->full.Aemb;
-    c.bt = b.bt;
-    c.stages = 0;
-    c.y = b.yB; c.r = b.rB; c.s = b.sB; c.p = b.pB; c.q = b.qB; c.rc = b.rcB;
-    c.nc = ctx->full.nc; c.npad = b.npad; c.nw = b.npad; c.nrhs = nrhs; c.maxit = maxit;
-    c.tol2 = tol * tol;
-    c.g = ctx->g;
-    c.S.scale = b.cgs; c.S.done = b.cgs + b.npad; c.S.iters = b.cgs + 2 * b.npad; c.S.r2 = b.cgs + 3 * b.npad;
-    c.S.gamma = b.cgs + 4 * b.npad; c.S.alpha = b.cgs + 5 * b.npad; c.S.beta = b.cgs + 6 * b.npad;
-    c.S.csp = b.cgs + 7 * b.npad; c.S.csr = b.cgs + 8 * b.npad;
-    c.xpart = b.xpart; c.rpart = b.rpart; c.active = b.flags; c.err = b.flags + 1;
-    return c;
-}
-
 // CGNR on the panel rcB -> yB for columns 0..nrhs-1 (zero columns stay zero).
 // iters_out[n] += coarse iterations of column n.
 int batched_coarse_solve(mg_ctx* ctx, int nrhs, double tol, int maxit, std::vector<double>& iters_out) {
     BatchWork& b = ctx->bw;
-    TRY(ensure_embedding(ctx, ctx->full));
-    CK(coarse_apply_tc_prepare(ctx->full.nc, b.npad));
-    BatchCg c = batch_cg(ctx, tol, maxit, nrhs);
-    {   // tile width from the autotuner (timed on the panel buffers once per shape)
-        TcApplyArgs t{c.Aemb, c.p, c.q, c.nc, c.npad, 0, 0, c.g, nullptr, c.err, nullptr, c.bt, 0};
-        c.nw = coarse_apply_tc_tune(t, ctx->st, &c.stages);
-        CKL();
-    }
-    long long tolbits = 0;
-    std::memcpy(&tolbits, &c.tol2, sizeof(tolbits));
-    long long key[6] = {(long long)(size_t)c.Aemb, b.npad, nrhs, maxit, tolbits,
-                        (ctx->full.nc * 1024 + c.nw) * 4 + c.stages};
-    if (!b.graph || std::memcmp(key, b.graph_key, sizeof(key)) != 0) {
-        if (b.graph) { cudaGraphExecDestroy(b.graph); b.graph = nullptr; }
-        cudaGraph_t gr;
-        CK(cudaStreamBeginCapture(b.cap, cudaStreamCaptureModeThreadLocal));
-        for (int j = 0; j < kBatchCheck; ++j) bcg_iteration(c, b.cap);
-        CK(cudaStreamEndCapture(b.cap, &gr));
-        // captured launches run only when the graph is replayed (counted there)
-        launch_counter().fetch_sub(kBatchCheck * kBcgKernelsPerIteration, std::memory_order_relaxed);
-        cudaError_t e = cudaGraphInstantiate(&b.graph, gr, 0);
-        cudaGraphDestroy(gr);
-        CK(e);
-        std::memcpy(b.graph_key, key, sizeof(key));
-    }
+    TRY(ensure_tiles(ctx, ctx->full));
+    BcgArgs c{};
+    c.At = ctx->full.At; c.bts = b.bts; c.btu = b.btu; c.rc = b.rcB;
+    c.y = b.yB; c.r = b.rB; c.s = b.sB; c.u = b.uB; c.p = b.pB; c.z = b.zB; c.q = b.qB;
+    c.nbr = ctx->cnbr; c.bar = b.sync; c.err = b.flags; c.iters = b.iters;
+    c.nc = ctx->full.nc; c.npad = b.npad; c.nrhs = nrhs; c.maxit = maxit; c.mode = BCG_SOLVE; c.tol2 = tol * tol;
+    c.g = ctx->g;
     PROF_BEGIN(MG_K_COARSE_SOLVE);
-    bcg_start(c, ctx->st);
-    CKL();
-    int done_its = 0;
-    for (;;) {
-        CK(cudaGraphLaunch(b.graph, ctx->st));
-        launch_counter().fetch_add(kBatchCheck * kBcgKernelsPerIteration, std::memory_order_relaxed);
-        done_its += kBatchCheck;
-        CK(cudaMemcpyAsync(b.h_flags, b.flags, sizeof(int) * 2, cudaMemcpyDeviceToHost, ctx->st));
-        CK(cudaStreamSynchronize(ctx->st));
-        if (b.h_flags[1]) return fail(ctx, MG_ERR_TIMEOUT, "batched coarse stencil: a bounded wait gave up");
-        if (b.h_flags[0] == 0 || done_its >= maxit) break;
-    }
-    bcg_finish(c, ctx->st);
+    CK(bcg_launch(c, ctx->st));
     PROF_END(MG_K_COARSE_SOLVE);
-    CKL();
-    CK(cudaMemcpyAsync(b.h_iters, c.S.iters, sizeof(double) * b.npad, cudaMemcpyDeviceToHost, ctx->st));
+    CK(cudaMemcpyAsync(b.h_flags, b.flags, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+    CK(cudaMemcpyAsync(b.h_iters, b.iters, sizeof(double) * b.npad, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
+    if (b.h_flags[0]) {
+        CK(cudaMemsetAsync(b.flags, 0, sizeof(int) * 4, ctx->st));
+        return fail(ctx, MG_ERR_TIMEOUT, "batched coarse solve: a bounded wait gave up");
+    }
     for (int n = 0; n < nrhs; ++n) iters_out[n] += b.h_iters[n];
     return MG_OK;
 }
@@ -2864,7 +2813,8 @@ int mg_solve_batched_device(mg_ctx* ctx, const double* b_dev, double* x_dev, int
     }
     if (nrhs > 256) return fail(ctx, MG_ERR_INVALID_ARG, "at most 256 sources per batch");
     if (ctx->prm.levels != 2) return fail(ctx, MG_ERR_INVALID_ARG, "the batched solve runs the two-level cycle");
-    if (!coarse_apply_tc_supported(ctx->full.nc, round16(nrhs)))
+    int nw = 0, stages = 0;
+    if (ctx->full.nc % 8 || !bcg_shape(ctx->full.nc, round16(nrhs), ctx->g.Vc, &nw, &stages))
         return fail(ctx, MG_ERR_INVALID_ARG, "batched coarse stencil needs 2*nvec a multiple of 16 and <= 128");
     TRY(ensure_batch(ctx, nrhs));
     for (int r = 0; r < nrhs; ++r)
@@ -2901,56 +2851,74 @@ int mg_solve_batched(mg_ctx* ctx, const double* b, double* x, int nrhs, mg_solve
     return st;
 }
 
+namespace {
+// arguments and scratch of one stencil application on a panel; the caller frees tmp
+int bcg_apply_args(mg_ctx* ctx, int npad, int nrhs, bool dag, BcgArgs* out, std::vector<void*>& tmp) {
+    CoarseLevel& L = ctx->full;
+    int nw = 0, stages = 0;
+    if (!bcg_shape(L.nc, npad, ctx->g.Vc, &nw, &stages)) return fail(ctx, MG_ERR_INVALID_ARG, "unsupported shape");
+    const size_t npanel = (size_t)ctx->g.Vc * L.nc * npad;
+    BcgArgs a{};
+    float2* x = nullptr;
+    int* fl = nullptr;
+    auto get = [&](auto** p, size_t bytes) {
+        int st = dalloc(ctx, p, bytes);
+        if (st == MG_OK) tmp.push_back(*p);
+        return st;
+    };
+    TRY(get(&x, sizeof(float2) * npanel));
+    TRY(get(&a.y, sizeof(float2) * npanel));
+    TRY(get(&a.bts, bcg_tile_bytes(L.nc, npad, ctx->g.Vc)));
+    TRY(get(&a.btu, bcg_tile_bytes(L.nc, npad, ctx->g.Vc)));
+    TRY(get(&a.bar, bcg_sync_bytes(npad)));
+    TRY(get(&fl, sizeof(int) * 4));
+    CK(cudaMemsetAsync(fl, 0, sizeof(int) * 4, ctx->st));
+    TRY(ensure_tiles(ctx, L));
+    a.At = L.At; a.rc = x; a.nbr = ctx->cnbr; a.err = fl;
+    a.nc = L.nc; a.npad = npad; a.nrhs = nrhs; a.mode = BCG_APPLY; a.dag = dag ? 1 : 0; a.g = ctx->g;
+    *out = a;
+    return MG_OK;
+}
+void release(mg_ctx* ctx, const std::vector<void*>& tmp) {
+    for (void* q : tmp) dfree(ctx, q);
+}
+}  // namespace
+
 int mg_time_coarse_batched(mg_ctx* ctx, int nrhs, int reps, double* ms_per_launch, double* bytes_per_launch,
                            double* flops_per_launch) {
     TRY(need_level(ctx));
     if (nrhs <= 0 || nrhs > 256 || reps <= 0 || !ms_per_launch) return MG_ERR_INVALID_ARG;
-    CoarseLevel& L = ctx->full;
+    const CoarseLevel& L = ctx->full;
     const int npad = round16(nrhs);
-    if (!coarse_apply_tc_supported(L.nc, npad)) return fail(ctx, MG_ERR_INVALID_ARG, "unsupported shape");
     const size_t npanel = (size_t)ctx->g.Vc * L.nc * npad;
-    float2 *pa = nullptr, *pb = nullptr;
-    int* err = nullptr;
-    __half* bt = nullptr;
-    TRY(dalloc(ctx, &pa, sizeof(float2) * npanel));
-    TRY(dalloc(ctx, &pb, sizeof(float2) * npanel));
-    TRY(dalloc(ctx, &err, sizeof(int) * 4));
-    TRY(dalloc(ctx, &bt, tc_split_bytes(L.nc, npad, ctx->g.Vc)));
-    auto release = [&]() {
-        for (void* q : {(void*)pa, (void*)pb, (void*)err, (void*)bt}) {
-            for (size_t i = 0; i < ctx->allocs.size(); ++i)
-                if (ctx->allocs[i] == q) { ctx->allocs.erase(ctx->allocs.begin() + i); break; }
-            cudaFree(q);
-        }
-    };
-    int st = MG_OK;
-    do {
-        if ((st = ensure_embedding(ctx, L)) != MG_OK) break;
-        if (cudaMemsetAsync(err, 0, sizeof(int) * 4, ctx->st) != cudaSuccess ||
-            cudaMemsetAsync(pb, 0, sizeof(float2) * npanel, ctx->st) != cudaSuccess ||
-            coarse_apply_tc_prepare(L.nc, npad) != cudaSuccess) { st = fail(ctx, MG_ERR_CUDA, "probe setup"); break; }
+    std::vector<void*> tmp;
+    BcgArgs a{};
+    int st = bcg_apply_args(ctx, npad, nrhs, false, &a, tmp);
+    while (st == MG_OK) {   // once
         // a zero panel (the values do not change the work or its timing)
-        panel_pack(pa, nullptr, (long long)ctx->g.Vc * L.nc, 0, npad, ctx->st);
-        TcApplyArgs a{L.Aemb, pa, pb, L.nc, npad, 0, 0, ctx->g, nullptr, err, nullptr, bt, 0};
-        a.nw = coarse_apply_tc_tune(a, ctx->st, &a.stages);
-        for (int i = 0; i < 2; ++i) coarse_apply_tc(a, ctx->st);
+        panel_pack(const_cast<float2*>(a.rc), nullptr, (long long)ctx->g.Vc * L.nc, 0, npad, ctx->st);
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < 2 && e == cudaSuccess; ++i) e = bcg_launch(a, ctx->st);
         cudaEventRecord(ctx->ev0, ctx->st);
-        for (int i = 0; i < reps; ++i) coarse_apply_tc(a, ctx->st);
+        for (int i = 0; i < reps && e == cudaSuccess; ++i) e = bcg_launch(a, ctx->st);
         cudaEventRecord(ctx->ev1, ctx->st);
-        if (cudaEventSynchronize(ctx->ev1) != cudaSuccess) { st = fail(ctx, MG_ERR_CUDA, "probe launch"); break; }
+        if (e != cudaSuccess || cudaEventSynchronize(ctx->ev1) != cudaSuccess) {
+            st = fail(ctx, MG_ERR_CUDA, "probe launch");
+            break;
+        }
         float ms = 0;
         cudaEventElapsedTime(&ms, ctx->ev0, ctx->ev1);
         int h_err = 0;
-        cudaMemcpy(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost);
+        cudaMemcpy(&h_err, a.err, sizeof(int), cudaMemcpyDeviceToHost);
         if (h_err) { st = fail(ctx, MG_ERR_TIMEOUT, "batched coarse stencil: a bounded wait gave up"); break; }
         *ms_per_launch = (double)ms / reps;
-        const double K = 2.0 * L.nc;
-        // algorithmic: the FP16 embedded operator once, the FP32 panel read once and written once
-        if (bytes_per_launch) *bytes_per_launch = (double)ctx->g.Vc * 9 * K * K * 2 + 2.0 * npanel * sizeof(float2);
+        // algorithmic: the FP16 operator once, the FP32 panel read once and written once
+        if (bytes_per_launch) *bytes_per_launch = (double)ctx->g.Vc * 9 * L.nc * L.nc * 4 + 2.0 * npanel * sizeof(float2);
         // useful work: 9 complex nc x nc blocks times nrhs columns per aggregate (8 real flops per complex MAC)
         if (flops_per_launch) *flops_per_launch = 8.0 * 9 * L.nc * (double)L.nc * ctx->g.Vc * nrhs;
-    } while (false);
-    release();
+        break;
+    }
+    release(ctx, tmp);
     return st;
 }
 
@@ -2962,7 +2930,6 @@ int mg_apply_coarse_batched(mg_ctx* ctx, const double* x, double* y, int nrhs, i
     long long rows = (long long)ctx->g.Vc * L.nc;
     size_t nin = (size_t)rows * nrhs, npanel = (size_t)rows * npad;
     double2 *hin = nullptr, *hout = nullptr, *p64a = nullptr, *p64b = nullptr;
-    float2 *pa = nullptr, *pb = nullptr;
     // each source scaled to max |x| = 1 (the FP16 panel of the tensor-core path has
     // no subnormal headroom), scaled back afterwards
     std::vector<double> scale(nrhs, 1.0), xs((size_t)2 * nin);
@@ -2978,26 +2945,16 @@ int mg_apply_coarse_batched(mg_ctx* ctx, const double* x, double* y, int nrhs, i
     std::vector<void*> tmp = {hin, hout};
     int st = MG_OK;
     if (impl == 0) {
-        if (!coarse_apply_tc_supported(L.nc, npad)) return fail(ctx, MG_ERR_INVALID_ARG, "unsupported shape");
-        TRY(dalloc(ctx, &pa, sizeof(float2) * npanel));
-        TRY(dalloc(ctx, &pb, sizeof(float2) * npanel));
-        tmp.push_back(pa);
-        tmp.push_back(pb);
-        TRY(dalloc(ctx, &p64a, sizeof(int) * 4));   // error flag
-        tmp.push_back(p64a);
-        __half* bt = nullptr;
-        TRY(dalloc(ctx, &bt, tc_split_bytes(L.nc, npad, ctx->g.Vc)));
-        tmp.push_back(bt);
-        CK(cudaMemsetAsync(p64a, 0, sizeof(int) * 4, ctx->st));
-        TRY(ensure_embedding(ctx, ctx->full));
-        panel_pack(pa, hin, rows, nrhs, npad, ctx->st);
-        CK(coarse_apply_tc_prepare(L.nc, npad));
-        TcApplyArgs a{L.Aemb, pa, pb, L.nc, npad, 0, dagger ? 1 : 0, ctx->g, nullptr, (int*)p64a, nullptr, bt, 0};
-        a.nw = coarse_apply_tc_tune(a, ctx->st, &a.stages);
-        CK(coarse_apply_tc(a, ctx->st));
-        panel_unpack(hout, pb, rows, nrhs, npad, ctx->st);
+        BcgArgs a{};
+        if ((st = bcg_apply_args(ctx, npad, nrhs, dagger != 0, &a, tmp)) != MG_OK) {
+            release(ctx, tmp);
+            return st;
+        }
+        panel_pack(const_cast<float2*>(a.rc), hin, rows, nrhs, npad, ctx->st);
+        CK(bcg_launch(a, ctx->st));
+        panel_unpack(hout, a.y, rows, nrhs, npad, ctx->st);
         int err = 0;
-        CK(cudaMemcpyAsync(&err, p64a, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+        CK(cudaMemcpyAsync(&err, a.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
         CK(cudaStreamSynchronize(ctx->st));
         if (err) st = fail(ctx, MG_ERR_TIMEOUT, "batched coarse stencil: a bounded wait gave up");
     } else {
@@ -3016,11 +2973,7 @@ int mg_apply_coarse_batched(mg_ctx* ctx, const double* x, double* y, int nrhs, i
         for (int r = 0; r < nrhs; ++r)
             for (long long i = 0; i < 2 * rows; ++i) y[(size_t)r * 2 * rows + i] *= scale[r];
     }
-    for (void* q : tmp) {
-        for (size_t i = 0; i < ctx->allocs.size(); ++i)
-            if (ctx->allocs[i] == q) { ctx->allocs.erase(ctx->allocs.begin() + i); break; }
-        cudaFree(q);
-    }
+    release(ctx, tmp);
     return st;
 }
 

@@ -321,75 +321,38 @@ void coarse_pack16(__half2* A16, float* s16, const double2* A, int nc, int Vc, c
 
 // ---------------------------------------------------------------- batched (multi-RHS) coarse level
 // Panel layout xB[X][b][n], n < npad (multiple of 16), complex FP32.
-// Aemb: per (X, d) the 2nc x 2nc real embedding of A[X][d] in FP16, tensor-core layout.
-void coarse_embed(__half* Aemb, const double2* A, int nc, int Vc, cudaStream_t st);
-struct TcApplyArgs {
-    const __half* Aemb;
-    const float2* x;
-    float2* y;
-    int nc;
-    int npad;
-    int nw;         // panel columns per CTA (multiple of 16 dividing npad; 0: all)
-    int dag;
-    Geom g;
-    float* norms;   // optional per-aggregate column sums of |y|^2: [Vc][npad]
-    int* err;       // set to 1 if a bounded wait gave up
-    const double* colscale;   // optional per-column power-of-two factor applied to x before the
-                              // FP16 hi/lo split (y is scaled back exactly); nullptr: 1
-    __half* bt;     // scratch for the split operand panel: tc_split_bytes(nc, npad) bytes
-    int stages;     // pipeline stages per CTA (2 or 3; 0: as many as fit, up to 3)
-};
-// bytes of the FP16 hi/lo operand tiles of one panel (any chunk width)
-inline size_t tc_split_bytes(int nc, int npad, long long Vc) { return (size_t)Vc * npad * (2 * nc) * 2 * sizeof(__half); }
-// y = D_c x (dag: sigma3 D_c sigma3 x) for the whole panel on tcgen05 tensor cores;
-// coarse_apply_tc_prepare(nc, npad) once per shape before launching (and before any capture)
-bool coarse_apply_tc_supported(int nc, int npad);
-cudaError_t coarse_apply_tc_prepare(int nc, int npad);
-cudaError_t coarse_apply_tc(const TcApplyArgs& args, cudaStream_t st);
-// autotuner: fastest chunk width (returned) and pipeline depth (*stages) for
-// args' (nc, npad), timed once and cached
-int coarse_apply_tc_tune(const TcApplyArgs& args, cudaStream_t st, int* stages);
-// kernels launched by one bcg_iteration
-constexpr int kBcgKernelsPerIteration = 10;   // two stencils of two launches each + six
+// At: per (X, d) the FP16 rows [Re A; Im A] of A[X][d] in tensor-core tiles (2 nc^2 halves each)
+void coarse_tiles(__half* At, const double2* A, int nc, int Vc, cudaStream_t st);
 // SIMT reference of the same contraction with the FP64 operator
 template <typename T>
 void coarse_apply_batched_simt(v2<T>* y, const double2* A, const v2<T>* x, int nc, int npad, bool dag, const Geom& g,
                                cudaStream_t st);
 
-struct BatchScal {   // per-RHS CG scalars, npad doubles each
-    double* scale;
-    double* done;
-    double* iters;
-    double* r2;
-    double* gamma;
-    double* alpha;
-    double* beta;
-    double* csp;     // power-of-two panel scales of p and r for the FP16 split (from |s|^2, |r|^2)
-    double* csr;
-};
-struct BatchCg {
-    const __half* Aemb;
-    __half* bt;      // split operand tiles of the stencil (scratch)
-    int stages;      // pipeline depth of the stencil (from the autotuner)
-    float2* y;
-    float2* r;
-    float2* s;
-    float2* p;
-    float2* q;
-    const float2* rc;
-    int nc, npad, nw, nrhs, maxit;
+// The batched coarse kernel (one persistent cooperative launch): BCG_SOLVE CGNR on
+// the panel rc -> y, BCG_APPLY y = D_c rc (dag: D_c^dag rc).
+enum { BCG_SOLVE = 0, BCG_APPLY = 1 };
+struct BcgArgs {
+    const __half* At;
+    __half *bts, *btu;       // operand tiles, bcg_tile_bytes each
+    const float2* rc;        // panels [Vc][nc][npad]
+    float2 *y, *r, *s, *u, *p, *z, *q;   // BCG_APPLY: y only
+    const int* nbr;          // coarse neighbour table [Vc][9]
+    unsigned int* bar;       // bcg_sync_bytes(npad), 8-byte aligned, cleared by the launcher: grid barrier
+                             // counter, then (set by the launcher)
+    unsigned int* mx;        // [npad] sizes of the right-hand sides and
+    unsigned long long* sums;   // [2][3][npad] fixed-point grid sums
+    int* err;                // set to 1 if a bounded wait gave up
+    double* iters;           // [npad] CG iterations (BCG_SOLVE)
+    int nc, npad, nrhs, maxit, mode, dag;
     double tol2;
     Geom g;
-    BatchScal S;
-    float* xpart;    // [Vc][npad]
-    float* rpart;    // [kBatchRowChunks][npad]
-    int* active;     // columns still iterating after the last check
-    int* err;
+    int nw, stages;          // columns per job, pipeline depth (set by the launcher)
+    uint32_t tmem_cols;      // (set by the launcher)
 };
-constexpr int kBatchRowChunks = 1216;   // row chunks of the batched CG's column sums (8 per SM: enough warps to stream the panel)
-void bcg_start(const BatchCg& c, cudaStream_t st);
-void bcg_iteration(const BatchCg& c, cudaStream_t st);
-void bcg_finish(const BatchCg& c, cudaStream_t st);
+inline size_t bcg_sync_bytes(int npad) { return 16 + (size_t)npad * (4 + 2 * 3 * 8); }
+bool bcg_shape(int nc, int npad, int Vc, int* nw, int* stages);   // false: no shape for this panel
+size_t bcg_tile_bytes(int nc, int npad, long long Vc);
+cudaError_t bcg_launch(const BcgArgs& args, cudaStream_t st);
 // nrhs stacked FP64 coarse vectors in[n][row] <-> panel [row][npad]
 void panel_pack(float2* out, const double2* in, long long rows, int nrhs, int npad, cudaStream_t st);
 void panel_unpack(double2* out, const float2* in, long long rows, int nrhs, int npad, cudaStream_t st);
