@@ -98,33 +98,52 @@ void block_orthonormalize(double2* P, const double2* V, int nv, const Geom& g, i
 // ================================================================ restriction / prolongation
 // r_c[X][s*Nv + i] = <P_(X,s,i), r>: one CTA per (X, s); the chirality-s half of
 // r on X (6*Vb contiguous) is staged in shared memory, warp w handles i = w, w+8, ...
-template <typename T>
+// Bound by the bytes of P, so a CTA serves NS sources of a batch (lanes) with one
+// read of its panel: 12 sources on 16^3x32 read P three times instead of twelve.
+template <typename T, int NS>
 __global__ void __launch_bounds__(256) k_restrict(v2<T>* __restrict__ rc, const v2<T>* __restrict__ P,
-                                                  const v2<T>* __restrict__ r, int nv, Geom g, int cstride, int coff) {
+                                                  const v2<T>* __restrict__ r, int nv, Geom g, int cstride, int coff,
+                                                  Lanes ln) {
     extern __shared__ unsigned char smem_raw[];
     v2<T>* rs = reinterpret_cast<v2<T>*>(smem_raw);
+    const int n0 = blockIdx.y * NS, ns = NS == 1 ? 1 : min(NS, ln.m - n0);
     int X = blockIdx.x >> 1, s = blockIdx.x & 1;
     int len = 6 * g.Vb;
-    const v2<T>* rX = r + ((size_t)X * 12 + 6 * s) * g.Vb;
-    for (int e = threadIdx.x; e < len; e += blockDim.x) rs[e] = rX[e];
+    const v2<T>* rX = r + n0 * ln.a + ((size_t)X * 12 + 6 * s) * g.Vb;
+#pragma unroll
+    for (int n = 0; n < NS; ++n)
+        if (n < ns)
+            for (int e = threadIdx.x; e < len; e += blockDim.x) rs[n * len + e] = rX[n * ln.a + e];
     __syncthreads();
     int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const v2<T>* panel = P + ((size_t)X * 2 + s) * nv * len;
     for (int i = warp; i < nv; i += nw) {
         const v2<T>* pi = panel + (size_t)i * len;
-        cx<T> a(0, 0);
-        for (int e = lane; e < len; e += 32) cmadc(a, ldg<T>(pi + e), ld<T>(rs + e));
-        double ar = warp_sum((double)a.r), ai = warp_sum((double)a.i);
-        if (lane == 0) {
-            v2<T> o; o.x = (T)ar; o.y = (T)ai;
-            rc[((size_t)X * 2 * nv + s * nv + i) * cstride + coff] = o;
+        cx<T> a[NS];
+#pragma unroll
+        for (int n = 0; n < NS; ++n) a[n] = cx<T>(0, 0);
+        for (int e = lane; e < len; e += 32) {
+            const cx<T> p = ldg<T>(pi + e);
+#pragma unroll
+            for (int n = 0; n < NS; ++n)
+                if (n < ns) cmadc(a[n], p, ld<T>(rs + n * len + e));
+        }
+#pragma unroll
+        for (int n = 0; n < NS; ++n) {
+            double ar = warp_sum((double)a[n].r), ai = warp_sum((double)a[n].i);
+            if (lane == 0 && n < ns) {
+                v2<T> o; o.x = (T)ar; o.y = (T)ai;
+                rc[((size_t)X * 2 * nv + s * nv + i) * cstride + coff + n0 + n] = o;
+            }
         }
     }
 }
-// e[X][k][l] = sum_i P[X][s(k)][i][k%6][l] y[X][s(k)*Nv + i]
-template <typename T>
+// e[X][k][l] = sum_i P[X][s(k)][i][k%6][l] y[X][s(k)*Nv + i], NS sources per read of P
+template <typename T, int NS>
 __global__ void __launch_bounds__(256) k_prolong(v2<T>* __restrict__ e, const v2<T>* __restrict__ P,
-                                                 const v2<T>* __restrict__ yc, int nv, Geom g, int cstride, int coff) {
+                                                 const v2<T>* __restrict__ yc, int nv, Geom g, int cstride, int coff,
+                                                 Lanes ln) {
+    const int n0 = blockIdx.y * NS, ns = NS == 1 ? 1 : min(NS, ln.m - n0);
     long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;   // over V*12 as (X, k, l)
     long long total = g.V * 12;
     if (idx >= total) return;
@@ -135,23 +154,44 @@ __global__ void __launch_bounds__(256) k_prolong(v2<T>* __restrict__ e, const v2
     int s = k / 6, kk = k - 6 * s;
     int len = 6 * g.Vb;
     const v2<T>* p = P + (((size_t)X * 2 + s) * nv * 6 + kk) * g.Vb + l;
-    const v2<T>* y = yc + ((size_t)X * 2 * nv + s * nv) * cstride + coff;
-    cx<T> a(0, 0);
-    for (int i = 0; i < nv; ++i) cmad(a, ldg<T>(p + (size_t)i * len), ldg<T>(y + (size_t)i * cstride));
-    st<T>(e + idx, a);
+    const v2<T>* y = yc + ((size_t)X * 2 * nv + s * nv) * cstride + coff + n0;
+    cx<T> a[NS];
+#pragma unroll
+    for (int n = 0; n < NS; ++n) a[n] = cx<T>(0, 0);
+    for (int i = 0; i < nv; ++i) {
+        const cx<T> pi = ldg<T>(p + (size_t)i * len);
+#pragma unroll
+        for (int n = 0; n < NS; ++n)
+            if (n < ns) cmad(a[n], pi, ldg<T>(y + (size_t)i * cstride + n));
+    }
+#pragma unroll
+    for (int n = 0; n < NS; ++n)
+        if (n < ns) st<T>(e + (n0 + n) * ln.a + idx, a[n]);
 }
 
+// sources per CTA: four, their staged halves within 48 KB of shared memory
+constexpr int kTransferSources = 4;
 template <typename T>
-void restrict_(v2<T>* rc, const v2<T>* P, const v2<T>* r, int nv, const Geom& g, cudaStream_t st, int cstride, int coff) {
-    size_t sm = sizeof(v2<T>) * 6 * g.Vb;
+void restrict_(v2<T>* rc, const v2<T>* P, const v2<T>* r, int nv, const Geom& g, cudaStream_t st, int cstride, int coff,
+               const Lanes& ln) {
+    constexpr int NS = kTransferSources;
+    const size_t sm = sizeof(v2<T>) * 6 * g.Vb;
     note_launch();
-    k_restrict<T><<<2 * g.Vc, kThreads, sm, st>>>(rc, P, r, nv, g, cstride, coff);
+    if (ln.m > 1 && NS * sm <= 48 * 1024)
+        k_restrict<T, NS><<<dim3(2 * g.Vc, (ln.m + NS - 1) / NS), kThreads, NS * sm, st>>>(rc, P, r, nv, g, cstride, coff, ln);
+    else
+        k_restrict<T, 1><<<dim3(2 * g.Vc, ln.m), kThreads, sm, st>>>(rc, P, r, nv, g, cstride, coff, ln);
 }
 template <typename T>
-void prolong(v2<T>* e, const v2<T>* P, const v2<T>* yc, int nv, const Geom& g, cudaStream_t st, int cstride, int coff) {
-    long long total = g.V * 12;
+void prolong(v2<T>* e, const v2<T>* P, const v2<T>* yc, int nv, const Geom& g, cudaStream_t st, int cstride, int coff,
+             const Lanes& ln) {
+    constexpr int NS = kTransferSources;
+    const unsigned int grid = (unsigned int)((g.V * 12 + kThreads - 1) / kThreads);
     note_launch();
-    k_prolong<T><<<(int)((total + kThreads - 1) / kThreads), kThreads, 0, st>>>(e, P, yc, nv, g, cstride, coff);
+    if (ln.m > 1)
+        k_prolong<T, NS><<<dim3(grid, (ln.m + NS - 1) / NS), kThreads, 0, st>>>(e, P, yc, nv, g, cstride, coff, ln);
+    else
+        k_prolong<T, 1><<<grid, kThreads, 0, st>>>(e, P, yc, nv, g, cstride, coff, ln);
 }
 
 // ================================================================ coarse operator build
@@ -536,8 +576,10 @@ void cg_step(v2<T>* y, v2<T>* r, v2<T>* s, v2<T>* p, v2<T>* q, const v2<T>* A, i
 }
 
 #define INST(T)                                                                                                     \
-    template void restrict_<T>(v2<T>*, const v2<T>*, const v2<T>*, int, const Geom&, cudaStream_t, int, int);       \
-    template void prolong<T>(v2<T>*, const v2<T>*, const v2<T>*, int, const Geom&, cudaStream_t, int, int);         \
+    template void restrict_<T>(v2<T>*, const v2<T>*, const v2<T>*, int, const Geom&, cudaStream_t, int, int,        \
+                               const Lanes&);                                                                       \
+    template void prolong<T>(v2<T>*, const v2<T>*, const v2<T>*, int, const Geom&, cudaStream_t, int, int,          \
+                             const Lanes&);                                                                         \
     template void coarse_apply<T>(v2<T>*, const v2<T>*, const v2<T>*, int, bool, int, const Geom&, const Reduce&,    \
                                   cudaStream_t);                                                                    \
     template void cg_init<T>(v2<T>*, v2<T>*, const v2<T>*, size_t, double, int, const Reduce&, cudaStream_t);       \

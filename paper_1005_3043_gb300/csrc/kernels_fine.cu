@@ -196,7 +196,11 @@ constexpr int kDslashOneWave = 7, kDslashMultiWave = 5;
 template <typename T, int MODE, int MINB>
 __global__ void __launch_bounds__(DslashShape<T, MINB>::threads, DslashShape<T, MINB>::blocks)
     k_dslash(v2<T>* __restrict__ out, const v2<T>* __restrict__ in, const v2<T>* __restrict__ U,
-             const v2<T>* __restrict__ src, Geom g, T diag, double omega, int slot, Reduce R) {
+             const v2<T>* __restrict__ src, Geom g, T diag, double omega, int slot, Reduce R, Lanes ln) {
+    out += blockIdx.y * ln.a;
+    in += blockIdx.y * ln.b;
+    src += blockIdx.y * ln.c;
+    R = R.lane(blockIdx.y);
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     T red[3] = {0, 0, 0};   // per-site partial sums in T, promoted once for the grid reduction
     if (s < g.V) {
@@ -252,34 +256,34 @@ __global__ void __launch_bounds__(DslashShape<T, MINB>::threads, DslashShape<T, 
 
 template <typename T, int MINB>
 static void dslash_launch(int mode, v2<T>* out, const v2<T>* in, const v2<T>* U, const v2<T>* src, const Geom& g,
-                          T diag, double omega, int slot, const Reduce& R, cudaStream_t st) {
+                          T diag, double omega, int slot, const Reduce& R, cudaStream_t st, const Lanes& ln) {
     // FP64 in CTAs of one or two warps: the pipe issues two FMAs per clock and SM,
     // so every SM has to have its share of the sites.  With 256 threads 8^4 ran on
     // 16 SMs (74 us) and 12^3 x 24 left half of the SMs with twice the sites of the
     // others (121 us); FP32 waits on memory, and its reductions on the CTA count,
     // so it keeps its shape on every lattice.
     const int thr = sizeof(T) == 8 && g.V <= 256LL * device_sm_count() ? 32 : DslashShape<T, MINB>::threads;
-    const int grid = grid_for(g.V, thr);
+    const dim3 grid(grid_for(g.V, thr), ln.m);
     note_launch();
     switch (mode) {
-        case DS_PLAIN: k_dslash<T, DS_PLAIN, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R); break;
-        case DS_XMY: k_dslash<T, DS_XMY, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R); break;
+        case DS_PLAIN: k_dslash<T, DS_PLAIN, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R, ln); break;
+        case DS_XMY: k_dslash<T, DS_XMY, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R, ln); break;
         case DS_XMY_NORM:
-            k_dslash<T, DS_XMY_NORM, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R);
+            k_dslash<T, DS_XMY_NORM, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R, ln);
             break;
-        case DS_MRDOT: k_dslash<T, DS_MRDOT, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R); break;
+        case DS_MRDOT: k_dslash<T, DS_MRDOT, MINB><<<grid, thr, 0, st>>>(out, in, U, src, g, diag, omega, slot, R, ln); break;
     }
 }
 
 template <typename T>
 void dslash(int mode, v2<T>* out, const v2<T>* in, const v2<T>* U, const v2<T>* src, const Geom& g, double mass,
-            double omega, int slot, const Reduce& R, cudaStream_t st) {
+            double omega, int slot, const Reduce& R, cudaStream_t st, const Lanes& ln) {
     const T diag = (T)(4.0 + mass);
     const long long one_wave = (long long)device_sm_count() * kDslashOneWave * DslashShape<T, kDslashOneWave>::threads;
-    if (sizeof(T) == 8 || g.V <= one_wave)
-        dslash_launch<T, kDslashOneWave>(mode, out, in, U, src, g, diag, omega, slot, R, st);
+    if (sizeof(T) == 8 || g.V * ln.m <= one_wave)
+        dslash_launch<T, kDslashOneWave>(mode, out, in, U, src, g, diag, omega, slot, R, st, ln);
     else
-        dslash_launch<T, kDslashMultiWave>(mode, out, in, U, src, g, diag, omega, slot, R, st);
+        dslash_launch<T, kDslashMultiWave>(mode, out, in, U, src, g, diag, omega, slot, R, st, ln);
 }
 
 // ================================================================ BLAS-1
@@ -289,7 +293,9 @@ template <typename T> __global__ void k_zero(v2<T>* x, size_t n) {
         x[i] = z;
     }
 }
-template <typename T> __global__ void k_norm2(const v2<T>* __restrict__ x, size_t n, int slot, Reduce R) {
+template <typename T> __global__ void k_norm2(const v2<T>* __restrict__ x, size_t n, int slot, Reduce R, Lanes ln) {
+    x += blockIdx.y * ln.a;
+    R = R.lane(blockIdx.y);
     T a = 0;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         a += norm2(ld<T>(x + i));
@@ -320,8 +326,12 @@ template <typename T> __global__ void k_axpy(v2<T>* y, const v2<T>* __restrict__
     }
 }
 template <typename T>
-__global__ void k_mr_update(v2<T>* e, v2<T>* r, const v2<T>* __restrict__ q, size_t n, bool update_r,
-                            const double* __restrict__ scal) {
+__global__ void k_mr_update(v2<T>* e, v2<T>* r, const v2<T>* __restrict__ q, size_t n, bool update_r, Reduce R,
+                            Lanes ln) {
+    const double* scal = R.lane(blockIdx.y).scal;
+    e += blockIdx.y * ln.a;
+    r += blockIdx.y * ln.b;
+    q += blockIdx.y * ln.b;
     cx<T> a((T)scal[S_MR_ALPHA], (T)scal[S_MR_ALPHA + 1]);
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         cx<T> ri = ld<T>(r + i);
@@ -350,9 +360,9 @@ template <typename T> void zero(v2<T>* x, size_t n, cudaStream_t st) {
     note_launch();
     k_zero<T><<<stream_grid(n), kThreads, 0, st>>>(x, n);
 }
-template <typename T> void norm2(const v2<T>* x, size_t n, int slot, const Reduce& R, cudaStream_t st) {
+template <typename T> void norm2(const v2<T>* x, size_t n, int slot, const Reduce& R, cudaStream_t st, const Lanes& ln) {
     note_launch();
-    k_norm2<T><<<reduce_grid(n), kThreads, 0, st>>>(x, n, slot, R);
+    k_norm2<T><<<dim3(reduce_grid(n), ln.m), kThreads, 0, st>>>(x, n, slot, R, ln);
 }
 template <typename T> void dot(const v2<T>* x, const v2<T>* y, size_t n, int slot, const Reduce& R, cudaStream_t st) {
     note_launch();
@@ -367,9 +377,10 @@ template <typename T> void axpy(v2<T>* y, const v2<T>* x, size_t n, double ar, d
     k_axpy<T><<<stream_grid(n), kThreads, 0, st>>>(y, x, n, (T)ar, (T)ai);
 }
 template <typename T>
-void mr_update(v2<T>* e, v2<T>* r, const v2<T>* q, size_t n, bool update_r, const Reduce& R, cudaStream_t st) {
+void mr_update(v2<T>* e, v2<T>* r, const v2<T>* q, size_t n, bool update_r, const Reduce& R, cudaStream_t st,
+               const Lanes& ln) {
     note_launch();
-    k_mr_update<T><<<stream_grid(n), kThreads, 0, st>>>(e, r, q, n, update_r, R.scal);
+    k_mr_update<T><<<dim3(stream_grid(n), ln.m), kThreads, 0, st>>>(e, r, q, n, update_r, R, ln);
 }
 template <typename T> void normalize_dev(v2<T>* x, size_t n, int slot, const Reduce& R, cudaStream_t st) {
     note_launch();
@@ -409,7 +420,9 @@ template <typename T> struct BasisVec {
 // Measured with the reductions of mg_common.cuh: the Krylov kernels of one solve
 // 35.6 -> 20.1 ms on 16^3x32 (FP32, GMRES(12)), 67 -> 39 ms on 12^3x24 (FP64).
 template <typename T, int NJ, bool GM>
-__global__ void __launch_bounds__(kThreads) k_gcr_multidot(const v2<T>* __restrict__ basis, size_t n, int k, Reduce R) {
+__global__ void __launch_bounds__(kThreads) k_gcr_multidot(const v2<T>* __restrict__ basis, size_t n, int k, Reduce R, Lanes ln) {
+    basis += blockIdx.y * ln.a;
+    R = R.lane(blockIdx.y);
     constexpr int E = BasisVec<T>::E;
     T a[2 * NJ];
 #pragma unroll
@@ -443,7 +456,9 @@ __global__ void __launch_bounds__(kThreads) k_gcr_multidot(const v2<T>* __restri
 // recorded as h_{k,k-1} (k = 0: the norm of the residual, nothing to subtract or
 // store) with its reciprocal f_k (0 for a zero vector: a breakdown ends the space).
 template <typename T, int NJ, bool GM>
-__global__ void __launch_bounds__(kThreads) k_gcr_orth_norm(v2<T>* basis, size_t n, int k, Reduce R) {
+__global__ void __launch_bounds__(kThreads) k_gcr_orth_norm(v2<T>* basis, size_t n, int k, Reduce R, Lanes ln) {
+    basis += blockIdx.y * ln.a;
+    R = R.lane(blockIdx.y);
     constexpr int E = BasisVec<T>::E;
     __shared__ T beta[2 * NJ];
     for (int j = threadIdx.x; j < k; j += blockDim.x) {
@@ -489,7 +504,11 @@ __global__ void __launch_bounds__(kThreads) k_gcr_orth_norm(v2<T>* basis, size_t
     });
 }
 template <typename T>
-__global__ void k_gcr_cdot(const v2<T>* __restrict__ basis, const v2<T>* __restrict__ r, size_t n, int k, Reduce R) {
+__global__ void k_gcr_cdot(const v2<T>* __restrict__ basis, const v2<T>* __restrict__ r, size_t n, int k, Reduce R,
+                           Lanes ln) {
+    basis += blockIdx.y * ln.a;
+    r += blockIdx.y * ln.b;
+    R = R.lane(blockIdx.y);
     const v2<T>* pk = basis + (size_t)k * n;
     cx<T> a(0, 0);
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -505,7 +524,10 @@ __global__ void k_gcr_cdot(const v2<T>* __restrict__ basis, const v2<T>* __restr
     });
 }
 template <typename T>
-__global__ void k_gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, Reduce R) {
+__global__ void k_gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, Reduce R, Lanes ln) {
+    basis += blockIdx.y * ln.a;
+    r += blockIdx.y * ln.b;
+    R = R.lane(blockIdx.y);
     double nk = sqrt(R.scal[S_GCR_PN2]);
     T f = (T)(nk > 0 ? 1.0 / nk : 0.0);
     cx<T> c((T)R.scal[S_GCR_C + 2 * k], (T)R.scal[S_GCR_C + 2 * k + 1]);
@@ -541,41 +563,41 @@ template <typename T> static int basis_grid(size_t n) {
     return (int)std::max<size_t>(1, std::min(need, most));
 }
 template <typename T, bool GM>
-static void multidot_launch(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    const int grid = basis_grid<T>(n);
+static void multidot_launch(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
+    const dim3 grid(basis_grid<T>(n), ln.m);
     note_launch();
-    if (k <= 4) k_gcr_multidot<T, 4, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
-    else if (k <= 8) k_gcr_multidot<T, 8, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
-    else if (k <= 16) k_gcr_multidot<T, 16, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
-    else k_gcr_multidot<T, 32, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    if (k <= 4) k_gcr_multidot<T, 4, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
+    else if (k <= 8) k_gcr_multidot<T, 8, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
+    else if (k <= 16) k_gcr_multidot<T, 16, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
+    else k_gcr_multidot<T, 32, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
 }
 template <typename T, bool GM>
-static void orth_launch(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    const int grid = basis_grid<T>(n);
+static void orth_launch(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
+    const dim3 grid(basis_grid<T>(n), ln.m);
     note_launch();
-    if (k <= 4) k_gcr_orth_norm<T, 4, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
-    else if (k <= 8) k_gcr_orth_norm<T, 8, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
-    else if (k <= 16) k_gcr_orth_norm<T, 16, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
-    else k_gcr_orth_norm<T, 32, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R);
+    if (k <= 4) k_gcr_orth_norm<T, 4, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
+    else if (k <= 8) k_gcr_orth_norm<T, 8, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
+    else if (k <= 16) k_gcr_orth_norm<T, 16, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
+    else k_gcr_orth_norm<T, 32, GM><<<grid, kThreads, 0, st>>>(basis, n, k, R, ln);
 }
-template <typename T> void gcr_multidot(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    multidot_launch<T, false>(basis, n, k, R, st);
+template <typename T> void gcr_multidot(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
+    multidot_launch<T, false>(basis, n, k, R, st, ln);
 }
-template <typename T> void gcr_orth_norm(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    orth_launch<T, false>(basis, n, k, R, st);
+template <typename T> void gcr_orth_norm(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
+    orth_launch<T, false>(basis, n, k, R, st, ln);
 }
-template <typename T> void gmres_orth(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    if (k > 0) multidot_launch<T, true>(basis, n, k, R, st);
-    orth_launch<T, true>(basis, n, k, R, st);
+template <typename T> void gmres_orth(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
+    if (k > 0) multidot_launch<T, true>(basis, n, k, R, st, ln);
+    orth_launch<T, true>(basis, n, k, R, st, ln);
 }
 template <typename T>
-void gcr_cdot(const v2<T>* basis, const v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st) {
+void gcr_cdot(const v2<T>* basis, const v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
     note_launch();
-    k_gcr_cdot<T><<<reduce_grid(n), kThreads, 0, st>>>(basis, r, n, k, R);
+    k_gcr_cdot<T><<<dim3(reduce_grid(n), ln.m), kThreads, 0, st>>>(basis, r, n, k, R, ln);
 }
-template <typename T> void gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st) {
+template <typename T> void gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
     note_launch();
-    k_gcr_update<T><<<reduce_grid(n), kThreads, 0, st>>>(basis, r, n, k, R);
+    k_gcr_update<T><<<dim3(reduce_grid(n), ln.m), kThreads, 0, st>>>(basis, r, n, k, R, ln);
 }
 template <typename T>
 void gcr_xupdate(double2* x, const v2<T>* Z, size_t n, int k, const GcrCoef& y, cudaStream_t st) {
@@ -594,14 +616,15 @@ void gcr_xupdate(double2* x, const v2<T>* Z, size_t n, int k, const GcrCoef& y, 
 // recorded when basis[0] was normalised).  The space ends at the first zero
 // h_{j+1,j}.
 constexpr int kGmresMax = 16;   // largest smoother Krylov dimension (mg_params check)
-__global__ void k_gmres_ls(double* scal, int k, double omega) {
+__global__ void k_gmres_ls(Reduce R, int k, double omega) {
+    double* scal = R.lane(blockIdx.x).scal;   // one CTA per lane
     // one warp: lane jj owns column jj of the Hessenberg matrix (lane kGmresMax
     // the right-hand side g), so each Givens rotation is applied to all columns at
     // once with the same arithmetic per column as a serial sweep
     __shared__ double hr[kGmresMax + 1][kGmresMax + 1], hi[kGmresMax + 1][kGmresMax + 1];
     __shared__ int s_dim;
     const int lane = threadIdx.x;
-    if (blockIdx.x != 0 || lane >= 32 || k > kGmresMax) return;
+    if (lane >= 32 || k > kGmresMax) return;
     // H[i][j] = scal[rslot(i, j + 1)], i <= j + 1; column kGmresMax holds g = beta e_0
     for (int e = lane; e < (kGmresMax + 1) * (kGmresMax + 1); e += 32) {
         const int i = e / (kGmresMax + 1), j = e - i * (kGmresMax + 1);
@@ -675,7 +698,10 @@ __global__ void k_gmres_ls(double* scal, int k, double omega) {
 // z += sum_{j<k} c_j f_j basis[j], c_j = scal[S_GCR_C + 2j], f_j = scal[S_GMRES_F + j]
 template <typename T, int NJ>
 __global__ void __launch_bounds__(kThreads) k_multi_axpy(v2<T>* z, const v2<T>* __restrict__ basis, size_t n, int k,
-                                                         const double* __restrict__ scal) {
+                                                         Reduce R, Lanes ln) {
+    const double* scal = R.lane(blockIdx.y).scal;
+    z += blockIdx.y * ln.a;
+    basis += blockIdx.y * ln.b;
     constexpr int E = BasisVec<T>::E;
     __shared__ T c[2 * NJ];
     for (int j = threadIdx.x; j < k; j += blockDim.x) {
@@ -699,15 +725,16 @@ __global__ void __launch_bounds__(kThreads) k_multi_axpy(v2<T>* z, const v2<T>* 
         v.store(z + i);
     }
 }
-void gmres_ls(const Reduce& R, int k, double omega, cudaStream_t st) {
+void gmres_ls(const Reduce& R, int k, double omega, cudaStream_t st, const Lanes& ln) {
     note_launch();
-    k_gmres_ls<<<1, 32, 0, st>>>(R.scal, k, omega);
+    k_gmres_ls<<<ln.m, 32, 0, st>>>(R, k, omega);
 }
-template <typename T> void multi_axpy(v2<T>* z, const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st) {
-    const int grid = basis_grid<T>(n);
+template <typename T> void multi_axpy(v2<T>* z, const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st,
+                                       const Lanes& ln) {
+    const dim3 grid(basis_grid<T>(n), ln.m);
     note_launch();
-    if (k <= 8) k_multi_axpy<T, 8><<<grid, kThreads, 0, st>>>(z, basis, n, k, R.scal);
-    else k_multi_axpy<T, kGmresMax><<<grid, kThreads, 0, st>>>(z, basis, n, k, R.scal);
+    if (k <= 8) k_multi_axpy<T, 8><<<grid, kThreads, 0, st>>>(z, basis, n, k, R, ln);
+    else k_multi_axpy<T, kGmresMax><<<grid, kThreads, 0, st>>>(z, basis, n, k, R, ln);
 }
 
 // ================================================================ instantiations
@@ -716,21 +743,21 @@ template <typename T> void multi_axpy(v2<T>* z, const v2<T>* basis, size_t n, in
     template void spinor_from_internal<T>(double2*, const v2<T>*, const Geom&, cudaStream_t);                       \
     template void links_to_internal<T>(v2<T>*, const double2*, const Geom&, cudaStream_t);                          \
     template void dslash<T>(int, v2<T>*, const v2<T>*, const v2<T>*, const v2<T>*, const Geom&, double, double, int, \
-                            const Reduce&, cudaStream_t);                                                           \
+                            const Reduce&, cudaStream_t, const Lanes&);                                             \
     template void zero<T>(v2<T>*, size_t, cudaStream_t);                                                            \
-    template void norm2<T>(const v2<T>*, size_t, int, const Reduce&, cudaStream_t);                                 \
+    template void norm2<T>(const v2<T>*, size_t, int, const Reduce&, cudaStream_t, const Lanes&);                                 \
     template void dot<T>(const v2<T>*, const v2<T>*, size_t, int, const Reduce&, cudaStream_t);                     \
     template void scale<T>(v2<T>*, size_t, double, cudaStream_t);                                                   \
     template void axpy<T>(v2<T>*, const v2<T>*, size_t, double, double, cudaStream_t);                              \
-    template void mr_update<T>(v2<T>*, v2<T>*, const v2<T>*, size_t, bool, const Reduce&, cudaStream_t);            \
+    template void mr_update<T>(v2<T>*, v2<T>*, const v2<T>*, size_t, bool, const Reduce&, cudaStream_t, const Lanes&);            \
     template void normalize_dev<T>(v2<T>*, size_t, int, const Reduce&, cudaStream_t);                               \
-    template void gcr_multidot<T>(const v2<T>*, size_t, int, const Reduce&, cudaStream_t);                          \
-    template void gcr_orth_norm<T>(v2<T>*, size_t, int, const Reduce&, cudaStream_t);                               \
-    template void gcr_cdot<T>(const v2<T>*, const v2<T>*, size_t, int, const Reduce&, cudaStream_t);                \
-    template void gcr_update<T>(v2<T>*, v2<T>*, size_t, int, const Reduce&, cudaStream_t);                          \
+    template void gcr_multidot<T>(const v2<T>*, size_t, int, const Reduce&, cudaStream_t, const Lanes&);                          \
+    template void gcr_orth_norm<T>(v2<T>*, size_t, int, const Reduce&, cudaStream_t, const Lanes&);                               \
+    template void gcr_cdot<T>(const v2<T>*, const v2<T>*, size_t, int, const Reduce&, cudaStream_t, const Lanes&);                \
+    template void gcr_update<T>(v2<T>*, v2<T>*, size_t, int, const Reduce&, cudaStream_t, const Lanes&);                          \
     template void gcr_xupdate<T>(double2*, const v2<T>*, size_t, int, const GcrCoef&, cudaStream_t);          \
-    template void gmres_orth<T>(v2<T>*, size_t, int, const Reduce&, cudaStream_t);                             \
-    template void multi_axpy<T>(v2<T>*, const v2<T>*, size_t, int, const Reduce&, cudaStream_t);
+    template void gmres_orth<T>(v2<T>*, size_t, int, const Reduce&, cudaStream_t, const Lanes&);                             \
+    template void multi_axpy<T>(v2<T>*, const v2<T>*, size_t, int, const Reduce&, cudaStream_t, const Lanes&);
 INST(float)
 INST(double)
 #undef INST

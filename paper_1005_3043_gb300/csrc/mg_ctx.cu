@@ -64,6 +64,10 @@ struct BatchWork {
     double2* b64 = nullptr;         // nrhs x n
     double* scal = nullptr;         // nrhs x S_COUNT
     double* h_scal = nullptr;       // pinned nrhs x S_COUNT
+    double* partials = nullptr;     // partial sums, counters and smoother scalars of `lanes` lanes
+    unsigned int* ticket = nullptr;
+    double* scal_s = nullptr;
+    int lanes = 0;
 };
 
 // Workspace of the red-black preconditioned CG (checkerboard layout).
@@ -130,8 +134,10 @@ template <typename T> struct Work {
     v2<T>* cr1 = nullptr;  // second buffers of the coarse CG
     v2<T>* cp1 = nullptr;
     unsigned long long* ctag = nullptr;   // epoch-tagged s and u of the on-chip coarse CG (T == float)
-    v2<T>* gm = nullptr;   // GMRES smoother basis, gm_k + 1 vectors
-    int gm_k = 0;
+    v2<T>* mr = nullptr;   // MR smoother of several lanes: mr_m residuals, then mr_m products
+    int mr_m = 0;
+    v2<T>* gm = nullptr;   // GMRES smoother basis, (gm_k + 1) vectors per lane
+    int gm_k = 0, gm_m = 0;
     int cnc = 0;           // coarse dof the coarse vectors are sized for
     bool ready = false;
 };
@@ -603,12 +609,26 @@ bool gmres_fp16(mg_ctx* ctx, int k) {
     return (double)ctx->g.V * 96.0 * (k + 1) > (double)l2;
 }
 
+// Sources of a batch smoothed by one launch: as many as keep the FP32 Krylov basis
+// (or the MR vectors) of all of them in L2 on a lattice that does not fill the SMs
+// by itself; one on lattices of 80000 sites and more (at 16^3x32 a second source's
+// basis would push out the first's) and with FP16 smoother storage.
+int smoother_lanes(mg_ctx* ctx, int nrhs) {
+    const int k = ctx->prm.smoother_steps;
+    if (ctx->prm.smoother == 1 && k > 0 ? gmres_fp16(ctx, k) : smoother_fp16(ctx)) return 1;
+    const long long most = std::max(1LL, 80000 / ctx->g.V);
+    const long long groups = (nrhs + most - 1) / most;
+    return (int)((nrhs + groups - 1) / groups);
+}
+
 // Post-smoothing of the V(0,n) cycle (Sec. III): r_s = r - D z, then n MR steps
 // q = D r_s, alpha = omega <q,r_s>/<q,q>, z += alpha r_s, r_s -= alpha q.  In
 // MG_FP16 mode r_s and q are stored in FP16 with a per-site scale and the
 // links in FP16 (FP32 arithmetic); z stays in the path's precision.
+// Several sources at once: ln.m lanes, a between their z, b between their r (m > 1 only
+// where smoother_lanes allows it; the counters are those of one source).
 template <typename T>
-int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt) {
+int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt, const Lanes& ln = {}) {
     Work<T>& w = work<T>(ctx);
     const size_t n = nfine(ctx);
     const int steps = ctx->prm.smoother_steps;
@@ -658,32 +678,36 @@ int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt
         // one GMRES(steps) application, under-relaxed by omega (Sec. III-IV):
         // Arnoldi with one classical Gram-Schmidt pass per vector, the small
         // least-squares problem on the device, z += omega V y
-        if (w.gm_k < steps) {
-            if (w.gm) { dfree(ctx, w.gm); w.gm = nullptr; w.gm_k = 0; }
-            TRY(dalloc(ctx, &w.gm, sizeof(v2<T>) * n * (size_t)(steps + 1)));
-            w.gm_k = steps;
+        if (w.gm_k < steps || w.gm_m < ln.m) {
+            if (w.gm) { dfree(ctx, w.gm); w.gm = nullptr; }
+            w.gm_k = std::max(w.gm_k, steps);
+            w.gm_m = std::max(w.gm_m, ln.m);
+            TRY(dalloc(ctx, &w.gm, sizeof(v2<T>) * n * (size_t)(w.gm_k + 1) * w.gm_m));
         }
         Reduce Rs = R;
-        Rs.scal = ctx->scal_s;
+        if (ln.m == 1) Rs.scal = ctx->scal_s;   // a batch brings its own
         const v2<T>* U = links<T>(ctx);
         v2<T>* V = w.gm;
+        const size_t nb = n * (size_t)(steps + 1);   // one lane's basis
+        const Lanes lb{ln.m, nb, nb, nb}, lz{ln.m, nb, ln.a, ln.b}, la{ln.m, ln.a, nb, 0};
         PROF_BEGIN(MG_K_DSLASH);
-        dslash<T>(DS_XMY, V, z, U, r, ctx->g, ctx->mass, 0.0, 0, Rs, ctx->st);
+        dslash<T>(DS_XMY, V, z, U, r, ctx->g, ctx->mass, 0.0, 0, Rs, ctx->st, lz);
         PROF_END(MG_K_DSLASH);
         PROF_BEGIN(MG_K_KRYLOV);
-        gmres_orth<T>(V, n, 0, Rs, ctx->st);
+        gmres_orth<T>(V, n, 0, Rs, ctx->st, lb);
         PROF_END(MG_K_KRYLOV);
         for (int j = 0; j < steps; ++j) {
             PROF_BEGIN(MG_K_DSLASH);
-            dslash<T>(DS_PLAIN, V + (size_t)(j + 1) * n, V + (size_t)j * n, U, V, ctx->g, ctx->mass, 0.0, 0, Rs, ctx->st);
+            dslash<T>(DS_PLAIN, V + (size_t)(j + 1) * n, V + (size_t)j * n, U, V, ctx->g, ctx->mass, 0.0, 0, Rs, ctx->st,
+                      lb);
             PROF_END(MG_K_DSLASH);
             PROF_BEGIN(MG_K_KRYLOV);
-            gmres_orth<T>(V, n, j + 1, Rs, ctx->st);
+            gmres_orth<T>(V, n, j + 1, Rs, ctx->st, lb);
             PROF_END(MG_K_KRYLOV);
         }
         PROF_BEGIN(MG_K_KRYLOV);
-        gmres_ls(Rs, steps, ctx->prm.omega, ctx->st);
-        multi_axpy<T>(z, V, n, steps, Rs, ctx->st);
+        gmres_ls(Rs, steps, ctx->prm.omega, ctx->st, lb);
+        multi_axpy<T>(z, V, n, steps, Rs, ctx->st, la);
         PROF_END(MG_K_KRYLOV);
         cnt.fine(steps + 1, dslash_site_bytes<T>());
         return MG_OK;
@@ -708,16 +732,27 @@ int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt
         return MG_OK;
     }
     const v2<T>* U = links<T>(ctx);
+    v2<T>*vr = w.vr, *vq = w.vq;
+    if (ln.m > 1) {   // r and q of every lane
+        if (w.mr_m < ln.m) {
+            if (w.mr) { dfree(ctx, w.mr); w.mr = nullptr; w.mr_m = 0; }
+            TRY(dalloc(ctx, &w.mr, sizeof(v2<T>) * n * 2 * (size_t)ln.m));
+            w.mr_m = ln.m;
+        }
+        vr = w.mr;
+        vq = w.mr + n * (size_t)ln.m;
+    }
+    const Lanes lv{ln.m, n, n, n}, lz{ln.m, n, ln.a, ln.b}, lu{ln.m, ln.a, n, 0};
     PROF_BEGIN(MG_K_DSLASH);
-    dslash<T>(DS_XMY, w.vr, z, U, r, ctx->g, ctx->mass, 0.0, 0, R, ctx->st);
+    dslash<T>(DS_XMY, vr, z, U, r, ctx->g, ctx->mass, 0.0, 0, R, ctx->st, lz);
     PROF_END(MG_K_DSLASH);
     cnt.fine(1, dslash_site_bytes<T>());
     for (int k = 0; k < steps; ++k) {
         PROF_BEGIN(MG_K_DSLASH);
-        dslash<T>(DS_MRDOT, w.vq, w.vr, U, w.vr, ctx->g, ctx->mass, ctx->prm.omega, 0, R, ctx->st);
+        dslash<T>(DS_MRDOT, vq, vr, U, vr, ctx->g, ctx->mass, ctx->prm.omega, 0, R, ctx->st, lv);
         PROF_END(MG_K_DSLASH);
         PROF_BEGIN(MG_K_KRYLOV);
-        mr_update<T>(z, w.vr, w.vq, n, k + 1 < steps, R, ctx->st);
+        mr_update<T>(z, vr, vq, n, k + 1 < steps, R, ctx->st, lu);
         PROF_END(MG_K_KRYLOV);
         cnt.fine(1, dslash_site_bytes<T>());
     }
@@ -2545,7 +2580,8 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
         CK(cudaStreamSynchronize(ctx->st));
         for (void* q : {(void*)b.rcB, (void*)b.yB, (void*)b.rB, (void*)b.sB, (void*)b.pB, (void*)b.qB, (void*)b.uB,
                         (void*)b.zB, (void*)b.bts, (void*)b.btu, (void*)b.sync, (void*)b.iters, (void*)b.flags,
-                        (void*)b.r32, (void*)b.Z, (void*)b.Pk, (void*)b.x64, (void*)b.b64, (void*)b.scal})
+                        (void*)b.r32, (void*)b.Z, (void*)b.Pk, (void*)b.x64, (void*)b.b64, (void*)b.scal,
+                        (void*)b.partials, (void*)b.ticket, (void*)b.scal_s})
             dfree(ctx, q);
         cudaFreeHost(b.h_flags);
         cudaFreeHost(b.h_iters);
@@ -2610,6 +2646,21 @@ int batched_coarse_solve(mg_ctx* ctx, int nrhs, double tol, int maxit, std::vect
     return MG_OK;
 }
 
+int ensure_lanes(mg_ctx* ctx, int m) {
+    BatchWork& b = ctx->bw;
+    if (b.lanes >= m) return MG_OK;
+    for (void* q : {(void*)b.partials, (void*)b.ticket, (void*)b.scal_s}) dfree(ctx, q);
+    b.partials = b.scal_s = nullptr;
+    b.ticket = nullptr;
+    b.lanes = 0;
+    TRY(dalloc(ctx, &b.partials, ctx->R.partial_bytes * m));
+    TRY(dalloc(ctx, &b.ticket, sizeof(unsigned int) * m));
+    TRY(dalloc(ctx, &b.scal_s, sizeof(double) * S_COUNT * m));
+    CK(cudaMemsetAsync(b.ticket, 0, sizeof(unsigned int) * m, ctx->st));
+    b.lanes = m;
+    return MG_OK;
+}
+
 // b64 (internal layout) -> x64 for nrhs sources, FP32 inner precision
 int solve_batched_impl(mg_ctx* ctx, int nrhs, mg_solve_info* infos) {
     TRY(ensure_work<float>(ctx));
@@ -2627,6 +2678,17 @@ int solve_batched_impl(mg_ctx* ctx, int nrhs, mg_solve_info* infos) {
     auto RR = [&](int r) {
         Reduce R = ctx->R;
         R.scal = b.scal + (size_t)r * S_COUNT;
+        return R;
+    };
+    // lanes of a launch: sources lane by lane for the fine-level steps
+    const int lanes = smoother_lanes(ctx, nrhs);
+    TRY(ensure_lanes(ctx, lanes));
+    auto lane_reduce = [&](double* scal) {
+        Reduce R = ctx->R;
+        R.partials = b.partials;
+        R.ticket = b.ticket;
+        R.scal = scal;
+        R.lane_scal = S_COUNT;
         return R;
     };
     CK(cudaEventRecord(ctx->ev0, ctx->st));
@@ -2652,43 +2714,65 @@ int solve_batched_impl(mg_ctx* ctx, int nrhs, mg_solve_info* infos) {
         if (stepping) {
             // restriction of every stepping source into its panel column
             CK(cudaMemsetAsync(b.rcB, 0, sizeof(float2) * (size_t)ctx->g.Vc * L.nc * b.npad, ctx->st));
+            auto steps_now = [&](int r) { return active[r] && !cycle_end[r] && kk[r] < K && iters[r] < p.max_outer; };
+            // runs of neighbouring stepping sources (they all step at the same kk), at most
+            // `most` long
+            auto run = [&](int r0, int most) {
+                int m = 0;
+                while (r0 + m < nrhs && m < most && steps_now(r0 + m) && kk[r0 + m] == kk[r0]) ++m;
+                return m;
+            };
             PROF_BEGIN(MG_K_RESTRICT);
-            for (int r = 0; r < nrhs; ++r)
-                if (active[r] && !cycle_end[r] && kk[r] < K && iters[r] < p.max_outer)
-                    restrict_<float>(b.rcB, L.P32, b.r32 + r * n, L.nv, ctx->g, ctx->st, b.npad, r);
+            for (int r = 0; r < nrhs;) {
+                const int m = run(r, nrhs);
+                if (m == 0) { ++r; continue; }
+                restrict_<float>(b.rcB, L.P32, b.r32 + r * n, L.nv, ctx->g, ctx->st, b.npad, r, Lanes{m, n, 0, 0});
+                r += m;
+            }
             PROF_END(MG_K_RESTRICT);
             CKL();
             TRY(batched_coarse_solve(ctx, nrhs, p.coarse_tol, p.max_coarse, coarse));
-            for (int r = 0; r < nrhs; ++r) {
-                if (!(active[r] && !cycle_end[r] && kk[r] < K && iters[r] < p.max_outer)) continue;
-                Reduce Rr = RR(r);
-                v2<float>* zk = b.Z + ((size_t)r * K + kk[r]) * n;
-                v2<float>* Pr = b.Pk + (size_t)r * K * n;
+            for (int r = 0; r < nrhs;) {
+                const int m = run(r, nrhs);
+                if (m == 0) { ++r; continue; }
                 PROF_BEGIN(MG_K_PROLONG);
-                prolong<float>(zk, L.P32, b.yB, L.nv, ctx->g, ctx->st, b.npad, r);
+                prolong<float>(b.Z + ((size_t)r * K + kk[r]) * n, L.P32, b.yB, L.nv, ctx->g, ctx->st, b.npad, r,
+                               Lanes{m, (size_t)K * n, 0, 0});
                 PROF_END(MG_K_PROLONG);
+                r += m;
+            }
+            for (int r = 0; r < nrhs;) {
+                const int m = run(r, lanes), k = kk[r];
+                if (m == 0) { ++r; continue; }
+                const size_t nK = (size_t)K * n;
+                v2<float>* zk = b.Z + ((size_t)r * K + k) * n;
+                v2<float>* Pr = b.Pk + (size_t)r * nK;
                 {
                     Counters scnt;
-                    TRY(smooth<float>(ctx, b.r32 + r * n, zk, Rr, scnt));
-                    mv[r] += scnt.matvecs;
-                    mvb[r] += scnt.site_bytes;
+                    TRY(smooth<float>(ctx, b.r32 + r * n, zk, m > 1 || ctx->prm.smoother == 0 ? lane_reduce(b.scal_s) : RR(r),
+                                      scnt, Lanes{m, nK, n, 0}));
+                    for (int q = r; q < r + m; ++q) {
+                        mv[q] += scnt.matvecs + 1;
+                        mvb[q] += scnt.site_bytes + kDslashBytesF32;
+                    }
                 }
+                const Reduce Rr = lane_reduce(b.scal + (size_t)r * S_COUNT);
+                const Lanes lk{m, nK, nK, nK}, lr{m, nK, n, 0};
                 PROF_BEGIN(MG_K_DSLASH);
-                dslash<float>(DS_PLAIN, Pr + (size_t)kk[r] * n, zk, U, zk, ctx->g, ctx->mass, 0.0, 0, Rr, ctx->st);
+                dslash<float>(DS_PLAIN, Pr + (size_t)k * n, zk, U, zk, ctx->g, ctx->mass, 0.0, 0, Rr, ctx->st, lk);
                 PROF_END(MG_K_DSLASH);
-                mv[r] += 1;
-                mvb[r] += kDslashBytesF32;
                 PROF_BEGIN(MG_K_KRYLOV);
-                if (kk[r] > 0) {
-                    gcr_multidot<float>(Pr, n, kk[r], Rr, ctx->st);
-                    gcr_orth_norm<float>(Pr, n, kk[r], Rr, ctx->st);
+                if (k > 0) {
+                    gcr_multidot<float>(Pr, n, k, Rr, ctx->st, lk);
+                    gcr_orth_norm<float>(Pr, n, k, Rr, ctx->st, lk);
                 } else {
-                    norm2<float>(Pr, n, S_GCR_PN2, Rr, ctx->st);
+                    norm2<float>(Pr, n, S_GCR_PN2, Rr, ctx->st, lk);
                 }
-                gcr_cdot<float>(Pr, b.r32 + r * n, n, kk[r], Rr, ctx->st);
-                gcr_update<float>(Pr, b.r32 + r * n, n, kk[r], Rr, ctx->st);
+                gcr_cdot<float>(Pr, b.r32 + r * n, n, k, Rr, ctx->st, lr);
+                gcr_update<float>(Pr, b.r32 + r * n, n, k, Rr, ctx->st, lr);
                 PROF_END(MG_K_KRYLOV);
                 CKL();
+                r += m;
             }
             CK(cudaMemcpyAsync(b.h_scal, b.scal, sizeof(double) * S_COUNT * nrhs, cudaMemcpyDeviceToHost, ctx->st));
             CK(cudaStreamSynchronize(ctx->st));

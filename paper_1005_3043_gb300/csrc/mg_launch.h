@@ -22,7 +22,24 @@ struct Reduce {
     double* partials;      // partial_bytes bytes (at least kReducePartialsBytes)
     unsigned int* ticket;  // one zeroed counter
     double* scal;          // device scalars, S_COUNT doubles (ScalarSlot)
-    size_t partial_bytes;  // capacity of partials
+    size_t partial_bytes;  // capacity of partials (of one lane)
+    size_t lane_scal = 0;  // doubles between the scalars of two lanes (see Lanes)
+    __host__ __device__ Reduce lane(int y) const {
+        Reduce r = *this;
+        r.partials += (size_t)y * (partial_bytes / sizeof(double));
+        r.ticket += y;
+        r.scal += (size_t)y * lane_scal;
+        return r;
+    }
+};
+// Several sources in one launch: lane y (blockIdx.y) of m works on its own vectors,
+// the arguments' pointers moved on by y times a stride each (a, b, c in the order
+// that the launcher names them), and on its own partial sums, counter and scalars
+// (Reduce::lane).  A lattice of a few thousand sites fills the SMs only with the
+// sources of a batch side by side, and each of its launches costs more than its work.
+struct Lanes {
+    int m = 1;
+    size_t a = 0, b = 0, c = 0;
 };
 // partial-sum buffer for a lattice of V sites: the widest per-block reduction of
 // the per-site kernels (32 floats per 128 sites) or kReducePartialsBytes
@@ -43,32 +60,33 @@ enum DslashMode { DS_PLAIN = 0, DS_XMY = 1, DS_XMY_NORM = 2, DS_MRDOT = 3 };
 // DS_XMY:       out = src - D in
 // DS_XMY_NORM:  out = src - D in, scal[slot] = ||out||^2
 // DS_MRDOT:     out = D in, scal[S_MR_ALPHA] = omega <out,in> / <out,out>
+// lanes: a out, b in, c src
 template <typename T>
 void dslash(int mode, v2<T>* out, const v2<T>* in, const v2<T>* U, const v2<T>* src, const Geom& g, double mass,
-            double omega, int slot, const Reduce& R, cudaStream_t st);
+            double omega, int slot, const Reduce& R, cudaStream_t st, const Lanes& ln = {});
 
 // ---------------------------------------------------------------- fine / generic BLAS (n complex)
 template <typename T> void zero(v2<T>* x, size_t n, cudaStream_t st);
-template <typename T> void norm2(const v2<T>* x, size_t n, int slot, const Reduce& R, cudaStream_t st);
+template <typename T> void norm2(const v2<T>* x, size_t n, int slot, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a x
 template <typename T> void dot(const v2<T>* x, const v2<T>* y, size_t n, int slot, const Reduce& R, cudaStream_t st);
 template <typename T> void scale(v2<T>* x, size_t n, double s, cudaStream_t st);
 // y += a x with a a host constant
 template <typename T> void axpy(v2<T>* y, const v2<T>* x, size_t n, double ar, double ai, cudaStream_t st);
 // MR update: e += alpha r; r -= alpha q (if update_r), alpha = scal[S_MR_ALPHA]
 template <typename T>
-void mr_update(v2<T>* e, v2<T>* r, const v2<T>* q, size_t n, bool update_r, const Reduce& R, cudaStream_t st);
+void mr_update(v2<T>* e, v2<T>* r, const v2<T>* q, size_t n, bool update_r, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a e, b r and q
 // normalise x in place by 1/sqrt(scal[slot])
 template <typename T> void normalize_dev(v2<T>* x, size_t n, int slot, const Reduce& R, cudaStream_t st);
 
 // ---------------------------------------------------------------- GCR (K_MAX basis vectors)
 // R[j][k] = <p_j, p_k> for j < k  (p_j = basis + j*n)
-template <typename T> void gcr_multidot(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st);
+template <typename T> void gcr_multidot(const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a basis
 // p_k -= sum_{j<k} R[j][k] p_j ; scal[S_GCR_PN2] = ||p_k||^2
-template <typename T> void gcr_orth_norm(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st);
+template <typename T> void gcr_orth_norm(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a basis
 // R[k][k] = ||p_k||; c_k = <p_k, r>/||p_k||
-template <typename T> void gcr_cdot(const v2<T>* basis, const v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st);
+template <typename T> void gcr_cdot(const v2<T>* basis, const v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a basis, b r
 // p_k /= ||p_k||; r -= c_k p_k; scal[S_GCR_R2] = ||r||^2
-template <typename T> void gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st);
+template <typename T> void gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a basis, b r
 // x (FP64) += sum_j y_j Z_j
 struct GcrCoef { double c[2 * K_MAX]; };
 template <typename T>
@@ -77,9 +95,9 @@ void gcr_xupdate(double2* x, const v2<T>* Z, size_t n, int k, const GcrCoef& y, 
 // residual for k = 0) against the vectors before it, column k - 1 of the Hessenberg
 // matrix and f_k = 1 / |basis[k]| (S_GMRES_F; vector k of the space is f_k basis[k]);
 // the small least-squares problem (omega y -> S_GCR_C); z += sum_j c_j f_j basis[j]
-template <typename T> void gmres_orth(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st);
-void gmres_ls(const Reduce& R, int k, double omega, cudaStream_t st);
-template <typename T> void multi_axpy(v2<T>* z, const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st);
+template <typename T> void gmres_orth(v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a basis
+void gmres_ls(const Reduce& R, int k, double omega, cudaStream_t st, const Lanes& ln = {});
+template <typename T> void multi_axpy(v2<T>* z, const v2<T>* basis, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln = {});   // lanes: a z, b basis
 
 // ---------------------------------------------------------------- transfer / coarse
 // P64[X][s][i][6][l] from prototypes V[i][X][12][l]; *status = 1 on rank deficiency
@@ -88,10 +106,10 @@ void block_orthonormalize(double2* P, const double2* V, int nv, const Geom& g, i
 // npad, n: column n of an RHS panel)
 template <typename T>
 void restrict_(v2<T>* rc, const v2<T>* P, const v2<T>* r, int nv, const Geom& g, cudaStream_t st, int cstride = 1,
-               int coff = 0);
+               int coff = 0, const Lanes& ln = {});   // lanes: a r, the panel column moves on by one
 template <typename T>
 void prolong(v2<T>* e, const v2<T>* P, const v2<T>* yc, int nv, const Geom& g, cudaStream_t st, int cstride = 1,
-             int coff = 0);
+             int coff = 0, const Lanes& ln = {});   // lanes: a e, the panel column moves on by one
 // A64 (column-major blocks) = P^dag D P; Aself scratch of Vc*8*nc*nc complex
 void coarse_build(double2* A, double2* Aself, const double2* P, const double2* U, int nv, double mass, const Geom& g,
                   cudaStream_t st);
