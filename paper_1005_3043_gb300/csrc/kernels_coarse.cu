@@ -3,6 +3,8 @@
 // prolongation e = P y, the Galerkin coarse operator D_c = P^dag D P and its
 // nearest-neighbour application, and the CGNR (CGLS) coarse solve steps.
 #include <atomic>
+#include <type_traits>
+
 #include "mg_launch.h"
 #include "mg_sync.cuh"
 
@@ -656,7 +658,13 @@ struct CgnrSplit {
 //   ST_R: rn = r_old - alpha * q; own entries -> r_new, y += alpha * p_cur;
 //         output s = D_c^dag rn;      partial sums: n0 = ||s||^2, n1 = ||rn||^2
 //   ST_PLAIN: operand = in;          output out = D_c(^dag) in, n0 = ||out||^2
+// Red-black form (a phase is one half of Dhat, see kernels_schur.cu): HALF_O
+// computes t = sum_{d >= 1} H x on the odd sites, the operand x (of the even
+// neighbours) formed as above; HALF_E computes y = H[0] x + sum_{d >= 1} H t on the
+// even sites, x formed for the site itself (with its own entries' updates) and t
+// read.  Only x and y carry sigma3 in the adjoint.
 enum { ST_PLAIN = 0, ST_P = 1, ST_R = 2 };
+enum { HALF_NONE = 0, HALF_O = 1, HALF_E = 2 };
 
 template <typename T, bool H16 = false> struct RowsPerThread { static constexpr int value = H16 ? 4 : 2; };
 
@@ -698,16 +706,18 @@ template <typename T> struct PhaseArgs {
     v2<T>* out;            // result
     T coef;                // beta (ST_P) or alpha (ST_R)
     bool first;            // ST_P, first iteration
+    const int* sites;      // red-black: the sites of this half, in the order of the units
+    v2<T>* t;              // red-black: t of the odd sites (HALF_O writes, HALF_E reads)
 };
 
-template <typename T, bool DAG, int STAGE, bool H16>
+template <typename T, bool DAG, int STAGE, bool H16, int HALF>
 __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, const __half2* __restrict__ A16,
                          const float* __restrict__ s16, int nc, const CgnrSplit& sp, const Geom& g, v2<T>* xs,
                          cx<T>* part, const int* __restrict__ nbr, T& n0, T& n1) {
     constexpr int R = RowsPerThread<T, H16>::value;
     const int rsp = sp.template parts<T>(), bs = sp.template cols<T>();
     const int nvh = nc >> 1, nrow = 9 * nc, ngl = nc / R / rsp, rows = sizeof(T) == 4 ? nc : ngl * R, nsum = 9 * bs;
-    const int tpu = nsum * ngl, nunit = g.Vc * rsp;
+    const int tpu = nsum * ngl, nsite = HALF ? g.Vc / 2 : g.Vc, nunit = nsite * rsp;
     const int ul = threadIdx.x / tpu, rem = threadIdx.x - ul * tpu;
     const int db = rem / ngl, a0 = (rem - db * ngl) * R;   // a0: row within the part
     const int d = db / bs, bp = db - d * bs;
@@ -717,14 +727,18 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
         for (int i = threadIdx.x; i < nall; i += blockDim.x) {
             int xi = i / nrow, ri = i - xi * nrow;
             int di = ri / nc, b = ri - di * nc;
-            int X = Xb + xi;
-            {
+            const int X = HALF ? __ldg(ph.sites + Xb + xi) : Xb + xi;
+            if (HALF != HALF_O || di > 0) {
                 // the CTA that owns row b of X does that entry's vector updates
-                const int u = X * rsp + b / rows;
+                const int u = (Xb + xi) * rsp + b / rows;
                 const bool own = di == 0 && (sizeof(T) == 4 || (u >= Ub && u < Ue));
                 int Y = __ldg(nbr + (size_t)X * 9 + di);
                 size_t o = (size_t)Y * nc + b;
                 cx<T> v;
+                if (HALF == HALF_E && di > 0) {
+                    st<T>(xs + i, ld<T>(ph.t + o));
+                    continue;
+                }
                 if (STAGE == ST_PLAIN) {
                     v = ld<T>(ph.in + o);
                 } else if (STAGE == ST_P) {
@@ -744,9 +758,10 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
             }
         }
         __syncthreads();
-        const int U0 = Ub + ul, X = U0 / rsp, ar = (U0 - X * rsp) * rows + a0;   // ar: row within the block
-        if (ul < sp.upb && U0 < nunit) {
-            const v2<T>* xd = xs + (X - Xb) * nrow + d * nc;
+        const int U0 = Ub + ul, Xi = U0 / rsp, ar = (U0 - Xi * rsp) * rows + a0;   // ar: row within the block
+        if (ul < sp.upb && U0 < nunit && (HALF != HALF_O || d > 0)) {
+            const int X = HALF ? __ldg(ph.sites + Xi) : Xi;
+            const v2<T>* xd = xs + (Xi - Xb) * nrow + d * nc;
             cx<T>* pd = part + (size_t)(ul * nsum + db) * rows + a0;
             cx<T> acc[R][2];
 #pragma unroll
@@ -795,12 +810,17 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
         }
         __syncthreads();
         for (int t = threadIdx.x; t < sp.upb * rows; t += blockDim.x) {
-            const int u2 = t / rows, U2 = Ub + u2, X2 = U2 / rsp, a2 = (U2 - X2 * rsp) * rows + (t - u2 * rows);
+            const int u2 = t / rows, U2 = Ub + u2, Xi2 = U2 / rsp, a2 = (U2 - Xi2 * rsp) * rows + (t - u2 * rows);
             if (U2 < nunit) {
+                const int X2 = HALF ? __ldg(ph.sites + Xi2) : Xi2, d0 = HALF == HALF_O ? bs : 0;   // no self block in t
                 const cx<T>* ps = part + (size_t)u2 * nsum * rows + (t - u2 * rows);
-                cx<T> sum = ps[0];
+                cx<T> sum = ps[d0 * rows];
 #pragma unroll 8
-                for (int dd = 1; dd < nsum; ++dd) sum = sum + ps[dd * rows];
+                for (int dd = d0 + 1; dd < nsum; ++dd) sum = sum + ps[dd * rows];
+                if (HALF == HALF_O) {
+                    st<T>(ph.t + (size_t)X2 * nc + a2, sum);
+                    continue;
+                }
                 if (DAG && a2 >= nvh) sum = cx<T>(-sum.r, -sum.i);
                 st<T>(ph.out + (size_t)X2 * nc + a2, sum);
                 n0 += norm2(sum);
@@ -819,7 +839,10 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
 // FP64: one CTA per SM, registers for all columns of a thread's loads in flight
 template <typename T> struct CgnrMaxThreads { static constexpr int value = 384, blocks = sizeof(T) == 8 ? 1 : 2; };
 
-template <typename T, bool H16>
+// EO: CG on the normal equations of Dhat (even entries of the vectors; each stencil
+// the two halves with a grid barrier between them); a.rc is then rhat and a.rc_full
+// the right-hand side whose norm the tolerance refers to.
+template <typename T, bool H16, bool EO>
 __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::blocks) k_cgnr_persistent(CgnrArgs<T> a) {
     extern __shared__ unsigned char smem_raw[];
     const int nc = a.nc;
@@ -832,18 +855,44 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
     unsigned int* gen = a.bar + 1;
     v2<T>* rbuf[2] = {a.r, a.r1};
     v2<T>* pbuf[2] = {a.p, a.p1};
-    // y = 0, r = rc on the aggregates of this CTA; ||rc||^2
+    const int nsite = EO ? a.g.Vc / 2 : a.g.Vc;
+    PhaseArgs<T> ph{};
+    // one stencil out = D x (or its adjoint), D = D_c or Dhat; false when a barrier gave up
+    auto stencil = [&](auto dag, auto stage, T& n0, T& n1) -> bool {
+        constexpr bool DAG = decltype(dag)::value != 0;
+        constexpr int STAGE = decltype(stage)::value;
+        ph.t = a.t;
+        if constexpr (EO) {
+            T u0 = 0, u1 = 0;
+            ph.sites = a.ord + nsite;
+            cg_phase<T, DAG, STAGE, H16, HALF_O>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, u0, u1);
+            if (!grid_sync(cnt, gen, G, a.err)) return false;
+            ph.sites = a.ord;
+            cg_phase<T, DAG, STAGE, H16, HALF_E>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
+        } else {
+            cg_phase<T, DAG, STAGE, H16, HALF_NONE>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
+        }
+        return true;
+    };
+    // y = 0, r = rc on the units of this CTA; ||rc||^2
     T loc = 0;
-    const int rows = nc / sp.rsp;   // rows of a unit: unit u holds entries u * rows ..
-    for (int Ub = blockIdx.x * sp.upb; Ub < a.g.Vc * sp.rsp; Ub += G * sp.upb)
+    const int rows = nc / sp.rsp;   // rows of a unit
+    for (int Ub = blockIdx.x * sp.upb; Ub < nsite * sp.rsp; Ub += G * sp.upb)
         for (int t = threadIdx.x; t < sp.upb * rows; t += blockDim.x) {
-            if (Ub + t / rows < a.g.Vc * sp.rsp) {
-                size_t o = (size_t)Ub * rows + t;
+            const int u = Ub + t / rows;
+            if (u < nsite * sp.rsp) {
+                const int Xi = u / sp.rsp, a0 = (u - Xi * sp.rsp) * rows + t % rows;
+                const size_t o = (size_t)(EO ? a.ord[Xi] : Xi) * nc + a0;
                 v2<T> v = a.rc[o];
                 a.r[o] = v;
                 v2<T> z; z.x = 0; z.y = 0;
                 a.y[o] = z;
-                loc += v.x * v.x + v.y * v.y;
+                if (EO) {
+                    const v2<T> e = a.rc_full[o], d = a.rc_full[(size_t)a.ord[nsite + Xi] * nc + a0];
+                    loc += e.x * e.x + e.y * e.y + d.x * d.x + d.y * d.y;
+                } else {
+                    loc += v.x * v.x + v.y * v.y;
+                }
             }
         }
     write_partial<T>(loc, a.partials, 0, shr);
@@ -852,12 +901,13 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
     int it = 0;
     T r2 = rc2;
     if (rc2 > T(0) && a.maxit > 0) {
-        PhaseArgs<T> ph{};
+        using Yes = std::integral_constant<int, 1>;
+        using No = std::integral_constant<int, 0>;
         T n0 = 0, n1 = 0;
         // s = D_c^dag r, gamma = ||s||^2
         ph.in = a.r;
         ph.out = a.s;
-        cg_phase<T, true, ST_PLAIN, H16>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
+        if (!stencil(Yes{}, std::integral_constant<int, ST_PLAIN>{}, n0, n1)) return;
         write_partial<T>(n0, a.partials, 1, shr);
         if (!grid_sync(cnt, gen, G, a.err)) return;
         T gamma = sum_partials<T>(a.partials, 1, G, shr);
@@ -869,7 +919,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
             ph.s = a.s; ph.p_old = pbuf[b ^ 1]; ph.p_new = pbuf[b]; ph.out = a.q;
             ph.coef = beta; ph.first = (it == 0);
             n0 = 0; n1 = 0;
-            cg_phase<T, false, ST_P, H16>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
+            if (!stencil(No{}, std::integral_constant<int, ST_P>{}, n0, n1)) return;
             write_partial<T>(n0, a.partials, 0, shr);
             if (!grid_sync(cnt, gen, G, a.err)) return;
             T qq = sum_partials<T>(a.partials, 0, G, shr);
@@ -880,7 +930,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
             ph.r_old = rbuf[b]; ph.q = a.q; ph.r_new = rbuf[b ^ 1]; ph.y = a.y; ph.p_new = pbuf[b];
             ph.out = a.s; ph.coef = alpha;
             n0 = 0; n1 = 0;
-            cg_phase<T, true, ST_R, H16>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
+            if (!stencil(Yes{}, std::integral_constant<int, ST_R>{}, n0, n1)) return;
             write_partial<T>(n0, a.partials, 1, shr);
             write_partial<T>(n1, a.partials, 2, shr);
             if (!grid_sync(cnt, gen, G, a.err)) return;
@@ -932,12 +982,13 @@ template <typename T, bool H16> CgnrSplit cgnr_split(int nc, int Vc, int sms) {
 
 // grid: co-resident CTAs for this split (FP64: one per SM), then the smallest
 // balanced grid covering all units
-template <typename T, bool H16> cudaError_t cgnr_launch(const CgnrArgs<T>& args, cudaStream_t st) {
+template <typename T, bool H16, bool EO> cudaError_t cgnr_launch(const CgnrArgs<T>& args, cudaStream_t st) {
     const int sms = device_sm_count();
-    const CgnrSplit sp = cgnr_split<T, H16>(args.nc, args.g.Vc, sms);
+    const int nsite = EO ? args.g.Vc / 2 : args.g.Vc;   // a red-black half
+    const CgnrSplit sp = cgnr_split<T, H16>(args.nc, nsite, sms);
     const int thr = cgnr_block_threads<T, H16>(args.nc, sp);
     const size_t sm = cgnr_smem<T, H16>(args.nc, sp);
-    const void* fn = (const void*)k_cgnr_persistent<T, H16>;
+    const void* fn = (const void*)k_cgnr_persistent<T, H16, EO>;
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
@@ -947,7 +998,7 @@ template <typename T, bool H16> cudaError_t cgnr_launch(const CgnrArgs<T>& args,
     if (e != cudaSuccess) return e;
     const int gmax = (sizeof(T) == 8 ? std::min(per, 1) : per) * sms;
     if (gmax <= 0) return cudaErrorCooperativeLaunchTooLarge;
-    const int batches = (args.g.Vc * sp.rsp + sp.upb - 1) / sp.upb;   // CTA-sized pieces of work
+    const int batches = (nsite * sp.rsp + sp.upb - 1) / sp.upb;   // CTA-sized pieces of work
     const int rounds = (batches + gmax - 1) / gmax;                    // pieces per CTA
     CgnrArgs<T> a = args;
     a.upb = sp.upb; a.rsp = sp.rsp; a.bs = sp.bs;
@@ -958,12 +1009,12 @@ template <typename T, bool H16> cudaError_t cgnr_launch(const CgnrArgs<T>& args,
 template <> cudaError_t cgnr_persistent<float>(const CgnrArgs<float>& a, cudaStream_t st) {
     if (a.A16) {
         if (a.nc % 4 != 0) return cudaErrorInvalidValue;
-        return cgnr_launch<float, true>(a, st);
+        return a.ord ? cgnr_launch<float, true, true>(a, st) : cgnr_launch<float, true, false>(a, st);
     }
-    return cgnr_launch<float, false>(a, st);
+    return a.ord ? cgnr_launch<float, false, true>(a, st) : cgnr_launch<float, false, false>(a, st);
 }
 template <> cudaError_t cgnr_persistent<double>(const CgnrArgs<double>& a, cudaStream_t st) {
-    return cgnr_launch<double, false>(a, st);
+    return a.ord ? cgnr_launch<double, false, true>(a, st) : cgnr_launch<double, false, false>(a, st);
 }
 
 // coarse neighbour table nbr[X][d] (d = 0 self, 1+2mu / 2+2mu: +mu / -mu)

@@ -40,6 +40,13 @@ struct CoarseLevel {
     float* su = nullptr;      // FP16 unit scales [X][d]
     size_t au_bytes = 0;
     bool au_valid = false, au_h16 = false;
+    double2* H64 = nullptr;   // red-black Schur form of A64 (kernels_schur.cu), built on demand
+    float2* H32 = nullptr;
+    __half2* H16 = nullptr;   // its FP16 copy and block scales
+    float* hs16 = nullptr;
+    size_t h_blocks = 0;      // nc x nc blocks the buffers hold
+    int h_state = 0;          // 0 not built, 1 FP32 products, 2 FP64 products, -1 a singular diagonal block
+    bool h16_valid = false;
     int au_mode = 0;
     CglsShape au_shape{};
     double mass = 0.0;
@@ -110,6 +117,7 @@ template <typename T> struct L1Work {
     int gm_k = 0;
     v2<T>*crc = nullptr, *cy = nullptr;                      // level-2 right-hand side and solution
     v2<T>*cr = nullptr, *cr1 = nullptr, *cs = nullptr, *cp = nullptr, *cp1 = nullptr, *cq = nullptr;
+    v2<T>*eb = nullptr, *et = nullptr;                       // its red-black form
     unsigned long long* ctag = nullptr;
     bool ready = false;
 };
@@ -133,6 +141,7 @@ template <typename T> struct Work {
     v2<T>* cq = nullptr;
     v2<T>* cr1 = nullptr;  // second buffers of the coarse CG
     v2<T>* cp1 = nullptr;
+    v2<T>*eb = nullptr, *et = nullptr;    // red-black form: right-hand side, odd-site scratch
     unsigned long long* ctag = nullptr;   // epoch-tagged s and u of the on-chip coarse CG (T == float)
     v2<T>* mr = nullptr;   // MR smoother of several lanes: mr_m residuals, then mr_m products
     int mr_m = 0;
@@ -173,6 +182,7 @@ struct mg_ctx {
     // third level (levels == 3)
     Geom g2{};                       // the level-1 lattice cut into level-2 aggregates
     int* cnbr2 = nullptr;            // level-2 neighbour table
+    int* cord2 = nullptr;            // level-2 sites by parity
     CoarseLevel full2, trunc2;       // P64/P32: level-2 prolongator panels; A64/A32: A2
     double2* protos2 = nullptr;      // level-2 prototypes [nv2][Vc1][2 nv1] FP64
     double2* protos2_t = nullptr;
@@ -186,6 +196,8 @@ struct mg_ctx {
     int* d_status = nullptr;
     unsigned int* bar = nullptr;     // persistent-kernel barrier: count, generation, error flag
     int* cnbr = nullptr;             // coarse neighbour table [Vc][9]
+    int* cord = nullptr;            // coarse sites by parity (even extents only)
+    bool in_solve = false;          // inside a solve: its preconditioner may use the red-black form
     unsigned long long* xch = nullptr;   // exchange slots of the on-chip coarse CGLS
     unsigned int xch_epoch = 1;          // next free epoch
     double* scal_s = nullptr;            // scalars of the GMRES smoother (its Hessenberg matrix)
@@ -258,6 +270,14 @@ void dfree(mg_ctx* ctx, void* q) {
 
 size_t nfine(const mg_ctx* c) { return (size_t)c->g.V * 12; }
 
+int make_parity_order(mg_ctx* ctx, const Geom& g, int** ord) {
+    if (!schur_supported(g)) return MG_OK;
+    TRY(dalloc(ctx, ord, sizeof(int) * (size_t)g.Vc));
+    parity_order(*ord, g, ctx->st);
+    CKL();
+    return MG_OK;
+}
+
 int read_scalars(mg_ctx* ctx, int first, int count) {
     CK(cudaMemcpyAsync(ctx->h_scal + first, ctx->R.scal + first, sizeof(double) * count, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
@@ -319,6 +339,8 @@ template <typename T> int ensure_work(mg_ctx* ctx) {
     TRY(dalloc(ctx, &w.cq, cb));
     TRY(dalloc(ctx, &w.cr1, cb));
     TRY(dalloc(ctx, &w.cp1, cb));
+    TRY(dalloc(ctx, &w.eb, cb));
+    TRY(dalloc(ctx, &w.et, cb));
     if (sizeof(T) == 4) {
         const size_t tb = sizeof(unsigned long long) * 4 * (size_t)ctx->g.Vc * (nc > 0 ? nc : 2);
         TRY(dalloc(ctx, &w.ctag, tb));
@@ -335,8 +357,11 @@ int ensure_level(mg_ctx* ctx, CoarseLevel& L, int nv) {
         // tensor-core tiles) are rebuilt at the new size on demand
         CK(cudaStreamSynchronize(ctx->st));
         for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.At, (void*)L.A16,
-                        (void*)L.s16})
+                        (void*)L.s16, (void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16})
             dfree(ctx, q);
+        L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr;
+        L.h_blocks = 0;
+        L.h_state = 0;
         L.P64 = nullptr; L.P32 = nullptr; L.A64 = nullptr; L.A32 = nullptr;
         L.At = nullptr; L.A16 = nullptr; L.s16 = nullptr;
         L.at_valid = L.a16_valid = L.au_valid = L.valid = false;
@@ -396,6 +421,7 @@ int build_level(mg_ctx* ctx, CoarseLevel& L, const double2* V, int nv) {
     L.at_valid = false;
     L.a16_valid = false;
     L.au_valid = false;
+    L.h_state = 0;
     return MG_OK;
 }
 
@@ -458,6 +484,13 @@ CgnrArgs<T> cgnr_args(const CoarseLevel& L, const Geom& g, const v2<T>* rc, v2<T
     return a;
 }
 
+// Inside a solve the preconditioner's coarse solves may use the red-black form.
+struct InSolve {
+    mg_ctx* ctx;
+    explicit InSolve(mg_ctx* c) : ctx(c) { c->in_solve = true; }
+    ~InSolve() { ctx->in_solve = false; }
+};
+
 // CGNR on D_c (one persistent cooperative launch).  With iters != nullptr the
 // call waits for the result; otherwise the count is only added to
 // scal[S_CG_TOTAL] and nothing synchronises.
@@ -470,10 +503,50 @@ template <typename T> struct CgSys {
     const int* nbr;    // its neighbour table [Vc][9]
     v2<T>*cr, *cr1, *cs, *cp, *cp1, *cq;
     unsigned long long* ctag;   // epoch-tagged vectors of the on-chip solver (T == float)
+    const int* ord;    // its sites by parity (nullptr: some extent is odd)
+    v2<T>*eb, *et;     // red-black form: right-hand side, odd-site scratch
 };
 template <typename T> CgSys<T> level1_sys(mg_ctx* ctx) {
     Work<T>& w = work<T>(ctx);
-    return CgSys<T>{ctx->g, ctx->cnbr, w.cr, w.cr1, w.cs, w.cp, w.cp1, w.cq, w.ctag};
+    return CgSys<T>{ctx->g, ctx->cnbr, w.cr, w.cr1, w.cs, w.cp, w.cp1, w.cq, w.ctag, ctx->cord, w.eb, w.et};
+}
+
+// The red-black Schur form of the level's operator (and, for FP16 storage, its FP16
+// copy); *ok false where it does not exist (a singular diagonal block).
+int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16, bool* ok) {
+    const int want = f64 ? 2 : 1;
+    if (L.h_state != -1 && L.h_state != want) {
+        const size_t blocks = (size_t)g.Vc * 9, n = blocks * L.nc * L.nc;
+        if (L.h_blocks < blocks) {
+            for (void* q : {(void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16}) dfree(ctx, q);
+            L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr;
+            L.h_blocks = 0;
+            const size_t most = blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap);
+            TRY(dalloc(ctx, &L.H64, sizeof(double2) * most));
+            TRY(dalloc(ctx, &L.H32, sizeof(float2) * most));
+            L.h_blocks = blocks;
+        }
+        CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->st));
+        CK(schur_build(L.H64, L.A64, L.nc, g, f64, ctx->d_status, ctx->st));
+        int status = 0;
+        CK(cudaMemcpyAsync(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+        convert<double, float>(L.H32, L.H64, n, ctx->st);
+        CKL();
+        CK(cudaStreamSynchronize(ctx->st));
+        L.h_state = status ? -1 : want;
+        L.h16_valid = false;
+    }
+    *ok = L.h_state == want;
+    if (*ok && h16 && !L.h16_valid) {
+        if (!L.H16) {
+            TRY(dalloc(ctx, &L.H16, sizeof(__half2) * L.h_blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)));
+            TRY(dalloc(ctx, &L.hs16, sizeof(float) * L.h_blocks));
+        }
+        coarse_pack16(L.H16, L.hs16, L.H64, L.nc, g.Vc, ctx->st);
+        CKL();
+        L.h16_valid = true;
+    }
+    return MG_OK;
 }
 
 template <typename T>
@@ -519,10 +592,32 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         a.s16 = Lm.s16;
     }
     if (!onchip) {
-        CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
+        // The preconditioner of a solve: CG on the red-black Schur complement, about
+        // half the iterations at the same bytes each (with a tolerance to reach: a
+        // fixed iteration count means iterations on D_c itself, as the single-step
+        // calls and the setup run them)
+        bool eo = false;
+        CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
+        const bool h16 = std::is_same<T, float>::value && ctx->coarse16;
+        if (ctx->in_solve && sys.ord && tol > 0)
+            TRY(ensure_schur(ctx, Lm, sys.g, std::is_same<T, double>::value, h16, &eo));
+        const int half = sys.g.Vc / 2;
         PROF_BEGIN(MG_K_COARSE_SOLVE);
+        if (eo) {
+            const v2<T>* H = std::is_same<T, double>::value ? (const v2<T>*)L.H64 : (const v2<T>*)L.H32;
+            // v_o = A_oo^-1 r_o, rhat_e = r_e - A_eo v_o
+            schur_rows<T>(sys.eb, nullptr, H, rc, sys.ord + half, half, sys.nbr, L.nc, 0, 1, 1.0, 1, 1, ctx->st);
+            schur_rows<T>(sys.eb, rc, H, sys.eb, sys.ord, half, sys.nbr, L.nc, 1, 9, 1.0, 1, 1, ctx->st);
+            a.A = H;
+            if (h16) { a.A16 = L.H16; a.s16 = L.hs16; }
+            a.rc = sys.eb; a.rc_full = rc; a.ord = sys.ord; a.t = sys.et;
+        }
+        CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
         CK(cgnr_persistent<T>(a, ctx->st));
+        if (eo)   // y_o = v_o - A_oo^-1 A_oe y_e
+            schur_rows<T>(y, sys.eb, a.A, y, sys.ord + half, half, sys.nbr, L.nc, 1, 9, -1.0, 1, 1, ctx->st);
         PROF_END(MG_K_COARSE_SOLVE);
+        CKL();
         ctx->coarse_kernel_used = MG_CK_REGISTER;
     }
     if (iters) {
@@ -774,7 +869,7 @@ template <typename T> int ensure_l1work(mg_ctx* ctx) {
     TRY(dalloc(ctx, &l.zero, b1));
     TRY(dalloc(ctx, &l.sv, b1));
     TRY(dalloc(ctx, &l.sz, b1));
-    for (v2<T>** q : {&l.crc, &l.cy, &l.cr, &l.cr1, &l.cs, &l.cp, &l.cp1, &l.cq}) TRY(dalloc(ctx, q, b2));
+    for (v2<T>** q : {&l.crc, &l.cy, &l.cr, &l.cr1, &l.cs, &l.cp, &l.cp1, &l.cq, &l.eb, &l.et}) TRY(dalloc(ctx, q, b2));
     zero<T>(l.zero, n1, ctx->st);
     if (sizeof(T) == 4) {
         const size_t tb = sizeof(unsigned long long) * 4 * n2;
@@ -786,7 +881,8 @@ template <typename T> int ensure_l1work(mg_ctx* ctx) {
 }
 template <typename T> CgSys<T> level2_sys(mg_ctx* ctx) {
     L1Work<T>& l = l1work<T>(ctx);
-    return CgSys<T>{ctx->g2, ctx->cnbr2, l.cr, l.cr1, l.cs, l.cp, l.cp1, l.cq, l.ctag};
+    return CgSys<T>{ctx->g2, ctx->cnbr2, l.cr, l.cr1, l.cs, l.cp, l.cp1, l.cq, l.ctag,
+                    ctx->cord2, l.eb, l.et};
 }
 
 int clear_epoch_tags(mg_ctx* ctx) {
@@ -802,8 +898,11 @@ int ensure_level2(mg_ctx* ctx, CoarseLevel& L, int nv2) {
     if (L.cap < nv2) {
         CK(cudaStreamSynchronize(ctx->st));
         for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.At, (void*)L.A16,
-                        (void*)L.s16})
+                        (void*)L.s16, (void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16})
             dfree(ctx, q);
+        L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr;
+        L.h_blocks = 0;
+        L.h_state = 0;
         L.P64 = nullptr; L.P32 = nullptr; L.A64 = nullptr; L.A32 = nullptr;
         L.At = nullptr; L.A16 = nullptr; L.s16 = nullptr;
         L.at_valid = L.a16_valid = L.au_valid = L.valid = false;
@@ -846,6 +945,7 @@ int build_level2(mg_ctx* ctx, CoarseLevel& L, const double2* V2, int nv2) {
     L.mass = ctx->mass;
     L.valid = true;
     L.at_valid = L.a16_valid = L.au_valid = false;
+    L.h_state = 0;
     return MG_OK;
 }
 
@@ -994,6 +1094,7 @@ int vcycle(mg_ctx* ctx, const CoarseLevel& L, const v2<T>* r, v2<T>* z, Counters
 
 // ---------------------------------------------------------------- flexible GCR
 template <typename T> int gcr_solve(mg_ctx* ctx, mg_solve_info* info) {
+    InSolve guard(ctx);
     TRY(ensure_work<T>(ctx));
     Work<T>& w = work<T>(ctx);
     const mg_params& p = ctx->prm;
@@ -1464,6 +1565,8 @@ int mg_create(const int dims[4], int t_antiperiodic, const mg_params* p, void* s
         cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 4, ctx->st) != cudaSuccess ||
         cudaMemsetAsync(ctx->xch, 0, sizeof(unsigned long long) * kXchWords, ctx->st) != cudaSuccess ||
         (coarse_neighbour_table(ctx->cnbr, ctx->g, ctx->st), cudaGetLastError()) != cudaSuccess ||
+        make_parity_order(ctx, ctx->g, &ctx->cord) != MG_OK ||
+        (p->levels == 3 && make_parity_order(ctx, ctx->g2, &ctx->cord2) != MG_OK) ||
         (p->levels == 3 && (dalloc(ctx, &ctx->cnbr2, sizeof(int) * 9 * (size_t)ctx->g2.Vc) != MG_OK ||
                             (coarse_neighbour_table(ctx->cnbr2, ctx->g2, ctx->st), cudaGetLastError()) != cudaSuccess)) ||
         cudaStreamSynchronize(ctx->st) != cudaSuccess) {
@@ -1544,6 +1647,7 @@ int mg_set_mass(mg_ctx* ctx, double m) {
         ctx->full.at_valid = false;
         ctx->full.a16_valid = false;
         ctx->full.au_valid = false;
+        ctx->full.h_state = 0;
     }
     if (ctx->full2.valid) {   // A2(m) = P2^dag D_c(m) P2 = A2(m0) + (m - m0) I, P2^dag P2 = I
         CoarseLevel& L = ctx->full2;
@@ -1552,6 +1656,7 @@ int mg_set_mass(mg_ctx* ctx, double m) {
         CKL();
         L.mass = m;
         L.at_valid = L.a16_valid = L.au_valid = false;
+        L.h_state = 0;
     }
     ctx->mass = m;
     CK(cudaStreamSynchronize(ctx->st));

@@ -154,6 +154,10 @@ template <typename T> struct CgnrArgs {
     const int* nbr;        // coarse neighbour table [Vc][9]
     const v2<T>* rc;
     int nc;
+    // red-black form (ord != nullptr): A / A16 the Schur operator H, rc = rhat (even entries)
+    const int* ord = nullptr;          // sites by parity (parity_order)
+    const v2<T>* rc_full = nullptr;    // right-hand side of D_c
+    v2<T>* t = nullptr;                // scratch of the odd sites
     int upb, rsp, bs;      // split of the rows over CTAs and threads (set by the launcher)
     Geom g;
     double tol2;
@@ -204,6 +208,17 @@ void h_multi_axpy(float2* z, const uint2* B, const float* S, const Geom& g, int 
 // e += alpha r; r -= alpha q when update_r (alpha from scal[S_MR_ALPHA])
 void mr_update_h(float2* e, HalfSpinor r, ConstHalfSpinor q, const Geom& g, bool update_r, const Reduce& R,
                  cudaStream_t st);
+
+// Red-black Schur form of a coarse operator (kernels_schur.cu)
+bool schur_supported(const Geom& g);   // every coarse extent even
+void parity_order(int* ord, const Geom& g, cudaStream_t st);   // ord[Vc]: even sites, then odd ones
+// H from A (both [X][9][b][a] FP64); products in FP32 unless f64; *status = 1: a singular block
+cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, bool f64, int* status, cudaStream_t st);
+// out[X] = base[X] + sign * sum_{d0 <= d < d1} H[X][d] in[X + d] for X in sites[0, nsites), `cols`
+// columns of panels with stride cstride (1, 1: plain coarse vectors)
+template <typename T>
+void schur_rows(v2<T>* out, const v2<T>* base, const v2<T>* H, const v2<T>* in, const int* sites, int nsites,
+                const int* nbr, int nc, int d0, int d1, double sign, int cols, int cstride, cudaStream_t st);
 
 // Coarse CGLS with the operator on chip (kernels_cgls.cu).  The operator rows
 // of each aggregate are cut into units of `ru` rows, Au[X*H + h][d][b][a].
