@@ -97,7 +97,7 @@ struct BcgSmem {
         off_acc = off_s2 + (size_t)nc * ts * 8;
         off_col = off_acc + (size_t)3 * rgs * npad * 8;
         off_col = (off_col + 15) & ~(size_t)15;
-        total = off_col + (size_t)npad * (3 * 8 + 12 * 4);
+        total = off_col + (size_t)npad * (3 * 8 + 13 * 4);
     }
 };
 
@@ -193,12 +193,27 @@ struct BcgCta {
     __device__ BcgCta(const BcgArgs& args, unsigned char* smem, uint64_t* bars, int* flags)
         : a(args), L(args.nc, args.nw, args.npad, args.stages), sm(smem) {
         nc = a.nc; nvh = nc >> 1; nw = a.nw; nch = a.npad / nw;
-        const long long NJ = (long long)a.g.Vc * nch;
+        const long long NJ = (long long)(a.ord ? a.g.Vc / 2 : a.g.Vc) * nch;
         j0 = (int)(blockIdx.x * NJ / gridDim.x);
         j1 = (int)((blockIdx.x + 1) * NJ / gridDim.x);
         full = bars; empty = bars + kBcgMaxStages; acc_full = bars + 2 * kBcgMaxStages; acc_empty = acc_full + 2;
         gate = acc_empty + 2;
         fail = flags; stop = flags + 1;
+    }
+
+    // Phases.  A stencil is one phase over all sites, or, in the red-black form, a phase
+    // over the odd sites (their eight neighbours, all even) and one over the even sites
+    // (the site itself and its neighbours); a phase has the same jobs in every CTA's
+    // share, nd items (directions 9 - nd ..) per job.
+    __device__ int dirs(int phase) const { return a.ord && !(phase & 1) ? 8 : 9; }
+    __device__ int site(int phase, int job) const {
+        const int i = job / nch;
+        return a.ord ? __ldg(a.ord + ((phase & 1) ? 0 : a.g.Vc / 2) + i) : i;
+    }
+    // operand of the phase's stencil: the adjoint's (btu) and D's (bts) take turns
+    __device__ const __half* operand(int phase) const {
+        const int stencil = a.ord ? phase >> 1 : phase;
+        return ((stencil & 1) != (a.first_dag != 0)) ? a.btu : a.bts;
     }
 
     // ------------------------------------------------------------ copies (two warps)
@@ -209,28 +224,30 @@ struct BcgCta {
     // iteration: its tiles run ahead across the grid barriers, as far as stages are
     // free; the operand's wait for the gate of each phase.
     __device__ void copy_operator(unsigned int* b_items) {
-        const int S = a.stages, R = min(S, 9), lane = threadIdx.x & 31;
+        const int S = a.stages, lane = threadIdx.x & 31;
         const size_t blk = (size_t)2 * nc * nc;
-        unsigned int next = 0;      // past the last item this lane armed
+        unsigned int next = 0;      // items armed
         bool ok = true;
-        for (unsigned int job = 0; ok; job += j1 - j0)
-            for (int j = j0; j < j1 && ok; ++j)
-                for (int d0 = 0; d0 < 9 && ok; d0 += R) {
-                    const int d = d0 + lane;
-                    bool mine = true;
-                    if (lane < R && d < 9) {
-                        const unsigned int i = (job + (j - j0)) * 9 + d, k = i / S;
-                        const int st = (int)(i - k * S);
-                        mine = i < (unsigned int)S || wait_stop(empty + st, (k - 1) & 1u);
-                        if (mine) {
+        for (int phase = 0; ok; ++phase) {
+            const int nd = dirs(phase), R = min(S, nd);
+            for (int j = j0; j < j1 && ok; ++j) {
+                const int X = site(phase, j);
+                for (int l0 = 0; l0 < nd && ok; l0 += R) {
+                    const int n = min(R, nd - l0);
+                    const unsigned int i = next + lane, k = i / S;
+                    const int st = (int)(i - k * S), d = 9 - nd + l0 + lane;
+                    // all lanes of a round or none, so that `next` is the number armed
+                    ok = __all_sync(0xffffffffu, lane >= n || i < (unsigned int)S || wait_stop(empty + st, (k - 1) & 1u));
+                    if (ok) {
+                        if (lane < n) {
                             mbar_expect_tx(full + st, L.a_copy);
-                            bulk_copy_g2s(sm + (size_t)st * L.stage, a.At + ((size_t)(j / nch) * 9 + d) * blk, L.a_copy,
-                                          full + st);
-                            next = i + 1;
+                            bulk_copy_g2s(sm + (size_t)st * L.stage, a.At + ((size_t)X * 9 + d) * blk, L.a_copy, full + st);
                         }
+                        next += n;
                     }
-                    ok = __all_sync(0xffffffffu, mine);
                 }
+            }
+        }
         // drain: the tiles that no operand joined (the arrival that is missing is made
         // here); after a failure, time enough for any copy to land
         asm volatile("barrier.cta.sync 2, 64;" ::: "memory");
@@ -238,32 +255,32 @@ struct BcgCta {
             for (int i = 0; i < 1000; ++i) __nanosleep(1000);
             return;
         }
-        const unsigned int b0 = *b_items;
-        for (unsigned int i = b0; i < b0 + S; ++i)
-            if (lane < R && (int)(i % 9) % R == lane && i < next) {
-                const unsigned int k = i / S;
-                const int st = (int)(i - k * S);
-                mbar_arrive(full + st);
-                mbar_wait(full + st, k & 1u, kBcgWait);
-            }
+        for (unsigned int i = *b_items + lane; i < next; i += 32) {
+            const unsigned int k = i / S;
+            const int st = (int)(i - k * S);
+            mbar_arrive(full + st);
+            mbar_wait(full + st, k & 1u, kBcgWait);
+        }
     }
-    __device__ void copy_operand(int phase, unsigned int* b_items) {   // phase odd: the adjoint's operand (btu)
-        const int S = a.stages, R = min(S, 9), lane = threadIdx.x & 31;
+    __device__ void copy_operand(unsigned int* b_items) {
+        const int S = a.stages, lane = threadIdx.x & 31;
         const size_t tile = (size_t)4 * nc * nw;
-        unsigned int job = 0;
-        for (uint32_t gate_par = 0;; ++phase, gate_par ^= 1u, job += j1 - j0) {
+        unsigned int next = 0;
+        uint32_t gate_par = 0;
+        bool ok = true;
+        for (int phase = 0; ok; ++phase, gate_par ^= 1u) {
             if (!__all_sync(0xffffffffu, bcg_wait(gate, gate_par, fail, a.err)) || *stop) break;
             fence_proxy_async_all();    // tiles written by other CTAs before the grid barrier
-            const __half* bt = (phase & 1) ? a.btu : a.bts;
-            bool ok = true;
-            for (int j = j0; j < j1 && ok; ++j)
-                for (int d0 = 0; d0 < 9 && ok; d0 += R) {
-                    const int d = d0 + lane;
+            const __half* bt = operand(phase);
+            const int nd = dirs(phase), R = min(S, nd);
+            for (int j = j0; j < j1 && ok; ++j) {
+                const int X = site(phase, j), c = j - j / nch * nch;
+                for (int l0 = 0; l0 < nd && ok; l0 += R, next += R) {
+                    const int n = min(R, nd - l0);
                     bool mine = true;
-                    if (lane < R && d < 9) {
-                        const unsigned int i = (job + (j - j0)) * 9 + d, k = i / S;
-                        const int st = (int)(i - k * S), X = j / nch, c = j - X * nch;
-                        const int Y = __ldg(a.nbr + (size_t)X * 9 + d);
+                    if (lane < n) {
+                        const unsigned int i = next + lane, k = i / S;
+                        const int st = (int)(i - k * S), Y = __ldg(a.nbr + (size_t)X * 9 + 9 - nd + l0 + lane);
                         mine = i < (unsigned int)S || bcg_wait(empty + st, (k - 1) & 1u, fail, a.err);
                         if (mine) {
                             mbar_expect_tx(full + st, L.b_copy);
@@ -272,10 +289,11 @@ struct BcgCta {
                         }
                     }
                     ok = __all_sync(0xffffffffu, mine);
+                    if (n < R) next -= R - n;
                 }
-            if (!ok) break;
+            }
         }
-        if (lane == 0) *b_items = job * 9;
+        if (lane == 0) *b_items = next;
         asm volatile("barrier.cta.sync 2, 64;" ::: "memory");
     }
     // as bcg_wait; false without an error when the launch has ended
@@ -300,19 +318,21 @@ struct BcgCta {
         const uint64_t step_a = lbo_a >> 3, step_b = lbo_b >> 3, step_st = L.stage >> 4;
         const uint32_t acc = tmem + (uint32_t)(which * 4 * nw);
         uint32_t gate_par = 0, acc_par = 1u;   // a fresh barrier passes a wait for parity 1
-        unsigned int job = 0;
-        for (bool ok = true; ok; job += jobs) {
+        unsigned int job = 0, base = 0;        // jobs and items before this phase
+        int phase = 0;
+        for (bool ok = true; ok; job += jobs, base += jobs * dirs(phase), ++phase) {
             if (!bcg_wait(gate, gate_par, fail, a.err) || *stop) break;
             gate_par ^= 1u;
+            const int nd = dirs(phase);
             for (unsigned int j = (job ^ which) & 1u; j < jobs && ok; j += 2) {   // this warp's jobs: (job + j) odd or even
                 if (!bcg_wait(acc_empty + which, acc_par, fail, a.err)) { ok = false; break; }
                 acc_par ^= 1u;
                 tc_fence_after();
-                const unsigned int i0 = (job + j) * 9, k0 = i0 / S;
+                const unsigned int i0 = base + j * nd, k0 = i0 / S;
                 unsigned int st = i0 - k0 * S;
                 uint32_t par = k0 & 1u;
                 uint64_t da = da0 + st * step_st, db = db0 + st * step_st;
-                for (int d = 0; d < 9; ++d) {
+                for (int d = 0; d < nd; ++d) {
                     if (!bcg_wait(full + st, par, fail, a.err)) { ok = false; break; }
                     tc_fence_after();
                     mma_f16(acc, da, db, idesc, d > 0 ? 1u : 0u);
@@ -488,7 +508,8 @@ struct BcgCta {
         float* sc_s = isu + np;                                    // scales for the next s and u tiles
         float* sc_u = sc_s + np;
         float* fr = sc_u + np;                                     // power of two that brings rc to unit size
-        int* done = reinterpret_cast<int*>(fr + np);               // 1: this column is frozen
+        float* sc_tu = fr + np;
+        int* done = reinterpret_cast<int*>(sc_tu + np);               // 1: this column is frozen
         int* its = done + np;
         const float rows = (float)((double)a.g.Vc * nc);
         for (int i = t; i < 3 * rgs * np; i += kEpi) acc[i] = Sum2{0.f, 0.f};
@@ -519,15 +540,26 @@ struct BcgCta {
             return;
         }
 
-        // the size of rc per column: the largest CTA's |rc|^2 (float bits order as integers)
+        // entry o of column col of the right-hand side that the tolerance refers to, at the
+        // job's site and, red-black, at its odd counterpart
+        const bool eo = a.ord != nullptr;
+        auto full2 = [&](int j, int r, int col) {
+            const int i = (j0 + j) / nch;
+            const float2 v = a.rc_full[((size_t)(eo ? __ldg(a.ord + i) : i) * nc + r) * np + col];
+            float q = v.x * v.x + v.y * v.y;
+            if (eo) {
+                const float2 w = a.rc_full[((size_t)__ldg(a.ord + a.g.Vc / 2 + i) * nc + r) * np + col];
+                q += w.x * w.x + w.y * w.y;
+            }
+            return q;
+        };
+        // the size of that right-hand side per column: the largest CTA's share of its
+        // norm (float bits order as integers)
         if (act)
             for (int j = 0; j < jobs; ++j) {
-                const int X = (j0 + j) / nch, col = (j0 + j - X * nch) * nw + n;
+                const int col = (j0 + j) % nch * nw + n;
                 float s = 0.f;
-                for (int r = rg; r < nc; r += rgs) {
-                    const float2 v = a.rc[((size_t)X * nc + r) * np + col];
-                    s += v.x * v.x + v.y * v.y;
-                }
+                for (int r = rg; r < nc; r += rgs) s += full2(j, r, col);
                 add2(col_acc(0, col), s);
             }
         epi_sync();
@@ -556,9 +588,27 @@ struct BcgCta {
             fx[i] = fx[np + i] = fx[2 * np + i] = 0x1p42f;
         }
         epi_sync();
+        int phase = 0;
+        // the odd half of a red-black stencil: t = sum H x, straight into the operand's tiles
+        // (the scale of x, so that both halves' operands add up in one accumulator)
+        auto odd_half = [&](__half* bt, const float* inv, const float* sc) {
+            if (!eo) return true;
+            for (int j = 0; j < jobs; ++j) {
+                const int X = site(phase, j0 + j), c = (j0 + j) % nch, col = c * nw + n;
+                if (!take(tmem)) return false;
+                if (act)
+                    for (int r = rg; r < nc; r += rgs) stage(r, product(r, inv[col], false), sc[col], false);
+                epi_sync();
+                write_tile(bt, X, c);
+            }
+            ++phase;
+            return grid_barrier(true);
+        };
+        // sites of the other phases
+        auto at = [&](int j) { return eo ? __ldg(a.ord + (j0 + j) / nch) : (j0 + j) / nch; };
         // r = rc 2^-e, y = 0; the tile of r for s = D_c^dag r
         for (int j = 0; j < jobs; ++j) {
-            const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+            const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
             if (act) {
                 float s = 0.f;
                 const float f = done[col] ? 0.f : fr[col], sc = sc_u[col];
@@ -570,7 +620,7 @@ struct BcgCta {
                     v = f != 0.f ? make_float2(f * v.x, f * v.y) : make_float2(0.f, 0.f);
                     a.r[o] = v;
                     a.y[o] = z;
-                    s += v.x * v.x + v.y * v.y;
+                    s += f * f * full2(j, r, col);   // |r_0|^2 of the full system
                     stage(r, v, sc, true);
                 }
                 add2(col_acc(2, col), s);
@@ -581,8 +631,9 @@ struct BcgCta {
         }
         if (!grid_barrier(true)) return;
         // s = D_c^dag r, its tile and norm
+        if (!odd_half(a.btu, isu, sc_u)) return;
         for (int j = 0; j < jobs; ++j) {
-            const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+            const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
             if (!take(tmem)) return;
             if (act) {
                 float s = 0.f;
@@ -598,11 +649,13 @@ struct BcgCta {
             epi_sync();
             write_tile(a.bts, X, c);
         }
+        ++phase;
         for (int it = 0;; ++it) {
             if (!grid_barrier(true)) return;
             // phase A: u = D_c s, its tile and norm
+            if (!odd_half(a.bts, iss, sc_s)) return;
             for (int j = 0; j < jobs; ++j) {
-                const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+                const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
                 if (!take(tmem)) return;
                 if (act) {
                     float s = 0.f;
@@ -618,6 +671,7 @@ struct BcgCta {
                 epi_sync();
                 write_tile(a.btu, X, c);
             }
+            ++phase;
             unsigned long long* sums = a.sums + (size_t)(it & 1) * 3 * np;
             publish(fx, sums);
             if (!grid_barrier(true)) return;
@@ -627,6 +681,7 @@ struct BcgCta {
             bool running = false;
             for (int i = t; i < np; i += kEpi) {
                 isu[i] = 1.f / sc_u[i];
+                sc_tu[i] = sc_u[i];   // the scale of the u tile, for the odd half's
                 if (!done[i]) {
                     double tot[3];
 #pragma unroll
@@ -662,8 +717,15 @@ struct BcgCta {
             running = epi_sync(running);
             // phase B: w = D_c^dag u and the updates on the own rows
             const bool first = it == 0;
+            if (eo && running) {
+                if (!odd_half(a.btu, isu, sc_tu)) return;
+            } else if (eo) {   // the odd half that was started; its even half never is
+                for (int j = 0; j < jobs; ++j)
+                    if (!take(tmem)) return;
+                break;
+            }
             for (int j = 0; j < jobs; ++j) {
-                const int X = (j0 + j) / nch, c = j0 + j - X * nch, col = c * nw + n;
+                const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
                 if (!take(tmem)) return;
                 if (!running) continue;   // nothing left to do but to take what was started
                 if (act) {
@@ -708,12 +770,13 @@ struct BcgCta {
                     alo[i] = 1.0 / alo[i];
                 }
             }
+            ++phase;
             if (!running) break;
         }
         // the solution in the units of rc
         if (act)
             for (int j = 0; j < jobs; ++j) {
-                const int X = (j0 + j) / nch, col = (j0 + j - X * nch) * nw + n;
+                const int X = at(j), col = (j0 + j) % nch * nw + n;
                 if (done[col] == 2) continue;
                 const float f = 1.f / fr[col];
                 for (int r = rg; r < nc; r += rgs) {
@@ -723,7 +786,13 @@ struct BcgCta {
                 }
             }
         if (blockIdx.x == 0)
-            for (int i = t; i < np; i += kEpi) a.iters[i] = (double)its[i];
+            for (int i = t; i < np; i += kEpi) {
+                a.iters[i] = (double)its[i];
+                if (i == 0 && a.scal) {
+                    a.scal[S_CG_ITERS] = (double)its[0];
+                    a.scal[S_CG_TOTAL] += (double)its[0];
+                }
+            }
         if (t == 0) *stop = 1;
         epi_sync();
         open_gate();
@@ -761,7 +830,7 @@ __global__ void __launch_bounds__(kBcgThreads, 1) k_bcg(BcgArgs a) {
     if (warp == 0) {
         c.copy_operator(&s_items);
     } else if (warp == 1) {
-        c.copy_operand(a.mode == BCG_APPLY ? (a.dag ? 1 : 0) : 1, &s_items);
+        c.copy_operand(&s_items);
     } else if (warp < 4) {
         if ((threadIdx.x & 31) == 0) c.multiply(tmem, warp - 2, c.gate + warp - 1);
     } else {
@@ -807,9 +876,11 @@ cudaError_t bcg_launch(const BcgArgs& args, cudaStream_t st) {
     BcgArgs a = args;
     a.mx = a.bar + 4;
     a.sums = reinterpret_cast<unsigned long long*>(a.bar + 4 + a.npad);
-    if (!bcg_shape(a.nc, a.npad, a.g.Vc, &a.nw, &a.stages)) return cudaErrorInvalidValue;
+    if (!bcg_shape(a.nc, a.npad, a.ord ? a.g.Vc / 2 : a.g.Vc, &a.nw, &a.stages)) return cudaErrorInvalidValue;
+    a.first_dag = a.mode == BCG_APPLY ? a.dag : 1;   // the CG starts with s = D_c^dag r
+    if (!a.rc_full) a.rc_full = a.rc;
     const int sms = device_sm_count();
-    const long long jobs = (long long)a.g.Vc * (a.npad / a.nw);
+    const long long jobs = (long long)(a.ord ? a.g.Vc / 2 : a.g.Vc) * (a.npad / a.nw);
     const int grid = (int)std::min<long long>(jobs, sms);
     // past half an SM, so that one CTA has the SM's tensor memory to itself
     const size_t sm = std::max<size_t>(BcgSmem(a.nc, a.nw, a.npad, a.stages).total, 116 * 1024);
@@ -913,6 +984,22 @@ __global__ void k_panel_unpack_t(double2* __restrict__ out, const v2<T>* __restr
         v2<T> v = in[r * npad + n];
         out[i] = make_double2((double)v.x, (double)v.y);
     }
+}
+__global__ void k_panel_column(float2* __restrict__ out, const float2* __restrict__ in, long long n, int npad) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n * npad; i += (long long)gridDim.x * blockDim.x)
+        out[i] = i % npad == 0 ? in[i / npad] : make_float2(0.f, 0.f);
+}
+__global__ void k_column_of_panel(float2* __restrict__ out, const float2* __restrict__ in, long long n, int npad) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = in[i * npad];
+}
+void panel_column(float2* out, const float2* in, long long n, int npad, cudaStream_t st) {
+    note_launch();
+    k_panel_column<<<ew_grid2(n * npad), 256, 0, st>>>(out, in, n, npad);
+}
+void column_of_panel(float2* out, const float2* in, long long n, int npad, cudaStream_t st) {
+    note_launch();
+    k_column_of_panel<<<ew_grid2(n), 256, 0, st>>>(out, in, n, npad);
 }
 void panel_pack(float2* out, const double2* in, long long rows, int nrhs, int npad, cudaStream_t st) {
     note_launch();

@@ -631,8 +631,8 @@ namespace wmg {
 // are cut into rsp parts of equal size; unit u = X * rsp + part.  A CTA works on
 // upb consecutive units at a time, tpu = 9 * bs * (row groups of a part) threads
 // each: thread (unit, d, column part, row group).
-// FP32 and FP16 operators (bound by the operator's bytes): rsp = bs = 1, whole
-// aggregates, as many as fit the CTA.  FP64 (bound by the FP64 pipe, two FMAs
+// FP32 and FP16 operators (bound by the operator's bytes): whole aggregates (rsp =
+// 1), as many as fit the CTA while every SM has two CTAs, then column parts.  FP64 (bound by the FP64 pipe, two FMAs
 // per clock and SM): every SM has to have an equal share of the rows.  With
 // whole aggregates an 8^4 lattice (16 aggregates) ran on 4 SMs and 12^3 x 24
 // (162 aggregates) on 54; cut into parts, one CTA per SM (its partial sums are
@@ -644,7 +644,6 @@ struct CgnrSplit {
     // the FP32 / FP16 split with its constants known to the compiler (index
     // arithmetic by run-time divisors cost 5-8 % of an iteration)
     template <typename T> __device__ int parts() const { return sizeof(T) == 4 ? 1 : rsp; }
-    template <typename T> __device__ int cols() const { return sizeof(T) == 4 ? 1 : bs; }
 };
 
 // One CG phase on the units of this CTA, upb at a time: stage the operand on
@@ -715,7 +714,7 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
                          const float* __restrict__ s16, int nc, const CgnrSplit& sp, const Geom& g, v2<T>* xs,
                          cx<T>* part, const int* __restrict__ nbr, T& n0, T& n1) {
     constexpr int R = RowsPerThread<T, H16>::value;
-    const int rsp = sp.template parts<T>(), bs = sp.template cols<T>();
+    const int rsp = sp.template parts<T>(), bs = sp.bs;
     const int nvh = nc >> 1, nrow = 9 * nc, ngl = nc / R / rsp, rows = sizeof(T) == 4 ? nc : ngl * R, nsum = 9 * bs;
     const int tpu = nsum * ngl, nsite = HALF ? g.Vc / 2 : g.Vc, nunit = nsite * rsp;
     const int ul = threadIdx.x / tpu, rem = threadIdx.x - ul * tpu;
@@ -814,9 +813,16 @@ __device__ void cg_phase(const PhaseArgs<T>& ph, const v2<T>* __restrict__ A, co
             if (U2 < nunit) {
                 const int X2 = HALF ? __ldg(ph.sites + Xi2) : Xi2, d0 = HALF == HALF_O ? bs : 0;   // no self block in t
                 const cx<T>* ps = part + (size_t)u2 * nsum * rows + (t - u2 * rows);
-                cx<T> sum = ps[d0 * rows];
-#pragma unroll 8
-                for (int dd = d0 + 1; dd < nsum; ++dd) sum = sum + ps[dd * rows];
+                // four chains: an FP64 add is some sixty clocks to the next that needs it
+                cx<T> c[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) c[q] = ps[(d0 + q) * rows];
+                int dd = d0 + 4;
+                for (; dd + 4 <= nsum; dd += 4)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) c[q] = c[q] + ps[(dd + q) * rows];
+                for (; dd < nsum; ++dd) c[0] = c[0] + ps[dd * rows];
+                cx<T> sum = (c[0] + c[1]) + (c[2] + c[3]);
                 if (HALF == HALF_O) {
                     st<T>(ph.t + (size_t)X2 * nc + a2, sum);
                     continue;
@@ -849,7 +855,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
     const CgnrSplit sp{a.upb, a.rsp, a.bs};
     v2<T>* xs = reinterpret_cast<v2<T>*>(smem_raw);
     cx<T>* part = reinterpret_cast<cx<T>*>(smem_raw + sizeof(v2<T>) * 9 * nc * ((sp.upb + 2 * sp.rsp - 2) / sp.rsp));
-    __shared__ T shr[33];
+    __shared__ T shr[66];
     const unsigned int G = gridDim.x;
     unsigned int* cnt = a.bar;
     unsigned int* gen = a.bar + 1;
@@ -934,8 +940,8 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
             write_partial<T>(n0, a.partials, 1, shr);
             write_partial<T>(n1, a.partials, 2, shr);
             if (!grid_sync(cnt, gen, G, a.err)) return;
-            T gnew = sum_partials<T>(a.partials, 1, G, shr);
-            r2 = sum_partials<T>(a.partials, 2, G, shr);
+            T gnew;
+            sum_partials2<T>(a.partials, 1, G, shr, gnew, r2);
             ++it;
             if (r2 <= (T)a.tol2 * rc2 || it >= a.maxit) break;
             beta = gnew / gamma;
@@ -958,12 +964,17 @@ template <typename T, bool H16> size_t cgnr_smem(int nc, const CgnrSplit& s) {
 }
 template <typename T, bool H16> int cgnr_block_threads(int nc, const CgnrSplit& s) {
     const int tpu = 9 * s.bs * (nc / RowsPerThread<T, H16>::value / s.rsp);
-    return (s.upb * tpu + 31) / 32 * 32;
+    return std::max(128, (s.upb * tpu + 31) / 32 * 32);   // at least four warps to stage the operand
 }
 template <typename T, bool H16> CgnrSplit cgnr_split(int nc, int Vc, int sms) {
     constexpr int most = CgnrMaxThreads<T>::value;
     const int ngrp = nc / RowsPerThread<T, H16>::value;
-    if (sizeof(T) == 4) return CgnrSplit{std::max(1, most / (9 * ngrp)), 1, 1};
+    if (sizeof(T) == 4) {
+        // as many aggregates as fit while every SM has one; small lattices' aggregates in
+        // column parts
+        const int fit = std::max(1, most / (9 * ngrp)), upb = std::max(1, std::min(fit, Vc / sms));
+        return CgnrSplit{upb, 1, std::max(1, std::min(most / (9 * ngrp * upb), nc / 8))};
+    }
     // FP64: the parts per aggregate that give the busiest SM the fewest rows
     // (2 % per part for the operand staged once per CTA that shares an aggregate)
     int rsp = 1;

@@ -184,31 +184,43 @@ cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, boo
 //   v_o = A_oo^-1 r_o,  rhat_e = r_e - A_eo v_o,  y_o = v_o - A_oo^-1 A_oe y_e.
 // One CTA per site, the rows over the lanes, the columns of the blocks over groups
 // of nc threads; bound by the blocks' bytes, read once.
-constexpr int kRowGroups = 8;
-template <typename T>
-__global__ void k_schur_rows(v2<T>* __restrict__ out, const v2<T>* base, const v2<T>* __restrict__ H,
-                             const v2<T>* __restrict__ in, const int* __restrict__ sites, const int* __restrict__ nbr,
-                             int nc, int d0, int d1, T sign, size_t cstride) {
+constexpr int kRowGroups = 8, kRowCols = 4;   // threads of a row, panel columns per read of the blocks
+template <typename T, int NC>
+__global__ void k_schur_rows(v2<T>* out, const v2<T>* base, const v2<T>* __restrict__ H, const v2<T>* in,
+                             const int* __restrict__ sites, const int* __restrict__ nbr, int nc, int d0, int d1, T sign,
+                             int cols, size_t cstride) {
     extern __shared__ unsigned char smem_raw[];
-    v2<T>* xs = reinterpret_cast<v2<T>*>(smem_raw);
-    v2<T>* part = xs + 8 * nc + nc;
-    const int X = sites[blockIdx.x], nd = d1 - d0, K = nd * nc, n = blockIdx.y;
-    for (int i = threadIdx.x; i < K; i += blockDim.x)
-        xs[i] = in[((size_t)__ldg(nbr + (size_t)X * 9 + d0 + i / nc) * nc + i % nc) * cstride + n];
-    __syncthreads();
-    const int a = threadIdx.x % nc, grp = threadIdx.x / nc;
-    cx<T> s(0, 0);
-    if (grp < kRowGroups) {
-        const v2<T>* h = H + ((size_t)X * 9 + d0) * nc * nc + a;
-#pragma unroll 4
-        for (int k = grp; k < K; k += kRowGroups) cmad(s, ldg<T>(h + (size_t)k * nc), ld<T>(xs + k));
-        st<T>(part + grp * nc + a, s);
+    v2<T>* xs = reinterpret_cast<v2<T>*>(smem_raw);       // [d][b][NC]
+    v2<T>* part = xs + 9 * nc * NC;                       // [group][a][NC]
+    const int X = sites[blockIdx.x], K = (d1 - d0) * nc, n0 = blockIdx.y * NC, ncol = min(NC, cols - n0);
+    for (int i = threadIdx.x; i < K * NC; i += blockDim.x) {
+        const int k = i / NC, n = i - k * NC;
+        v2<T> v; v.x = 0; v.y = 0;
+        if (n < ncol) v = in[((size_t)__ldg(nbr + (size_t)X * 9 + d0 + k / nc) * nc + k % nc) * cstride + n0 + n];
+        xs[i] = v;
     }
     __syncthreads();
-    if (threadIdx.x < nc) {
-        s = ld<T>(part + a);
-        for (int q = 1; q < kRowGroups; ++q) s = s + ld<T>(part + q * nc + a);
-        const size_t o = ((size_t)X * nc + a) * cstride + n;
+    const int a = threadIdx.x % nc, grp = threadIdx.x / nc;
+    if (grp < kRowGroups) {
+        cx<T> s[NC];
+#pragma unroll
+        for (int n = 0; n < NC; ++n) s[n] = cx<T>(0, 0);
+        const v2<T>* h = H + ((size_t)X * 9 + d0) * nc * nc + a;
+#pragma unroll 4
+        for (int k = grp; k < K; k += kRowGroups) {
+            const cx<T> hk = ldg<T>(h + (size_t)k * nc);
+#pragma unroll
+            for (int n = 0; n < NC; ++n) cmad(s[n], hk, ld<T>(xs + k * NC + n));
+        }
+#pragma unroll
+        for (int n = 0; n < NC; ++n) st<T>(part + (grp * nc + a) * NC + n, s[n]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nc * ncol; i += blockDim.x) {
+        const int r = i / ncol, n = i - r * ncol;
+        cx<T> s = ld<T>(part + r * NC + n);
+        for (int q = 1; q < kRowGroups; ++q) s = s + ld<T>(part + (q * nc + r) * NC + n);
+        const size_t o = ((size_t)X * nc + r) * cstride + n0 + n;
         s = sign * s;
         if (base) s = s + ld<T>(base + o);
         st<T>(out + o, s);
@@ -217,9 +229,14 @@ __global__ void k_schur_rows(v2<T>* __restrict__ out, const v2<T>* base, const v
 template <typename T>
 void schur_rows(v2<T>* out, const v2<T>* base, const v2<T>* H, const v2<T>* in, const int* sites, int nsites,
                 const int* nbr, int nc, int d0, int d1, double sign, int cols, int cstride, cudaStream_t st) {
+    const int thr = (kRowGroups * nc + 31) / 32 * 32;
+    const size_t sm = sizeof(v2<T>) * (9 + kRowGroups) * nc;
     note_launch();
-    k_schur_rows<T><<<dim3(nsites, cols), (kRowGroups * nc + 31) / 32 * 32, sizeof(v2<T>) * (9 + kRowGroups) * nc, st>>>(
-        out, base, H, in, sites, nbr, nc, d0, d1, (T)sign, cstride);
+    if (cols > 1)
+        k_schur_rows<T, kRowCols><<<dim3(nsites, (cols + kRowCols - 1) / kRowCols), thr, kRowCols * sm, st>>>(
+            out, base, H, in, sites, nbr, nc, d0, d1, (T)sign, cols, cstride);
+    else
+        k_schur_rows<T, 1><<<nsites, thr, sm, st>>>(out, base, H, in, sites, nbr, nc, d0, d1, (T)sign, cols, cstride);
 }
 template void schur_rows<float>(v2<float>*, const v2<float>*, const v2<float>*, const v2<float>*, const int*, int, const int*,
                                 int, int, int, double, int, int, cudaStream_t);

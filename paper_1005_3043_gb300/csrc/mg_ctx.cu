@@ -44,6 +44,8 @@ struct CoarseLevel {
     float2* H32 = nullptr;
     __half2* H16 = nullptr;   // its FP16 copy and block scales
     float* hs16 = nullptr;
+    __half* Ht = nullptr;     // its FP16 tensor-core tiles (batched path)
+    bool ht_valid = false;
     size_t h_blocks = 0;      // nc x nc blocks the buffers hold
     int h_state = 0;          // 0 not built, 1 FP32 products, 2 FP64 products, -1 a singular diagonal block
     bool h16_valid = false;
@@ -53,15 +55,21 @@ struct CoarseLevel {
     bool valid = false;
 };
 
-// Workspace of the batched (multi-RHS) solve, sized for npad panel columns.
-struct BatchWork {
-    int npad = 0, nrhs_cap = 0, K = 0, nc = 0;
-    float2 *rcB = nullptr, *yB = nullptr, *rB = nullptr, *sB = nullptr, *pB = nullptr, *qB = nullptr, *uB = nullptr,
-           *zB = nullptr;
+// Workspace of the panel coarse solver (kernels_batched.cu) for npad columns.
+struct PanelWork {
+    int npad = 0, nc = 0, Vc = 0;
+    float2 *rc = nullptr, *y = nullptr, *r = nullptr, *s = nullptr, *p = nullptr, *q = nullptr, *u = nullptr, *z = nullptr;
+    float2* e = nullptr;            // red-black form: rhat (even sites) and A_oo^-1 r (odd sites)
     __half *bts = nullptr, *btu = nullptr;   // operand tiles of the tensor-core stencil
-    unsigned int* sync = nullptr;   // grid barrier and grid sums of the coarse kernel
+    unsigned int* sync = nullptr;   // grid barrier and grid sums
     double* iters = nullptr;        // npad
     int* flags = nullptr;           // [0] error
+};
+
+// Workspace of the batched (multi-RHS) solve.
+struct BatchWork {
+    PanelWork pw;
+    int nrhs_cap = 0, K = 0;
     int* h_flags = nullptr;         // pinned
     double* h_iters = nullptr;      // pinned, npad
     float2* r32 = nullptr;          // nrhs x n
@@ -178,6 +186,7 @@ struct mg_ctx {
     double setup_ms = 0.0;           // device time of the last adaptive setup (CUDA events)
     CoarseLevel full, trunc;
     BatchWork bw;
+    PanelWork pw1;                   // one right-hand side (FP16 operators that do not fit on chip)
     EoWork eo;
     // third level (levels == 3)
     Geom g2{};                       // the level-1 lattice cut into level-2 aggregates
@@ -357,8 +366,9 @@ int ensure_level(mg_ctx* ctx, CoarseLevel& L, int nv) {
         // tensor-core tiles) are rebuilt at the new size on demand
         CK(cudaStreamSynchronize(ctx->st));
         for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.At, (void*)L.A16,
-                        (void*)L.s16, (void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16})
+                        (void*)L.s16, (void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16, (void*)L.Ht})
             dfree(ctx, q);
+        L.Ht = nullptr;
         L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr;
         L.h_blocks = 0;
         L.h_state = 0;
@@ -518,7 +528,8 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16,
     if (L.h_state != -1 && L.h_state != want) {
         const size_t blocks = (size_t)g.Vc * 9, n = blocks * L.nc * L.nc;
         if (L.h_blocks < blocks) {
-            for (void* q : {(void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16}) dfree(ctx, q);
+            for (void* q : {(void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16, (void*)L.Ht}) dfree(ctx, q);
+            L.Ht = nullptr;
             L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr;
             L.h_blocks = 0;
             const size_t most = blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap);
@@ -534,7 +545,7 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16,
         CKL();
         CK(cudaStreamSynchronize(ctx->st));
         L.h_state = status ? -1 : want;
-        L.h16_valid = false;
+        L.h16_valid = L.ht_valid = false;
     }
     *ok = L.h_state == want;
     if (*ok && h16 && !L.h16_valid) {
@@ -546,6 +557,76 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16,
         CKL();
         L.h16_valid = true;
     }
+    return MG_OK;
+}
+
+// ---------------------------------------------------------------- coarse solve of a panel
+int ensure_tiles(mg_ctx* ctx, CoarseLevel& L, int Vc) {
+    if (L.at_valid) return MG_OK;
+    const size_t nc = (size_t)2 * L.cap;
+    if (!L.At) TRY(dalloc(ctx, &L.At, sizeof(__half) * (size_t)Vc * 9 * 2 * nc * nc));
+    coarse_tiles(L.At, L.A64, L.nc, Vc, ctx->st);
+    CKL();
+    L.at_valid = true;
+    return MG_OK;
+}
+int ensure_panel(mg_ctx* ctx, PanelWork& w, int npad, int nc, int Vc) {
+    if (w.npad >= npad && w.nc == nc && w.Vc == Vc) return MG_OK;
+    if (w.npad) {   // grow: release the smaller workspace first
+        CK(cudaStreamSynchronize(ctx->st));
+        for (void* q : {(void*)w.rc, (void*)w.y, (void*)w.r, (void*)w.s, (void*)w.p, (void*)w.q, (void*)w.u, (void*)w.z,
+                        (void*)w.e, (void*)w.bts, (void*)w.btu, (void*)w.sync, (void*)w.iters, (void*)w.flags})
+            dfree(ctx, q);
+        w = PanelWork{};
+    }
+    const size_t pe = sizeof(float2) * (size_t)Vc * nc * npad;
+    for (float2** q : {&w.rc, &w.y, &w.r, &w.s, &w.p, &w.q, &w.u, &w.z, &w.e}) {
+        TRY(dalloc(ctx, q, pe));
+        CK(cudaMemsetAsync(*q, 0, pe, ctx->st));
+    }
+    TRY(dalloc(ctx, &w.bts, bcg_tile_bytes(nc, npad, Vc)));
+    TRY(dalloc(ctx, &w.btu, bcg_tile_bytes(nc, npad, Vc)));
+    TRY(dalloc(ctx, &w.sync, bcg_sync_bytes(npad)));
+    TRY(dalloc(ctx, &w.iters, sizeof(double) * npad));
+    TRY(dalloc(ctx, &w.flags, sizeof(int) * 4));
+    CK(cudaMemsetAsync(w.flags, 0, sizeof(int) * 4, ctx->st));
+    w.npad = npad;
+    w.nc = nc;
+    w.Vc = Vc;
+    return MG_OK;
+}
+// CG on the normal equations of the level's operator for nrhs columns of the panel
+// w.rc -> w.y, red-black where the lattice allows it (see coarse_solve).  *err is
+// raised on a timed-out wait; scal (optional) receives column 0's iterations.
+int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, const int* ord, PanelWork& w, int nrhs,
+                double tol, int maxit, int* err, double* scal) {
+    BcgArgs c{};
+    c.bts = w.bts; c.btu = w.btu; c.rc = w.rc;
+    c.y = w.y; c.r = w.r; c.s = w.s; c.u = w.u; c.p = w.p; c.z = w.z; c.q = w.q;
+    c.nbr = nbr; c.bar = w.sync; c.err = err; c.iters = w.iters; c.scal = scal;
+    c.nc = L.nc; c.npad = w.npad; c.nrhs = nrhs; c.maxit = maxit; c.mode = BCG_SOLVE; c.tol2 = tol * tol;
+    c.g = g;
+    const int half = g.Vc / 2;
+    bool eo = false;
+    if (ord && tol > 0) TRY(ensure_schur(ctx, L, g, false, false, &eo));
+    if (!eo) {
+        TRY(ensure_tiles(ctx, L, g.Vc));
+    } else if (!L.ht_valid) {
+        if (!L.Ht) TRY(dalloc(ctx, &L.Ht, sizeof(__half) * L.h_blocks * 2 * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)));
+        coarse_tiles(L.Ht, L.H64, L.nc, g.Vc, ctx->st);
+        L.ht_valid = true;
+    }
+    c.At = eo ? L.Ht : L.At;
+    PROF_BEGIN(MG_K_COARSE_SOLVE);
+    if (eo) {
+        schur_rows<float>(w.e, nullptr, L.H32, w.rc, ord + half, half, nbr, L.nc, 0, 1, 1.0, nrhs, w.npad, ctx->st);
+        schur_rows<float>(w.e, w.rc, L.H32, w.e, ord, half, nbr, L.nc, 1, 9, 1.0, nrhs, w.npad, ctx->st);
+        c.ord = ord; c.rc = w.e; c.rc_full = w.rc;
+    }
+    CK(bcg_launch(c, ctx->st));
+    if (eo) schur_rows<float>(w.y, w.e, L.H32, w.y, ord + half, half, nbr, L.nc, 1, 9, -1.0, nrhs, w.npad, ctx->st);
+    PROF_END(MG_K_COARSE_SOLVE);
+    CKL();
     return MG_OK;
 }
 
@@ -590,6 +671,26 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         TRY(ensure_a16(ctx, Lm, sys.g.Vc));
         a.A16 = Lm.A16;
         a.s16 = Lm.s16;
+    }
+    int nw = 0, stages = 0;
+    if (!onchip && std::is_same<T, float>::value && ctx->coarse16 && ctx->in_solve && tol > 0 && !iters &&
+        ctx->prm.coarse_kernel != 1 &&
+        bcg_shape(L.nc, 8, sys.g.Vc / 2, &nw, &stages)) {
+        // FP16 operator larger than the chip: the panel solver with one column of eight in
+        // use, its operator tiles streaming ahead across the grid barriers (24^3x32, Nv =
+        // 24: 249 -> 114 ms of coarse solves per solve against the
+        // register-streaming kernel on D_c, 177 with that kernel red-black)
+        TRY(ensure_panel(ctx, ctx->pw1, 8, L.nc, sys.g.Vc));
+        PanelWork& w = ctx->pw1;
+        const long long n = (long long)sys.g.Vc * L.nc;
+        panel_column(w.rc, (const float2*)rc, n, w.npad, ctx->st);
+        CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
+        TRY(panel_solve(ctx, const_cast<CoarseLevel&>(L), sys.g, sys.nbr, sys.ord, w, 1, tol, maxit, (int*)(ctx->bar + 2),
+                        ctx->R.scal));
+        column_of_panel((float2*)y, w.y, n, w.npad, ctx->st);
+        CKL();
+        ctx->coarse_kernel_used = MG_CK_REGISTER;
+        return MG_OK;
     }
     if (!onchip) {
         // The preconditioner of a solve: CG on the red-black Schur complement, about
@@ -898,8 +999,9 @@ int ensure_level2(mg_ctx* ctx, CoarseLevel& L, int nv2) {
     if (L.cap < nv2) {
         CK(cudaStreamSynchronize(ctx->st));
         for (void* q : {(void*)L.P64, (void*)L.P32, (void*)L.A64, (void*)L.A32, (void*)L.At, (void*)L.A16,
-                        (void*)L.s16, (void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16})
+                        (void*)L.s16, (void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16, (void*)L.Ht})
             dfree(ctx, q);
+        L.Ht = nullptr;
         L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr;
         L.h_blocks = 0;
         L.h_state = 0;
@@ -2665,49 +2767,25 @@ namespace {
 
 int round16(int n) { return ((n + 15) / 16) * 16; }
 
-int ensure_tiles(mg_ctx* ctx, CoarseLevel& L) {
-    if (L.at_valid) return MG_OK;
-    const size_t nc = (size_t)2 * L.cap;
-    if (!L.At) TRY(dalloc(ctx, &L.At, sizeof(__half) * (size_t)ctx->g.Vc * 9 * 2 * nc * nc));
-    coarse_tiles(L.At, L.A64, L.nc, ctx->g.Vc, ctx->st);
-    CKL();
-    L.at_valid = true;
-    return MG_OK;
-}
-
 int ensure_batch(mg_ctx* ctx, int nrhs) {
     BatchWork& b = ctx->bw;
     int npad = round16(nrhs), nc = ctx->full.nc;
     size_t n = nfine(ctx);
     int K = std::min(ctx->prm.gcr_restart, ctx->K);
-    if (b.npad >= npad && b.nrhs_cap >= nrhs && b.nc == nc && b.K >= K) return MG_OK;
-    if (b.npad || b.nrhs_cap) {   // grow: release the smaller workspace first
+    TRY(ensure_panel(ctx, b.pw, npad, nc, ctx->g.Vc));
+    if (b.nrhs_cap >= nrhs && b.K >= K) return MG_OK;
+    if (b.nrhs_cap) {   // grow: release the smaller workspace first
         CK(cudaStreamSynchronize(ctx->st));
-        for (void* q : {(void*)b.rcB, (void*)b.yB, (void*)b.rB, (void*)b.sB, (void*)b.pB, (void*)b.qB, (void*)b.uB,
-                        (void*)b.zB, (void*)b.bts, (void*)b.btu, (void*)b.sync, (void*)b.iters, (void*)b.flags,
-                        (void*)b.r32, (void*)b.Z, (void*)b.Pk, (void*)b.x64, (void*)b.b64, (void*)b.scal,
-                        (void*)b.partials, (void*)b.ticket, (void*)b.scal_s})
+        for (void* q : {(void*)b.r32, (void*)b.Z, (void*)b.Pk, (void*)b.x64, (void*)b.b64, (void*)b.scal, (void*)b.partials,
+                        (void*)b.ticket, (void*)b.scal_s})
             dfree(ctx, q);
         cudaFreeHost(b.h_flags);
         cudaFreeHost(b.h_iters);
         cudaFreeHost(b.h_scal);
+        const PanelWork pw = b.pw;
         b = BatchWork{};
-        npad = std::max(npad, round16(nrhs));
+        b.pw = pw;
     }
-    size_t pe = (size_t)ctx->g.Vc * nc * npad;
-    TRY(dalloc(ctx, &b.rcB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.yB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.rB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.sB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.pB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.qB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.uB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.zB, sizeof(float2) * pe));
-    TRY(dalloc(ctx, &b.bts, bcg_tile_bytes(nc, npad, ctx->g.Vc)));
-    TRY(dalloc(ctx, &b.btu, bcg_tile_bytes(nc, npad, ctx->g.Vc)));
-    TRY(dalloc(ctx, &b.sync, bcg_sync_bytes(npad)));
-    TRY(dalloc(ctx, &b.iters, sizeof(double) * npad));
-    TRY(dalloc(ctx, &b.flags, sizeof(int) * 4));
     TRY(dalloc(ctx, &b.r32, sizeof(float2) * n * nrhs));
     TRY(dalloc(ctx, &b.Z, sizeof(float2) * n * nrhs * K));
     TRY(dalloc(ctx, &b.Pk, sizeof(float2) * n * nrhs * K));
@@ -2715,36 +2793,24 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
     TRY(dalloc(ctx, &b.b64, sizeof(double2) * n * nrhs));
     TRY(dalloc(ctx, &b.scal, sizeof(double) * S_COUNT * nrhs));
     CK(cudaMallocHost(&b.h_flags, sizeof(int) * 4));
-    CK(cudaMallocHost(&b.h_iters, sizeof(double) * npad));
+    CK(cudaMallocHost(&b.h_iters, sizeof(double) * nrhs));
     CK(cudaMallocHost(&b.h_scal, sizeof(double) * S_COUNT * nrhs));
     CK(cudaMemsetAsync(b.scal, 0, sizeof(double) * S_COUNT * nrhs, ctx->st));
-    CK(cudaMemsetAsync(b.flags, 0, sizeof(int) * 4, ctx->st));
-    b.npad = npad;
     b.nrhs_cap = nrhs;
-    b.nc = nc;
     b.K = K;
     return MG_OK;
 }
 
-// CGNR on the panel rcB -> yB for columns 0..nrhs-1 (zero columns stay zero).
+// CGNR on the panel pw.rc -> pw.y for columns 0..nrhs-1 (zero columns stay zero).
 // iters_out[n] += coarse iterations of column n.
 int batched_coarse_solve(mg_ctx* ctx, int nrhs, double tol, int maxit, std::vector<double>& iters_out) {
     BatchWork& b = ctx->bw;
-    TRY(ensure_tiles(ctx, ctx->full));
-    BcgArgs c{};
-    c.At = ctx->full.At; c.bts = b.bts; c.btu = b.btu; c.rc = b.rcB;
-    c.y = b.yB; c.r = b.rB; c.s = b.sB; c.u = b.uB; c.p = b.pB; c.z = b.zB; c.q = b.qB;
-    c.nbr = ctx->cnbr; c.bar = b.sync; c.err = b.flags; c.iters = b.iters;
-    c.nc = ctx->full.nc; c.npad = b.npad; c.nrhs = nrhs; c.maxit = maxit; c.mode = BCG_SOLVE; c.tol2 = tol * tol;
-    c.g = ctx->g;
-    PROF_BEGIN(MG_K_COARSE_SOLVE);
-    CK(bcg_launch(c, ctx->st));
-    PROF_END(MG_K_COARSE_SOLVE);
-    CK(cudaMemcpyAsync(b.h_flags, b.flags, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
-    CK(cudaMemcpyAsync(b.h_iters, b.iters, sizeof(double) * b.npad, cudaMemcpyDeviceToHost, ctx->st));
+    TRY(panel_solve(ctx, ctx->full, ctx->g, ctx->cnbr, ctx->cord, b.pw, nrhs, tol, maxit, b.pw.flags, nullptr));
+    CK(cudaMemcpyAsync(b.h_flags, b.pw.flags, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+    CK(cudaMemcpyAsync(b.h_iters, b.pw.iters, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     if (b.h_flags[0]) {
-        CK(cudaMemsetAsync(b.flags, 0, sizeof(int) * 4, ctx->st));
+        CK(cudaMemsetAsync(b.pw.flags, 0, sizeof(int), ctx->st));
         return fail(ctx, MG_ERR_TIMEOUT, "batched coarse solve: a bounded wait gave up");
     }
     for (int n = 0; n < nrhs; ++n) iters_out[n] += b.h_iters[n];
@@ -2818,7 +2884,7 @@ int solve_batched_impl(mg_ctx* ctx, int nrhs, mg_solve_info* infos) {
             if (active[r] && !cycle_end[r] && kk[r] < K && iters[r] < p.max_outer) stepping = true;
         if (stepping) {
             // restriction of every stepping source into its panel column
-            CK(cudaMemsetAsync(b.rcB, 0, sizeof(float2) * (size_t)ctx->g.Vc * L.nc * b.npad, ctx->st));
+            CK(cudaMemsetAsync(b.pw.rc, 0, sizeof(float2) * (size_t)ctx->g.Vc * L.nc * b.pw.npad, ctx->st));
             auto steps_now = [&](int r) { return active[r] && !cycle_end[r] && kk[r] < K && iters[r] < p.max_outer; };
             // runs of neighbouring stepping sources (they all step at the same kk), at most
             // `most` long
@@ -2831,7 +2897,7 @@ int solve_batched_impl(mg_ctx* ctx, int nrhs, mg_solve_info* infos) {
             for (int r = 0; r < nrhs;) {
                 const int m = run(r, nrhs);
                 if (m == 0) { ++r; continue; }
-                restrict_<float>(b.rcB, L.P32, b.r32 + r * n, L.nv, ctx->g, ctx->st, b.npad, r, Lanes{m, n, 0, 0});
+                restrict_<float>(b.pw.rc, L.P32, b.r32 + r * n, L.nv, ctx->g, ctx->st, b.pw.npad, r, Lanes{m, n, 0, 0});
                 r += m;
             }
             PROF_END(MG_K_RESTRICT);
@@ -2841,7 +2907,7 @@ int solve_batched_impl(mg_ctx* ctx, int nrhs, mg_solve_info* infos) {
                 const int m = run(r, nrhs);
                 if (m == 0) { ++r; continue; }
                 PROF_BEGIN(MG_K_PROLONG);
-                prolong<float>(b.Z + ((size_t)r * K + kk[r]) * n, L.P32, b.yB, L.nv, ctx->g, ctx->st, b.npad, r,
+                prolong<float>(b.Z + ((size_t)r * K + kk[r]) * n, L.P32, b.pw.y, L.nv, ctx->g, ctx->st, b.pw.npad, r,
                                Lanes{m, (size_t)K * n, 0, 0});
                 PROF_END(MG_K_PROLONG);
                 r += m;
@@ -3062,7 +3128,7 @@ int bcg_apply_args(mg_ctx* ctx, int npad, int nrhs, bool dag, BcgArgs* out, std:
     TRY(get(&a.bar, bcg_sync_bytes(npad)));
     TRY(get(&fl, sizeof(int) * 4));
     CK(cudaMemsetAsync(fl, 0, sizeof(int) * 4, ctx->st));
-    TRY(ensure_tiles(ctx, L));
+    TRY(ensure_tiles(ctx, L, ctx->g.Vc));
     a.At = L.At; a.rc = x; a.nbr = ctx->cnbr; a.err = fl;
     a.nc = L.nc; a.npad = npad; a.nrhs = nrhs; a.mode = BCG_APPLY; a.dag = dag ? 1 : 0; a.g = ctx->g;
     *out = a;

@@ -376,16 +376,24 @@ struct BcgArgs {
     unsigned long long* sums;   // [2][3][npad] fixed-point grid sums
     int* err;                // set to 1 if a bounded wait gave up
     double* iters;           // [npad] CG iterations (BCG_SOLVE)
+    double* scal;            // optional: solver scalars that receive column 0's iterations
+    // red-black form: sites by parity, At the tiles of the Schur operator, rc = rhat (even
+    // entries), rc_full the right-hand side of D_c; nullptr: the full operator
+    const int* ord;
+    const float2* rc_full;
     int nc, npad, nrhs, maxit, mode, dag;
     double tol2;
     Geom g;
-    int nw, stages;          // columns per job, pipeline depth (set by the launcher)
+    int nw, stages, first_dag;   // columns per job, pipeline depth, first operand (set by the launcher)
     uint32_t tmem_cols;      // (set by the launcher)
 };
 inline size_t bcg_sync_bytes(int npad) { return 16 + (size_t)npad * (4 + 2 * 3 * 8); }
 bool bcg_shape(int nc, int npad, int Vc, int* nw, int* stages);   // false: no shape for this panel
 size_t bcg_tile_bytes(int nc, int npad, long long Vc);
 cudaError_t bcg_launch(const BcgArgs& args, cudaStream_t st);
+// a coarse vector of n entries <-> column 0 of a panel (its other columns zero)
+void panel_column(float2* out, const float2* in, long long n, int npad, cudaStream_t st);
+void column_of_panel(float2* out, const float2* in, long long n, int npad, cudaStream_t st);
 // nrhs stacked FP64 coarse vectors in[n][row] <-> panel [row][npad]
 void panel_pack(float2* out, const double2* in, long long rows, int nrhs, int npad, cudaStream_t st);
 void panel_unpack(double2* out, const float2* in, long long rows, int nrhs, int npad, cudaStream_t st);

@@ -69,6 +69,32 @@ template <typename T> __device__ __forceinline__ T sum_partials(const double* pa
     for (int c = threadIdx.x; c < G; c += blockDim.x) a += (T)__ldcg(partials + (size_t)c * 4 + slot);
     return block_sum_t<T>(a, sh);
 }
+// the sums of slots slot and slot + 1 together (sh: 66 entries)
+template <typename T>
+__device__ __forceinline__ void sum_partials2(const double* partials, int slot, int G, T* sh, T& u, T& v) {
+    T a = 0, b = 0;
+    for (int c = threadIdx.x; c < G; c += blockDim.x) {
+        a += (T)__ldcg(partials + (size_t)c * 4 + slot);
+        b += (T)__ldcg(partials + (size_t)c * 4 + slot + 1);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    a = warp_sum_t(a);
+    b = warp_sum_t(b);
+    if (lane == 0) {
+        sh[warp] = a;
+        sh[33 + warp] = b;
+    }
+    __syncthreads();
+    if (warp < 2) {
+        T x = lane < nw ? sh[33 * warp + lane] : T(0);
+        x = warp_sum_t(x);
+        if (lane == 0) sh[33 * warp + 32] = x;
+    }
+    __syncthreads();
+    u = sh[32];
+    v = sh[65];
+    __syncthreads();
+}
 template <typename T> __device__ __forceinline__ void write_partial(T v, double* partials, int slot, T* sh) {
     T a = block_sum_t<T>(v, sh);
     if (threadIdx.x == 0) partials[(size_t)blockIdx.x * 4 + slot] = (double)a;
