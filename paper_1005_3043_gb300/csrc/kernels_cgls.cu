@@ -120,6 +120,12 @@ struct NoPre {
 enum { EPI_STORE = 0, EPI_TAG = 1, EPI_CG_TAG = 2 };
 enum { OV_P = 0, OV_Z = 1, OV_Q = 2, OV_Y = 3, OV_R = 4, OV_S = 5, OV_U = 6, OV_COUNT = 7 };
 
+// TM == 1: a thread's share of the operator in 32-word chunks, the first four in its
+// 128 TMEM columns, the rest in shared memory (64 KB per chunk).  FP32 at 16^3x32
+// (Nv = 20, six chunks, 394 KB per SM) stays on chip this way, 9.3 us per CG
+// iteration against 26.4 with the operator read from L2 twice an iteration (a solve
+// with 3943 iterations 113 -> 64 ms, although the latter ran red-black).
+constexpr int kTmemChunks = 4;
 constexpr int kStageRegs = 4;   // staged operand entries per thread kept as precomputed offsets
 
 // Tensor-core products (TM == 2, FP16 operator): the first kMmaRows rows of a
@@ -199,6 +205,7 @@ template <bool H16, int TM> struct CglsCta {
     // TMEM-resident operator (TM): this thread's quad qd and column split ks
     // (k = ks, ks + KS, ...), its TMEM lane/column base and the CTA-wide chunk count
     int q_ks = 0, q_qd = 0, q_KS = 1, q_quads = 0, q_nch = 0;
+    unsigned char* ext = nullptr;   // chunks past the thread's TMEM columns
     bool q_act = false;
     uint32_t q_taddr = 0, tm_base = 0;
     int st_o[kStageRegs];
@@ -242,6 +249,7 @@ template <bool H16, int TM> struct CglsCta {
             ov = reinterpret_cast<cx<float>*>(sm + a.sh.own_off);
             ov_n = a.sh.nu_max * RU;
         }
+        if (TM == 1) ext = sm + a.sh.ext_off;
         if (TM == 2) {
             bt = sm + a.sh.bt_off;
             rop = reinterpret_cast<uint32_t*>(sm + a.sh.rop_off);
@@ -392,13 +400,22 @@ template <bool H16, int TM> struct CglsCta {
 #pragma unroll
                 for (int v = 0; v < kWpq; ++v) w[i * kWpq + v] = ok ? __ldg(src + (size_t)k * RU * (kWpq / 4) + v) : 0u;
             }
-            tmem_st32(q_taddr + 32 * c, w);
+            if (c < kTmemChunks)
+                tmem_st32(q_taddr + 32 * c, w);
+            else
+#pragma unroll
+                for (int i = 0; i < 8; ++i) q_ext(c)[i * T] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
         }
         tmem_wait_st();
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
         loaded = true;
+    }
+    // TM == 1: this thread's words of chunk c >= kTmemChunks in shared memory, eight
+    // 16-byte words a CTA's threads apart
+    __device__ uint4* q_ext(int c) const {
+        return reinterpret_cast<uint4*>(ext) + (size_t)(c - kTmemChunks) * 8 * blockDim.x + threadIdx.x;
     }
     // thread 0: wait for every copy still in flight (before the CTA may exit);
     // TM: release the tensor memory
@@ -747,7 +764,15 @@ template <bool H16, int TM> struct CglsCta {
             for (int q = 0; q < 4; ++q) { P[q] = make_float2(0.f, 0.f); Q[q] = make_float2(0.f, 0.f); }
             for (int c = 0; c < q_nch; ++c) {
                 uint32_t w[32];
-                tmem_ld32(q_taddr + 32 * c, w);
+                if (c < kTmemChunks) {
+                    tmem_ld32(q_taddr + 32 * c, w);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const uint4 v = q_ext(c)[i * T];
+                        w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+                    }
+                }
                 if (q_act) {
 #pragma unroll
                     for (int i = 0; i < kQpc; ++i) {
@@ -1235,7 +1260,7 @@ bool cgls_shape(int nc, int Vc, bool h16, int mode, CglsShape* out) {
             s.groups = 1;
             off = mma_smem(off, s, K, lim.smem);
             score = (long long)s.nu_max * ru;
-        } else if ((mode == CGLS_AUTO || mode == CGLS_TMEM_CORES) && chunks <= 4 && off <= budget) {
+        } else if ((mode == CGLS_AUTO || mode == CGLS_TMEM_CORES) && chunks <= 2 * kTmemChunks && off <= budget) {
             // the operator in tensor memory; shared memory padded past half an SM
             // so that no second CTA of this kernel (and no second all-column TMEM
             // allocation) shares the SM.  Padding to the whole SM would also keep
@@ -1251,9 +1276,12 @@ bool cgls_shape(int nc, int Vc, bool h16, int mode, CglsShape* out) {
             s.groups = 1;
             // the own-row vectors of the tagged form after the exchange scratch
             s.own_off = (int)off;
-            off = std::max(off + (size_t)OV_COUNT * s.nu_max * ru * 8, (size_t)lim.smem / 2 + 4096);
+            s.ext_off = (int)round_up(off + (size_t)OV_COUNT * s.nu_max * ru * 8, 128);
+            const int ext = std::max(0, chunks - kTmemChunks);
+            off = std::max((size_t)s.ext_off + (size_t)ext * 32 * 4 * T, (size_t)lim.smem / 2 + 4096);
             if (off > budget) continue;
-            score = (long long)s.nu_max * ru + (mode == CGLS_AUTO ? (1LL << 38) : 0);   // tensor-core shapes first
+            // tensor-core shapes first, then those that need tensor memory alone
+            score = (long long)s.nu_max * ru + (mode == CGLS_AUTO ? (1LL << 38) : 0) + ((long long)ext << 39);
         } else if (mode != CGLS_TMEM_CORES && off + (size_t)s.nu_max * s.stride <= budget) {
             s.resident = 1;
             s.slots = s.nu_max;

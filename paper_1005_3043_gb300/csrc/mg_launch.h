@@ -236,7 +236,8 @@ struct CglsShape {
     int red_n;       // complex entries per reduction buffer
     int tm;          // the operator in tensor memory (all 512 columns of the SM): 1 products on the
                      // CUDA cores, 2 products on the tensor cores (tcgen05.mma, A from TMEM)
-    int tm_chunks;   // 32-column TMEM chunks per thread (tm 1)
+    int tm_chunks;   // 32-word chunks of a thread's share of the operator (tm 1): four in tensor memory,
+    int ext_off;     // the rest in shared memory from this byte offset on
     int own_off;     // byte offset of the own-row vectors of the tagged form in shared memory (0: global)
     int bt_off;      // tm 2: byte offset of the FP16 hi/lo operand tile (MMA B) in shared memory
     int mma_lbo;     // tm 2: its byte distance between core matrices adjacent in K
