@@ -110,14 +110,24 @@ struct CglsPhase {
     unsigned int etag, etag_out;
     int own_out;   // EPI_TAG with own-row vectors in shared memory: the one (OV_S, OV_U) that keeps out
     bool stop;   // set by phase when its pre-emit step declined the epilogue
+    // red-black halves (HALF_*): the tagged t of the odd sites that the even half reads
+    const unsigned long long* tt;
+    unsigned int etag_t;
 };
+// A stencil of the red-black form (kernels_schur.cu) is two phases: HALF_O computes t
+// of the odd sites from x of their neighbours (tagged tin), HALF_E the even rows from
+// x of the site itself (tin) and t of the neighbours (tt).  A CTA stages and emits only
+// the aggregates of the half's parity; only x and the even rows carry sigma3.
+enum { HALF_NONE = 0, HALF_O = 1, HALF_E = 2 };
+// roles of a staged entry in the halves (bits 24.. of st_f)
+enum { IN_O = 1 << 24, ZERO_O = 1 << 25, SELF_E = 1 << 26, T_E = 1 << 27 };
 enum { ST_IN = 0, ST_P = 1, ST_R = 2, ST_TAG = 3 };
 // pre-emit step of a phase: runs (collectively) between the stencil's products
 // and its epilogue; 1 = emit, 0 = stop without emitting, -1 = failure
 struct NoPre {
     __device__ int operator()() const { return 1; }
 };
-enum { EPI_STORE = 0, EPI_TAG = 1, EPI_CG_TAG = 2 };
+enum { EPI_STORE = 0, EPI_TAG = 1, EPI_CG_TAG = 2, EPI_T = 3 };   // EPI_T: t of the odd half
 enum { OV_P = 0, OV_Z = 1, OV_Q = 2, OV_Y = 3, OV_R = 4, OV_S = 5, OV_U = 6, OV_COUNT = 7 };
 
 // TM == 1: a thread's share of the operator in 32-word chunks, the first four in its
@@ -228,6 +238,10 @@ template <bool H16, int TM> struct CglsCta {
     // the row whose accumulator columns it reads (-1: none)
     int e_row = -1, e_o = 0, e_xl = 0, p_xl = -1;
     bool e_neg = false;
+    // red-black (TM == 1): parity of the CTA's aggregates (shared memory) and of the row
+    // quad this thread multiplies
+    unsigned char* par = nullptr;
+    int q_par = 0;
 
     __device__ CglsCta(const CglsArgs& args, unsigned char* sm) : a(args) {
         nc = a.nc; K = 9 * nc; nvh = nc >> 1; RU = a.sh.ru; H = nc / RU;
@@ -288,6 +302,27 @@ template <bool H16, int TM> struct CglsCta {
                 }
             }
         }
+    }
+    __device__ int parity_of(int X) const {
+        int xc[4];
+        coarse_coords(a.g, X, xc);
+        return (xc[0] + xc[1] + xc[2] + xc[3]) & 1;
+    }
+    // collective, before start(): the red-black roles of aggregates, entries and rows
+    __device__ void start_halves(unsigned char* sm) {
+        par = sm + 128;   // nX <= 128 (checked by the launcher)
+        for (int i = threadIdx.x; i < nX; i += blockDim.x) par[i] = (unsigned char)parity_of(X0 + i);
+        if (pre) {
+#pragma unroll
+            for (int q = 0; q < kStageRegs; ++q)
+                if (st_o[q] >= 0) {
+                    const int i = threadIdx.x + q * blockDim.x, xl = i / K;
+                    st_f[q] |= role(xl, (i - xl * K) / nc);
+                }
+        }
+    }
+    __device__ int role(int xl, int d) const {
+        return parity_of(X0 + xl) ? (d > 0 ? IN_O : ZERO_O) : (d > 0 ? T_E : SELF_E);
     }
     __device__ bool owned(int X, int b) const {
         long long u = (long long)X * H + b / RU;
@@ -389,6 +424,7 @@ template <bool H16, int TM> struct CglsCta {
         q_nch = ((K + q_KS - 1) / q_KS + kQpc - 1) / kQpc;   // chunks of the thread with ks = 0
         q_taddr = base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(128 * (warp >> 2));
         const int r = 4 * q_qd, j = r / RU, ain = r - j * RU;
+        if (par && q_act) q_par = par[(u0 + j) / H - X0];
         const uint32_t* src = reinterpret_cast<const uint32_t*>(
             reinterpret_cast<const unsigned char*>(a.Au) + (size_t)(u0 + j) * unit_bytes()) + (size_t)ain * (kWpq / 4);
         for (int c = 0; c < q_nch; ++c) {
@@ -476,6 +512,8 @@ template <bool H16, int TM> struct CglsCta {
             tag_store(ph.tout + 2 * o, w.r, w.i, ph.etag_out);
             if (ov) ov[ph.own_out * ov_n + j] = w;
             n0 += norm2(w);
+        } else if (EPI == EPI_T) {
+            tag_store(ph.tout + 2 * o, w.r, w.i, ph.etag_out);
         } else if (EPI == EPI_CG_TAG) {
             cx<float> s, u, p0, z0, q0, y0, r0;
             if (ov) {
@@ -693,7 +731,7 @@ template <bool H16, int TM> struct CglsCta {
     // n0 accumulates |out|^2 over the CTA's rows.  pre_emit() runs after the
     // products and before the first output row is emitted (see NoPre); false
     // on a failed wait.
-    template <int STAGE, bool DAG, int EPI = EPI_STORE, typename Pre = NoPre>
+    template <int STAGE, bool DAG, int EPI = EPI_STORE, int HALF = HALF_NONE, typename Pre = NoPre>
     __device__ bool phase(CglsPhase& ph, float& n0, float& n1, Pre&& pre_emit = Pre()) {
         ph.stop = false;
         const int T = blockDim.x;
@@ -702,10 +740,18 @@ template <bool H16, int TM> struct CglsCta {
             if (STAGE == ST_TAG) {
                 // all loads first, then re-poll only the entries not yet at epoch etag
                 unsigned int okm = 0;
+                // entries of this half, and where they come from
+                auto wanted = [&](int q) {
+                    return st_o[q] >= 0 && (HALF == HALF_NONE || (st_f[q] & (HALF == HALF_O ? IN_O : SELF_E | T_E)));
+                };
+                auto look = [&](int q, float2& t) {
+                    if (HALF == HALF_E && (st_f[q] & T_E)) return tag_load(ph.tt + 2 * (size_t)st_o[q], ph.etag_t, t);
+                    return tag_load(ph.tin + 2 * (size_t)st_o[q], ph.etag, t);
+                };
 #pragma unroll
                 for (int q = 0; q < kStageRegs; ++q) {
                     float2 t = make_float2(0.f, 0.f);
-                    if (st_o[q] < 0 || tag_load(ph.tin + 2 * (size_t)st_o[q], ph.etag, t)) okm |= 1u << q;
+                    if (!wanted(q) || look(q, t)) okm |= 1u << q;
                     v[q] = cx<float>(t.x, t.y);
                 }
                 long long spins = 0;
@@ -714,7 +760,7 @@ template <bool H16, int TM> struct CglsCta {
                     for (int q = 0; q < kStageRegs; ++q)
                         if (!((okm >> q) & 1u)) {
                             float2 t;
-                            if (tag_load(ph.tin + 2 * (size_t)st_o[q], ph.etag, t)) {
+                            if (look(q, t)) {
                                 okm |= 1u << q;
                                 v[q] = cx<float>(t.x, t.y);
                             }
@@ -734,9 +780,9 @@ template <bool H16, int TM> struct CglsCta {
             } else {
 #pragma unroll
                 for (int q = 0; q < kStageRegs; ++q)
-                    if (st_o[q] >= 0) {
+                    if (st_o[q] >= 0 && (HALF == HALF_NONE || (st_f[q] & (HALF == HALF_O ? IN_O | ZERO_O : SELF_E | T_E)))) {
                         cx<float> w = v[q];
-                        if (DAG && (st_f[q] & 2)) w = cx<float>(-w.r, -w.i);
+                        if (DAG && (st_f[q] & 2) && !(HALF == HALF_E && (st_f[q] & T_E))) w = cx<float>(-w.r, -w.i);
                         if (H16) w = st_s[q] * w;
                         xs[threadIdx.x + q * T] = w;
                     }
@@ -746,8 +792,20 @@ template <bool H16, int TM> struct CglsCta {
                 const int xl = i / K, kk = i - xl * K, d = kk / nc, b = kk - d * nc;
                 const int X = X0 + xl;
                 const int o = __ldg(a.nbr + (size_t)X * 9 + d) * nc + b;
-                cx<float> w = form<STAGE>(ph, o, d == 0 && owned(X, b), n1);
-                if (DAG && b >= nvh) w = cx<float>(-w.r, -w.i);
+                cx<float> w;
+                bool flip = DAG && b >= nvh;
+                if (HALF == HALF_NONE) {
+                    w = form<STAGE>(ph, o, d == 0 && owned(X, b), n1);
+                } else {
+                    if (par[xl] != (HALF == HALF_O ? 1 : 0)) continue;
+                    const bool tside = HALF == HALF_E && d > 0;
+                    float2 t = make_float2(0.f, 0.f);
+                    if (HALF == HALF_E || d > 0)
+                        if (!tag_wait((tside ? ph.tt : ph.tin) + 2 * (size_t)o, tside ? ph.etag_t : ph.etag, a.err, t)) sfail = true;
+                    w = cx<float>(t.x, t.y);
+                    flip = flip && !tside;
+                }
+                if (flip) w = cx<float>(-w.r, -w.i);
                 if (H16) w = __ldg(a.su + (size_t)X * 9 + d) * w;
                 xs[i] = w;
             }
@@ -773,7 +831,7 @@ template <bool H16, int TM> struct CglsCta {
                         w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
                     }
                 }
-                if (q_act) {
+                if (q_act && (HALF == HALF_NONE || q_par == (HALF == HALF_O ? 1 : 0))) {
 #pragma unroll
                     for (int i = 0; i < kQpc; ++i) {
                         const int k = q_ks + (c * kQpc + i) * q_KS;
@@ -802,10 +860,11 @@ template <bool H16, int TM> struct CglsCta {
                 return true;
             }
             for (int rr = threadIdx.x; rr < rows; rr += T) {
+                const int jj = rr / RU, ain = rr - jj * RU, u = u0 + jj, X = u / H, row = (u - X * H) * RU + ain;
+                if (HALF != HALF_NONE && par[X - X0] != (HALF == HALF_O ? 1 : 0)) continue;
                 cx<float> sum = red[rr];
                 for (int ks = 1; ks < q_KS; ++ks) sum = sum + red[ks * rows + rr];
-                const int jj = rr / RU, ain = rr - jj * RU, u = u0 + jj, X = u / H, row = (u - X * H) * RU + ain;
-                if (DAG && row >= nvh) sum = cx<float>(-sum.r, -sum.i);
+                if (DAG && HALF != HALF_O && row >= nvh) sum = cx<float>(-sum.r, -sum.i);
                 emit<EPI>(ph, (size_t)X * nc + row, rr, sum, n0, n1);
             }
             return true;
@@ -1067,6 +1126,130 @@ template <bool H16, int TM> __device__ void cgls_body_tag(const CglsArgs& a, Cgl
     }
 }
 
+// The same CG on the red-black Schur complement (kernels_schur.cu): a.rc = rhat on the
+// even sites, a.rc_full the right-hand side of D_c, whose norm the tolerance refers
+// to.  A stencil is two half-phases through the tagged t of the odd sites; everything
+// else, the ordering argument included, is as in cgls_body_tag: an entry of t is
+// overwritten only after staging x of all its eight neighbours, which each neighbour's
+// owner wrote after staging the old t.  Less than half the iterations, each of four
+// half-stencils instead of two stencils, and a half-stencil takes nearly as long as a
+// stencil (the round trip through L2, the barriers): 16^3x32 FP32 9.3 -> 17.5 us per
+// iteration, 3943 -> 1822 iterations, 36.7 -> 32.4 ms per solve; 8^4 30 -> 26 ms.  With
+// the tensor-core products it takes 20 us against 8.4 and does not pay.
+template <bool H16, int TM> __device__ void cgls_body_schur(const CglsArgs& a, CglsCta<H16, TM>& c) {
+    unsigned int ex = a.epoch0;
+    const unsigned int E = a.epoch0, Er = E + (unsigned int)a.maxit + 2u, Et = E + 2u * (unsigned int)a.maxit + 3u;
+    float* shr = reinterpret_cast<float*>(c.xs + (size_t)a.sh.nx_max * c.K);
+    const size_t nw = 2 * (size_t)a.g.Vc * a.nc;
+    unsigned long long *ts = a.tag, *tu = a.tag + nw, *tt = a.tag + 2 * nw;
+    float one[1] = {0.f}, rpart0 = 0.f;
+    for (int i = threadIdx.x; i < c.nu * c.RU; i += blockDim.x) {
+        const int j = i / c.RU, ain = i - j * c.RU, u = c.u0 + j, X = u / c.H;
+        const size_t o = (size_t)X * c.nc + (u - X * c.H) * c.RU + ain;
+        const bool even = c.par[X - c.X0] == 0;
+        const float2 f = a.rc_full[o], v = even ? a.rc[o] : make_float2(0.f, 0.f);
+        if (c.ov) {
+            c.ov[OV_R * c.ov_n + i] = cx<float>(v.x, v.y);
+            c.ov[OV_Y * c.ov_n + i] = cx<float>(0.f, 0.f);
+        } else {
+            a.r[o] = v;
+            a.y[o] = make_float2(0.f, 0.f);
+        }
+        if (even) tag_store(tu + 2 * o, v.x, v.y, Er);   // r_0, the operand of s_0 = Dhat^dag r_0
+        one[0] += f.x * f.x + f.y * f.y;
+        rpart0 += v.x * v.x + v.y * v.y;
+    }
+    xch_post_packed<1>(one, a.xch, ex, shr);
+    if (!xch_collect_packed<1>(one, a.xch, ex++, a.err, shr)) return;
+    const float rc2 = one[0];
+    int it = 0;
+    float r2 = rc2;
+    if (rc2 > 0.f && a.maxit > 0) {
+        CglsPhase ph{};
+        float n0 = 0.f, n1 = 0.f;
+        ph.tin = tu; ph.etag = Er;
+        ph.tout = tt; ph.etag_out = Et;
+        if (!c.template phase<ST_TAG, true, EPI_T, HALF_O>(ph, n0, n1)) return;
+        ph.tt = tt; ph.etag_t = Et;
+        ph.tout = ts; ph.etag_out = E; ph.own_out = OV_S;
+        if (!c.template phase<ST_TAG, true, EPI_TAG, HALF_E>(ph, n0, n1)) return;
+        float gpart = n0, rpart = rpart0;
+        float gamma_old = 0.f, alpha_old = 0.f;
+        for (int i = 0;; ++i) {
+            ph = CglsPhase{};
+            n0 = 0.f; n1 = 0.f;
+            ph.tin = ts; ph.etag = E + (unsigned int)i;
+            ph.tout = tt; ph.etag_out = E + 2u * (unsigned int)i;
+            if (!c.template phase<ST_TAG, false, EPI_T, HALF_O>(ph, n0, n1)) return;
+            ph.tt = tt; ph.etag_t = E + 2u * (unsigned int)i;
+            ph.tout = tu; ph.etag_out = E + (unsigned int)i; ph.own_out = OV_U;
+            if (!c.template phase<ST_TAG, false, EPI_TAG, HALF_E>(ph, n0, n1)) return;   // u = Dhat s
+            float three[3] = {n0, gpart, rpart};
+            const unsigned int ex_i = ex++;
+            xch_post_packed<3>(three, a.xch, ex_i, shr);
+            ph = CglsPhase{};
+            n0 = 0.f; n1 = 0.f;
+            ph.tin = tu; ph.etag = E + (unsigned int)i;
+            ph.tout = tt; ph.etag_out = E + 2u * (unsigned int)i + 1u;
+            if (!c.template phase<ST_TAG, true, EPI_T, HALF_O>(ph, n0, n1)) return;
+            float gamma = 0.f, alpha = 0.f;
+            ph.tt = tt; ph.etag_t = E + 2u * (unsigned int)i + 1u;
+            ph.ts = ts; ph.tu = tu;
+            ph.cp = a.p; ph.cz = a.p1; ph.cq = a.q; ph.cy = a.y; ph.cr = a.r;
+            ph.etag_out = E + (unsigned int)i + 1u;
+            ph.first = (i == 0);
+            auto pre = [&]() -> int {
+                if (!xch_collect_packed<3>(three, a.xch, ex_i, a.err, shr)) return -1;
+                const float delta = three[0];
+                gamma = three[1];
+                r2 = three[2];
+                it = i;
+                if ((i > 0 && r2 <= a.tol2 * rc2) || i >= a.maxit) return 0;
+                const float beta = i > 0 ? gamma / gamma_old : 0.f;
+                const float den = i > 0 ? delta - beta * gamma / alpha_old : delta;
+                if (!(gamma > 0.f) || !(den > 0.f)) return 0;
+                alpha = gamma / den;
+                ph.alpha = alpha;
+                ph.beta = beta;
+                return 1;
+            };
+            n0 = 0.f; n1 = 0.f;
+            if (!c.template phase<ST_TAG, true, EPI_CG_TAG, HALF_E>(ph, n0, n1, pre)) return;   // w = Dhat^dag u, updates
+            if (ph.stop) break;
+            gpart = n0;
+            rpart = n1;
+            gamma_old = gamma;
+            alpha_old = alpha;
+        }
+    }
+    if (c.ov) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < c.nu * c.RU; i += blockDim.x) {
+            const int j = i / c.RU, ain = i - j * c.RU, u = c.u0 + j, X = u / c.H;
+            const size_t o = (size_t)X * c.nc + (u - X * c.H) * c.RU + ain;
+            const cx<float> y = c.ov[OV_Y * c.ov_n + i], r = c.ov[OV_R * c.ov_n + i];
+            a.y[o] = make_float2(y.r, y.i);
+            a.r[o] = make_float2(r.r, r.i);
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.scal[S_CG_ITERS] = (double)it;
+        a.scal[S_CG_R2] = (double)r2;
+        a.scal[S_CG_RC2] = (double)rc2;
+        a.scal[S_CG_DONE] = 1.0;
+        a.scal[S_CG_TOTAL] += (double)it;
+    }
+}
+template <bool H16> __global__ void __launch_bounds__(kCglsThreads, 1) k_cgls_schur(CglsArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    CglsCta<H16, 1> c(a, smem_raw);
+    c.start_halves(smem_raw);
+    __syncthreads();
+    c.start();
+    cgls_body_schur<H16, 1>(a, c);
+    c.drain();
+}
+
 // Latency probes (see CGLS_PROBE_*): maxit rounds of the tagged form's two
 // stencils (u = D_c s, s' = D_c^dag u, tagged staging and emission, values
 // unnormalised and unused) or of its three-value exchange.  Same epochs and
@@ -1312,14 +1495,16 @@ cudaError_t cgls_onchip(const CglsArgs& args, cudaStream_t st) {
     const void* fns[2][3] = {{(const void*)k_cgls_onchip<false, 0>, (const void*)k_cgls_onchip<false, 1>, nullptr},
                              {(const void*)k_cgls_onchip<true, 0>, (const void*)k_cgls_onchip<true, 1>,
                               (const void*)k_cgls_onchip<true, 2>}};
-    const void* fn = fns[h16][tmk];
-    static std::atomic<bool> attr[kCglsDevs][2][3];   // per device: the attribute is set on the current one
+    const bool eo = args.rc_full != nullptr;   // red-black form: tensor memory, CUDA-core products
+    const void* fn = !eo ? fns[h16][tmk] : h16 ? (const void*)k_cgls_schur<true> : (const void*)k_cgls_schur<false>;
+    if (eo && (tmk != 1 || args.form != CGLS_CG_TAGGED || args.sh.nx_max > 128)) return cudaErrorInvalidValue;
+    static std::atomic<bool> attr[kCglsDevs][2][2][3];   // per device: the attribute is set on the current one
     const DevLimits lim = dev_limits();
     if (lim.dev < 0) return cudaErrorInvalidDevice;
-    if (!attr[lim.dev][h16][tmk].load(std::memory_order_acquire)) {
+    if (!attr[lim.dev][eo][h16][tmk].load(std::memory_order_acquire)) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lim.smem - 1024);
         if (e != cudaSuccess) return e;
-        attr[lim.dev][h16][tmk].store(true, std::memory_order_release);
+        attr[lim.dev][eo][h16][tmk].store(true, std::memory_order_release);
     }
     if (((args.form == CGLS_CG_TAGGED || args.form == CGLS_PROBE_STENCILS) && !args.tag) || args.sh.smem > (size_t)lim.smem - 1024 || args.sh.grid <= 0 ||
         args.sh.grid > lim.sms ||

@@ -46,6 +46,11 @@ struct CoarseLevel {
     float* hs16 = nullptr;
     __half* Ht = nullptr;     // its FP16 tensor-core tiles (batched path)
     bool ht_valid = false;
+    void* Hu = nullptr;       // its CGLS units, as Au
+    float* hsu = nullptr;
+    size_t hu_bytes = 0;
+    bool hu_valid = false, hu_h16 = false;
+    int hu_mode = 0;
     size_t h_blocks = 0;      // nc x nc blocks the buffers hold
     int h_state = 0;          // 0 not built, 1 FP32 products, 2 FP64 products, -1 a singular diagonal block
     bool h16_valid = false;
@@ -351,7 +356,7 @@ template <typename T> int ensure_work(mg_ctx* ctx) {
     TRY(dalloc(ctx, &w.eb, cb));
     TRY(dalloc(ctx, &w.et, cb));
     if (sizeof(T) == 4) {
-        const size_t tb = sizeof(unsigned long long) * 4 * (size_t)ctx->g.Vc * (nc > 0 ? nc : 2);
+        const size_t tb = sizeof(unsigned long long) * 6 * (size_t)ctx->g.Vc * (nc > 0 ? nc : 2);
         TRY(dalloc(ctx, &w.ctag, tb));
         CK(cudaMemsetAsync(w.ctag, 0, tb, ctx->st));   // epoch 0 is never awaited
     }
@@ -545,7 +550,7 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16,
         CKL();
         CK(cudaStreamSynchronize(ctx->st));
         L.h_state = status ? -1 : want;
-        L.h16_valid = L.ht_valid = false;
+        L.h16_valid = L.ht_valid = L.hu_valid = false;
     }
     *ok = L.h_state == want;
     if (*ok && h16 && !L.h16_valid) {
@@ -645,6 +650,35 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
     if (onchip) {
         CglsArgs c{};
         c.Au = L.Au; c.su = ctx->coarse16 ? L.su : nullptr; c.nbr = sys.nbr;
+        // the preconditioner of a solve runs red-black (see below)
+        bool eo = false;
+        CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
+        if (ctx->in_solve && sys.ord && tol > 0 && !iters && ctx->prm.coarse_form == 0 && L.au_shape.tm == 1 &&
+            L.au_shape.nx_max <= 128)
+            TRY(ensure_schur(ctx, Lm, sys.g, false, false, &eo));
+        const int half = sys.g.Vc / 2;
+        if (eo) {
+            const int mode = cgls_mode(ctx->prm.coarse_kernel);
+            if (!(L.hu_valid && L.hu_h16 == ctx->coarse16 && L.hu_mode == mode)) {
+                const size_t bytes = (size_t)sys.g.Vc * 9 * L.nc * L.nc * (ctx->coarse16 ? 4 : 8);
+                if (Lm.hu_bytes < bytes) {
+                    dfree(ctx, Lm.Hu);
+                    Lm.Hu = nullptr;
+                    Lm.hu_bytes = 0;
+                    TRY(dalloc(ctx, &Lm.Hu, bytes));
+                    Lm.hu_bytes = bytes;
+                }
+                if (ctx->coarse16 && !L.hsu) TRY(dalloc(ctx, &Lm.hsu, sizeof(float) * (size_t)sys.g.Vc * 9));
+                coarse_pack_units(Lm.Hu, ctx->coarse16 ? Lm.hsu : nullptr, L.H64, L.nc, L.au_shape.ru, sys.g.Vc, ctx->coarse16,
+                                  ctx->st);
+                CKL();
+                Lm.hu_h16 = ctx->coarse16;
+                Lm.hu_mode = mode;
+                Lm.hu_valid = true;
+            }
+            c.Au = L.Hu;
+            c.su = ctx->coarse16 ? L.hsu : nullptr;
+        }
         c.rc = (const float2*)a.rc; c.y = (float2*)a.y; c.r = (float2*)a.r; c.r1 = (float2*)a.r1;
         c.s = (float2*)a.s; c.p = (float2*)a.p; c.p1 = (float2*)a.p1; c.q = (float2*)a.q;
         c.nc = L.nc; c.g = sys.g; c.tol2 = (float)(tol * tol); c.maxit = maxit;
@@ -663,7 +697,18 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         ctx->xch_epoch += (unsigned int)reserve;
         CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
         PROF_BEGIN(MG_K_COARSE_SOLVE);
+        if (eo) {
+            v2<float>* eb = (v2<float>*)sys.eb;
+            const v2<float>* b = (const v2<float>*)rc;
+            schur_rows<float>(eb, nullptr, L.H32, b, sys.ord + half, half, sys.nbr, L.nc, 0, 1, 1.0, 1, 1, ctx->st);
+            schur_rows<float>(eb, b, L.H32, eb, sys.ord, half, sys.nbr, L.nc, 1, 9, 1.0, 1, 1, ctx->st);
+            c.rc = eb;
+            c.rc_full = b;
+        }
         CK(cgls_onchip(c, ctx->st));
+        if (eo)
+            schur_rows<float>((v2<float>*)y, (v2<float>*)sys.eb, L.H32, (v2<float>*)y, sys.ord + half, half, sys.nbr, L.nc, 1, 9,
+                              -1.0, 1, 1, ctx->st);
         PROF_END(MG_K_COARSE_SOLVE);
         ctx->coarse_kernel_used = c.sh.tm == 2 ? MG_CK_TMEM_MMA : c.sh.tm ? MG_CK_TMEM : c.sh.resident ? MG_CK_SMEM : MG_CK_STREAM;
     } else if (std::is_same<T, float>::value && ctx->coarse16) {
@@ -973,7 +1018,7 @@ template <typename T> int ensure_l1work(mg_ctx* ctx) {
     for (v2<T>** q : {&l.crc, &l.cy, &l.cr, &l.cr1, &l.cs, &l.cp, &l.cp1, &l.cq, &l.eb, &l.et}) TRY(dalloc(ctx, q, b2));
     zero<T>(l.zero, n1, ctx->st);
     if (sizeof(T) == 4) {
-        const size_t tb = sizeof(unsigned long long) * 4 * n2;
+        const size_t tb = sizeof(unsigned long long) * 6 * n2;
         TRY(dalloc(ctx, &l.ctag, tb));
         CK(cudaMemsetAsync(l.ctag, 0, tb, ctx->st));   // epoch 0 is never awaited
     }
@@ -988,9 +1033,9 @@ template <typename T> CgSys<T> level2_sys(mg_ctx* ctx) {
 
 int clear_epoch_tags(mg_ctx* ctx) {
     if (ctx->wf.ctag)
-        CK(cudaMemsetAsync(ctx->wf.ctag, 0, sizeof(unsigned long long) * 4 * (size_t)ctx->g.Vc * ctx->wf.cnc, ctx->st));
+        CK(cudaMemsetAsync(ctx->wf.ctag, 0, sizeof(unsigned long long) * 6 * (size_t)ctx->g.Vc * ctx->wf.cnc, ctx->st));
     if (ctx->l1f.ctag)
-        CK(cudaMemsetAsync(ctx->l1f.ctag, 0, sizeof(unsigned long long) * 4 * (size_t)ctx->g2.Vc * 2 * ctx->prm.nvec2,
+        CK(cudaMemsetAsync(ctx->l1f.ctag, 0, sizeof(unsigned long long) * 6 * (size_t)ctx->g2.Vc * 2 * ctx->prm.nvec2,
                            ctx->st));
     return MG_OK;
 }

@@ -267,7 +267,9 @@ struct CglsArgs {
     unsigned long long* xch;   // exchange slots, kXchWords words
     unsigned int epoch0;       // first epoch of this launch; 2 * maxit + 4 are reserved
     int form;                  // CGLS_TEXTBOOK or CGLS_CG_TAGGED
-    unsigned long long* tag;   // CGLS_CG_TAGGED: epoch-tagged s and u, 4 * Vc * nc words
+    unsigned long long* tag;   // CGLS_CG_TAGGED: epoch-tagged s, u and t, 6 * Vc * nc words
+    const float2* rc_full;     // red-black form (Au: units of the Schur operator, rc: rhat): the right-hand
+                               // side of D_c; nullptr: the full operator
     double* scal;
     int* err;                  // error flag (zeroed before the launch)
     CglsShape sh;

@@ -22,7 +22,7 @@ SHAPES = [((8, 8, 8, 8), (4, 4, 4, 4), 4), ((4, 4, 8, 8), (2, 2, 2, 2), 6), ((8,
           ((4, 4, 4, 8), (2, 2, 2, 2), 24)]
 
 
-def run(L, B, nv, prec, tol, batch=False):
+def run(L, B, nv, prec, tol, batch=False, kernel=1):
     U = rough_gauge(L, seed=8)
     V0 = synth.gaussian_vectors(L, nv, 97)
     b = np.stack([synth.gaussian_spinor(L, 98, stream=i) for i in range(3)])
@@ -31,7 +31,7 @@ def run(L, B, nv, prec, tol, batch=False):
         p.block[i] = B[i]
     p.nvec, p.setup_group, p.prec_inner = nv, 2, prec
     p.coarse_tol, p.max_outer = tol, 1
-    p.coarse_kernel = 1                      # the operator from global memory
+    p.coarse_kernel = kernel                 # 1: the operator from global memory
     p.smoother_fp16 = 2
     with wmg.WilsonMG(L, p) as mg:
         mg.set_links(U)
@@ -52,6 +52,16 @@ def run(L, B, nv, prec, tol, batch=False):
                                           (wmg.MG_FP16, 1e-5, 2.0 ** -11)])
 def test_schur_solve_is_the_full_solve(L, B, nv, prec, tol, eps):
     assert run(L, B, nv, prec, tol) < 20 * eps
+
+
+# on chip: tensor-core products where the shape allows them (0), CUDA-core products (4);
+# the last shape has several aggregates and both parities in every CTA, the first ones
+# parts of one aggregate
+@pytest.mark.parametrize("L,B,nv", SHAPES + [((8, 8, 8, 8), (2, 2, 2, 2), 10)])
+@pytest.mark.parametrize("prec,tol,eps", [(wmg.MG_FP32, 1e-5, 1e-5), (wmg.MG_FP16, 1e-5, 2.0 ** -11)])
+@pytest.mark.parametrize("kernel", [0, 4])
+def test_schur_solve_on_chip(L, B, nv, prec, tol, eps, kernel):
+    assert run(L, B, nv, prec, tol, kernel=kernel) < 20 * eps
 
 
 @pytest.mark.parametrize("L,B,nv", [s for s in SHAPES if s[2] % 4 == 0])
