@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(kHalfThreads) k_h_orth(uint2* __restrict__ B, 
         const size_t self6 = (size_t)X * 6 * g.Vb + l, V6 = (size_t)6 * g.V;
         cx<float> w[12];
         ld_site_h(B + (size_t)k * V6 + self6, S[(size_t)k * g.V + s], g.Vb, w);
+#pragma unroll 4
         for (int j = 0; j < k; ++j) {
             cx<float> v[12];
             ld_site_h(B + (size_t)j * V6 + self6, S[(size_t)j * g.V + s] * fac[j], g.Vb, v);
@@ -382,8 +383,10 @@ void dslash_h_mrdot(HalfSpinor out, ConstHalfSpinor in, const uint2* U16, const 
 void h_multidot(const uint2* B, const float* S, const Geom& g, int k, const Reduce& R, cudaStream_t st) {
     note_launch();
     // at most the CTAs that the SMs hold at once, with equal numbers of sites: each
-    // ends with a reduction of up to 32 sums, and the last one adds all of them
-    const long long need = half_grid(g.V), most = 4LL * device_sm_count();
+    // ends with a reduction of up to 32 sums, and the last one adds all of them.
+    // 16^3x32, k <= 4: 1024 CTAs 9.6 us, 512 11.5; k <= 8: 512 24.7, 1024 28.6;
+    // k <= 12: 512 23.5, 1024 27.0; two threads per site 10.4, 18.3 and 44.9
+    const long long need = half_grid(g.V), most = (k <= 4 ? 7LL : 4LL) * device_sm_count();
     const int grid = (int)((need + (need + most - 1) / most - 1) / ((need + most - 1) / most));
     if (k <= 4) k_h_multidot<4><<<grid, kHalfThreads, 0, st>>>(B, S, g, k, R);
     else if (k <= 8) k_h_multidot<8><<<grid, kHalfThreads, 0, st>>>(B, S, g, k, R);

@@ -284,10 +284,7 @@ __device__ __forceinline__ void grid_reduce(TA (&v)[N], double* partials, unsign
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double t[N];
-#pragma unroll
-        for (int q = 0; q < N; ++q) t[q] = tot[q];
-        fin(t);
+        fin(tot);
         *ticket = 0u;
     }
 }
