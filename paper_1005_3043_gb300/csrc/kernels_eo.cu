@@ -23,17 +23,20 @@ namespace wmg {
 
 constexpr int kEoThreads = 256;
 
+// 32-bit arithmetic (see site_of): the six 64-bit divisions here and the 64-bit
+// products of the eight neighbours were a good part of a hop
 __host__ __device__ inline void eo_coords(const EoGeom& e, int p, long long i, int c[4]) {
-    long long r = i / e.Lh0;
-    const int xh = (int)(i - r * e.Lh0);
-    c[1] = (int)(r % e.L[1]);
-    r /= e.L[1];
-    c[2] = (int)(r % e.L[2]);
-    c[3] = (int)(r / e.L[2]);
+    unsigned int r = (unsigned int)i / (unsigned int)e.Lh0;
+    const int xh = (int)((unsigned int)i - r * (unsigned int)e.Lh0);
+    unsigned int q = r / (unsigned int)e.L[1];
+    c[1] = (int)(r - q * (unsigned int)e.L[1]);
+    r = q / (unsigned int)e.L[2];
+    c[2] = (int)(q - r * (unsigned int)e.L[2]);
+    c[3] = (int)r;
     c[0] = 2 * xh + ((c[1] + c[2] + c[3] + p) & 1);
 }
-__host__ __device__ inline long long eo_lex(const EoGeom& e, const int c[4]) {
-    return c[0] + (long long)e.L[0] * (c[1] + (long long)e.L[1] * (c[2] + (long long)e.L[2] * c[3]));
+__host__ __device__ inline int eo_lex(const EoGeom& e, const int c[4]) {
+    return c[0] + e.L[0] * (c[1] + e.L[1] * (c[2] + e.L[2] * c[3]));
 }
 
 // ---------------------------------------------------------------- layout conversion
@@ -129,7 +132,7 @@ __device__ __forceinline__ void eo_hop1(cx<T> (&acc)[4][3], const v2<T>* __restr
     cn[MU] += FWD ? 1 : -1;
     if (cn[MU] == e.L[MU]) { cn[MU] = 0; flip = (MU == 3) && e.tap; }
     if (cn[MU] < 0) { cn[MU] = e.L[MU] - 1; flip = (MU == 3) && e.tap; }
-    const long long j = eo_lex(e, cn) >> 1;
+    const int j = eo_lex(e, cn) >> 1;
     cx<T> ps[4][3];
 #pragma unroll
     for (int s = 0; s < 4; ++s)

@@ -24,7 +24,8 @@ template <typename T>
 __global__ void k_spinor_to_internal(v2<T>* out, const double2* __restrict__ in, Geom g) {
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     long long lex = lex_site(g, X, l);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
@@ -37,7 +38,8 @@ template <typename T>
 __global__ void k_spinor_from_internal(double2* out, const v2<T>* __restrict__ in, Geom g) {
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     long long lex = lex_site(g, X, l);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
@@ -49,7 +51,8 @@ template <typename T>
 __global__ void k_links_to_internal(v2<T>* out, const double2* __restrict__ in, Geom g) {
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     long long lex = lex_site(g, X, l);
     for (int mu = 0; mu < 4; ++mu)
 #pragma unroll
@@ -212,7 +215,8 @@ __global__ void __launch_bounds__(DslashShape<T, MINB>::threads, DslashShape<T, 
     long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     T red[3] = {0, 0, 0};   // per-site partial sums in T, promoted once for the grid reduction
     if (s < g.V) {
-        int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+        int X, l;
+        site_of(g, s, X, l);
         int lc[4], xc[4];
         local_coords(g, l, lc);
         coarse_coords(g, X, xc);
@@ -315,7 +319,8 @@ __global__ void __launch_bounds__(kSplitThreads)
     R = R.lane(blockIdx.y);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long s = blockIdx.x * (long long)kSplitSites + lane;
-    const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     if (s < g.V) {
         int lc[4], xc[4];
         local_coords(g, l, lc);

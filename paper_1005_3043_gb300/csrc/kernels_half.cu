@@ -127,7 +127,8 @@ __global__ void __launch_bounds__(kHalfThreads, MODE == HMODE_MRDOT ? 6 : 7)
     const float fin = IN16 ? inv_norm(fnorm) : 1.f;   // the input's site scales times fin
     float red[3] = {0.f, 0.f, 0.f};
     if (s < g.V) {
-        const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+        int X, l;
+        site_of(g, s, X, l);
         int lc[4], xc[4];
         local_coords(g, l, lc);
         coarse_coords(g, X, xc);
@@ -185,7 +186,8 @@ __global__ void __launch_bounds__(kHalfThreads) k_mr_update_h(float2* __restrict
                                                                const double* __restrict__ scal) {
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     const size_t self = (size_t)X * 12 * g.Vb + l, self6 = (size_t)X * 6 * g.Vb + l;
     const cx<float> a((float)scal[S_MR_ALPHA], (float)scal[S_MR_ALPHA + 1]);
     cx<float> rv[12];
@@ -208,7 +210,8 @@ __global__ void __launch_bounds__(kHalfThreads) k_mr_update_h(float2* __restrict
 __global__ void k_to_half(uint2* __restrict__ h, float* __restrict__ sc, const float2* __restrict__ x, Geom g) {
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     const size_t self = (size_t)X * 12 * g.Vb + l;
     cx<float> v[12];
 #pragma unroll
@@ -218,7 +221,8 @@ __global__ void k_to_half(uint2* __restrict__ h, float* __restrict__ sc, const f
 __global__ void k_from_half(float2* __restrict__ x, const uint2* __restrict__ h, const float* __restrict__ sc, Geom g) {
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     const size_t self = (size_t)X * 12 * g.Vb + l;
     cx<float> v[12];
     ld_site_h(h + (size_t)X * 6 * g.Vb + l, sc[(size_t)X * g.Vb + l], g.Vb, v);
@@ -257,7 +261,8 @@ __global__ void __launch_bounds__(kHalfThreads) k_h_multidot(const uint2* __rest
 #pragma unroll
     for (int j = 0; j < 2 * NJ; ++j) a[j] = 0.f;
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < g.V; s += (long long)gridDim.x * blockDim.x) {
-        const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+        int X, l;
+        site_of(g, s, X, l);
         const size_t self6 = (size_t)X * 6 * g.Vb + l, V6 = (size_t)6 * g.V;
         cx<float> w[12];
         ld_site_h(B + (size_t)k * V6 + self6, S[(size_t)k * g.V + s], g.Vb, w);
@@ -295,7 +300,8 @@ __global__ void __launch_bounds__(kHalfThreads) k_h_orth(uint2* __restrict__ B, 
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     float a = 0.f;
     if (s < g.V) {
-        const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+        int X, l;
+        site_of(g, s, X, l);
         const size_t self6 = (size_t)X * 6 * g.Vb + l, V6 = (size_t)6 * g.V;
         cx<float> w[12];
         ld_site_h(B + (size_t)k * V6 + self6, S[(size_t)k * g.V + s], g.Vb, w);
@@ -329,7 +335,8 @@ __global__ void __launch_bounds__(kHalfThreads) k_h_multi_axpy(float2* __restric
     __syncthreads();
     const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    const int X = (int)(s / g.Vb), l = (int)(s - (long long)X * g.Vb);
+    int X, l;
+    site_of(g, s, X, l);
     const size_t self = (size_t)X * 12 * g.Vb + l, self6 = (size_t)X * 6 * g.Vb + l, V6 = (size_t)6 * g.V;
     cx<float> acc[12];
 #pragma unroll

@@ -78,6 +78,14 @@ __host__ __device__ inline void coarse_coords(const Geom& g, int X, int xc[4]) {
     xc[2] = X % g.Lc[2];
     xc[3] = X / g.Lc[2];
 }
+// aggregate and local index of internal site s, in 32 bits (a lattice of 2^31 sites
+// would be a terabyte of links): a 64-bit division by a run-time divisor is some
+// eighty instructions at the start of every thread
+__device__ __forceinline__ void site_of(const Geom& g, long long s, int& X, int& l) {
+    const unsigned int u = (unsigned int)s, v = (unsigned int)g.Vb, q = u / v;
+    X = (int)q;
+    l = (int)(u - q * v);
+}
 // lexicographic (boundary) site index of internal (X, l)
 __host__ __device__ inline long long lex_site(const Geom& g, int X, int l) {
     int lc[4], xc[4];
