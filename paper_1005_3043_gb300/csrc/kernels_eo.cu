@@ -16,6 +16,8 @@
 // U4[p][mu][j 4][Vh] (entries 2j, 2j+1) then float2 U8[p][mu][Vh] (entry 8).
 // One thread per output site; consecutive threads read consecutive cb
 // indices of every component.
+#include <algorithm>
+
 #include "mg_launch.h"
 #include "mg_wilson.cuh"
 
@@ -260,14 +262,21 @@ __global__ void __launch_bounds__(kEoThreads) k_eo_cg_update1(v2<T>* __restrict_
     const double qq = R.scal[s.q2];
     const T alpha = qq > 0 ? (T)(R.scal[s.gamma] / qq) : T(0);
     T acc = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        cx<T> xv = ld<T>(x + i), rv = ld<T>(r + i);
-        const cx<T> pv = ld<T>(p + i), qv = ld<T>(q + i);
-        xv = xv + alpha * pv;
-        rv = rv - alpha * qv;
-        st<T>(x + i, xv);
-        st<T>(r + i, rv);
-        acc += norm2(rv);
+    constexpr int E = BasisVec<T>::E;   // 16 bytes per load; n = 12 Vh is even
+    for (long long i = E * (blockIdx.x * (long long)blockDim.x + threadIdx.x); i < n; i += E * (long long)gridDim.x * blockDim.x) {
+        BasisVec<T> xv, rv, pv, qv;
+        pv.load(p + i);
+        qv.load(q + i);
+        xv.load_rw(x + i);
+        rv.load_rw(r + i);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            xv.c[e] = xv.c[e] + alpha * pv.c[e];
+            rv.c[e] = rv.c[e] - alpha * qv.c[e];
+            acc += norm2(rv.c[e]);
+        }
+        xv.store(x + i);
+        rv.store(r + i);
     }
     T v1[1] = {acc};
     grid_reduce<1, T>(v1, R.partials, R.ticket, R.partial_bytes, [&](double (&t)[1]) {
@@ -285,24 +294,32 @@ __global__ void __launch_bounds__(kEoThreads) k_eo_cg_update2(v2<T>* __restrict_
     if (R.scal[done] != 0.0) return;
     const double g0 = R.scal[gamma_old];
     const T beta = g0 > 0 ? (T)(R.scal[gamma_new] / g0) : T(0);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        st<T>(p + i, ld<T>(sv + i) + beta * ld<T>(p + i));
+    constexpr int E = BasisVec<T>::E;
+    for (long long i = E * (blockIdx.x * (long long)blockDim.x + threadIdx.x); i < n; i += E * (long long)gridDim.x * blockDim.x) {
+        BasisVec<T> s, v;
+        s.load(sv + i);
+        v.load_rw(p + i);
+#pragma unroll
+        for (int e = 0; e < E; ++e) v.c[e] = s.c[e] + beta * v.c[e];
+        v.store(p + i);
+    }
+}
+// CTAs of the updates: 16 bytes per thread and vector, at most four per SM
+template <typename T> static int eo_update_grid(long long n) {
+    const long long b = (n / BasisVec<T>::E + kEoThreads - 1) / kEoThreads;
+    return (int)std::max(1LL, std::min(b, 4LL * device_sm_count()));
 }
 template <typename T>
 void eo_cg_update1(v2<T>* x, v2<T>* r, const v2<T>* p, const v2<T>* q, long long n, const EoCgSlots& s, int iter,
                    const Reduce& R, cudaStream_t st) {
-    long long b = (n + kEoThreads - 1) / kEoThreads;
-    if (b > kMaxReduceBlocks) b = kMaxReduceBlocks;
     note_launch();
-    k_eo_cg_update1<T><<<(int)b, kEoThreads, 0, st>>>(x, r, p, q, n, s, iter, R);
+    k_eo_cg_update1<T><<<eo_update_grid<T>(n), kEoThreads, 0, st>>>(x, r, p, q, n, s, iter, R);
 }
 template <typename T>
 void eo_cg_update2(v2<T>* p, const v2<T>* sv, long long n, int gamma_old, int gamma_new, int done, const Reduce& R,
                    cudaStream_t st) {
-    long long b = (n + kEoThreads - 1) / kEoThreads;
-    if (b > kMaxReduceBlocks) b = kMaxReduceBlocks;
     note_launch();
-    k_eo_cg_update2<T><<<(int)b, kEoThreads, 0, st>>>(p, sv, n, gamma_old, gamma_new, done, R);
+    k_eo_cg_update2<T><<<eo_update_grid<T>(n), kEoThreads, 0, st>>>(p, sv, n, gamma_old, gamma_new, done, R);
 }
 template void eo_cg_update1<float>(v2<float>*, v2<float>*, const v2<float>*, const v2<float>*, long long,
                                    const EoCgSlots&, int, const Reduce&, cudaStream_t);

@@ -484,14 +484,19 @@ __global__ void k_mr_update(v2<T>* e, v2<T>* r, const v2<T>* __restrict__ q, siz
     r += blockIdx.y * ln.b;
     q += blockIdx.y * ln.b;
     cx<T> a((T)scal[S_MR_ALPHA], (T)scal[S_MR_ALPHA + 1]);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        cx<T> ri = ld<T>(r + i);
-        cx<T> ei = ld<T>(e + i);
-        cmad(ei, a, ri);
-        st<T>(e + i, ei);
+    constexpr int E = BasisVec<T>::E;
+    for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
+        BasisVec<T> rv, ev, qv;
+        rv.load_rw(r + i);
+        ev.load_rw(e + i);
+        if (update_r) qv.load(q + i);
+#pragma unroll
+        for (int k = 0; k < E; ++k) cmad(ev.c[k], a, rv.c[k]);
+        ev.store(e + i);
         if (update_r) {
-            cx<T> qa = a * ld<T>(q + i);
-            st<T>(r + i, ri - qa);
+#pragma unroll
+            for (int k = 0; k < E; ++k) rv.c[k] = rv.c[k] - a * qv.c[k];
+            rv.store(r + i);
         }
     }
 }
@@ -531,7 +536,7 @@ template <typename T>
 void mr_update(v2<T>* e, v2<T>* r, const v2<T>* q, size_t n, bool update_r, const Reduce& R, cudaStream_t st,
                const Lanes& ln) {
     note_launch();
-    k_mr_update<T><<<dim3(stream_grid(n), ln.m), kThreads, 0, st>>>(e, r, q, n, update_r, R, ln);
+    k_mr_update<T><<<dim3(stream_grid(n / BasisVec<T>::E), ln.m), kThreads, 0, st>>>(e, r, q, n, update_r, R, ln);
 }
 template <typename T> void normalize_dev(v2<T>* x, size_t n, int slot, const Reduce& R, cudaStream_t st) {
     note_launch();
@@ -540,26 +545,6 @@ template <typename T> void normalize_dev(v2<T>* x, size_t n, int slot, const Red
 
 // ================================================================ GCR
 __device__ __forceinline__ int rslot(int j, int k) { return S_GCR_R + 2 * (k * K_MAX + j); }
-
-// Entries per thread and step of the basis passes: 16 bytes of one vector (FP32:
-// two complex entries; fine and coarse vectors have an even number of entries).
-template <typename T> struct BasisVec {
-    static constexpr int E = sizeof(T) == 4 ? 2 : 1;
-    cx<T> c[E];
-    __device__ __forceinline__ void load(const v2<T>* p) {
-        if constexpr (E == 2) {
-            const float4 q = __ldg(reinterpret_cast<const float4*>(p));
-            c[0] = cx<T>(q.x, q.y);
-            c[1] = cx<T>(q.z, q.w);
-        } else {
-            c[0] = ldg<T>(p);
-        }
-    }
-    __device__ __forceinline__ void store(v2<T>* p) const {
-        if constexpr (E == 2) *reinterpret_cast<float4*>(p) = make_float4(c[0].r, c[0].i, c[1].r, c[1].i);
-        else st<T>(p, c[0]);
-    }
-};
 
 // Projections <basis_j, basis_k>, j < k, in one pass.  GM (the GMRES smoother):
 // basis vector j stands for f_j basis_j, f_j = 1 / |basis_j| in scal[S_GMRES_F + j],
@@ -623,8 +608,7 @@ __global__ void __launch_bounds__(kThreads) k_gcr_orth_norm(v2<T>* basis, size_t
     T a = 0;
     for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
         BasisVec<T> v;
-#pragma unroll
-        for (int e = 0; e < E; ++e) v.c[e] = ld<T>(pk + i + e);
+        v.load_rw(pk + i);
         if (GM)
 #pragma unroll
             for (int e = 0; e < E; ++e) v.c[e] = fk * v.c[e];
@@ -662,8 +646,14 @@ __global__ void k_gcr_cdot(const v2<T>* __restrict__ basis, const v2<T>* __restr
     R = R.lane(blockIdx.y);
     const v2<T>* pk = basis + (size_t)k * n;
     cx<T> a(0, 0);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        cmadc(a, ld<T>(pk + i), ld<T>(r + i));
+    constexpr int E = BasisVec<T>::E;
+    for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
+        BasisVec<T> p, v;
+        p.load(pk + i);
+        v.load(r + i);
+#pragma unroll
+        for (int e = 0; e < E; ++e) cmadc(a, p.c[e], v.c[e]);
+    }
     T acc[2] = {a.r, a.i};
     grid_reduce<2, T>(acc, R.partials, R.ticket, R.partial_bytes, [&](double (&t)[2]) {
         double nk = sqrt(R.scal[S_GCR_PN2]);
@@ -684,12 +674,19 @@ __global__ void k_gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, Reduce R, 
     cx<T> c((T)R.scal[S_GCR_C + 2 * k], (T)R.scal[S_GCR_C + 2 * k + 1]);
     v2<T>* pk = basis + (size_t)k * n;
     T a = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        cx<T> p = f * ld<T>(pk + i);
-        st<T>(pk + i, p);
-        cx<T> v = ld<T>(r + i) - c * p;
-        st<T>(r + i, v);
-        a += norm2(v);
+    constexpr int E = BasisVec<T>::E;
+    for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
+        BasisVec<T> p, v;
+        p.load_rw(pk + i);
+        v.load_rw(r + i);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            p.c[e] = f * p.c[e];
+            v.c[e] = v.c[e] - c * p.c[e];
+            a += norm2(v.c[e]);
+        }
+        p.store(pk + i);
+        v.store(r + i);
     }
     T acc[1] = {a};
     grid_reduce<1, T>(acc, R.partials, R.ticket, R.partial_bytes, [&](double (&t)[1]) { R.scal[S_GCR_R2] = t[0]; });
@@ -744,11 +741,11 @@ template <typename T> void gmres_orth(v2<T>* basis, size_t n, int k, const Reduc
 template <typename T>
 void gcr_cdot(const v2<T>* basis, const v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
     note_launch();
-    k_gcr_cdot<T><<<dim3(reduce_grid(n), ln.m), kThreads, 0, st>>>(basis, r, n, k, R, ln);
+    k_gcr_cdot<T><<<dim3(basis_grid<T>(n), ln.m), kThreads, 0, st>>>(basis, r, n, k, R, ln);
 }
 template <typename T> void gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, const Reduce& R, cudaStream_t st, const Lanes& ln) {
     note_launch();
-    k_gcr_update<T><<<dim3(reduce_grid(n), ln.m), kThreads, 0, st>>>(basis, r, n, k, R, ln);
+    k_gcr_update<T><<<dim3(basis_grid<T>(n), ln.m), kThreads, 0, st>>>(basis, r, n, k, R, ln);
 }
 template <typename T>
 void gcr_xupdate(double2* x, const v2<T>* Z, size_t n, int k, const GcrCoef& y, cudaStream_t st) {
@@ -863,8 +860,7 @@ __global__ void __launch_bounds__(kThreads) k_multi_axpy(v2<T>* z, const v2<T>* 
     __syncthreads();
     for (size_t i = E * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i < n; i += E * (size_t)gridDim.x * blockDim.x) {
         BasisVec<T> v;
-#pragma unroll
-        for (int e = 0; e < E; ++e) v.c[e] = ld<T>(z + i + e);
+        v.load_rw(z + i);
 #pragma unroll
         for (int j = 0; j < NJ; ++j)
             if (j < k) {

@@ -55,6 +55,36 @@ template <typename T> __device__ __forceinline__ cx<T> ld(const v2<T>* p) { v2<T
 template <typename T> __device__ __forceinline__ cx<T> ldg(const v2<T>* p) { v2<T> v = __ldg(p); return cx<T>(v.x, v.y); }
 template <typename T> __device__ __forceinline__ void st(v2<T>* p, cx<T> a) { v2<T> v; v.x = a.r; v.y = a.i; *p = v; }
 
+// Entries per thread and step of a pass over vectors: 16 bytes of one vector (FP32:
+// two complex entries; fine and coarse vectors have an even number of entries).
+template <typename T> struct BasisVec {
+    static constexpr int E = sizeof(T) == 4 ? 2 : 1;
+    cx<T> c[E];
+    __device__ __forceinline__ void load(const v2<T>* p) {
+        if constexpr (E == 2) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+            c[0] = cx<T>(q.x, q.y);
+            c[1] = cx<T>(q.z, q.w);
+        } else {
+            c[0] = ldg<T>(p);
+        }
+    }
+    // of a vector that the kernel also writes
+    __device__ __forceinline__ void load_rw(const v2<T>* p) {
+        if constexpr (E == 2) {
+            const float4 q = *reinterpret_cast<const float4*>(p);
+            c[0] = cx<T>(q.x, q.y);
+            c[1] = cx<T>(q.z, q.w);
+        } else {
+            c[0] = ld<T>(p);
+        }
+    }
+    __device__ __forceinline__ void store(v2<T>* p) const {
+        if constexpr (E == 2) *reinterpret_cast<float4*>(p) = make_float4(c[0].r, c[0].i, c[1].r, c[1].i);
+        else st<T>(p, c[0]);
+    }
+};
+
 // lattice geometry, passed by value to kernels
 struct Geom {
     int L[4], B[4], Lc[4];
