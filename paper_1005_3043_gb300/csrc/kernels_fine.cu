@@ -554,7 +554,8 @@ __device__ __forceinline__ int rslot(int j, int k) { return S_GCR_R + 2 * (k * K
 // 20 us per cycle.)  Bound by the bytes of the basis: all k + 1 loads of a step
 // are independent, the grid is what an SM holds (a few hundred partial sums).
 // Measured with the reductions of mg_common.cuh: the Krylov kernels of one solve
-// 35.6 -> 20.1 ms on 16^3x32 (FP32, GMRES(12)), 67 -> 39 ms on 12^3x24 (FP64).
+// 35.6 -> 18.0 ms on 16^3x32 (FP32, GMRES(12)), 67 -> 32.6 ms on 12^3x24 (FP64,
+// where the FP64 pipe bounds them: two operations a clock and SM).
 template <typename T, int NJ, bool GM>
 __global__ void __launch_bounds__(kThreads) k_gcr_multidot(const v2<T>* __restrict__ basis, size_t n, int k, Reduce R, Lanes ln) {
     basis += blockIdx.y * ln.a;
@@ -617,9 +618,9 @@ __global__ void __launch_bounds__(kThreads) k_gcr_orth_norm(v2<T>* basis, size_t
             if (j < k) {
                 BasisVec<T> pj;
                 pj.load(basis + (size_t)j * n + i);
-                const cx<T> b(beta[2 * j], beta[2 * j + 1]);
+                const cx<T> b(-beta[2 * j], -beta[2 * j + 1]);   // four fused products; w - b p is six operations
 #pragma unroll
-                for (int e = 0; e < E; ++e) v.c[e] = v.c[e] - b * pj.c[e];
+                for (int e = 0; e < E; ++e) cmad(v.c[e], b, pj.c[e]);
             }
         }
         if (k > 0) v.store(pk + i);
@@ -682,7 +683,7 @@ __global__ void k_gcr_update(v2<T>* basis, v2<T>* r, size_t n, int k, Reduce R, 
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             p.c[e] = f * p.c[e];
-            v.c[e] = v.c[e] - c * p.c[e];
+            cmad(v.c[e], cx<T>(-c.r, -c.i), p.c[e]);
             a += norm2(v.c[e]);
         }
         p.store(pk + i);

@@ -309,9 +309,9 @@ __global__ void __launch_bounds__(kHalfThreads) k_h_orth(uint2* __restrict__ B, 
         for (int j = 0; j < k; ++j) {
             cx<float> v[12];
             ld_site_h(B + (size_t)j * V6 + self6, S[(size_t)j * g.V + s] * fac[j], g.Vb, v);
-            const cx<float> b((float)beta[2 * j], (float)beta[2 * j + 1]);
+            const cx<float> b(-(float)beta[2 * j], -(float)beta[2 * j + 1]);
 #pragma unroll
-            for (int q = 0; q < 12; ++q) w[q] = w[q] - b * v[q];
+            for (int q = 0; q < 12; ++q) cmad(w[q], b, v[q]);
         }
         store_site_h(B + (size_t)k * V6 + self6, S + (size_t)k * g.V + s, w, g.Vb,
                      [&](int, cx<float> q) { a += norm2(q); });

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kL2Threads) k_block_ortho_l2(double2* __restri
             __syncthreads();
             for (int k = threadIdx.x; k < len; k += blockDim.x) {
                 cx<double> w = ld<double>(wi + k);
-                for (int j = 0; j < i; ++j) w = w - cx<double>(cj[j].x, cj[j].y) * ld<double>(panel + (size_t)j * len + k);
+                for (int j = 0; j < i; ++j) cmad(w, cx<double>(-cj[j].x, -cj[j].y), ld<double>(panel + (size_t)j * len + k));
                 st<double>(wi + k, w);
             }
             __syncthreads();
