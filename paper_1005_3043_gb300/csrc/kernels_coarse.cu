@@ -27,8 +27,9 @@ static inline int reduce_grid(size_t n) {
 // rounding.  The column being orthogonalised sits in shared memory; warp w
 // forms the projections on columns w, w + 8, ... with warp shuffles, so a
 // pass costs three CTA barriers instead of one block reduction per column.
-// Bound by the FP64 pipe (16 operations per entry and pair of columns): 16^4, 4^4
-// aggregates, nv = 24: 8.3 -> 6.5 ms with the updates fused, 6.0 at the pipe's rate.
+// Bound by the FP64 pipe (16 operations per entry and pair of columns): the six
+// calls of a setup on 16^3x32, 4^4 aggregates, 16 to 20 columns: 50 -> 39 ms with the
+// updates fused, 32 at the pipe's rate.
 constexpr int kOrthoMaxNv = 64;   // nvec <= 25 (parameter check)
 
 __device__ __forceinline__ double block_sum(double v, double* sh) {
@@ -206,11 +207,11 @@ void prolong(v2<T>* e, const v2<T>* P, const v2<T>* yc, int nv, const Geom& g, c
 // hop of eq. 2 from x to y = x +/- mu, P_b column b at y) and accumulates
 // conj(P_a(x)) . W_b(x) over the 6 components of chirality s_a.  Hops leaving
 // X through its face in direction h go to A[X][1+h]; hops staying inside X go
-// to Aself[X][h] (summed later with the diagonal (4+m)).  FP64 throughout.
+// to Aself[X][h] (summed later with the diagonal (4+m)).
 constexpr int kBuildChunk = 8;
 // stride (complex entries) of one (site, column) spinor in the build's shared
-// memory: 13, not 12, so the lanes of a warp (consecutive columns) fall on
-// distinct banks in the product loop (12 put every fourth lane on one bank)
+// memory: 13, not 12, so the lanes of a warp (sixteen consecutive columns) fall on
+// distinct banks in the product loop
 constexpr int kWStride = 13;
 
 template <typename TC, int MU, bool FWD>
@@ -264,110 +265,154 @@ __device__ __forceinline__ void hop_column(const cx<TC> (&p)[4][3], const v2<TC>
     }
 }
 
-// TC: precision of the products (double, or float with FP64 accumulation of
-// the per-chunk sums).
-template <typename TC, int MU, bool FWD>
-__device__ void build_hop(double2* __restrict__ A, double2* __restrict__ Aself, const v2<TC>* __restrict__ P,
-                          const v2<TC>* __restrict__ U, int nv, const Geom& g, int X, int h, v2<TC>* Wsh,
-                          v2<TC>* Psh, unsigned char* leaves) {
-    const int nc = 2 * nv, len = 6 * g.Vb;
-    const int npair = nc * nc;
-    constexpr int kMaxPairs = 10;                      // nc <= 50 with 256 threads
-    cx<double> acc_out[kMaxPairs], acc_in[kMaxPairs];
-#pragma unroll
-    for (int q = 0; q < kMaxPairs; ++q) { acc_out[q] = cx<double>(0, 0); acc_in[q] = cx<double>(0, 0); }
-    int xcX[4];
-    coarse_coords(g, X, xcX);
-    for (int l0 = 0; l0 < g.Vb; l0 += kBuildChunk) {
-        int cs = min(kBuildChunk, g.Vb - l0);
-        // W_b(x) for x in chunk, all columns b: Wsh[(xi*nc + b)*kWStride + k]
-        for (int t = threadIdx.x; t < cs * nc; t += blockDim.x) {
-            int xi = t / nc, b = t - xi * nc;
-            int l = l0 + xi;
-            int lc[4];
-            local_coords(g, l, lc);
-            int Xn, ln;
-            bool flip;
-            neighbour(g, X, l, lc, xcX, MU, FWD ? 1 : -1, Xn, ln, flip);
-            if (b == 0) leaves[xi] = (FWD ? lc[MU] == g.B[MU] - 1 : lc[MU] == 0) ? 1 : 0;
-            int sb = b / nv, ib = b - sb * nv;
-            cx<TC> p[4][3];
-            const v2<TC>* col = P + (((size_t)Xn * 2 + sb) * nv + ib) * len;
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    int s_sp = sp >> 1;
-                    p[sp][c] = (s_sp == sb) ? ld<TC>(col + ((sp & 1) * 3 + c) * g.Vb + ln) : cx<TC>(0, 0);
-                }
-            const v2<TC>* u = FWD ? U + ((size_t)MU * g.Vc + X) * 9 * g.Vb + l : U + ((size_t)MU * g.Vc + Xn) * 9 * g.Vb + ln;
-            cx<TC> o[4][3];
-            hop_column<TC, MU, FWD>(p, u, g.Vb, flip ? TC(0.5) : TC(-0.5), o);
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) st<TC>(Wsh + ((size_t)xi * nc + b) * kWStride + 3 * sp + c, o[sp][c]);
-        }
-        // P_a(x) for x in chunk: Psh[(xi*nc + a)*6 + kk]
-        for (int t = threadIdx.x; t < cs * nc * 6; t += blockDim.x) {
-            int kk = t % 6, r = t / 6;
-            int a = r % nc, xi = r / nc;
-            int sa = a / nv, ia = a - sa * nv;
-            Psh[t] = P[(((size_t)X * 2 + sa) * nv + ia) * len + kk * g.Vb + l0 + xi];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < kMaxPairs; ++q) {
-            int pr = threadIdx.x + q * blockDim.x;
-            if (pr < npair) {
-                int a = pr / nc, b = pr - a * nc;
-                int sa = a / nv;
-                cx<TC> co(0, 0), ci(0, 0);
-                for (int xi = 0; xi < cs; ++xi) {
-                    cx<TC> t(0, 0);
-#pragma unroll
-                    for (int kk = 0; kk < 6; ++kk)
-                        cmadc(t, ld<TC>(Psh + ((size_t)xi * nc + a) * 6 + kk),
-                              ld<TC>(Wsh + ((size_t)xi * nc + b) * kWStride + 6 * sa + kk));
-                    if (leaves[xi]) co = co + t;
-                    else ci = ci + t;
-                }
-                acc_out[q] = acc_out[q] + cx<double>((double)co.r, (double)co.i);
-                acc_in[q] = acc_in[q] + cx<double>((double)ci.r, (double)ci.i);
-            }
-        }
-        __syncthreads();
+// Sites of an aggregate in the build's order for direction MU: first those whose hop
+// leaves the aggregate (count Vb / B_MU), then the others, each set in lexicographic
+// order.  One accumulator set then serves both sums: it is written out where the
+// first set ends.
+template <int MU, bool FWD> __device__ __forceinline__ int build_site(const Geom& g, int m) {
+    const unsigned int ls = g.lstride[MU], Bm = g.B[MU], nface = g.Vb / Bm;
+    unsigned int q = m, c = FWD ? Bm - 1 : 0, hi;
+    if (q < nface) {
+        hi = q / ls;
+        q -= hi * ls;
+    } else {
+        q -= nface;
+        hi = q / ls;
+        q -= hi * ls;
+        c = hi % (Bm - 1) + (FWD ? 0 : 1);
+        hi /= Bm - 1;
     }
-    // column-major output: A[X][d][b][a]
+    return (int)(q + ls * (c + Bm * hi));
+}
+// strides (complex entries) between the sites of a chunk: two (FP32) or one (FP64)
+// above a multiple of 16, so that the lanes of a store (sites fastest) fall on
+// distinct banks
+template <typename TC> __host__ __device__ constexpr int build_stride(int n) {
+    constexpr int off = sizeof(TC) == 4 ? 2 : 1;
+    return (n + 15 - off) / 16 * 16 + off;
+}
+
+// W_b(x) of the chunk's sites, all columns b: Wsh[xi * ws + b * kWStride + k].  Lanes
+// run over the sites first: P and U are read in segments of consecutive sites.
+template <typename TC, int MU, bool FWD>
+__device__ __forceinline__ void build_stage(const v2<TC>* __restrict__ P, const v2<TC>* __restrict__ U, int nv, const Geom& g,
+                                            int X, const int (&xcX)[4], int m0, int cs, v2<TC>* Wsh, v2<TC>* Psh, int ws,
+                                            int ps) {
+    const int nc = 2 * nv, len = 6 * g.Vb;
+    for (int t = threadIdx.x; t < kBuildChunk * nc; t += blockDim.x) {
+        const int xi = t % kBuildChunk, b = t / kBuildChunk;
+        if (xi >= cs) continue;
+        const int l = build_site<MU, FWD>(g, m0 + xi);
+        int lc[4];
+        local_coords(g, l, lc);
+        int Xn, ln;
+        bool flip;
+        neighbour(g, X, l, lc, xcX, MU, FWD ? 1 : -1, Xn, ln, flip);
+        const int sb = b >= nv, ib = b - sb * nv;
+        cx<TC> p[4][3];
+        const v2<TC>* col = P + (((size_t)Xn * 2 + sb) * nv + ib) * len + ln;
 #pragma unroll
-    for (int q = 0; q < kMaxPairs; ++q) {
-        int pr = threadIdx.x + q * blockDim.x;
-        if (pr < npair) {
-            int a = pr / nc, b = pr - a * nc;
-            st<double>(A + (((size_t)X * 9 + 1 + h) * nc + b) * nc + a, acc_out[q]);
-            st<double>(Aself + (((size_t)X * 8 + h) * nc + b) * nc + a, acc_in[q]);
-        }
+        for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+                p[sp][c] = ((sp >> 1) == sb) ? ld<TC>(col + ((sp & 1) * 3 + c) * g.Vb) : cx<TC>(0, 0);
+        const v2<TC>* u = FWD ? U + ((size_t)MU * g.Vc + X) * 9 * g.Vb + l : U + ((size_t)MU * g.Vc + Xn) * 9 * g.Vb + ln;
+        cx<TC> o[4][3];
+        hop_column<TC, MU, FWD>(p, u, g.Vb, flip ? TC(0.5) : TC(-0.5), o);
+#pragma unroll
+        for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) st<TC>(Wsh + (size_t)xi * ws + b * kWStride + 3 * sp + c, o[sp][c]);
+    }
+    // P_a(x): Psh[xi * ps + a * 6 + kk]
+    for (int t = threadIdx.x; t < kBuildChunk * nc * 6; t += blockDim.x) {
+        const int xi = t % kBuildChunk, r = t / kBuildChunk;
+        if (xi < cs) Psh[xi * ps + r] = P[((size_t)X * nc * 6 + r) * g.Vb + build_site<MU, FWD>(g, m0 + xi)];
     }
 }
 
-template <typename TC>
-__global__ void __launch_bounds__(256) k_coarse_hop(double2* A, double2* Aself, const v2<TC>* __restrict__ P,
-                                                    const v2<TC>* __restrict__ U, int nv, Geom g) {
+// One CTA per (aggregate, direction).  TC: precision of the products (double, or
+// float with the sums over a chunk's sites added up in FP64).  Threads: chirality
+// of the row (2) x 8 x 16, each with NT x NT products, rows ta + 8 i, columns
+// tb + 16 j (NT = ceil(nv / 8), at most 4 for nv <= 25): an entry of shared memory
+// feeds NT products.  (With one product per two entries the shared-memory pipe, not
+// the FMA units, was at work: the six builds of a setup on 16^3x32, 4^4 aggregates,
+// 16 to 20 columns, FP32: 40 -> 22 ms; the products alone take 5, their sums and
+// conversions in FP64 another 6.)
+template <typename TC, int NT>
+__global__ void __launch_bounds__(256, sizeof(TC) == 4 && NT <= 3 ? 2 : 1)
+k_coarse_hop(double2* __restrict__ A, double2* __restrict__ Aself, const v2<TC>* __restrict__ P, const v2<TC>* __restrict__ U,
+             int nv, Geom g) {
     extern __shared__ unsigned char smem_raw[];
-    const int nc = 2 * nv;
+    const int nc = 2 * nv, ws = build_stride<TC>(nc * kWStride), ps = build_stride<TC>(nc * 6);
     v2<TC>* Wsh = reinterpret_cast<v2<TC>*>(smem_raw);
-    v2<TC>* Psh = Wsh + (size_t)kBuildChunk * nc * kWStride;
-    unsigned char* leaves = reinterpret_cast<unsigned char*>(Psh + (size_t)kBuildChunk * nc * 6);
-    int X = blockIdx.x >> 3, h = blockIdx.x & 7;
-    switch (h) {
-        case 0: build_hop<TC, 0, true>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
-        case 1: build_hop<TC, 0, false>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
-        case 2: build_hop<TC, 1, true>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
-        case 3: build_hop<TC, 1, false>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
-        case 4: build_hop<TC, 2, true>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
-        case 5: build_hop<TC, 2, false>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
-        case 6: build_hop<TC, 3, true>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
-        default: build_hop<TC, 3, false>(A, Aself, P, U, nv, g, X, h, Wsh, Psh, leaves); break;
+    v2<TC>* Psh = Wsh + (size_t)kBuildChunk * ws;
+    const int X = blockIdx.x >> 3, h = blockIdx.x & 7;
+    const int sa = threadIdx.x >> 7, ta = (threadIdx.x >> 4) & 7, tb = threadIdx.x & 15;
+    int xcX[4], pa[NT], pb[NT];
+    coarse_coords(g, X, xcX);
+#pragma unroll
+    for (int i = 0; i < NT; ++i) {   // rows and columns past the last repeat it and are not stored
+        pa[i] = (sa * nv + min(ta + 8 * i, nv - 1)) * 6;
+        pb[i] = min(tb + 16 * i, nc - 1) * kWStride + 6 * sa;
+    }
+    const int nface = g.Vb / (h < 2 ? g.B[0] : h < 4 ? g.B[1] : h < 6 ? g.B[2] : g.B[3]);
+    for (int set = 0; set < 2; ++set) {
+        const int end = set ? g.Vb : nface;
+        cx<double> acc[NT][NT];
+#pragma unroll
+        for (int i = 0; i < NT; ++i)
+#pragma unroll
+            for (int j = 0; j < NT; ++j) acc[i][j] = cx<double>(0, 0);
+        for (int m0 = set ? nface : 0; m0 < end; m0 += kBuildChunk) {
+            const int cs = min(kBuildChunk, end - m0);
+            switch (h) {
+                case 0: build_stage<TC, 0, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+                case 1: build_stage<TC, 0, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+                case 2: build_stage<TC, 1, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+                case 3: build_stage<TC, 1, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+                case 4: build_stage<TC, 2, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+                case 5: build_stage<TC, 2, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+                case 6: build_stage<TC, 3, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+                default: build_stage<TC, 3, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+            }
+            __syncthreads();
+            cx<TC> t[NT][NT];
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+#pragma unroll
+                for (int j = 0; j < NT; ++j) t[i][j] = cx<TC>(0, 0);
+            for (int xi = 0; xi < cs; ++xi) {
+                const v2<TC>* wx = Wsh + (size_t)xi * ws;
+                const v2<TC>* px = Psh + xi * ps;
+#pragma unroll
+                for (int kk = 0; kk < 6; ++kk) {
+                    cx<TC> w[NT], p[NT];
+#pragma unroll
+                    for (int i = 0; i < NT; ++i) {
+                        w[i] = ld<TC>(wx + pb[i] + kk);
+                        p[i] = ld<TC>(px + pa[i] + kk);
+                    }
+#pragma unroll
+                    for (int i = 0; i < NT; ++i)
+#pragma unroll
+                        for (int j = 0; j < NT; ++j) cmadc(t[i][j], p[i], w[j]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+#pragma unroll
+                for (int j = 0; j < NT; ++j) acc[i][j] = acc[i][j] + cx<double>((double)t[i][j].r, (double)t[i][j].i);
+            __syncthreads();
+        }
+        // column-major: A[X][1 + h][b][a], Aself[X][h][b][a]
+        double2* out = set ? Aself + ((size_t)X * 8 + h) * nc * nc : A + ((size_t)X * 9 + 1 + h) * nc * nc;
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int i = 0; i < NT; ++i)
+                if (ta + 8 * i < nv && tb + 16 * j < nc)
+                    st<double>(out + (size_t)(tb + 16 * j) * nc + sa * nv + ta + 8 * i, acc[i][j]);
     }
 }
 // A[X][0] = (4+m) I + sum_h Aself[X][h] (fixed order)
@@ -387,10 +432,11 @@ template <typename TC>
 void coarse_build_t(double2* A, double2* Aself, const v2<TC>* P, const v2<TC>* U, int nv, double mass, const Geom& g,
                     cudaStream_t st) {
     int nc = 2 * nv;
-    size_t sm = sizeof(v2<TC>) * kBuildChunk * nc * (kWStride + 6) + kBuildChunk + 16;
-    cudaFuncSetAttribute(k_coarse_hop<TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = sizeof(v2<TC>) * kBuildChunk * (build_stride<TC>(nc * kWStride) + build_stride<TC>(nc * 6));
+    auto kern = nv <= 8 ? k_coarse_hop<TC, 1> : nv <= 16 ? k_coarse_hop<TC, 2> : nv <= 24 ? k_coarse_hop<TC, 3> : k_coarse_hop<TC, 4>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     note_launch();
-    k_coarse_hop<TC><<<g.Vc * 8, kThreads, sm, st>>>(A, Aself, P, U, nv, g);
+    kern<<<g.Vc * 8, kThreads, sm, st>>>(A, Aself, P, U, nv, g);
     long long total = (long long)g.Vc * nc * nc;
     note_launch();
     k_coarse_diag<<<(int)((total + kThreads - 1) / kThreads), kThreads, 0, st>>>(A, Aself, nc, 4.0 + mass, g);
