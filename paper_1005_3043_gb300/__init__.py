@@ -496,7 +496,7 @@ def mg_kernel_launches() -> int:
     return int(load().mg_kernel_launches())
 
 
-COARSE_KERNELS = {-1: "none", 0: "k_cgnr_persistent (operator from global memory)",
+COARSE_KERNELS = {-1: "none", 0: "k_cgnr_persistent (operator from global memory; FP64: resident in shared memory where it fits)",
                   1: "k_cgls_onchip (operator resident in shared memory)",
                   2: "k_cgls_onchip (operator streamed through shared memory)",
                   3: "k_cgls_onchip (operator resident in tensor memory, products on the CUDA cores)",

@@ -99,6 +99,22 @@ template <typename T> __device__ __forceinline__ void write_partial(T v, double*
     T a = block_sum_t<T>(v, sh);
     if (threadIdx.x == 0) partials[(size_t)blockIdx.x * 4 + slot] = (double)a;
 }
+// the CTA's sums of u and v into slots slot and slot + 1 (sh: 66 entries)
+template <typename T> __device__ __forceinline__ void write_partial2(T u, T v, double* partials, int slot, T* sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    u = warp_sum_t(u);
+    v = warp_sum_t(v);
+    if (lane == 0) {
+        sh[warp] = u;
+        sh[33 + warp] = v;
+    }
+    __syncthreads();
+    if (warp < 2) {
+        T x = lane < nw ? sh[33 * warp + lane] : T(0);
+        x = warp_sum_t(x);
+        if (lane == 0) partials[(size_t)blockIdx.x * 4 + slot + warp] = (double)x;
+    }
+}
 
 
 // ---------------------------------------------------------------- epoch exchange

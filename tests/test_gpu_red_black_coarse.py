@@ -67,3 +67,32 @@ def test_schur_solve_on_chip(L, B, nv, prec, tol, eps, kernel):
 @pytest.mark.parametrize("L,B,nv", [s for s in SHAPES if s[2] % 4 == 0])
 def test_schur_solve_of_a_batch(L, B, nv):
     assert run(L, B, nv, wmg.MG_FP32, 1e-5, batch=True) < 20 * 2.0 ** -11
+
+
+# CG on D_c itself in FP64: the operator in shared memory (all but the last shape, 92 MB),
+# units that share aggregates, a last CTA with fewer units, odd coarse extents.  At mass 1
+# an iteration amplifies the rounding of its two stencils, 9 nc 2^-53 < 1e-13 each, by less
+# than the squared condition number, 100: four iterations stay within 1e-10.
+@pytest.mark.parametrize("L,B,nv", SHAPES + [((6, 6, 6, 12), (2, 2, 2, 2), 12), ((6, 2, 4, 4), (2, 2, 2, 2), 1),
+                                             ((6, 4, 4, 10), (2, 2, 2, 2), 25), ((8, 8, 8, 8), (2, 2, 2, 2), 25)])
+def test_fp64_iterations_match_oracle(L, B, nv):
+    U = rough_gauge(L, seed=8)
+    V0 = synth.gaussian_vectors(L, nv, 97)
+    P, st = oracle.block_orthonormalize(V0, L, B)
+    assert st == 0
+    A = oracle.coarse_build(U, P, MASS, L, B)
+    Lc = oracle.coarse_dims(L, B)
+    rc = synth.gaussian(oracle.volume(Lc) * 2 * nv, 8, 0).reshape(-1, 2 * nv)
+    p = wmg.mg_default_params()
+    for i in range(4):
+        p.block[i] = B[i]
+    p.nvec, p.setup_group = nv, 1
+    with wmg.WilsonMG(L, p) as mg:
+        mg.set_links(U)
+        mg.set_mass(MASS)
+        mg.set_null_vectors(V0)
+        for k in (1, 4):
+            ref, _, _ = oracle.cgnr(A, rc, Lc, 0.0, k)
+            y, it, _ = mg.coarse_solve(rc, 0.0, k, wmg.MG_FP64)
+            assert it == k
+            assert np.abs(y - ref).max() <= 1e-10 * np.abs(ref).max(), k
