@@ -1598,7 +1598,7 @@ __global__ void k_wait_probe(int kind, unsigned long long* words, unsigned int* 
         float v[1] = {1.f};
         xch_allreduce<1>(v, words, 1u, err, sc, G + 1, limit);
     } else if (kind == 1) {
-        grid_sync(ctr, ctr + 1, (unsigned int)G + 1u, err, limit);
+        grid_sync(ctr, (unsigned int)G + 1u, err, limit);
     } else if (kind == 2) {
         if (threadIdx.x == 0) {
             mbar_init(&bar, 1);

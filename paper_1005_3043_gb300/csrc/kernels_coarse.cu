@@ -1044,8 +1044,6 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
     cx<T>* part = reinterpret_cast<cx<T>*>(xs + nstage);
     __shared__ T shr[66];
     const unsigned int G = gridDim.x;
-    unsigned int* cnt = a.bar;
-    unsigned int* gen = a.bar + 1;
     v2<T>* rbuf[2] = {a.r, a.r1};
     v2<T>* pbuf[2] = {a.p, a.p1};
     const int nsite = EO ? a.g.Vc / 2 : a.g.Vc;
@@ -1070,7 +1068,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
             ph.sites = a.ord + nsite;
             if constexpr (RES) cg_phase_res<DAG, STAGE, HALF_O>(ph, As + nres, src + nstage, nc, sp, nsite, xs, part, u0, u1);
             else cg_phase<T, DAG, STAGE, H16, HALF_O>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, u0, u1);
-            if (!grid_sync(cnt, gen, G, a.err)) return false;
+            if (!grid_sync(a.bar, G, a.err)) return false;
             ph.sites = a.ord;
             if constexpr (RES) cg_phase_res<DAG, STAGE, HALF_E>(ph, As, src, nc, sp, nsite, xs, part, n0, n1);
             else cg_phase<T, DAG, STAGE, H16, HALF_E>(ph, a.A, a.A16, a.s16, nc, sp, a.g, xs, part, a.nbr, n0, n1);
@@ -1102,7 +1100,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
             }
         }
     write_partial<T>(loc, a.partials, 0, shr);
-    if (!grid_sync(cnt, gen, G, a.err)) return;
+    if (!grid_sync(a.bar, G, a.err)) return;
     const T rc2 = sum_partials<T>(a.partials, 0, G, shr);
     int it = 0;
     T r2 = rc2;
@@ -1115,7 +1113,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
         ph.out = a.s;
         if (!stencil(Yes{}, std::integral_constant<int, ST_PLAIN>{}, n0, n1)) return;
         write_partial<T>(n0, a.partials, 1, shr);
-        if (!grid_sync(cnt, gen, G, a.err)) return;
+        if (!grid_sync(a.bar, G, a.err)) return;
         T gamma = sum_partials<T>(a.partials, 1, G, shr);
         T beta = 0;
         for (;;) {
@@ -1127,7 +1125,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
             n0 = 0; n1 = 0;
             if (!stencil(No{}, std::integral_constant<int, ST_P>{}, n0, n1)) return;
             write_partial<T>(n0, a.partials, 0, shr);
-            if (!grid_sync(cnt, gen, G, a.err)) return;
+            if (!grid_sync(a.bar, G, a.err)) return;
             T qq = sum_partials<T>(a.partials, 0, G, shr);
             if (!(qq > T(0))) break;
             T alpha = gamma / qq;
@@ -1138,7 +1136,7 @@ __global__ void __launch_bounds__(CgnrMaxThreads<T>::value, CgnrMaxThreads<T>::b
             n0 = 0; n1 = 0;
             if (!stencil(Yes{}, std::integral_constant<int, ST_R>{}, n0, n1)) return;
             write_partial2<T>(n0, n1, a.partials, 1, shr);
-            if (!grid_sync(cnt, gen, G, a.err)) return;
+            if (!grid_sync(a.bar, G, a.err)) return;
             T gnew;
             sum_partials2<T>(a.partials, 1, G, shr, gnew, r2);
             ++it;
