@@ -395,15 +395,16 @@ struct BcgCta {
     }
 
     // grid barrier of the epilogue warps (all writes before it visible to all reads
-    // after it, tile writes to the bulk copies too); opens the gate of the next phase
+    // after it, tile writes to the bulk copies too); opens the gate of the next phase.
+    // One thread's release covers the warps' writes (they are ordered before it by the
+    // barrier of the warps), its acquire their reads.
     __device__ bool grid_barrier(bool open) {
         fence_proxy_async_all();
         if (epi_sync(*fail != 0)) return false;
         if (t == 0) {
-            __threadfence();
             ++arrived;
             const unsigned int want = arrived * gridDim.x;
-            atomicAdd(a.bar, 1u);
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
             long long spins = 0;
             unsigned int got;
             for (;;) {
@@ -413,7 +414,6 @@ struct BcgCta {
                 if (++spins > kBcgWait) { *fail = 1; atomicExch(a.err, 1); break; }
                 if (spins > 64) __nanosleep(20);
             }
-            __threadfence();
             fence_proxy_async_all();
             if (open && !*fail) mbar_arrive(gate);
         }
@@ -484,7 +484,6 @@ struct BcgCta {
             const long long q = fabsf(h) < 0x1p55f ? __float2ll_rn(h) + __float2ll_rn(l) : -(1LL << 54);
             if (q != 0) atomicAdd(sums + i, (unsigned long long)q);
         }
-        __threadfence();
     }
 
     __device__ void epilogue(uint32_t tmem) {
@@ -572,7 +571,6 @@ struct BcgCta {
             }
             atomicMax(a.mx + i, __float_as_uint(fabsf(s)));   // fabs: one sign for every NaN
         }
-        __threadfence();
         if (!grid_barrier(false)) return;
         for (int i = t; i < np; i += kEpi) {
             const unsigned int m = __ldcg(a.mx + i);
