@@ -287,19 +287,16 @@ __device__ __forceinline__ void grid_reduce(TA (&v)[N], double* partials, unsign
     __shared__ bool is_last;
     const TA mine = block_sums<N, TA>(v, sh);
     TA* part = reinterpret_cast<TA*>(partials);
-    if ((int)threadIdx.x < N) {
-        part[(size_t)blockIdx.x * N + threadIdx.x] = mine;
-        __threadfence();
-    }
+    if ((int)threadIdx.x < N) part[(size_t)blockIdx.x * N + threadIdx.x] = mine;
     if (N > 32) __syncthreads();
     else __syncwarp();
-    if (threadIdx.x == 0) {
-        unsigned int t = atomicAdd(ticket, 1u);
+    if (threadIdx.x == 0) {   // releases the partial sums of the threads synchronised above
+        unsigned int t;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
         is_last = (t == gridDim.x - 1);
     }
     __syncthreads();
     if (!is_last) return;
-    __threadfence();
     const int k = threadIdx.x % P2, nch = max((int)blockDim.x / P2, 1);
     TA acc[4] = {TA(0), TA(0), TA(0), TA(0)};
     if (k < N) {
