@@ -152,6 +152,23 @@ __device__ __forceinline__ bool bcg_wait(uint64_t* bar, uint32_t parity, volatil
     atomicExch(err, 1);
     return false;
 }
+// until *count reaches want (it only grows); false as bcg_wait.  The counts order waits
+// on mbarriers, no data: what a thread reads after its wait it acquires there.  Not
+// inlined: the loop of the MMA threads stays as short as it was (0.5 us per phase).
+__device__ __noinline__ bool wait_count(const unsigned int* count, unsigned int want, volatile int* fail, int* err) {
+    for (long long i = 0;; ++i) {
+        unsigned int have;
+        asm volatile("ld.relaxed.cta.shared::cta.u32 %0, [%1];" : "=r"(have) : "r"(smem_u32(count)) : "memory");
+        if ((int)(have - want) >= 0) return true;
+        if (*fail) return false;
+        if (i > kBcgWait) {
+            *fail = 1;
+            atomicExch(err, 1);
+            return false;
+        }
+        if (i > 64) __nanosleep(20);
+    }
+}
 // sum in two floats (Knuth's two-sum): the column sums run over many aggregates
 // and CTAs, and FP64 adds are two per clock and SM here
 struct Sum2 {
@@ -189,6 +206,7 @@ struct BcgCta {
     unsigned char* sm;
     uint64_t *full, *empty, *acc_full, *acc_empty, *gate;
     volatile int *fail, *stop;
+    unsigned int *passed, *entered;   // progress of the two MMA threads: items, phases
 
     __device__ BcgCta(const BcgArgs& args, unsigned char* smem, uint64_t* bars, int* flags)
         : a(args), L(args.nc, args.nw, args.npad, args.stages), sm(smem) {
@@ -199,6 +217,7 @@ struct BcgCta {
         full = bars; empty = bars + kBcgMaxStages; acc_full = bars + 2 * kBcgMaxStages; acc_empty = acc_full + 2;
         gate = acc_empty + 2;
         fail = flags; stop = flags + 1;
+        passed = reinterpret_cast<unsigned int*>(flags) + 2; entered = passed + 2;
     }
 
     // Phases.  A stencil is one phase over all sites, or, in the red-black form, a phase
@@ -308,7 +327,19 @@ struct BcgCta {
         return false;
     }
 
+    __device__ void set_count(unsigned int* count, unsigned int v) {
+        asm volatile("st.relaxed.cta.shared::cta.u32 [%0], %1;" ::"r"(smem_u32(count)), "r"(v) : "memory");
+    }
+
     // ------------------------------------------------------------ MMAs (one thread of two warps)
+    // A wait by parity tells a phase of a barrier from its neighbours only.  So a thread
+    // waits for a stage that the job before also used only after the other thread has
+    // passed its waits of that job (`passed`; without it a thread a job ahead took a
+    // stage that had yet to be filled for that job for a full one: certain with fewer
+    // stages than a job has directions; the copies come in order, so the other thread
+    // is past them when the stage's tiles arrive), and the next
+    // phase's gate opens only after both have passed this one's (`entered`; a phase of
+    // one job has work for one of them).
     __device__ void multiply(uint32_t tmem, int which, uint64_t* drain) {
         const unsigned int S = a.stages, jobs = j1 - j0;
         const int nks = L.kcp >> 1;
@@ -321,9 +352,11 @@ struct BcgCta {
         unsigned int job = 0, base = 0;        // jobs and items before this phase
         int phase = 0;
         for (bool ok = true; ok; job += jobs, base += jobs * dirs(phase), ++phase) {
-            if (!bcg_wait(gate, gate_par, fail, a.err) || *stop) break;
+            if (!bcg_wait(gate, gate_par, fail, a.err)) break;
+            set_count(entered + which, phase + 1);
+            if (*stop) break;
             gate_par ^= 1u;
-            const int nd = dirs(phase);
+            const int nd = dirs(phase), dw = max((int)S - nd, 0);
             for (unsigned int j = (job ^ which) & 1u; j < jobs && ok; j += 2) {   // this warp's jobs: (job + j) odd or even
                 if (!bcg_wait(acc_empty + which, acc_par, fail, a.err)) { ok = false; break; }
                 acc_par ^= 1u;
@@ -332,23 +365,33 @@ struct BcgCta {
                 unsigned int st = i0 - k0 * S;
                 uint32_t par = k0 & 1u;
                 uint64_t da = da0 + st * step_st, db = db0 + st * step_st;
-                for (int d = 0; d < nd; ++d) {
-                    if (!bcg_wait(full + st, par, fail, a.err)) { ok = false; break; }
-                    tc_fence_after();
-                    mma_f16(acc, da, db, idesc, d > 0 ? 1u : 0u);
-                    if (nks > 1) mma_f16(acc, da + step_a, db + step_b, idesc, 1u);
-                    if (nks > 2) mma_f16(acc, da + 2 * step_a, db + 2 * step_b, idesc, 1u);
-                    mma_commit(empty + st);
-                    da += step_st;
-                    db += step_st;
-                    if (++st == S) {
-                        st = 0;
-                        par ^= 1u;
-                        da = da0;
-                        db = db0;
+                // items from dw on use stages that the job before used (item i0 + d - S)
+                int d = 0, end = j > 0 ? min(dw, nd) : nd;
+                for (;;) {
+                    for (; d < end; ++d) {
+                        if (!bcg_wait(full + st, par, fail, a.err)) { ok = false; break; }
+                        tc_fence_after();
+                        mma_f16(acc, da, db, idesc, d > 0 ? 1u : 0u);
+                        if (nks > 1) mma_f16(acc, da + step_a, db + step_b, idesc, 1u);
+                        if (nks > 2) mma_f16(acc, da + 2 * step_a, db + 2 * step_b, idesc, 1u);
+                        mma_commit(empty + st);
+                        da += step_st;
+                        db += step_st;
+                        if (++st == S) {
+                            st = 0;
+                            par ^= 1u;
+                            da = da0;
+                            db = db0;
+                        }
                     }
+                    if (!ok || end == nd) break;
+                    if (!wait_count(passed + (which ^ 1), i0, fail, a.err)) { ok = false; break; }
+                    end = nd;
                 }
-                if (ok) mma_commit(acc_full + which);
+                if (ok) {
+                    set_count(passed + which, i0 + nd);
+                    mma_commit(acc_full + which);
+                }
             }
         }
         mma_commit(drain);
@@ -360,7 +403,7 @@ struct BcgCta {
     Sum2* acc;
     int t, n, rg, rgs;
     long long job_count = 0;
-    unsigned int arrived = 0;
+    unsigned int arrived = 0, opened = 0;
 
     // entries staged in S2[row][n] (scaled) -> the four FP16 rows of the tile
     __device__ void write_tile(__half* bt, int X, int c) {
@@ -415,12 +458,18 @@ struct BcgCta {
                 if (spins > 64) __nanosleep(20);
             }
             fence_proxy_async_all();
-            if (open && !*fail) mbar_arrive(gate);
+            if (open && !*fail) next_phase();
         }
         return !epi_sync(*fail != 0);
     }
+    __device__ void next_phase() {   // thread 0
+        if (wait_count(entered, opened, fail, a.err) && wait_count(entered + 1, opened, fail, a.err)) {
+            ++opened;
+            mbar_arrive(gate);
+        }
+    }
     __device__ void open_gate() {
-        if (t == 0) mbar_arrive(gate);
+        if (t == 0) next_phase();
     }
 
     // products of the next job into T; false on failure (uniform over the warps)
@@ -802,7 +851,7 @@ __global__ void __launch_bounds__(kBcgThreads, 1) k_bcg(BcgArgs a) {
     __shared__ __align__(8) uint64_t bars[2 * kBcgMaxStages + 7];
     __shared__ uint32_t s_taddr;
     __shared__ unsigned int s_items;
-    __shared__ int s_flags[2];
+    __shared__ int s_flags[6];
     BcgCta c(a, smem, bars, s_flags);
     const int warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
@@ -810,7 +859,7 @@ __global__ void __launch_bounds__(kBcgThreads, 1) k_bcg(BcgArgs a) {
         for (int i = 0; i < 2; ++i) { mbar_init(c.acc_full + i, 1); mbar_init(c.acc_empty + i, kEpiWarps); }
         for (int i = 0; i < 3; ++i) mbar_init(c.gate + i, 1);   // the gate, the MMA threads' drains
         fence_mbar_init();
-        s_flags[0] = s_flags[1] = 0;
+        for (int i = 0; i < 6; ++i) s_flags[i] = 0;
         s_items = 0;
     }
     // zero the stages: the padding K group stays zero, the copies fill the rest

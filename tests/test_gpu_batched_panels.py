@@ -26,7 +26,9 @@ def params(nv, B, **kw):
 
 @pytest.mark.parametrize("L,B,nv,nrhs", [((4, 4, 4, 8), (2, 2, 2, 2), 4, 1), ((8, 8, 8, 8), (2, 2, 2, 2), 4, 17),
                                          ((4, 4, 4, 8), (2, 2, 2, 2), 12, 40), ((8, 8, 8, 8), (4, 4, 4, 4), 20, 100),
-                                         ((4, 4, 4, 8), (4, 4, 4, 4), 20, 256), ((4, 4, 4, 8), (2, 2, 2, 2), 24, 224)])
+                                         ((4, 4, 4, 8), (4, 4, 4, 4), 20, 256), ((4, 4, 4, 8), (2, 2, 2, 2), 24, 224),
+                                         # several jobs per CTA in six and in three stages, fewer than directions
+                                         ((8, 8, 8, 8), (2, 2, 2, 2), 24, 80), ((8, 8, 8, 8), (2, 2, 2, 2), 24, 192)])
 def test_stencil_on_panels(L, B, nv, nrhs):
     """Against the oracle's stencil with the operator rounded to FP16: the operand is
     kept to 2^-22 and the FP32 sums over 9 * 2 Nv products add some 1e-6."""
@@ -65,3 +67,19 @@ def test_sources_of_any_size():
     for i in (0, 1, 3):
         assert np.linalg.norm(b[i] - oracle.dslash(U, x[i], 0.1, L)) <= 1e-10 * np.linalg.norm(b[i]), i
     assert not x[2].any()
+
+
+def test_many_sources_of_a_wide_operator():
+    """The whole batched solve where a stage of the pipeline is used more than once per job."""
+    L, B, nv, nrhs = (8, 8, 8, 8), (2, 2, 2, 2), 24, 76
+    U = rough_gauge(L, seed=7)
+    V0 = synth.gaussian_vectors(L, nv, 95)
+    b = np.stack([synth.gaussian_spinor(L, 96, stream=i) for i in range(nrhs)])
+    with wmg.WilsonMG(L, params(nv, B, prec_inner=wmg.MG_FP16, delta=1e-4)) as mg:
+        mg.set_links(U)
+        mg.set_mass(0.1)
+        mg.setup(V0)
+        x, infos = mg.solve_batched(b)
+    assert all(i["status"] == wmg.MG_OK for i in infos)
+    for i in range(0, nrhs, 15):
+        assert np.linalg.norm(b[i] - oracle.dslash(U, x[i], 0.1, L)) <= 1e-10 * np.linalg.norm(b[i]), i
