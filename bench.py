@@ -212,7 +212,7 @@ def batched_leg(wmg, torch, stream, prec, name="wilson_24x24x24x64_nv24_beta6_76
     dB = torch.from_numpy(src.view(np.float64)).cuda()
     dX = torch.empty_like(dB)
     del src
-    mg.solve_batched_device(dB[:2], dX[:2], 2)       # warm-up: workspace, graph capture, autotuner
+    mg.solve_batched_device(dB[:2], dX[:2], 2)       # warm-up: workspace
     e0.record(stream)
     binfo = mg.solve_batched_device(dB, dX, dB.shape[0])
     e1.record(stream)
@@ -639,7 +639,7 @@ def run_ours(args, w):
         mgb.set_mass(masses[-1])
         dbb = torch.from_numpy(bsrc.view(np.float64)).cuda()
         dxb = torch.empty_like(dbb)
-        mgb.solve_batched_device(dbb[:2], dxb[:2], 2)          # warm-up (graph capture, autotuner)
+        mgb.solve_batched_device(dbb[:2], dxb[:2], 2)          # warm-up
         eb0, eb1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         eb0.record(stream)
         binfo = mgb.solve_batched_device(dbb, dxb, len(bsrc))

@@ -81,9 +81,10 @@ typedef struct {
     int prec_inner;        /* MG_FP64, MG_FP32 or MG_FP16: smoother, dslash, transfers, coarse solve, Krylov basis */
     int coarse_check;      /* coarse iterations between convergence checks read by the host */
     int coarse_kernel;     /* FP32/FP16 coarse solve: 0 (default) operator held on chip for the
-                              whole solve, in tensor memory when each SM's share fits (FP16: its
-                              products on the tensor cores when each SM holds at most 140 rows),
-                              else in shared memory, else as 1; 1 operator read from global
+                              whole solve, in tensor memory as far as each SM's share fits and the
+                              rest in shared memory (FP16: its products on the tensor cores when
+                              each SM holds at most 140 rows), else as 1 (FP16 inside a solve: one
+                              column of the batched kernel); 1 operator read from global
                               memory into registers every iteration; 2 operator streamed through
                               a shared-memory ring (tests); 3 shared memory only (tests); 4 tensor
                               memory with the products on the CUDA cores (tests) */
@@ -112,7 +113,8 @@ typedef struct {
 /* Outcome of one solve (Sec. IV reports outer iterations and fine matvecs). */
 typedef struct {
     int outer_iters;       /* preconditioner applications (the paper's outer GCR count, Table I) */
-    int coarse_iters;      /* total coarse-solver iterations */
+    int coarse_iters;      /* total coarse-solver iterations (of the red-black system where the
+                              solve uses it: two half stencils each way per iteration) */
     int fine_matvecs;      /* fine D applications, all precisions (the work unit of Fig. 1) */
     int restarts;          /* true-residual recomputations */
     double true_rel_res;   /* ||b - D x|| / ||b|| in FP64 */
@@ -453,8 +455,9 @@ int mg_profile_classes(mg_ctx* ctx, unsigned int mask);
 long long mg_kernel_launches(void);
 
 /* Which coarse CGNR kernel the last coarse solve of this context ran (a
- * diagnostic; no counterpart in the paper): MG_CK_REGISTER operator read from
- * global memory every iteration, MG_CK_SMEM operator resident in shared
+ * diagnostic; no counterpart in the paper): MG_CK_REGISTER the kernel that reads
+ * the operator from global memory (in FP64 once per launch where the SMs' shared
+ * memory holds it), MG_CK_SMEM operator resident in shared
  * memory, MG_CK_STREAM operator streamed through a shared-memory ring,
  * MG_CK_TMEM operator resident in tensor memory, products on the CUDA cores,
  * MG_CK_TMEM_MMA operator resident in tensor memory, products on the tensor
