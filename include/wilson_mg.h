@@ -479,6 +479,13 @@ int mg_coarse_kernel(mg_ctx* ctx);
  * MG_OK if it unexpectedly completed, another status on a CUDA error. */
 int mg_check_wait_timeout(mg_ctx* ctx, int kind, long long spin_limit);
 
+/* Check of what a call leaves behind when device memory runs out (the paper has no
+ * counterpart): the context's nth device allocation from now on is refused as if no
+ * memory were left, once (0: none).  The call that asked for it returns MG_ERR_OOM
+ * or does without; the context stays usable.  Returns what was still pending (0: the
+ * refusal has happened, or none was asked for), -1 on bad arguments. */
+int mg_fail_allocation(mg_ctx* ctx, int nth);
+
 /* Name of a status code; last error message of a context (NUL-terminated,
  * owned by the library: valid until the next call on that context).  No
  * counterpart in the paper. */

@@ -115,6 +115,7 @@ _SIGS = {
     "mg_kernel_launches": ([], ctypes.c_longlong),
     "mg_coarse_kernel": ([ctypes.c_void_p], ctypes.c_int),
     "mg_check_wait_timeout": ([_P, _I, ctypes.c_longlong], _I),
+    "mg_fail_allocation": ([_P, _I], _I),
     "mg_status_string": ([_I], ctypes.c_char_p),
     "mg_last_error": ([_P], ctypes.c_char_p),
 }
@@ -510,6 +511,11 @@ def mg_coarse_kernel(ctx) -> int:
 def mg_check_wait_timeout(ctx, kind: int, spin_limit: int = 20000) -> int:
     """Status of one bounded device wait driven to give up (MG_ERR_TIMEOUT expected)."""
     return int(load().mg_check_wait_timeout(ctx, int(kind), int(spin_limit)))
+
+
+def mg_fail_allocation(ctx, nth: int) -> int:
+    """Refuse the context's nth device allocation from now on, once (0: none); returns what was pending."""
+    return int(load().mg_fail_allocation(ctx, int(nth)))
 
 
 def mg_profile_enable(ctx, on: bool = True) -> None:

@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -170,6 +171,7 @@ struct mg_ctx {
     Geom g{};
     mg_params prm{};
     int K = 16;                      // GCR restart capacity
+    int refuse_alloc = 0;            // mg_fail_allocation: the allocation that is refused counts this down to 0
     cudaStream_t st = nullptr;
     std::string err;
     double mass = 0.0;
@@ -265,7 +267,8 @@ int fail(mg_ctx* c, int code, const std::string& msg) {
 
 template <typename P> int dalloc(mg_ctx* ctx, P** p, size_t bytes) {
     void* q = nullptr;
-    cudaError_t e = cudaMalloc(&q, bytes > 0 ? bytes : 16);
+    const bool refuse = ctx->refuse_alloc > 0 && --ctx->refuse_alloc == 0;   // mg_fail_allocation
+    cudaError_t e = refuse ? cudaErrorMemoryAllocation : cudaMalloc(&q, bytes > 0 ? bytes : 16);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(ctx, MG_ERR_OOM, std::string("cudaMalloc ") + std::to_string(bytes) + " bytes: " + cudaGetErrorString(e));
@@ -280,6 +283,32 @@ void dfree(mg_ctx* ctx, void* q) {
     for (size_t i = 0; i < ctx->allocs.size(); ++i)
         if (ctx->allocs[i] == q) { ctx->allocs.erase(ctx->allocs.begin() + i); break; }
     cudaFree(q);
+}
+
+// Buffers that belong together, in place of what their pointers held: all of them or, after
+// a failed allocation, none (every pointer null).  A size or a flag that describes them is
+// cleared before the call and set after it, so that a call after MG_ERR_OOM allocates again.
+struct Buf {
+    void** p;
+    size_t bytes;
+    template <typename P> Buf(P** q, size_t n) : p((void**)q), bytes(n) {}
+};
+int dalloc_all(mg_ctx* ctx, std::initializer_list<Buf> bufs) {
+    auto drop = [&]() {
+        for (const Buf& b : bufs) {
+            dfree(ctx, *b.p);
+            *b.p = nullptr;
+        }
+    };
+    drop();
+    for (const Buf& b : bufs) {
+        const int st = dalloc(ctx, b.p, b.bytes);
+        if (st != MG_OK) {
+            drop();
+            return st;
+        }
+    }
+    return MG_OK;
 }
 
 size_t nfine(const mg_ctx* c) { return (size_t)c->g.V * 12; }
@@ -333,31 +362,17 @@ template <typename T> int ensure_work(mg_ctx* ctx) {
     size_t n = nfine(ctx), vb = sizeof(v2<T>) * n;
     if (!w.ready) {
         if (std::is_same<T, double>::value) w.r = (v2<T>*)ctx->r64;
-        else TRY(dalloc(ctx, &w.r, vb));
-        TRY(dalloc(ctx, &w.Z, vb * ctx->K));
-        TRY(dalloc(ctx, &w.Pk, vb * ctx->K));
-        TRY(dalloc(ctx, &w.vr, vb));
-        TRY(dalloc(ctx, &w.vq, vb));
-        TRY(dalloc(ctx, &w.sv, vb));
-        TRY(dalloc(ctx, &w.sr, vb));
-        TRY(dalloc(ctx, &w.sz, vb));
-        TRY(dalloc(ctx, &w.tin, vb));
-        TRY(dalloc(ctx, &w.tout, vb));
+        else TRY(dalloc_all(ctx, {{&w.r, vb}}));
+        TRY(dalloc_all(ctx, {{&w.Z, vb * ctx->K}, {&w.Pk, vb * ctx->K}, {&w.vr, vb}, {&w.vq, vb}, {&w.sv, vb}, {&w.sr, vb},
+                             {&w.sz, vb}, {&w.tin, vb}, {&w.tout, vb}}));
     }
-    size_t cb = sizeof(v2<T>) * (size_t)ctx->g.Vc * (nc > 0 ? nc : 2);
-    TRY(dalloc(ctx, &w.crc, cb));
-    TRY(dalloc(ctx, &w.cy, cb));
-    TRY(dalloc(ctx, &w.cr, cb));
-    TRY(dalloc(ctx, &w.cs, cb));
-    TRY(dalloc(ctx, &w.cp, cb));
-    TRY(dalloc(ctx, &w.cq, cb));
-    TRY(dalloc(ctx, &w.cr1, cb));
-    TRY(dalloc(ctx, &w.cp1, cb));
-    TRY(dalloc(ctx, &w.eb, cb));
-    TRY(dalloc(ctx, &w.et, cb));
+    const size_t nco = (size_t)ctx->g.Vc * (nc > 0 ? nc : 2), cb = sizeof(v2<T>) * nco;
+    w.ready = false;
+    TRY(dalloc_all(ctx, {{&w.crc, cb}, {&w.cy, cb}, {&w.cr, cb}, {&w.cs, cb}, {&w.cp, cb}, {&w.cq, cb}, {&w.cr1, cb},
+                         {&w.cp1, cb}, {&w.eb, cb}, {&w.et, cb}}));
     if (sizeof(T) == 4) {
-        const size_t tb = sizeof(unsigned long long) * 6 * (size_t)ctx->g.Vc * (nc > 0 ? nc : 2);
-        TRY(dalloc(ctx, &w.ctag, tb));
+        const size_t tb = sizeof(unsigned long long) * 6 * nco;
+        TRY(dalloc_all(ctx, {{&w.ctag, tb}}));
         CK(cudaMemsetAsync(w.ctag, 0, tb, ctx->st));   // epoch 0 is never awaited
     }
     w.cnc = nc;
@@ -382,10 +397,9 @@ int ensure_level(mg_ctx* ctx, CoarseLevel& L, int nv) {
         L.at_valid = L.a16_valid = L.au_valid = L.valid = false;
         size_t np = (size_t)nv * nfine(ctx);
         size_t na = (size_t)ctx->g.Vc * 9 * (2 * nv) * (2 * nv);
-        TRY(dalloc(ctx, &L.P64, sizeof(double2) * np));
-        TRY(dalloc(ctx, &L.P32, sizeof(float2) * np));
-        TRY(dalloc(ctx, &L.A64, sizeof(double2) * na));
-        TRY(dalloc(ctx, &L.A32, sizeof(float2) * na));
+        L.cap = 0;
+        TRY(dalloc_all(ctx, {{&L.P64, sizeof(double2) * np}, {&L.P32, sizeof(float2) * np}, {&L.A64, sizeof(double2) * na},
+                             {&L.A32, sizeof(float2) * na}}));
         L.cap = nv;
     }
     L.nv = nv;
@@ -397,12 +411,10 @@ int ensure_protos(mg_ctx* ctx) {
     int nv = ctx->prm.nvec;
     if (ctx->protos) return MG_OK;
     size_t n = nfine(ctx);
-    TRY(dalloc(ctx, &ctx->protos, sizeof(double2) * n * nv));
-    TRY(dalloc(ctx, &ctx->protos_t, sizeof(double2) * n * nv));
-    TRY(dalloc(ctx, &ctx->protos_stage, sizeof(double2) * n * nv));
-    TRY(dalloc(ctx, &ctx->Aself, sizeof(double2) * (size_t)ctx->g.Vc * 8 * (2 * nv) * (2 * nv)));
-    TRY(dalloc(ctx, &ctx->cstage, sizeof(double2) * (size_t)ctx->g.Vc * 9 * (2 * nv) * (2 * nv)));
-    return MG_OK;
+    return dalloc_all(ctx, {{&ctx->protos, sizeof(double2) * n * nv}, {&ctx->protos_t, sizeof(double2) * n * nv},
+                            {&ctx->protos_stage, sizeof(double2) * n * nv},
+                            {&ctx->Aself, sizeof(double2) * (size_t)ctx->g.Vc * 8 * (2 * nv) * (2 * nv)},
+                            {&ctx->cstage, sizeof(double2) * (size_t)ctx->g.Vc * 9 * (2 * nv) * (2 * nv)}});
 }
 
 // P, D_c of a level from nv prototypes (internal FP64 layout)
@@ -444,10 +456,9 @@ int build_level(mg_ctx* ctx, CoarseLevel& L, const double2* V, int nv) {
 int ensure_a16(mg_ctx* ctx, CoarseLevel& L, int Vc) {
     if (L.a16_valid) return MG_OK;
     if (L.nc % 4 != 0) return fail(ctx, MG_ERR_INVALID_ARG, "FP16 coarse storage needs an even nvec");
-    if (!L.A16) {
-        TRY(dalloc(ctx, &L.A16, sizeof(__half2) * (size_t)Vc * 9 * (2 * L.cap) * (2 * L.cap)));
-        TRY(dalloc(ctx, &L.s16, sizeof(float) * (size_t)Vc * 9));
-    }
+    if (!L.A16)
+        TRY(dalloc_all(ctx, {{&L.A16, sizeof(__half2) * (size_t)Vc * 9 * (2 * L.cap) * (2 * L.cap)},
+                             {&L.s16, sizeof(float) * (size_t)Vc * 9}}));
     coarse_pack16(L.A16, L.s16, L.A64, L.nc, Vc, ctx->st);
     CKL();
     L.a16_valid = true;
@@ -471,9 +482,10 @@ int ensure_units(mg_ctx* ctx, CoarseLevel& L, int Vc, bool h16, int mode, bool* 
     CglsShape sh{};
     if (!cgls_shape(L.nc, Vc, h16, mode, &sh)) return MG_OK;
     const size_t bytes = (size_t)Vc * 9 * L.nc * L.nc * (h16 ? 4 : 8);
+    L.au_valid = false;
     if (L.au_bytes < bytes) {
-        if (L.Au) { dfree(ctx, L.Au); L.Au = nullptr; L.au_bytes = 0; }
-        TRY(dalloc(ctx, &L.Au, bytes));
+        L.au_bytes = 0;
+        TRY(dalloc_all(ctx, {{&L.Au, bytes}}));
         L.au_bytes = bytes;
     }
     if (h16 && !L.su) TRY(dalloc(ctx, &L.su, sizeof(float) * (size_t)Vc * 9));
@@ -533,13 +545,11 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16,
     if (L.h_state != -1 && L.h_state != want) {
         const size_t blocks = (size_t)g.Vc * 9, n = blocks * L.nc * L.nc;
         if (L.h_blocks < blocks) {
-            for (void* q : {(void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16, (void*)L.Ht}) dfree(ctx, q);
-            L.Ht = nullptr;
-            L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr;
+            for (void* q : {(void*)L.H16, (void*)L.hs16, (void*)L.Ht}) dfree(ctx, q);
+            L.H16 = nullptr; L.hs16 = nullptr; L.Ht = nullptr;
             L.h_blocks = 0;
             const size_t most = blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap);
-            TRY(dalloc(ctx, &L.H64, sizeof(double2) * most));
-            TRY(dalloc(ctx, &L.H32, sizeof(float2) * most));
+            TRY(dalloc_all(ctx, {{&L.H64, sizeof(double2) * most}, {&L.H32, sizeof(float2) * most}}));
             L.h_blocks = blocks;
         }
         CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->st));
@@ -554,10 +564,9 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16,
     }
     *ok = L.h_state == want;
     if (*ok && h16 && !L.h16_valid) {
-        if (!L.H16) {
-            TRY(dalloc(ctx, &L.H16, sizeof(__half2) * L.h_blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)));
-            TRY(dalloc(ctx, &L.hs16, sizeof(float) * L.h_blocks));
-        }
+        if (!L.H16)
+            TRY(dalloc_all(ctx, {{&L.H16, sizeof(__half2) * L.h_blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)},
+                                 {&L.hs16, sizeof(float) * L.h_blocks}}));
         coarse_pack16(L.H16, L.hs16, L.H64, L.nc, g.Vc, ctx->st);
         CKL();
         L.h16_valid = true;
@@ -577,23 +586,13 @@ int ensure_tiles(mg_ctx* ctx, CoarseLevel& L, int Vc) {
 }
 int ensure_panel(mg_ctx* ctx, PanelWork& w, int npad, int nc, int Vc) {
     if (w.npad >= npad && w.nc == nc && w.Vc == Vc) return MG_OK;
-    if (w.npad) {   // grow: release the smaller workspace first
-        CK(cudaStreamSynchronize(ctx->st));
-        for (void* q : {(void*)w.rc, (void*)w.y, (void*)w.r, (void*)w.s, (void*)w.p, (void*)w.q, (void*)w.u, (void*)w.z,
-                        (void*)w.e, (void*)w.bts, (void*)w.btu, (void*)w.sync, (void*)w.iters, (void*)w.flags})
-            dfree(ctx, q);
-        w = PanelWork{};
-    }
+    if (w.npad) CK(cudaStreamSynchronize(ctx->st));   // grow: the smaller workspace goes first
+    w.npad = 0;
     const size_t pe = sizeof(float2) * (size_t)Vc * nc * npad;
-    for (float2** q : {&w.rc, &w.y, &w.r, &w.s, &w.p, &w.q, &w.u, &w.z, &w.e}) {
-        TRY(dalloc(ctx, q, pe));
-        CK(cudaMemsetAsync(*q, 0, pe, ctx->st));
-    }
-    TRY(dalloc(ctx, &w.bts, bcg_tile_bytes(nc, npad, Vc)));
-    TRY(dalloc(ctx, &w.btu, bcg_tile_bytes(nc, npad, Vc)));
-    TRY(dalloc(ctx, &w.sync, bcg_sync_bytes(npad)));
-    TRY(dalloc(ctx, &w.iters, sizeof(double) * npad));
-    TRY(dalloc(ctx, &w.flags, sizeof(int) * 4));
+    TRY(dalloc_all(ctx, {{&w.rc, pe}, {&w.y, pe}, {&w.r, pe}, {&w.s, pe}, {&w.p, pe}, {&w.q, pe}, {&w.u, pe}, {&w.z, pe},
+                         {&w.e, pe}, {&w.bts, bcg_tile_bytes(nc, npad, Vc)}, {&w.btu, bcg_tile_bytes(nc, npad, Vc)},
+                         {&w.sync, bcg_sync_bytes(npad)}, {&w.iters, sizeof(double) * npad}, {&w.flags, sizeof(int) * 4}}));
+    for (float2* q : {w.rc, w.y, w.r, w.s, w.p, w.q, w.u, w.z, w.e}) CK(cudaMemsetAsync(q, 0, pe, ctx->st));
     CK(cudaMemsetAsync(w.flags, 0, sizeof(int) * 4, ctx->st));
     w.npad = npad;
     w.nc = nc;
@@ -661,11 +660,10 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
             const int mode = cgls_mode(ctx->prm.coarse_kernel);
             if (!(L.hu_valid && L.hu_h16 == ctx->coarse16 && L.hu_mode == mode)) {
                 const size_t bytes = (size_t)sys.g.Vc * 9 * L.nc * L.nc * (ctx->coarse16 ? 4 : 8);
+                Lm.hu_valid = false;
                 if (Lm.hu_bytes < bytes) {
-                    dfree(ctx, Lm.Hu);
-                    Lm.Hu = nullptr;
                     Lm.hu_bytes = 0;
-                    TRY(dalloc(ctx, &Lm.Hu, bytes));
+                    TRY(dalloc_all(ctx, {{&Lm.Hu, bytes}}));
                     Lm.hu_bytes = bytes;
                 }
                 if (ctx->coarse16 && !L.hsu) TRY(dalloc(ctx, &Lm.hsu, sizeof(float) * (size_t)sys.g.Vc * 9));
@@ -808,13 +806,10 @@ struct Counters {
 // FP16 links and the FP16 smoother vectors (MG_FP16 mode), built on first use
 int ensure_fine16(mg_ctx* ctx) {
     const size_t V = (size_t)ctx->g.V;
-    if (!ctx->U16) {
-        TRY(dalloc(ctx, &ctx->U16, sizeof(uint2) * 20 * V));
-        TRY(dalloc(ctx, &ctx->h_r, sizeof(uint2) * 6 * V));
-        TRY(dalloc(ctx, &ctx->h_q, sizeof(uint2) * 6 * V));
-        TRY(dalloc(ctx, &ctx->h_sr, sizeof(float) * V));
-        TRY(dalloc(ctx, &ctx->h_sq, sizeof(float) * V));
-    }
+    if (!ctx->U16)
+        TRY(dalloc_all(ctx, {{&ctx->U16, sizeof(uint2) * 20 * V}, {&ctx->h_r, sizeof(uint2) * 6 * V},
+                             {&ctx->h_q, sizeof(uint2) * 6 * V}, {&ctx->h_sr, sizeof(float) * V},
+                             {&ctx->h_sq, sizeof(float) * V}}));
     if (!ctx->u16_valid) {
         links_to_half(ctx->U16, ctx->U32, ctx->g, ctx->st);
         CKL();
@@ -879,9 +874,9 @@ int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt
         TRY(ensure_fine16(ctx));
         const size_t V = (size_t)ctx->g.V;
         if (ctx->h_bk < steps) {
-            if (ctx->h_basis) { dfree(ctx, ctx->h_basis); dfree(ctx, ctx->h_bscale); ctx->h_basis = nullptr; }
-            TRY(dalloc(ctx, &ctx->h_basis, sizeof(uint2) * 6 * V * (size_t)(steps + 1)));
-            TRY(dalloc(ctx, &ctx->h_bscale, sizeof(float) * V * (size_t)(steps + 1)));
+            ctx->h_bk = 0;
+            TRY(dalloc_all(ctx, {{&ctx->h_basis, sizeof(uint2) * 6 * V * (size_t)(steps + 1)},
+                                 {&ctx->h_bscale, sizeof(float) * V * (size_t)(steps + 1)}}));
             ctx->h_bk = steps;
         }
         Reduce Rs = R;
@@ -920,10 +915,11 @@ int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt
         // Arnoldi with one classical Gram-Schmidt pass per vector, the small
         // least-squares problem on the device, z += omega V y
         if (w.gm_k < steps || w.gm_m < ln.m) {
-            if (w.gm) { dfree(ctx, w.gm); w.gm = nullptr; }
-            w.gm_k = std::max(w.gm_k, steps);
-            w.gm_m = std::max(w.gm_m, ln.m);
-            TRY(dalloc(ctx, &w.gm, sizeof(v2<T>) * n * (size_t)(w.gm_k + 1) * w.gm_m));
+            const int k = std::max(w.gm_k, steps), m = std::max(w.gm_m, ln.m);
+            w.gm_k = w.gm_m = 0;
+            TRY(dalloc_all(ctx, {{&w.gm, sizeof(v2<T>) * n * (size_t)(k + 1) * m}}));
+            w.gm_k = k;
+            w.gm_m = m;
         }
         Reduce Rs = R;
         if (ln.m == 1) Rs.scal = ctx->scal_s;   // a batch brings its own
@@ -976,8 +972,8 @@ int smooth(mg_ctx* ctx, const v2<T>* r, v2<T>* z, const Reduce& R, Counters& cnt
     v2<T>*vr = w.vr, *vq = w.vq;
     if (ln.m > 1) {   // r and q of every lane
         if (w.mr_m < ln.m) {
-            if (w.mr) { dfree(ctx, w.mr); w.mr = nullptr; w.mr_m = 0; }
-            TRY(dalloc(ctx, &w.mr, sizeof(v2<T>) * n * 2 * (size_t)ln.m));
+            w.mr_m = 0;
+            TRY(dalloc_all(ctx, {{&w.mr, sizeof(v2<T>) * n * 2 * (size_t)ln.m}}));
             w.mr_m = ln.m;
         }
         vr = w.mr;
@@ -1010,16 +1006,13 @@ template <typename T> int ensure_l1work(mg_ctx* ctx) {
     if (l.ready) return MG_OK;
     const size_t n1 = (size_t)ctx->g.Vc * 2 * ctx->prm.nvec, n2 = (size_t)ctx->g2.Vc * 2 * ctx->prm.nvec2;
     const size_t b1 = sizeof(v2<T>) * n1, b2 = sizeof(v2<T>) * n2;
-    TRY(dalloc(ctx, &l.z, b1));
-    TRY(dalloc(ctx, &l.res, b1));
-    TRY(dalloc(ctx, &l.zero, b1));
-    TRY(dalloc(ctx, &l.sv, b1));
-    TRY(dalloc(ctx, &l.sz, b1));
-    for (v2<T>** q : {&l.crc, &l.cy, &l.cr, &l.cr1, &l.cs, &l.cp, &l.cp1, &l.cq, &l.eb, &l.et}) TRY(dalloc(ctx, q, b2));
+    TRY(dalloc_all(ctx, {{&l.z, b1}, {&l.res, b1}, {&l.zero, b1}, {&l.sv, b1}, {&l.sz, b1}, {&l.crc, b2}, {&l.cy, b2},
+                         {&l.cr, b2}, {&l.cr1, b2}, {&l.cs, b2}, {&l.cp, b2}, {&l.cp1, b2}, {&l.cq, b2}, {&l.eb, b2},
+                         {&l.et, b2}}));
     zero<T>(l.zero, n1, ctx->st);
     if (sizeof(T) == 4) {
         const size_t tb = sizeof(unsigned long long) * 6 * n2;
-        TRY(dalloc(ctx, &l.ctag, tb));
+        TRY(dalloc_all(ctx, {{&l.ctag, tb}}));
         CK(cudaMemsetAsync(l.ctag, 0, tb, ctx->st));   // epoch 0 is never awaited
     }
     l.ready = true;
@@ -1055,10 +1048,9 @@ int ensure_level2(mg_ctx* ctx, CoarseLevel& L, int nv2) {
         L.at_valid = L.a16_valid = L.au_valid = L.valid = false;
         const size_t np = (size_t)nv2 * ctx->g.Vc * 2 * ctx->prm.nvec;
         const size_t na = (size_t)ctx->g2.Vc * 9 * (2 * nv2) * (2 * nv2);
-        TRY(dalloc(ctx, &L.P64, sizeof(double2) * np));
-        TRY(dalloc(ctx, &L.P32, sizeof(float2) * np));
-        TRY(dalloc(ctx, &L.A64, sizeof(double2) * na));
-        TRY(dalloc(ctx, &L.A32, sizeof(float2) * na));
+        L.cap = 0;
+        TRY(dalloc_all(ctx, {{&L.P64, sizeof(double2) * np}, {&L.P32, sizeof(float2) * np}, {&L.A64, sizeof(double2) * na},
+                             {&L.A32, sizeof(float2) * na}}));
         L.cap = nv2;
     }
     L.nv = nv2;
@@ -1102,8 +1094,8 @@ template <typename T> int smooth_l1(mg_ctx* ctx, const v2<T>* r1, v2<T>* z, int 
     L1Work<T>& l = l1work<T>(ctx);
     const size_t n1 = (size_t)ctx->g.Vc * ctx->full.nc;
     if (l.gm_k < k) {
-        if (l.gm) { dfree(ctx, l.gm); l.gm = nullptr; l.gm_k = 0; }
-        TRY(dalloc(ctx, &l.gm, sizeof(v2<T>) * n1 * (size_t)(k + 1)));
+        l.gm_k = 0;
+        TRY(dalloc_all(ctx, {{&l.gm, sizeof(v2<T>) * n1 * (size_t)(k + 1)}}));
         l.gm_k = k;
     }
     Reduce Rs = ctx->R;
@@ -1891,20 +1883,15 @@ int ensure_nn(mg_ctx* ctx) {
     for (int k = 0; k < NnState::kLayers; ++k) {
         q.off[k] = o;
         const int c = NnState::kCh[k] * NnState::kCh[k + 1] * 144;
-        TRY(dalloc(ctx, &q.W[k], sizeof(float2) * c));
-        TRY(dalloc(ctx, &q.Wt[k], sizeof(float2) * c));
+        TRY(dalloc_all(ctx, {{&q.W[k], sizeof(float2) * c}, {&q.Wt[k], sizeof(float2) * c}}));
         o += c;
     }
     q.off[NnState::kLayers] = o;
-    TRY(dalloc(ctx, &q.Wm, sizeof(double2) * o));
-    TRY(dalloc(ctx, &q.G, sizeof(double2) * o));
-    TRY(dalloc(ctx, &q.m, sizeof(double2) * o));
-    TRY(dalloc(ctx, &q.v, sizeof(double2) * o));
-    TRY(dalloc(ctx, &q.act, sizeof(float2) * n * 26));
-    TRY(dalloc(ctx, &q.ga, sizeof(float2) * n * 8));
-    TRY(dalloc(ctx, &q.gb, sizeof(float2) * n * 8));
-    TRY(dalloc(ctx, &q.part, sizeof(float2) * (size_t)nn_wgrad_blocks(ctx->g) * 576 * 16));
-    TRY(dalloc(ctx, &q.r, sizeof(float2) * n));
+    TRY(dalloc_all(ctx, {{&q.Wm, sizeof(double2) * o}, {&q.G, sizeof(double2) * o}, {&q.m, sizeof(double2) * o},
+                         {&q.v, sizeof(double2) * o}, {&q.act, sizeof(float2) * n * 26}, {&q.ga, sizeof(float2) * n * 8},
+                         {&q.gb, sizeof(float2) * n * 8},
+                         {&q.part, sizeof(float2) * (size_t)nn_wgrad_blocks(ctx->g) * 576 * 16},
+                         {&q.r, sizeof(float2) * n}}));
     CK(cudaMemsetAsync(q.m, 0, sizeof(double2) * o, ctx->st));
     CK(cudaMemsetAsync(q.v, 0, sizeof(double2) * o, ctx->st));
     q.ready = true;
@@ -1941,11 +1928,9 @@ int nn_loss_grad(mg_ctx* ctx, bool grad, double gscale) {
     const size_t n = nfine(ctx);
     const CoarseLevel& L = ctx->full;
     if (q.cvec_nv < L.nv) {   // sized by the current level (nvec may change with mg_set_params)
-        if (q.cvec) {
-            CK(cudaStreamSynchronize(ctx->st));
-            dfree(ctx, q.cvec);
-        }
-        TRY(dalloc(ctx, &q.cvec, sizeof(float2) * (size_t)ctx->g.Vc * 2 * L.nv));
+        if (q.cvec) CK(cudaStreamSynchronize(ctx->st));
+        q.cvec_nv = 0;
+        TRY(dalloc_all(ctx, {{&q.cvec, sizeof(float2) * (size_t)ctx->g.Vc * 2 * L.nv}}));
         q.cvec_nv = L.nv;
     }
     float2* v = reinterpret_cast<float2*>(nn_act(ctx, NnState::kLayers));
@@ -2104,10 +2089,8 @@ int need_three_levels(mg_ctx* ctx) {
 }
 int upload_protos2(mg_ctx* ctx, const double* V2) {
     const size_t n1 = (size_t)ctx->g.Vc * ctx->full.nc, nv2 = ctx->prm.nvec2;
-    if (!ctx->protos2) {
-        TRY(dalloc(ctx, &ctx->protos2, sizeof(double2) * n1 * nv2));
-        TRY(dalloc(ctx, &ctx->protos2_t, sizeof(double2) * n1 * nv2));
-    }
+    if (!ctx->protos2)
+        TRY(dalloc_all(ctx, {{&ctx->protos2, sizeof(double2) * n1 * nv2}, {&ctx->protos2_t, sizeof(double2) * n1 * nv2}}));
     CK(cudaMemcpyAsync(ctx->protos2, V2, sizeof(double2) * n1 * nv2, cudaMemcpyHostToDevice, ctx->st));
     return MG_OK;
 }
@@ -2483,8 +2466,8 @@ int mg_check_wait_timeout(mg_ctx* ctx, int kind, long long spin_limit) {
     const size_t words = (size_t)2 * 3 * (G + 1) * 16;   // two parities x three values x (G + 1) padded slots
     unsigned long long* w = nullptr;
     unsigned int* ctr = nullptr;
-    TRY(dalloc(ctx, &w, sizeof(unsigned long long) * words));
-    TRY(dalloc(ctx, &ctr, sizeof(unsigned int) * 4));   // [0] count, [1] generation, [2] error flag
+    // ctr: [0] count, [2] error flag
+    TRY(dalloc_all(ctx, {{&w, sizeof(unsigned long long) * words}, {&ctr, sizeof(unsigned int) * 4}}));
     int st = MG_OK;
     CK(cudaMemsetAsync(w, 0, sizeof(unsigned long long) * words, ctx->st));
     CK(cudaMemsetAsync(ctr, 0, sizeof(unsigned int) * 4, ctx->st));
@@ -2496,6 +2479,12 @@ int mg_check_wait_timeout(mg_ctx* ctx, int kind, long long spin_limit) {
     dfree(ctx, ctr);
     if (flag) st = fail(ctx, MG_ERR_TIMEOUT, "bounded wait gave up as expected (kind " + std::to_string(kind) + ")");
     return st;
+}
+int mg_fail_allocation(mg_ctx* ctx, int nth) {
+    if (!ctx || nth < 0) return -1;
+    const int pending = ctx->refuse_alloc;
+    ctx->refuse_alloc = nth;
+    return pending;
 }
 int mg_coarse_kernel(mg_ctx* ctx) { return ctx ? ctx->coarse_kernel_used : MG_CK_NONE; }
 
@@ -2620,21 +2609,14 @@ int ensure_eo(mg_ctx* ctx, int inner_bytes) {
         w.e.Vh = g.V / 2;
         w.e.tap = g.tap;
         const size_t nf = (size_t)24 * w.e.Vh;
-        TRY(dalloc(ctx, &w.U64, sizeof(double2) * 36 * (size_t)g.V));
-        TRY(dalloc(ctx, &w.U32, sizeof(float2) * 36 * (size_t)g.V));
-        TRY(dalloc(ctx, &w.b, sizeof(double2) * nf));
-        TRY(dalloc(ctx, &w.x, sizeof(double2) * nf));
-        TRY(dalloc(ctx, &w.res, sizeof(double2) * nf));
-        TRY(dalloc(ctx, &w.t, sizeof(double2) * nf));
+        TRY(dalloc_all(ctx, {{&w.U64, sizeof(double2) * 36 * (size_t)g.V}, {&w.U32, sizeof(float2) * 36 * (size_t)g.V},
+                             {&w.b, sizeof(double2) * nf}, {&w.x, sizeof(double2) * nf}, {&w.res, sizeof(double2) * nf},
+                             {&w.t, sizeof(double2) * nf}}));
     }
     if (w.inner_bytes != inner_bytes) {
-        for (void* q : {w.xe, w.r, w.s, w.p, w.q, w.t1}) dfree(ctx, q);
         const size_t nh = (size_t)12 * w.e.Vh * inner_bytes;
-        for (void** q : {&w.xe, &w.r, &w.s, &w.p, &w.q, &w.t1}) {
-            unsigned char* a = nullptr;
-            TRY(dalloc(ctx, &a, nh));
-            *q = a;
-        }
+        w.inner_bytes = 0;
+        TRY(dalloc_all(ctx, {{&w.xe, nh}, {&w.r, nh}, {&w.s, nh}, {&w.p, nh}, {&w.q, nh}, {&w.t1, nh}}));
         w.inner_bytes = inner_bytes;
     }
     if (!w.links_valid) {
@@ -2819,24 +2801,16 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
     int K = std::min(ctx->prm.gcr_restart, ctx->K);
     TRY(ensure_panel(ctx, b.pw, npad, nc, ctx->g.Vc));
     if (b.nrhs_cap >= nrhs && b.K >= K) return MG_OK;
-    if (b.nrhs_cap) {   // grow: release the smaller workspace first
-        CK(cudaStreamSynchronize(ctx->st));
-        for (void* q : {(void*)b.r32, (void*)b.Z, (void*)b.Pk, (void*)b.x64, (void*)b.b64, (void*)b.scal, (void*)b.partials,
-                        (void*)b.ticket, (void*)b.scal_s})
-            dfree(ctx, q);
-        cudaFreeHost(b.h_flags);
-        cudaFreeHost(b.h_iters);
-        cudaFreeHost(b.h_scal);
-        const PanelWork pw = b.pw;
-        b = BatchWork{};
-        b.pw = pw;
-    }
-    TRY(dalloc(ctx, &b.r32, sizeof(float2) * n * nrhs));
-    TRY(dalloc(ctx, &b.Z, sizeof(float2) * n * nrhs * K));
-    TRY(dalloc(ctx, &b.Pk, sizeof(float2) * n * nrhs * K));
-    TRY(dalloc(ctx, &b.x64, sizeof(double2) * n * nrhs));
-    TRY(dalloc(ctx, &b.b64, sizeof(double2) * n * nrhs));
-    TRY(dalloc(ctx, &b.scal, sizeof(double) * S_COUNT * nrhs));
+    if (b.nrhs_cap) CK(cudaStreamSynchronize(ctx->st));   // grow: the smaller workspace goes first
+    b.nrhs_cap = 0;
+    cudaFreeHost(b.h_flags);
+    cudaFreeHost(b.h_iters);
+    cudaFreeHost(b.h_scal);
+    b.h_flags = nullptr;
+    b.h_iters = b.h_scal = nullptr;
+    TRY(dalloc_all(ctx, {{&b.r32, sizeof(float2) * n * nrhs}, {&b.Z, sizeof(float2) * n * nrhs * K},
+                         {&b.Pk, sizeof(float2) * n * nrhs * K}, {&b.x64, sizeof(double2) * n * nrhs},
+                         {&b.b64, sizeof(double2) * n * nrhs}, {&b.scal, sizeof(double) * S_COUNT * nrhs}}));
     CK(cudaMallocHost(&b.h_flags, sizeof(int) * 4));
     CK(cudaMallocHost(&b.h_iters, sizeof(double) * nrhs));
     CK(cudaMallocHost(&b.h_scal, sizeof(double) * S_COUNT * nrhs));
@@ -2865,13 +2839,9 @@ int batched_coarse_solve(mg_ctx* ctx, int nrhs, double tol, int maxit, std::vect
 int ensure_lanes(mg_ctx* ctx, int m) {
     BatchWork& b = ctx->bw;
     if (b.lanes >= m) return MG_OK;
-    for (void* q : {(void*)b.partials, (void*)b.ticket, (void*)b.scal_s}) dfree(ctx, q);
-    b.partials = b.scal_s = nullptr;
-    b.ticket = nullptr;
     b.lanes = 0;
-    TRY(dalloc(ctx, &b.partials, ctx->R.partial_bytes * m));
-    TRY(dalloc(ctx, &b.ticket, sizeof(unsigned int) * m));
-    TRY(dalloc(ctx, &b.scal_s, sizeof(double) * S_COUNT * m));
+    TRY(dalloc_all(ctx, {{&b.partials, ctx->R.partial_bytes * m}, {&b.ticket, sizeof(unsigned int) * m},
+                         {&b.scal_s, sizeof(double) * S_COUNT * m}}));
     CK(cudaMemsetAsync(b.ticket, 0, sizeof(unsigned int) * m, ctx->st));
     b.lanes = m;
     return MG_OK;
@@ -3134,8 +3104,7 @@ int mg_solve_batched(mg_ctx* ctx, const double* b, double* x, int nrhs, mg_solve
     if (!b || !x || nrhs <= 0) return fail(ctx, MG_ERR_INVALID_ARG, "null buffer or nrhs <= 0");
     size_t n = nfine(ctx);
     double2 *db = nullptr, *dx = nullptr;
-    TRY(dalloc(ctx, &db, sizeof(double2) * n * nrhs));
-    TRY(dalloc(ctx, &dx, sizeof(double2) * n * nrhs));
+    TRY(dalloc_all(ctx, {{&db, sizeof(double2) * n * nrhs}, {&dx, sizeof(double2) * n * nrhs}}));
     CK(cudaMemcpyAsync(db, b, sizeof(double2) * n * nrhs, cudaMemcpyHostToDevice, ctx->st));
     int st = mg_solve_batched_device(ctx, (const double*)db, (double*)dx, nrhs, infos);
     if (st == MG_OK || st == MG_ERR_NOT_CONVERGED) {
@@ -3239,8 +3208,7 @@ int mg_apply_coarse_batched(mg_ctx* ctx, const double* x, double* y, int nrhs, i
         scale[r] = mx > 0 ? mx : 1.0;
         for (long long i = 0; i < 2 * rows; ++i) xs[(size_t)r * 2 * rows + i] = x[(size_t)r * 2 * rows + i] / scale[r];
     }
-    TRY(dalloc(ctx, &hin, sizeof(double2) * nin));
-    TRY(dalloc(ctx, &hout, sizeof(double2) * nin));
+    TRY(dalloc_all(ctx, {{&hin, sizeof(double2) * nin}, {&hout, sizeof(double2) * nin}}));
     CK(cudaMemcpyAsync(hin, xs.data(), sizeof(double2) * nin, cudaMemcpyHostToDevice, ctx->st));
     std::vector<void*> tmp = {hin, hout};
     int st = MG_OK;
@@ -3258,8 +3226,10 @@ int mg_apply_coarse_batched(mg_ctx* ctx, const double* x, double* y, int nrhs, i
         CK(cudaStreamSynchronize(ctx->st));
         if (err) st = fail(ctx, MG_ERR_TIMEOUT, "batched coarse stencil: a bounded wait gave up");
     } else {
-        TRY(dalloc(ctx, &p64a, sizeof(double2) * npanel));
-        TRY(dalloc(ctx, &p64b, sizeof(double2) * npanel));
+        if ((st = dalloc_all(ctx, {{&p64a, sizeof(double2) * npanel}, {&p64b, sizeof(double2) * npanel}})) != MG_OK) {
+            release(ctx, tmp);
+            return st;
+        }
         tmp.push_back(p64a);
         tmp.push_back(p64b);
         panel_pack64(p64a, hin, rows, nrhs, npad, ctx->st);
