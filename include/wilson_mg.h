@@ -268,6 +268,13 @@ int mg_get_null_vectors(mg_ctx* ctx, double* V);
  * layout). */
 int mg_get_coarse_op(mg_ctx* ctx, double* A);
 
+/* Read back the red-black form of D_c on which the coarse solves of a solve run (FP64,
+ * host, the layout of the coarse operator): on an even aggregate the diagonal block
+ * A_ee and -A_eo, on an odd one A_oo^-1 and A_oo^-1 A_oe.  MG_ERR_INVALID_ARG when a
+ * coarse extent is odd, MG_ERR_NUMERIC when the solves use D_c itself because the form
+ * does not exist (a singular diagonal block). */
+int mg_get_schur_op(mg_ctx* ctx, double* H);
+
 /* Solve D x = b by MG-preconditioned flexible GCR (Sec. III), x0 = 0.
  * b, x: host fine spinors (FP64).  Returns MG_ERR_NOT_CONVERGED with x the
  * last iterate when max_outer is reached. */

@@ -90,6 +90,7 @@ _SIGS = {
     "mg_get_level2_op": ([_P, _P], _I),
     "mg_kcycle": ([_P, _P, _P, _I], _I),
     "mg_get_coarse_op": ([_P, _P], _I),
+    "mg_get_schur_op": ([_P, _P], _I),
     "mg_solve": ([_P, _P, _P, _P], _I),
     "mg_solve_device": ([_P, _P, _P, _P], _I),
     "mg_solve_batched": ([_P, _P, _P, _I, _P], _I),
@@ -328,6 +329,12 @@ def mg_kcycle(ctx, r1, prec: int = MG_FP64) -> np.ndarray:
 def mg_get_coarse_op(ctx, Vc: int, nc: int) -> np.ndarray:
     out = np.empty((Vc, 9, nc, nc), dtype=np.complex128)
     _check(load().mg_get_coarse_op(ctx, _ptr(out)), ctx)
+    return out
+
+
+def mg_get_schur_op(ctx, Vc: int, nc: int) -> np.ndarray:
+    out = np.empty((Vc, 9, nc, nc), dtype=np.complex128)
+    _check(load().mg_get_schur_op(ctx, _ptr(out)), ctx)
     return out
 
 
@@ -636,6 +643,9 @@ class WilsonMG:
 
     def coarse_op(self):
         return mg_get_coarse_op(self.ctx, self.Vc, self.nc)
+
+    def schur_op(self):
+        return mg_get_schur_op(self.ctx, self.Vc, self.nc)
 
     def solve(self, b, out=None):
         return mg_solve(self.ctx, b, out)

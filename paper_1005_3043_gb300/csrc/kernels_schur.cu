@@ -42,21 +42,19 @@ void parity_order(int* ord, const Geom& g, cudaStream_t st) {
     k_parity_order<<<(g.Vc / 2 + 255) / 256, 256, 0, st>>>(ord, g);
 }
 
-// One CTA per site; an odd one inverts its diagonal block in FP64 (Gauss-Jordan in
-// place with row pivoting, the block in shared memory) and multiplies it with the
-// hop blocks in TC: FP64, or FP32 where the solver holds the operator in 32 or 16
-// bits anyway (FP64 products are two per clock and SM: 1.8 M clocks per site at
-// nc = 48, against 60 k).
+// One CTA per site; an odd one inverts its diagonal block (Gauss-Jordan in place with
+// row pivoting, the block in shared memory) and multiplies it with the hop blocks, all
+// in FP64: an operator stored in 32 or 16 bits is then rounded once, as D_c is.  Bound
+// by the FP64 pipe, two operations per clock and SM: 1.8 M clocks per site at nc = 48.
 constexpr int kSchurThreads = 256;
-template <typename TC>
 __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H, const double2* __restrict__ A, int nc,
                                                          Geom g, int* status) {
     extern __shared__ unsigned char smem_raw[];
     double2* M = reinterpret_cast<double2*>(smem_raw);          // M[i * nc + j]
     double2* col = M + (size_t)nc * nc;
     int* piv = reinterpret_cast<int*>(col + 2 * nc);
-    v2<TC>* Bs = reinterpret_cast<v2<TC>*>(piv + ((nc + 3) & ~3));   // the inverse in TC, [c][a]
-    v2<TC>* As = Bs + (size_t)nc * nc;                          // a hop block, [b][c]
+    double2* Bs = reinterpret_cast<double2*>(piv + ((nc + 3) & ~3));   // the inverse, [c][a]
+    double2* As = Bs + (size_t)nc * nc;                         // a hop block, [b][c]
     __shared__ int s_p;
     const int X = blockIdx.x, t = threadIdx.x, nn = nc * nc;
     const double2* Ax = A + (size_t)X * 9 * nn;
@@ -136,46 +134,38 @@ __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H
         const int b = i / nc, a = i - b * nc;
         const double2 v = M[a * nc + b];
         Hx[i] = v;
-        Bs[i].x = (TC)v.x;
-        Bs[i].y = (TC)v.y;
+        Bs[i] = v;
     }
     for (int dd = 1; dd < 9; ++dd) {
         __syncthreads();
-        for (int i = t; i < nn; i += kSchurThreads) {
-            const double2 v = Ax[(size_t)dd * nn + i];
-            As[i].x = (TC)v.x;
-            As[i].y = (TC)v.y;
-        }
+        for (int i = t; i < nn; i += kSchurThreads) As[i] = Ax[(size_t)dd * nn + i];
         __syncthreads();
         // two rows and two columns per thread (nc is even)
         for (int i = t; i < nn / 4; i += kSchurThreads) {
             const int b = 2 * (i / (nc / 2)), a = 2 * (i % (nc / 2));
-            cx<TC> s00(0, 0), s01(0, 0), s10(0, 0), s11(0, 0);
+            cx<double> s00(0, 0), s01(0, 0), s10(0, 0), s11(0, 0);
             for (int c = 0; c < nc; ++c) {
-                const cx<TC> b0 = ld<TC>(Bs + c * nc + a), b1 = ld<TC>(Bs + c * nc + a + 1);
-                const cx<TC> a0 = ld<TC>(As + b * nc + c), a1 = ld<TC>(As + (b + 1) * nc + c);
+                const cx<double> b0 = ld<double>(Bs + c * nc + a), b1 = ld<double>(Bs + c * nc + a + 1);
+                const cx<double> a0 = ld<double>(As + b * nc + c), a1 = ld<double>(As + (b + 1) * nc + c);
                 cmad(s00, b0, a0);
                 cmad(s01, b1, a0);
                 cmad(s10, b0, a1);
                 cmad(s11, b1, a1);
             }
             double2* o = Hx + (size_t)dd * nn + (size_t)b * nc + a;
-            o[0] = make_double2((double)s00.r, (double)s00.i);
-            o[1] = make_double2((double)s01.r, (double)s01.i);
-            o[nc] = make_double2((double)s10.r, (double)s10.i);
-            o[nc + 1] = make_double2((double)s11.r, (double)s11.i);
+            st<double>(o, s00);
+            st<double>(o + 1, s01);
+            st<double>(o + nc, s10);
+            st<double>(o + nc + 1, s11);
         }
     }
 }
-cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, bool f64, int* status, cudaStream_t st) {
-    const size_t sz = f64 ? 16 : 8;
-    const size_t sm = sizeof(double2) * ((size_t)nc * nc + 2 * nc) + 4 * ((nc + 3) & ~3) + 2 * sz * nc * nc;
-    const void* fn = f64 ? (const void*)k_schur<double> : (const void*)k_schur<float>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, int* status, cudaStream_t st) {
+    const size_t sm = sizeof(double2) * (3 * (size_t)nc * nc + 2 * nc) + 4 * ((nc + 3) & ~3);
+    cudaError_t e = cudaFuncSetAttribute(k_schur, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     note_launch();
-    if (f64) k_schur<double><<<g.Vc, kSchurThreads, sm, st>>>(H, A, nc, g, status);
-    else k_schur<float><<<g.Vc, kSchurThreads, sm, st>>>(H, A, nc, g, status);
+    k_schur<<<g.Vc, kSchurThreads, sm, st>>>(H, A, nc, g, status);
     return cudaGetLastError();
 }
 

@@ -53,7 +53,7 @@ struct CoarseLevel {
     bool hu_valid = false, hu_h16 = false;
     int hu_mode = 0;
     size_t h_blocks = 0;      // nc x nc blocks the buffers hold
-    int h_state = 0;          // 0 not built, 1 FP32 products, 2 FP64 products, -1 a singular diagonal block
+    int h_state = 0;          // 0 not built, 1 built, -1 a singular diagonal block
     bool h16_valid = false;
     int au_mode = 0;
     CglsShape au_shape{};
@@ -540,9 +540,8 @@ template <typename T> CgSys<T> level1_sys(mg_ctx* ctx) {
 
 // The red-black Schur form of the level's operator (and, for FP16 storage, its FP16
 // copy); *ok false where it does not exist (a singular diagonal block).
-int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16, bool* ok) {
-    const int want = f64 ? 2 : 1;
-    if (L.h_state != -1 && L.h_state != want) {
+int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool h16, bool* ok) {
+    if (L.h_state == 0) {
         const size_t blocks = (size_t)g.Vc * 9, n = blocks * L.nc * L.nc;
         if (L.h_blocks < blocks) {
             for (void* q : {(void*)L.H16, (void*)L.hs16, (void*)L.Ht}) dfree(ctx, q);
@@ -553,16 +552,16 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool f64, bool h16,
             L.h_blocks = blocks;
         }
         CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->st));
-        CK(schur_build(L.H64, L.A64, L.nc, g, f64, ctx->d_status, ctx->st));
+        CK(schur_build(L.H64, L.A64, L.nc, g, ctx->d_status, ctx->st));
         int status = 0;
         CK(cudaMemcpyAsync(&status, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
         convert<double, float>(L.H32, L.H64, n, ctx->st);
         CKL();
         CK(cudaStreamSynchronize(ctx->st));
-        L.h_state = status ? -1 : want;
+        L.h_state = status ? -1 : 1;
         L.h16_valid = L.ht_valid = L.hu_valid = false;
     }
-    *ok = L.h_state == want;
+    *ok = L.h_state == 1;
     if (*ok && h16 && !L.h16_valid) {
         if (!L.H16)
             TRY(dalloc_all(ctx, {{&L.H16, sizeof(__half2) * L.h_blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)},
@@ -612,7 +611,7 @@ int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, cons
     c.g = g;
     const int half = g.Vc / 2;
     bool eo = false;
-    if (ord && tol > 0) TRY(ensure_schur(ctx, L, g, false, false, &eo));
+    if (ord && tol > 0) TRY(ensure_schur(ctx, L, g, false, &eo));
     if (!eo) {
         TRY(ensure_tiles(ctx, L, g.Vc));
     } else if (!L.ht_valid) {
@@ -654,7 +653,7 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
         if (ctx->in_solve && sys.ord && tol > 0 && !iters && ctx->prm.coarse_form == 0 && L.au_shape.tm == 1 &&
             L.au_shape.nx_max <= 128)
-            TRY(ensure_schur(ctx, Lm, sys.g, false, false, &eo));
+            TRY(ensure_schur(ctx, Lm, sys.g, false, &eo));
         const int half = sys.g.Vc / 2;
         if (eo) {
             const int mode = cgls_mode(ctx->prm.coarse_kernel);
@@ -744,7 +743,7 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
         const bool h16 = std::is_same<T, float>::value && ctx->coarse16;
         if (ctx->in_solve && sys.ord && tol > 0)
-            TRY(ensure_schur(ctx, Lm, sys.g, std::is_same<T, double>::value, h16, &eo));
+            TRY(ensure_schur(ctx, Lm, sys.g, h16, &eo));
         const int half = sys.g.Vc / 2;
         PROF_BEGIN(MG_K_COARSE_SOLVE);
         if (eo) {
@@ -2201,6 +2200,21 @@ int mg_get_coarse_op(mg_ctx* ctx, double* A) {
     coarse_op_transpose(ctx->cstage, ctx->full.A64, nc, ctx->g.Vc, ctx->st);
     CKL();
     CK(cudaMemcpyAsync(A, ctx->cstage, sizeof(double2) * (size_t)ctx->g.Vc * 9 * nc * nc, cudaMemcpyDeviceToHost, ctx->st));
+    CK(cudaStreamSynchronize(ctx->st));
+    return MG_OK;
+}
+
+int mg_get_schur_op(mg_ctx* ctx, double* H) {
+    TRY(need_level(ctx));
+    if (!H) return MG_ERR_INVALID_ARG;
+    if (!ctx->cord) return fail(ctx, MG_ERR_INVALID_ARG, "the red-black form needs even coarse extents");
+    CoarseLevel& L = ctx->full;
+    bool ok = false;
+    TRY(ensure_schur(ctx, L, ctx->g, false, &ok));
+    if (!ok) return fail(ctx, MG_ERR_NUMERIC, "the coarse operator has no red-black form");
+    coarse_op_transpose(ctx->cstage, L.H64, L.nc, ctx->g.Vc, ctx->st);
+    CKL();
+    CK(cudaMemcpyAsync(H, ctx->cstage, sizeof(double2) * (size_t)ctx->g.Vc * 9 * L.nc * L.nc, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     return MG_OK;
 }
