@@ -272,7 +272,7 @@ int mg_get_coarse_op(mg_ctx* ctx, double* A);
  * host, the layout of the coarse operator): on an even aggregate the diagonal block
  * A_ee and -A_eo, on an odd one A_oo^-1 and A_oo^-1 A_oe.  MG_ERR_INVALID_ARG when a
  * coarse extent is odd, MG_ERR_NUMERIC when the solves use D_c itself because the form
- * does not exist (a singular diagonal block). */
+ * does not exist or has lost too many bits (a singular or nearly singular A_oo). */
 int mg_get_schur_op(mg_ctx* ctx, double* H);
 
 /* Solve D x = b by MG-preconditioned flexible GCR (Sec. III), x0 = 0.

@@ -46,9 +46,17 @@ void parity_order(int* ord, const Geom& g, cudaStream_t st) {
 // row pivoting, the block in shared memory) and multiplies it with the hop blocks, all
 // in FP64: an operator stored in 32 or 16 bits is then rounded once, as D_c is.  Bound
 // by the FP64 pipe, two operations per clock and SM: 1.8 M clocks per site at nc = 48.
+// *growth receives, as the bits of a float, the largest over the odd sites of
+// max |H[o][d]|, d >= 1, and max |A_oo^-1| max |A_oo|: how much larger than D_c's own the
+// errors of the form's stored blocks can be (infinite for a singular block).
 constexpr int kSchurThreads = 256;
+constexpr float kInfinite = 3.0e38f;   // "no bound": above every accepted growth
+__device__ __forceinline__ float finite_or_infinite(float x) { return x < kInfinite ? x : kInfinite; }   // NaN too
+__device__ __forceinline__ float abs_bound(double2 v) {
+    return finite_or_infinite((float)fabs(v.x) + (float)fabs(v.y));
+}
 __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H, const double2* __restrict__ A, int nc,
-                                                         Geom g, int* status) {
+                                                         Geom g, int* growth) {
     extern __shared__ unsigned char smem_raw[];
     double2* M = reinterpret_cast<double2*>(smem_raw);          // M[i * nc + j]
     double2* col = M + (size_t)nc * nc;
@@ -56,6 +64,7 @@ __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H
     double2* Bs = reinterpret_cast<double2*>(piv + ((nc + 3) & ~3));   // the inverse, [c][a]
     double2* As = Bs + (size_t)nc * nc;                         // a hop block, [b][c]
     __shared__ int s_p;
+    __shared__ float s_max[kSchurThreads / 32];
     const int X = blockIdx.x, t = threadIdx.x, nn = nc * nc;
     const double2* Ax = A + (size_t)X * 9 * nn;
     double2* Hx = H + (size_t)X * 9 * nn;
@@ -66,7 +75,11 @@ __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H
         }
         return;
     }
-    for (int i = t; i < nn; i += kSchurThreads) M[(i % nc) * nc + i / nc] = Ax[i];   // A[b][a] -> M[a][b]
+    float ma = 0.f, mi = 0.f, mh = 0.f;   // this thread's max |A_oo|, |A_oo^-1|, |H[o][d]|
+    for (int i = t; i < nn; i += kSchurThreads) {   // A[b][a] -> M[a][b]
+        M[(i % nc) * nc + i / nc] = Ax[i];
+        ma = fmaxf(ma, abs_bound(Ax[i]));
+    }
     __syncthreads();
     for (int k = 0; k < nc; ++k) {
         if (t < 32) {   // pivot: the largest |M[i][k]|^2, i >= k (the first of equals)
@@ -85,7 +98,7 @@ __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H
             if (t == 0) {
                 s_p = at;
                 piv[k] = at;
-                if (!(best > 0.0) || best > 1e300) atomicExch(status, 1);
+                if (!(best > 0.0) || best > 1e300) atomicMax(growth, __float_as_int(kInfinite));
             }
         }
         __syncthreads();
@@ -135,6 +148,7 @@ __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H
         const double2 v = M[a * nc + b];
         Hx[i] = v;
         Bs[i] = v;
+        mi = fmaxf(mi, abs_bound(v));
     }
     for (int dd = 1; dd < 9; ++dd) {
         __syncthreads();
@@ -157,15 +171,29 @@ __global__ void __launch_bounds__(kSchurThreads) k_schur(double2* __restrict__ H
             st<double>(o + 1, s01);
             st<double>(o + nc, s10);
             st<double>(o + nc + 1, s11);
+            for (int q = 0; q < 4; ++q) mh = fmaxf(mh, abs_bound(o[(q >> 1) * nc + (q & 1)]));
         }
     }
+    // one value per CTA: fmax((max ma) (max mi), max mh)
+    auto block_max = [&](float v) {
+        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+        __syncthreads();
+        if ((t & 31) == 0) s_max[t >> 5] = v;
+        __syncthreads();
+        for (int w = 0; w < kSchurThreads / 32; ++w) v = fmaxf(v, s_max[w]);
+        return v;
+    };
+    ma = block_max(ma);
+    mi = block_max(mi);
+    mh = block_max(mh);
+    if (t == 0) atomicMax(growth, __float_as_int(finite_or_infinite(fmaxf(ma * mi, mh))));
 }
-cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, int* status, cudaStream_t st) {
+cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, int* growth, cudaStream_t st) {
     const size_t sm = sizeof(double2) * (3 * (size_t)nc * nc + 2 * nc) + 4 * ((nc + 3) & ~3);
     cudaError_t e = cudaFuncSetAttribute(k_schur, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     note_launch();
-    k_schur<<<g.Vc, kSchurThreads, sm, st>>>(H, A, nc, g, status);
+    k_schur<<<g.Vc, kSchurThreads, sm, st>>>(H, A, nc, g, growth);
     return cudaGetLastError();
 }
 

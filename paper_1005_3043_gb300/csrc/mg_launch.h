@@ -212,8 +212,9 @@ void mr_update_h(float2* e, HalfSpinor r, ConstHalfSpinor q, const Geom& g, bool
 // Red-black Schur form of a coarse operator (kernels_schur.cu)
 bool schur_supported(const Geom& g);   // every coarse extent even
 void parity_order(int* ord, const Geom& g, cudaStream_t st);   // ord[Vc]: even sites, then odd ones
-// H from A (both [X][9][b][a] FP64); *status = 1: a singular block
-cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, int* status, cudaStream_t st);
+// H from A (both [X][9][b][a] FP64); *growth (zeroed before): bits of the float that bounds
+// how much larger than D_c's own the errors of H's blocks are, 3e38 for a singular block
+cudaError_t schur_build(double2* H, const double2* A, int nc, const Geom& g, int* growth, cudaStream_t st);
 // out[X] = base[X] + sign * sum_{d0 <= d < d1} H[X][d] in[X + d] for X in sites[0, nsites), `cols`
 // columns of panels with stride cstride (1, 1: plain coarse vectors)
 template <typename T>
