@@ -194,6 +194,7 @@ struct mg_ctx {
     CoarseLevel full, trunc;
     BatchWork bw;
     PanelWork pw1;                   // one right-hand side (FP16 operators that do not fit on chip)
+    bool panel_refused = false;      // no memory for pw1 since the last level was built
     EoWork eo;
     // third level (levels == 3)
     Geom g2{};                       // the level-1 lattice cut into level-2 aggregates
@@ -449,6 +450,7 @@ int build_level(mg_ctx* ctx, CoarseLevel& L, const double2* V, int nv) {
     L.a16_valid = false;
     L.au_valid = false;
     L.h_state = 0;
+    ctx->panel_refused = false;
     return MG_OK;
 }
 
@@ -544,6 +546,20 @@ template <typename T> CgSys<T> level1_sys(mg_ctx* ctx) {
 // the growth that k_schur measures: below 6 on thermalised fields between mass 0.3
 // and -0.84; at 64 the form's blocks are off by at most six bits more than D_c's.
 constexpr float kSchurGrowth = 64.f;
+// After a failed allocation (st) of something that the form needs: its memory is given
+// back and the solves use D_c until the operator changes.
+int without_schur(mg_ctx* ctx, CoarseLevel& L, int st, bool* ok) {
+    if (st != MG_ERR_OOM) return st;
+    CK(cudaStreamSynchronize(ctx->st));
+    for (void* q : {(void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16, (void*)L.Ht, L.Hu, (void*)L.hsu}) dfree(ctx, q);
+    L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr; L.Ht = nullptr; L.Hu = nullptr; L.hsu = nullptr;
+    L.h_blocks = L.hu_bytes = 0;
+    L.h16_valid = L.ht_valid = L.hu_valid = false;
+    L.h_state = -1;
+    ctx->err.clear();
+    *ok = false;
+    return MG_OK;
+}
 int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool h16, bool* ok) {
     if (L.h_state == 0) {
         const size_t blocks = (size_t)g.Vc * 9, n = blocks * L.nc * L.nc;
@@ -552,7 +568,8 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool h16, bool* ok)
             L.H16 = nullptr; L.hs16 = nullptr; L.Ht = nullptr;
             L.h_blocks = 0;
             const size_t most = blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap);
-            TRY(dalloc_all(ctx, {{&L.H64, sizeof(double2) * most}, {&L.H32, sizeof(float2) * most}}));
+            const int st = dalloc_all(ctx, {{&L.H64, sizeof(double2) * most}, {&L.H32, sizeof(float2) * most}});
+            if (st != MG_OK) return without_schur(ctx, L, st, ok);
             L.h_blocks = blocks;
         }
         CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(int), ctx->st));
@@ -567,9 +584,11 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool h16, bool* ok)
     }
     *ok = L.h_state == 1;
     if (*ok && h16 && !L.h16_valid) {
-        if (!L.H16)
-            TRY(dalloc_all(ctx, {{&L.H16, sizeof(__half2) * L.h_blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)},
-                                 {&L.hs16, sizeof(float) * L.h_blocks}}));
+        if (!L.H16) {
+            const int st = dalloc_all(ctx, {{&L.H16, sizeof(__half2) * L.h_blocks * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)},
+                                            {&L.hs16, sizeof(float) * L.h_blocks}});
+            if (st != MG_OK) return without_schur(ctx, L, st, ok);
+        }
         coarse_pack16(L.H16, L.hs16, L.H64, L.nc, g.Vc, ctx->st);
         CKL();
         L.h16_valid = true;
@@ -605,6 +624,7 @@ int ensure_panel(mg_ctx* ctx, PanelWork& w, int npad, int nc, int Vc) {
 // CG on the normal equations of the level's operator for nrhs columns of the panel
 // w.rc -> w.y, red-black where the lattice allows it (see coarse_solve).  *err is
 // raised on a timed-out wait; scal (optional) receives column 0's iterations.
+// MG_ERR_OOM before anything is launched.
 int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, const int* ord, PanelWork& w, int nrhs,
                 double tol, int maxit, int* err, double* scal) {
     BcgArgs c{};
@@ -616,10 +636,13 @@ int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, cons
     const int half = g.Vc / 2;
     bool eo = false;
     if (ord && tol > 0) TRY(ensure_schur(ctx, L, g, false, &eo));
+    if (eo && !L.Ht) {
+        const int st = dalloc(ctx, &L.Ht, sizeof(__half) * L.h_blocks * 2 * (2 * (size_t)L.cap) * (2 * (size_t)L.cap));
+        if (st != MG_OK) TRY(without_schur(ctx, L, st, &eo));
+    }
     if (!eo) {
         TRY(ensure_tiles(ctx, L, g.Vc));
     } else if (!L.ht_valid) {
-        if (!L.Ht) TRY(dalloc(ctx, &L.Ht, sizeof(__half) * L.h_blocks * 2 * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)));
         coarse_tiles(L.Ht, L.H64, L.nc, g.Vc, ctx->st);
         L.ht_valid = true;
     }
@@ -659,17 +682,22 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
             L.au_shape.nx_max <= 128)
             TRY(ensure_schur(ctx, Lm, sys.g, false, &eo));
         const int half = sys.g.Vc / 2;
+        const int mode = cgls_mode(ctx->prm.coarse_kernel);
+        const bool packed = L.hu_valid && L.hu_h16 == ctx->coarse16 && L.hu_mode == mode;
+        const size_t bytes = (size_t)sys.g.Vc * 9 * L.nc * L.nc * (ctx->coarse16 ? 4 : 8);
+        if (eo && !packed) {
+            Lm.hu_valid = false;
+            int st = MG_OK;
+            if (Lm.hu_bytes < bytes) {
+                Lm.hu_bytes = 0;
+                st = dalloc_all(ctx, {{&Lm.Hu, bytes}});
+                if (st == MG_OK) Lm.hu_bytes = bytes;
+            }
+            if (st == MG_OK && ctx->coarse16 && !L.hsu) st = dalloc(ctx, &Lm.hsu, sizeof(float) * (size_t)sys.g.Vc * 9);
+            if (st != MG_OK) TRY(without_schur(ctx, Lm, st, &eo));
+        }
         if (eo) {
-            const int mode = cgls_mode(ctx->prm.coarse_kernel);
-            if (!(L.hu_valid && L.hu_h16 == ctx->coarse16 && L.hu_mode == mode)) {
-                const size_t bytes = (size_t)sys.g.Vc * 9 * L.nc * L.nc * (ctx->coarse16 ? 4 : 8);
-                Lm.hu_valid = false;
-                if (Lm.hu_bytes < bytes) {
-                    Lm.hu_bytes = 0;
-                    TRY(dalloc_all(ctx, {{&Lm.Hu, bytes}}));
-                    Lm.hu_bytes = bytes;
-                }
-                if (ctx->coarse16 && !L.hsu) TRY(dalloc(ctx, &Lm.hsu, sizeof(float) * (size_t)sys.g.Vc * 9));
+            if (!packed) {
                 coarse_pack_units(Lm.Hu, ctx->coarse16 ? Lm.hsu : nullptr, L.H64, L.nc, L.au_shape.ru, sys.g.Vc, ctx->coarse16,
                                   ctx->st);
                 CKL();
@@ -720,23 +748,29 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
     }
     int nw = 0, stages = 0;
     if (!onchip && std::is_same<T, float>::value && ctx->coarse16 && ctx->in_solve && tol > 0 && !iters &&
-        ctx->prm.coarse_kernel != 1 &&
+        ctx->prm.coarse_kernel != 1 && !ctx->panel_refused &&
         bcg_shape(L.nc, 8, sys.g.Vc / 2, &nw, &stages)) {
         // FP16 operator larger than the chip: the panel solver with one column of eight in
         // use, its operator tiles streaming ahead across the grid barriers (24^3x32, Nv =
         // 24: 249 -> 114 ms of coarse solves per solve against the
         // register-streaming kernel on D_c, 177 with that kernel red-black)
-        TRY(ensure_panel(ctx, ctx->pw1, 8, L.nc, sys.g.Vc));
         PanelWork& w = ctx->pw1;
+        int st = ensure_panel(ctx, w, 8, L.nc, sys.g.Vc);
         const long long n = (long long)sys.g.Vc * L.nc;
-        panel_column(w.rc, (const float2*)rc, n, w.npad, ctx->st);
-        CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
-        TRY(panel_solve(ctx, const_cast<CoarseLevel&>(L), sys.g, sys.nbr, sys.ord, w, 1, tol, maxit, (int*)(ctx->bar + 2),
-                        ctx->R.scal));
-        column_of_panel((float2*)y, w.y, n, w.npad, ctx->st);
-        CKL();
-        ctx->coarse_kernel_used = MG_CK_REGISTER;
-        return MG_OK;
+        if (st == MG_OK) {
+            panel_column(w.rc, (const float2*)rc, n, w.npad, ctx->st);
+            CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
+            st = panel_solve(ctx, const_cast<CoarseLevel&>(L), sys.g, sys.nbr, sys.ord, w, 1, tol, maxit,
+                             (int*)(ctx->bar + 2), ctx->R.scal);
+        }
+        if (st == MG_OK) {
+            column_of_panel((float2*)y, w.y, n, w.npad, ctx->st);
+            CKL();
+            ctx->coarse_kernel_used = MG_CK_REGISTER;
+        }
+        if (st != MG_ERR_OOM) return st;
+        ctx->panel_refused = true;   // no memory for its panels or tiles: the register-streaming kernel
+        ctx->err.clear();
     }
     if (!onchip) {
         // The preconditioner of a solve: CG on the red-black Schur complement, about
@@ -1088,6 +1122,7 @@ int build_level2(mg_ctx* ctx, CoarseLevel& L, const double2* V2, int nv2) {
     L.valid = true;
     L.at_valid = L.a16_valid = L.au_valid = false;
     L.h_state = 0;
+    ctx->panel_refused = false;
     return MG_OK;
 }
 

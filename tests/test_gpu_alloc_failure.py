@@ -89,3 +89,39 @@ def test_calls_after_a_refused_allocation(name):
             if wmg.mg_fail_allocation(mg.ctx, 0):
                 break   # fewer than nth allocations: every one has been refused once
     assert refused > 10
+
+
+# (precision, coarse_kernel, lattice, aggregates, nvec): the red-black form in global memory, its
+# FP16 copy, its units on chip with and without scales, and FP16 operators larger than the chip
+# (76 MB, even and odd coarse extents: panels and tiles of the batched kernel)
+FORMS = {"global_fp64": (wmg.MG_FP64, 0, L, B, 8), "global_fp32": (wmg.MG_FP32, 1, L, B, 8),
+         "global_fp16": (wmg.MG_FP16, 1, L, B, 8), "chip_fp32": (wmg.MG_FP32, 0, L, B, 8),
+         "chip_fp16": (wmg.MG_FP16, 4, L, B, 8), "panel_even": (wmg.MG_FP16, 0, (16, 16, 16, 8), (2, 2, 2, 2), 16),
+         "panel_odd": (wmg.MG_FP16, 0, (12, 16, 16, 10), (2, 2, 2, 2), 16)}
+
+
+@pytest.mark.parametrize("name", FORMS)
+def test_solve_without_memory_for_its_fast_forms(name):
+    """What a solve allocates beyond the V-cycle's buffers are faster forms of the coarse
+    solve: it does without those that are refused."""
+    prec, kernel, dims, block, nv = FORMS[name]
+    U, b = rough_gauge(dims, seed=8), synth.gaussian_spinor(dims, 98)
+    V0 = synth.gaussian_vectors(dims, nv, 97)
+    p = params(prec, coarse_kernel=kernel, nvec=nv)
+    for i in range(4):
+        p.block[i] = block[i]
+    nth, pending = 0, 0
+    while not pending:
+        nth += 1
+        assert nth < 50
+        with wmg.WilsonMG(dims, p) as mg:
+            mg.set_links(U)
+            mg.set_mass(MASS)
+            mg.set_null_vectors(V0)
+            mg.vcycle(b, prec)
+            wmg.mg_fail_allocation(mg.ctx, nth)
+            x, info = mg.solve(b)
+            pending = wmg.mg_fail_allocation(mg.ctx, 0)
+        assert info["status"] == wmg.MG_OK
+        assert np.linalg.norm(b - oracle.dslash(U, x, MASS, dims)) <= 2 * TOL * np.linalg.norm(b)
+    assert nth > 1
