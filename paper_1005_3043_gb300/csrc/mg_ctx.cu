@@ -56,7 +56,9 @@ struct CoarseLevel {
     int h_state = 0;          // 0 not built, 1 built, -1 not used (ensure_schur)
     bool h16_valid = false;
     int au_mode = 0;
-    CglsShape au_shape{};
+    CglsShape sh{};           // shape of the on-chip solver for (sh_nc, sh_h16, sh_mode), if sh_ok
+    int sh_nc = 0, sh_mode = 0;
+    bool sh_h16 = false, sh_ok = false;
     double mass = 0.0;
     bool valid = false;
 };
@@ -473,16 +475,20 @@ int cgls_mode(int coarse_kernel) {
                                                                                                     : CGLS_AUTO;
 }
 
-// The operator in the unit layout of the on-chip CGLS kernel; false when no
-// shape fits this device (the register-streaming kernel is used instead).
-int ensure_units(mg_ctx* ctx, CoarseLevel& L, int Vc, bool h16, int mode, bool* ok) {
-    *ok = false;
-    if (L.au_valid && L.au_h16 == h16 && L.au_mode == mode) {
-        *ok = true;
-        return MG_OK;
+// Shape of the on-chip CGLS kernel (L.sh); false when none fits this device (the
+// register-streaming kernel is used instead).
+bool unit_shape(CoarseLevel& L, int Vc, bool h16, int mode) {
+    if (L.sh_nc != L.nc || L.sh_h16 != h16 || L.sh_mode != mode) {
+        L.sh_ok = cgls_shape(L.nc, Vc, h16, mode, &L.sh);
+        L.sh_nc = L.nc;
+        L.sh_h16 = h16;
+        L.sh_mode = mode;
     }
-    CglsShape sh{};
-    if (!cgls_shape(L.nc, Vc, h16, mode, &sh)) return MG_OK;
+    return L.sh_ok;
+}
+// The operator in that kernel's unit layout, for the shape in L.sh.
+int ensure_units(mg_ctx* ctx, CoarseLevel& L, int Vc, bool h16, int mode) {
+    if (L.au_valid && L.au_h16 == h16 && L.au_mode == mode) return MG_OK;
     const size_t bytes = (size_t)Vc * 9 * L.nc * L.nc * (h16 ? 4 : 8);
     L.au_valid = false;
     if (L.au_bytes < bytes) {
@@ -491,13 +497,11 @@ int ensure_units(mg_ctx* ctx, CoarseLevel& L, int Vc, bool h16, int mode, bool* 
         L.au_bytes = bytes;
     }
     if (h16 && !L.su) TRY(dalloc(ctx, &L.su, sizeof(float) * (size_t)Vc * 9));
-    coarse_pack_units(L.Au, h16 ? L.su : nullptr, L.A64, L.nc, sh.ru, Vc, h16, ctx->st);
+    coarse_pack_units(L.Au, h16 ? L.su : nullptr, L.A64, L.nc, L.sh.ru, Vc, h16, ctx->st);
     CKL();
-    L.au_shape = sh;
     L.au_h16 = h16;
     L.au_mode = mode;
     L.au_valid = true;
-    *ok = true;
     return MG_OK;
 }
 
@@ -666,23 +670,19 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
     CgnrArgs<T> a = cgnr_args<T>(L, sys.g, rc, y, sys.cr, sys.cr1, sys.cs, sys.cp, sys.cp1, sys.cq, tol, maxit,
                                  ctx->R.partials, ctx->bar, ctx->R.scal);
     a.nbr = sys.nbr;
-    bool onchip = false;
-    if (std::is_same<T, float>::value && ctx->prm.coarse_kernel != 1) {
-        CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
-        const int mode = cgls_mode(ctx->prm.coarse_kernel);
-        TRY(ensure_units(ctx, Lm, sys.g.Vc, ctx->coarse16, mode, &onchip));
-    }
+    CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
+    const int mode = cgls_mode(ctx->prm.coarse_kernel);
+    const bool onchip = std::is_same<T, float>::value && ctx->prm.coarse_kernel != 1 &&
+                        unit_shape(Lm, sys.g.Vc, ctx->coarse16, mode);
     if (onchip) {
         CglsArgs c{};
-        c.Au = L.Au; c.su = ctx->coarse16 ? L.su : nullptr; c.nbr = sys.nbr;
+        c.nbr = sys.nbr;
         // the preconditioner of a solve runs red-black (see below)
         bool eo = false;
-        CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
-        if (ctx->in_solve && sys.ord && tol > 0 && !iters && ctx->prm.coarse_form == 0 && L.au_shape.tm == 1 &&
-            L.au_shape.nx_max <= 128)
+        if (ctx->in_solve && sys.ord && tol > 0 && !iters && ctx->prm.coarse_form == 0 && L.sh.tm == 1 &&
+            L.sh.nx_max <= 128)
             TRY(ensure_schur(ctx, Lm, sys.g, false, &eo));
         const int half = sys.g.Vc / 2;
-        const int mode = cgls_mode(ctx->prm.coarse_kernel);
         const bool packed = L.hu_valid && L.hu_h16 == ctx->coarse16 && L.hu_mode == mode;
         const size_t bytes = (size_t)sys.g.Vc * 9 * L.nc * L.nc * (ctx->coarse16 ? 4 : 8);
         if (eo && !packed) {
@@ -698,7 +698,7 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         }
         if (eo) {
             if (!packed) {
-                coarse_pack_units(Lm.Hu, ctx->coarse16 ? Lm.hsu : nullptr, L.H64, L.nc, L.au_shape.ru, sys.g.Vc, ctx->coarse16,
+                coarse_pack_units(Lm.Hu, ctx->coarse16 ? Lm.hsu : nullptr, L.H64, L.nc, L.sh.ru, sys.g.Vc, ctx->coarse16,
                                   ctx->st);
                 CKL();
                 Lm.hu_h16 = ctx->coarse16;
@@ -707,12 +707,16 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
             }
             c.Au = L.Hu;
             c.su = ctx->coarse16 ? L.hsu : nullptr;
+        } else {
+            TRY(ensure_units(ctx, Lm, sys.g.Vc, ctx->coarse16, mode));
+            c.Au = L.Au;
+            c.su = ctx->coarse16 ? L.su : nullptr;
         }
         c.rc = (const float2*)a.rc; c.y = (float2*)a.y; c.r = (float2*)a.r; c.r1 = (float2*)a.r1;
         c.s = (float2*)a.s; c.p = (float2*)a.p; c.p1 = (float2*)a.p1; c.q = (float2*)a.q;
         c.nc = L.nc; c.g = sys.g; c.tol2 = (float)(tol * tol); c.maxit = maxit;
         c.scal = ctx->R.scal; c.err = (int*)(ctx->bar + 2);
-        c.sh = L.au_shape;
+        c.sh = L.sh;
         const unsigned long long reserve = 2ull * (unsigned long long)(maxit > 0 ? maxit : 0) + 4ull;
         if ((unsigned long long)ctx->xch_epoch + reserve >= 0xFFFFFFFFull) {   // 32-bit epochs would wrap
             CK(cudaMemsetAsync(ctx->xch, 0, sizeof(unsigned long long) * kXchWords, ctx->st));
@@ -740,11 +744,6 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
                               -1.0, 1, 1, ctx->st);
         PROF_END(MG_K_COARSE_SOLVE);
         ctx->coarse_kernel_used = c.sh.tm == 2 ? MG_CK_TMEM_MMA : c.sh.tm ? MG_CK_TMEM : c.sh.resident ? MG_CK_SMEM : MG_CK_STREAM;
-    } else if (std::is_same<T, float>::value && ctx->coarse16) {
-        CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
-        TRY(ensure_a16(ctx, Lm, sys.g.Vc));
-        a.A16 = Lm.A16;
-        a.s16 = Lm.s16;
     }
     int nw = 0, stages = 0;
     if (!onchip && std::is_same<T, float>::value && ctx->coarse16 && ctx->in_solve && tol > 0 && !iters &&
@@ -760,7 +759,7 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         if (st == MG_OK) {
             panel_column(w.rc, (const float2*)rc, n, w.npad, ctx->st);
             CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
-            st = panel_solve(ctx, const_cast<CoarseLevel&>(L), sys.g, sys.nbr, sys.ord, w, 1, tol, maxit,
+            st = panel_solve(ctx, Lm, sys.g, sys.nbr, sys.ord, w, 1, tol, maxit,
                              (int*)(ctx->bar + 2), ctx->R.scal);
         }
         if (st == MG_OK) {
@@ -778,10 +777,10 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         // fixed iteration count means iterations on D_c itself, as the single-step
         // calls and the setup run them)
         bool eo = false;
-        CoarseLevel& Lm = const_cast<CoarseLevel&>(L);
         const bool h16 = std::is_same<T, float>::value && ctx->coarse16;
         if (ctx->in_solve && sys.ord && tol > 0)
             TRY(ensure_schur(ctx, Lm, sys.g, h16, &eo));
+        if (h16 && !eo) TRY(ensure_a16(ctx, Lm, sys.g.Vc));
         const int half = sys.g.Vc / 2;
         PROF_BEGIN(MG_K_COARSE_SOLVE);
         if (eo) {
@@ -792,6 +791,9 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
             a.A = H;
             if (h16) { a.A16 = L.H16; a.s16 = L.hs16; }
             a.rc = sys.eb; a.rc_full = rc; a.ord = sys.ord; a.t = sys.et;
+        } else if (h16) {
+            a.A16 = L.A16;
+            a.s16 = L.s16;
         }
         CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
         CK(cgnr_persistent<T>(a, ctx->st));
@@ -2405,9 +2407,8 @@ int mg_time_coarse_floor(mg_ctx* ctx, int rounds, double* us_stencils, double* u
     CoarseLevel& L = ctx->full;
     const CgSys<float> sys = level1_sys<float>(ctx);
     const int mode = cgls_mode(ctx->prm.coarse_kernel);
-    bool onchip = false;
-    TRY(ensure_units(ctx, L, sys.g.Vc, ctx->coarse16, mode, &onchip));
-    if (!onchip) return fail(ctx, MG_ERR_INVALID_ARG, "no on-chip shape for this coarse level");
+    if (!unit_shape(L, sys.g.Vc, ctx->coarse16, mode)) return fail(ctx, MG_ERR_INVALID_ARG, "no on-chip shape for this coarse level");
+    TRY(ensure_units(ctx, L, sys.g.Vc, ctx->coarse16, mode));
     double* outs[2] = {us_stencils, us_exchange};
     const int forms[2] = {CGLS_PROBE_STENCILS, CGLS_PROBE_EXCHANGE};
     for (int f = 0; f < 2; ++f) {
@@ -2417,7 +2418,7 @@ int mg_time_coarse_floor(mg_ctx* ctx, int rounds, double* us_stencils, double* u
         c.s = (float2*)sys.cs; c.p = (float2*)sys.cp; c.p1 = (float2*)sys.cp1; c.q = (float2*)sys.cq;
         c.nc = L.nc; c.g = sys.g; c.tol2 = 0.f; c.maxit = rounds;
         c.scal = ctx->scal_s; c.err = (int*)(ctx->bar + 2);
-        c.sh = L.au_shape;
+        c.sh = L.sh;
         const unsigned long long reserve = 2ull * (unsigned long long)rounds + 4ull;
         if ((unsigned long long)ctx->xch_epoch + reserve >= 0xFFFFFFFFull) {
             CK(cudaMemsetAsync(ctx->xch, 0, sizeof(unsigned long long) * kXchWords, ctx->st));
