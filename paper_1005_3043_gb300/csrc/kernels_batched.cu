@@ -45,24 +45,35 @@ namespace wmg {
 // ---------------------------------------------------------------- operator tiles
 // At[X][d][kc][rg][8][8]: core matrices (8 rows x 8 K, 128 bytes) of one K group
 // kc adjacent over the row groups rg; row a the real part of row a of A, row
-// nc + a the imaginary part.
-__global__ void k_coarse_tiles(__half* At, const double2* __restrict__ A, int nc, long long nblk) {
-    const long long total = nblk * nc * nc;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const long long blk = i / (nc * nc);
-        const int rem = (int)(i - blk * nc * nc), b = rem / nc, a = rem - b * nc;
-        const double2 v = A[i];   // column-major block: A[b][a] = A_ab
-        __half* t = At + blk * 2 * nc * nc + (size_t)(b >> 3) * (nc >> 2) * 64 + (b & 7);
+// nc + a the imaginary part.  The nine blocks of an aggregate add up in one
+// accumulator, so they share one scale: a power of two that brings the largest of
+// their entries to [2^14, 2^15), its inverse in as[X].  An entry keeps its 11 bits down
+// to 2^-28 of the largest, and none overflows.
+__global__ void __launch_bounds__(256) k_coarse_tiles(__half* At, float* as, const double2* __restrict__ A, int nc) {
+    __shared__ float s_max[8];
+    const int X = blockIdx.x, n = 9 * nc * nc;
+    const double2* Ax = A + (size_t)X * n;
+    float mx = 0.f;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) mx = fmaxf(mx, (float)fmax(fabs(Ax[i].x), fabs(Ax[i].y)));
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    for (int w = 0; w < 8; ++w) mx = fmaxf(mx, s_max[w]);
+    const int e = mx > 1e-30f && mx < 1e30f ? 14 - ilogbf(mx) : 0;
+    const double f = ldexp(1.0, e);
+    if (threadIdx.x == 0) as[X] = (float)ldexp(1.0, -e);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const int blk = i / (nc * nc), rem = i - blk * nc * nc, b = rem / nc, a = rem - b * nc;
+        const double2 v = Ax[i];   // column-major block: A[b][a] = A_ab
+        __half* t = At + ((size_t)X * 9 + blk) * 2 * nc * nc + (size_t)(b >> 3) * (nc >> 2) * 64 + (b & 7);
         const int m = nc + a;
-        t[((a >> 3) << 6) + ((a & 7) << 3)] = __double2half(v.x);
-        t[((m >> 3) << 6) + ((m & 7) << 3)] = __double2half(v.y);
+        t[((a >> 3) << 6) + ((a & 7) << 3)] = __double2half(f * v.x);
+        t[((m >> 3) << 6) + ((m & 7) << 3)] = __double2half(f * v.y);
     }
 }
-void coarse_tiles(__half* At, const double2* A, int nc, int Vc, cudaStream_t st) {
-    const long long total = (long long)Vc * 9 * nc * nc;
+void coarse_tiles(__half* At, float* as, const double2* A, int nc, int Vc, cudaStream_t st) {
     note_launch();
-    k_coarse_tiles<<<(int)std::min<long long>((total + 255) / 256, 32LL * device_sm_count()), 256, 0, st>>>(
-        At, A, nc, (long long)Vc * 9);
+    k_coarse_tiles<<<Vc, 256, 0, st>>>(At, as, A, nc);
 }
 
 // ---------------------------------------------------------------- the persistent kernel
@@ -473,8 +484,10 @@ struct BcgCta {
         if (t == 0) next_phase();
     }
 
-    // products of the next job into T; false on failure (uniform over the warps)
-    __device__ bool take(uint32_t tmem) {
+    // products of the next job (at site X) into T, in the operator's units; false on
+    // failure (uniform over the warps)
+    __device__ bool take(uint32_t tmem, int X) {
+        const float f = __ldg(a.as + X);
         const int buf = (int)(job_count & 1), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         const int quad = warp & 3, half = (warp - 4) >> 2, m = 32 * quad + lane;
         const bool ok = __all_sync(0xffffffffu, bcg_wait(acc_full + buf, (uint32_t)((job_count >> 1) & 1), fail, a.err));
@@ -491,8 +504,8 @@ struct BcgCta {
                 if (m < 2 * nc)
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
-                        T[(size_t)m * L.ts + c0 + e] = make_float2(__uint_as_float(rh[e]) + __uint_as_float(rl[e]),
-                                                                   __uint_as_float(ih[e]) + __uint_as_float(il[e]));
+                        T[(size_t)m * L.ts + c0 + e] = make_float2(f * (__uint_as_float(rh[e]) + __uint_as_float(rl[e])),
+                                                                   f * (__uint_as_float(ih[e]) + __uint_as_float(il[e])));
             }
         }
         tc_fence_before();
@@ -577,7 +590,7 @@ struct BcgCta {
             if (!grid_barrier(true)) return;
             for (int j = 0; j < jobs; ++j) {
                 const int X = (j0 + j) / nch, c = j0 + j - X * nch;
-                if (!take(tmem)) return;
+                if (!take(tmem, X)) return;
                 if (act)
                     for (int r = rg; r < nc; r += rgs)
                         a.y[((size_t)X * nc + r) * np + c * nw + n] = product(r, 1.f, a.dag != 0);
@@ -643,7 +656,7 @@ struct BcgCta {
             if (!eo) return true;
             for (int j = 0; j < jobs; ++j) {
                 const int X = site(phase, j0 + j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem)) return false;
+                if (!take(tmem, X)) return false;
                 if (act)
                     for (int r = rg; r < nc; r += rgs) stage(r, product(r, inv[col], false), sc[col], false);
                 epi_sync();
@@ -682,7 +695,7 @@ struct BcgCta {
         if (!odd_half(a.btu, isu, sc_u)) return;
         for (int j = 0; j < jobs; ++j) {
             const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-            if (!take(tmem)) return;
+            if (!take(tmem, X)) return;
             if (act) {
                 float s = 0.f;
                 const float inv = isu[col], sc = sc_s[col];
@@ -704,7 +717,7 @@ struct BcgCta {
             if (!odd_half(a.bts, iss, sc_s)) return;
             for (int j = 0; j < jobs; ++j) {
                 const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem)) return;
+                if (!take(tmem, X)) return;
                 if (act) {
                     float s = 0.f;
                     const float inv = iss[col], sc = sc_u[col];
@@ -769,12 +782,12 @@ struct BcgCta {
                 if (!odd_half(a.btu, isu, sc_tu)) return;
             } else if (eo) {   // the odd half that was started; its even half never is
                 for (int j = 0; j < jobs; ++j)
-                    if (!take(tmem)) return;
+                    if (!take(tmem, site(phase, j0 + j))) return;
                 break;
             }
             for (int j = 0; j < jobs; ++j) {
                 const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem)) return;
+                if (!take(tmem, X)) return;
                 if (!running) continue;   // nothing left to do but to take what was started
                 if (act) {
                     float sg = 0.f, sr = 0.f;

@@ -33,6 +33,7 @@ struct CoarseLevel {
     double2* A64 = nullptr;   // [X][9][nc][nc] column-major blocks
     float2* A32 = nullptr;
     __half* At = nullptr;     // FP16 tensor-core tiles of A64 (batched path), built on demand
+    float* as = nullptr;      // and their scales [X]
     bool at_valid = false;
     __half2* A16 = nullptr;   // FP16 copy with per-block scales s16 (FP16-storage mode), built on demand
     float* s16 = nullptr;
@@ -45,7 +46,8 @@ struct CoarseLevel {
     float2* H32 = nullptr;
     __half2* H16 = nullptr;   // its FP16 copy and block scales
     float* hs16 = nullptr;
-    __half* Ht = nullptr;     // its FP16 tensor-core tiles (batched path)
+    __half* Ht = nullptr;     // its FP16 tensor-core tiles (batched path) and their scales
+    float* hts = nullptr;
     bool ht_valid = false;
     void* Hu = nullptr;       // its CGLS units, as Au
     float* hsu = nullptr;
@@ -555,8 +557,10 @@ constexpr float kSchurGrowth = 64.f;
 int without_schur(mg_ctx* ctx, CoarseLevel& L, int st, bool* ok) {
     if (st != MG_ERR_OOM) return st;
     CK(cudaStreamSynchronize(ctx->st));
-    for (void* q : {(void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16, (void*)L.Ht, L.Hu, (void*)L.hsu}) dfree(ctx, q);
-    L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr; L.Ht = nullptr; L.Hu = nullptr; L.hsu = nullptr;
+    for (void* q : {(void*)L.H64, (void*)L.H32, (void*)L.H16, (void*)L.hs16, (void*)L.Ht, (void*)L.hts, L.Hu, (void*)L.hsu})
+        dfree(ctx, q);
+    L.H64 = nullptr; L.H32 = nullptr; L.H16 = nullptr; L.hs16 = nullptr; L.Ht = nullptr; L.hts = nullptr;
+    L.Hu = nullptr; L.hsu = nullptr;
     L.h_blocks = L.hu_bytes = 0;
     L.h16_valid = L.ht_valid = L.hu_valid = false;
     L.h_state = -1;
@@ -604,8 +608,8 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool h16, bool* ok)
 int ensure_tiles(mg_ctx* ctx, CoarseLevel& L, int Vc) {
     if (L.at_valid) return MG_OK;
     const size_t nc = (size_t)2 * L.cap;
-    if (!L.At) TRY(dalloc(ctx, &L.At, sizeof(__half) * (size_t)Vc * 9 * 2 * nc * nc));
-    coarse_tiles(L.At, L.A64, L.nc, Vc, ctx->st);
+    if (!L.At) TRY(dalloc_all(ctx, {{&L.At, sizeof(__half) * (size_t)Vc * 9 * 2 * nc * nc}, {&L.as, sizeof(float) * Vc}}));
+    coarse_tiles(L.At, L.as, L.A64, L.nc, Vc, ctx->st);
     CKL();
     L.at_valid = true;
     return MG_OK;
@@ -641,16 +645,18 @@ int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, cons
     bool eo = false;
     if (ord && tol > 0) TRY(ensure_schur(ctx, L, g, false, &eo));
     if (eo && !L.Ht) {
-        const int st = dalloc(ctx, &L.Ht, sizeof(__half) * L.h_blocks * 2 * (2 * (size_t)L.cap) * (2 * (size_t)L.cap));
+        const int st = dalloc_all(ctx, {{&L.Ht, sizeof(__half) * L.h_blocks * 2 * (2 * (size_t)L.cap) * (2 * (size_t)L.cap)},
+                                        {&L.hts, sizeof(float) * g.Vc}});
         if (st != MG_OK) TRY(without_schur(ctx, L, st, &eo));
     }
     if (!eo) {
         TRY(ensure_tiles(ctx, L, g.Vc));
     } else if (!L.ht_valid) {
-        coarse_tiles(L.Ht, L.H64, L.nc, g.Vc, ctx->st);
+        coarse_tiles(L.Ht, L.hts, L.H64, L.nc, g.Vc, ctx->st);
         L.ht_valid = true;
     }
     c.At = eo ? L.Ht : L.At;
+    c.as = eo ? L.hts : L.as;
     PROF_BEGIN(MG_K_COARSE_SOLVE);
     if (eo) {
         schur_rows<float>(w.e, nullptr, L.H32, w.rc, ord + half, half, nbr, L.nc, 0, 1, 1.0, nrhs, w.npad, ctx->st);
@@ -3197,7 +3203,7 @@ int bcg_apply_args(mg_ctx* ctx, int npad, int nrhs, bool dag, BcgArgs* out, std:
     TRY(get(&fl, sizeof(int) * 4));
     CK(cudaMemsetAsync(fl, 0, sizeof(int) * 4, ctx->st));
     TRY(ensure_tiles(ctx, L, ctx->g.Vc));
-    a.At = L.At; a.rc = x; a.nbr = ctx->cnbr; a.err = fl;
+    a.At = L.At; a.as = L.as; a.rc = x; a.nbr = ctx->cnbr; a.err = fl;
     a.nc = L.nc; a.npad = npad; a.nrhs = nrhs; a.mode = BCG_APPLY; a.dag = dag ? 1 : 0; a.g = ctx->g;
     *out = a;
     return MG_OK;

@@ -358,8 +358,9 @@ void coarse_pack16(__half2* A16, float* s16, const double2* A, int nc, int Vc, c
 
 // ---------------------------------------------------------------- batched (multi-RHS) coarse level
 // Panel layout xB[X][b][n], n < npad (multiple of 16), complex FP32.
-// At: per (X, d) the FP16 rows [Re A; Im A] of A[X][d] in tensor-core tiles (2 nc^2 halves each)
-void coarse_tiles(__half* At, const double2* A, int nc, int Vc, cudaStream_t st);
+// At: per (X, d) the FP16 rows [Re A; Im A] of A[X][d] in tensor-core tiles (2 nc^2 halves
+// each), times 1 / as[X], a power of two
+void coarse_tiles(__half* At, float* as, const double2* A, int nc, int Vc, cudaStream_t st);
 // SIMT reference of the same contraction with the FP64 operator
 template <typename T>
 void coarse_apply_batched_simt(v2<T>* y, const double2* A, const v2<T>* x, int nc, int npad, bool dag, const Geom& g,
@@ -370,6 +371,7 @@ void coarse_apply_batched_simt(v2<T>* y, const double2* A, const v2<T>* x, int n
 enum { BCG_SOLVE = 0, BCG_APPLY = 1 };
 struct BcgArgs {
     const __half* At;
+    const float* as;         // scales of the operator's tiles per site
     __half *bts, *btu;       // operand tiles, bcg_tile_bytes each
     const float2* rc;        // panels [Vc][nc][npad]
     float2 *y, *r, *s, *u, *p, *z, *q;   // BCG_APPLY: y only
