@@ -7,7 +7,8 @@
 //   y[X][a][n] = sum_d sum_b A[X][d][a][b] x[X+d][b][n].
 // As a real GEMM the rows are the real parts of A followed by the imaginary
 // parts (M = 2 nc <= 96 of the MMA's 128), K = b, and a right-hand side is four
-// columns: Re x and Im x, each split into FP16 hi + lo (x = hi + lo to ~22 bits):
+// columns: Re x and Im x, each split into FP16 hi + 2^-11 lo (22 bits; lo is kept times
+// 2^11, so that it is a normal number wherever hi is):
 //   D[a] = Re A x, D[nc + a] = Im A x,
 //   Re y = D[a][Re] - D[nc + a][Im],  Im y = D[a][Im] + D[nc + a][Re].
 // So neither the operator nor the operand is stored twice (the embedding
@@ -191,11 +192,11 @@ __device__ __forceinline__ void add2(Sum2& s, float x) {
     s.l += (s.h - (t - b)) + (x - b);
     s.h = t;
 }
-// power of two near sqrt(rows / s): entries of a column with |x|^2 = s then have
-// rms about 1, far above the FP16 subnormal range, with room for a column
-// concentrated on one site
+// power of two near 2^-5 sqrt(rows / s): entries of a column with |x|^2 = s then have
+// rms about 2^-5, 2^9 above the FP16 subnormal range, with room for a column
+// concentrated on one site that grows some 10^3 times from one scale to the next
 __device__ __forceinline__ float col_scale(double s, float rows) {
-    const float x = rows / (float)s;
+    const float x = 0x1p-10f * rows / (float)s;
     if (!(x > 1e-38f) || !(x < 1e38f)) return 1.f;
     return __int_as_float((127 + ((((__float_as_int(x) >> 23) & 255) - 127) >> 1)) << 23);
 }
@@ -417,9 +418,12 @@ struct BcgCta {
     long long job_count = 0;
     unsigned int arrived = 0, opened = 0;
 
-    // entries staged in S2[row][n] (scaled) -> the four FP16 rows of the tile
+    // entries staged in S2[row][n] (scaled) -> the four FP16 rows of the tile.  A single
+    // right-hand side (a.third): what its hi and lo leave, times 2^22, goes into the hi
+    // rows of the unused column 1, so that its operand has the 24 bits of an FP32 number.
     __device__ void write_tile(__half* bt, int X, int c) {
         __half* base = bt + ((size_t)X * nch + c) * 4 * nc * nw;
+        const bool third = a.third && c == 0;
         for (int i = t; i < (nc >> 3) * nw; i += kEpi) {
             const int kc = i / nw, m = i - kc * nw;
             uint32_t w[4][4];
@@ -429,16 +433,23 @@ struct BcgCta {
                 float hr[2], hi[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    v[q] = S2[(kc * 8 + 2 * e + q) * L.ts + m];
+                    v[q] = S2[(kc * 8 + 2 * e + q) * L.ts + (third && m == 1 ? 0 : m)];
                     v[q].x = fminf(fmaxf(v[q].x, -65504.f), 65504.f);
                     v[q].y = fminf(fmaxf(v[q].y, -65504.f), 65504.f);
                     hr[q] = __half2float(__float2half_rn(v[q].x));
                     hi[q] = __half2float(__float2half_rn(v[q].y));
+                    v[q].x = 0x1p11f * (v[q].x - hr[q]);
+                    v[q].y = 0x1p11f * (v[q].y - hi[q]);
+                    if (third && m == 1) {
+                        hr[q] = 0x1p11f * (v[q].x - __half2float(__float2half_rn(v[q].x)));
+                        hi[q] = 0x1p11f * (v[q].y - __half2float(__float2half_rn(v[q].y)));
+                        v[q] = make_float2(0.f, 0.f);
+                    }
                 }
                 w[0][e] = half_pair(hr[0], hr[1]);
                 w[1][e] = half_pair(hi[0], hi[1]);
-                w[2][e] = half_pair(v[0].x - hr[0], v[1].x - hr[1]);
-                w[3][e] = half_pair(v[0].y - hi[0], v[1].y - hi[1]);
+                w[2][e] = half_pair(v[0].x, v[1].x);
+                w[3][e] = half_pair(v[0].y, v[1].y);
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -486,7 +497,7 @@ struct BcgCta {
 
     // products of the next job (at site X) into T, in the operator's units; false on
     // failure (uniform over the warps)
-    __device__ bool take(uint32_t tmem, int X) {
+    __device__ bool take(uint32_t tmem, int X, int c) {
         const float f = __ldg(a.as + X);
         const int buf = (int)(job_count & 1), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         const int quad = warp & 3, half = (warp - 4) >> 2, m = 32 * quad + lane;
@@ -501,11 +512,17 @@ struct BcgCta {
                 tmem_ld8(base + 2 * nw + c0, rl);
                 tmem_ld8(base + 3 * nw + c0, il);
                 tmem_wait_ld8(rh, ih, rl, il);
+                if (a.third && c == 0 && c0 == 0) {
+                    rl[0] = __float_as_uint(__uint_as_float(rl[0]) + 0x1p-11f * __uint_as_float(rh[1]));
+                    il[0] = __float_as_uint(__uint_as_float(il[0]) + 0x1p-11f * __uint_as_float(ih[1]));
+                    rh[1] = ih[1] = 0u;
+                }
                 if (m < 2 * nc)
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
-                        T[(size_t)m * L.ts + c0 + e] = make_float2(f * (__uint_as_float(rh[e]) + __uint_as_float(rl[e])),
-                                                                   f * (__uint_as_float(ih[e]) + __uint_as_float(il[e])));
+                        T[(size_t)m * L.ts + c0 + e] =
+                            make_float2(f * (__uint_as_float(rh[e]) + 0x1p-11f * __uint_as_float(rl[e])),
+                                        f * (__uint_as_float(ih[e]) + 0x1p-11f * __uint_as_float(il[e])));
             }
         }
         tc_fence_before();
@@ -590,7 +607,7 @@ struct BcgCta {
             if (!grid_barrier(true)) return;
             for (int j = 0; j < jobs; ++j) {
                 const int X = (j0 + j) / nch, c = j0 + j - X * nch;
-                if (!take(tmem, X)) return;
+                if (!take(tmem, X, c)) return;
                 if (act)
                     for (int r = rg; r < nc; r += rgs)
                         a.y[((size_t)X * nc + r) * np + c * nw + n] = product(r, 1.f, a.dag != 0);
@@ -656,7 +673,7 @@ struct BcgCta {
             if (!eo) return true;
             for (int j = 0; j < jobs; ++j) {
                 const int X = site(phase, j0 + j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem, X)) return false;
+                if (!take(tmem, X, c)) return false;
                 if (act)
                     for (int r = rg; r < nc; r += rgs) stage(r, product(r, inv[col], false), sc[col], false);
                 epi_sync();
@@ -695,7 +712,7 @@ struct BcgCta {
         if (!odd_half(a.btu, isu, sc_u)) return;
         for (int j = 0; j < jobs; ++j) {
             const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-            if (!take(tmem, X)) return;
+            if (!take(tmem, X, c)) return;
             if (act) {
                 float s = 0.f;
                 const float inv = isu[col], sc = sc_s[col];
@@ -717,7 +734,7 @@ struct BcgCta {
             if (!odd_half(a.bts, iss, sc_s)) return;
             for (int j = 0; j < jobs; ++j) {
                 const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem, X)) return;
+                if (!take(tmem, X, c)) return;
                 if (act) {
                     float s = 0.f;
                     const float inv = iss[col], sc = sc_u[col];
@@ -782,12 +799,12 @@ struct BcgCta {
                 if (!odd_half(a.btu, isu, sc_tu)) return;
             } else if (eo) {   // the odd half that was started; its even half never is
                 for (int j = 0; j < jobs; ++j)
-                    if (!take(tmem, site(phase, j0 + j))) return;
+                    if (!take(tmem, site(phase, j0 + j), (j0 + j) % nch)) return;
                 break;
             }
             for (int j = 0; j < jobs; ++j) {
                 const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem, X)) return;
+                if (!take(tmem, X, c)) return;
                 if (!running) continue;   // nothing left to do but to take what was started
                 if (act) {
                     float sg = 0.f, sr = 0.f;
@@ -940,6 +957,7 @@ cudaError_t bcg_launch(const BcgArgs& args, cudaStream_t st) {
     if (!bcg_shape(a.nc, a.npad, a.ord ? a.g.Vc / 2 : a.g.Vc, &a.nw, &a.stages)) return cudaErrorInvalidValue;
     a.first_dag = a.mode == BCG_APPLY ? a.dag : 1;   // the CG starts with s = D_c^dag r
     if (!a.rc_full) a.rc_full = a.rc;
+    a.third = a.nrhs == 1;
     const int sms = device_sm_count();
     const long long jobs = (long long)(a.ord ? a.g.Vc / 2 : a.g.Vc) * (a.npad / a.nw);
     const int grid = (int)std::min<long long>(jobs, sms);

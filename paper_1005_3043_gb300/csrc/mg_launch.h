@@ -391,6 +391,7 @@ struct BcgArgs {
     double tol2;
     Geom g;
     int nw, stages, first_dag;   // columns per job, pipeline depth, first operand (set by the launcher)
+    int third;               // one right-hand side: third part of its operand in column 1 (set by the launcher)
     uint32_t tmem_cols;      // (set by the launcher)
 };
 inline size_t bcg_sync_bytes(int npad) { return 16 + (size_t)npad * (4 + 2 * 3 * 8); }

@@ -38,3 +38,41 @@ def test_operator_of_any_size(size, m0, dagger):
         y, ref = (mg.coarse_batched(x, dagger=dagger, impl=i) for i in (0, 1))
     for i in range(nrhs):
         assert np.linalg.norm(y[i] - ref[i]) <= 2.0 ** -11 * np.linalg.norm(ref[i]), i
+
+
+def exact_context(L, mass, **kw):
+    """D_c with entries that FP16 holds exactly: unit links, prototypes constant on each
+    spin-colour component (P = 1/4 on 2^4 aggregates), a dyadic mass.  On an extent that is
+    even a column of D_c then has entries on the site itself and its neighbours only."""
+    V = np.zeros((4, int(np.prod(L)), 4, 3), complex)
+    for i in range(4):
+        V[i, :, i // 3, i % 3] = V[i, :, 2 + i // 3, i % 3] = 1.0
+    return context(L, (2, 2, 2, 2), 4, synth.unit_gauge(L), mass, V, **kw)
+
+
+@pytest.mark.parametrize("nrhs,bits", [(1, 23), (3, 21)])
+def test_operand_keeps_its_bits(nrhs, bits):
+    """Columns of one entry per neighbourhood, so that an entry of y is one product (twice
+    the same entry where two neighbours are one site): y / A is the operand as the kernel
+    holds it.  FP32 for a single right-hand side, 22 bits in a batch, rounded to nearest and
+    the product once more, for entries down to 2^-12 of the largest."""
+    with exact_context((8, 8, 8, 16), -0.5) as mg:
+        A = mg.coarse_op()
+        assert np.array_equal(A, A.real.astype(np.float16) + 1j * A.imag.astype(np.float16).astype(float))
+        rng = np.random.default_rng(3)
+        X = np.arange(mg.Vc)
+        t = X // 64
+        x = np.zeros((nrhs, mg.Vc, mg.nc), complex)
+        x[:, 0, 0] = 1.0
+        far = np.flatnonzero((X % 64 == 42) & (t == 4))[0]   # (2, 2, 2, 4), four and more hops from 0
+        for k in range(13):
+            for i in range(nrhs):
+                v = rng.uniform(1, 2, 2).astype(np.float32).astype(float)
+                x[i, far, 5] = 2.0 ** -k * (v[0] + 1j * v[1]) / 2
+            y, ref = (mg.coarse_batched(x, impl=q) for q in (0, 1))
+            for i in range(nrhs):
+                z = np.abs(ref[i, far]) > 0
+                assert z.any()
+                for part in (np.real, np.imag):
+                    p, q = part(y[i, far][z]), part(ref[i, far][z])
+                    assert np.all(np.abs(p - q) <= 2.0 ** -bits * np.abs(q)), (k, i)
