@@ -546,9 +546,9 @@ struct BcgCta {
     // sum in any order, so a CTA adds its share with one atomic per value and reads the
     // sums after the grid barrier.  (Every CTA adding up all CTAs' partial sums in a
     // fixed order took 5-7 us per iteration at 152 x 48 values.)  The unit of a value
-    // is 2^-36 of its last grid sum (fx; 2^-42 of |r|^2 before the first), so a sum
-    // keeps more bits than its FP32 terms have; a value out of range (it grew 2^19
-    // times in one iteration, or is not finite) ends its column.
+    // is 2^-36 of its last grid sum, at first of the largest CTA's share (publish_size),
+    // so a sum keeps more bits than its FP32 terms have; a value out of range (it grew
+    // 2^19 times in one iteration, or is not finite) marks its column, which ends there.
     __device__ void publish(const float* fx, unsigned long long* sums) {
         epi_sync();
         for (int i = t; i < 3 * a.npad; i += kEpi) {
@@ -561,8 +561,26 @@ struct BcgCta {
                 e = Sum2{0.f, 0.f};
             }
             const float h = s.h * fx[i], l = s.l * fx[i];
-            const long long q = fabsf(h) < 0x1p55f ? __float2ll_rn(h) + __float2ll_rn(l) : -(1LL << 54);
+            if (!(fabsf(h) < 0x1p55f)) {
+                atomicOr(a.bad + c, 1u);
+                continue;
+            }
+            const long long q = __float2ll_rn(h) + __float2ll_rn(l);
             if (q != 0) atomicAdd(sums + i, (unsigned long long)q);
+        }
+    }
+    // The largest CTA's share of a value's column sums into mx (float bits order as
+    // integers; fabs: one sign for every NaN).
+    __device__ void publish_size(int val, unsigned int* mx, bool clear) {
+        epi_sync();
+        for (int i = t; i < a.npad; i += kEpi) {
+            float s = 0.f;
+            for (int g = 0; g < rgs; ++g) {
+                Sum2& e = acc[((size_t)val * rgs + g) * a.npad + i];
+                s += e.h;
+                if (clear) e = Sum2{0.f, 0.f};
+            }
+            atomicMax(mx + i, __float_as_uint(fabsf(s)));
         }
     }
 
@@ -632,8 +650,7 @@ struct BcgCta {
             }
             return q;
         };
-        // the size of that right-hand side per column: the largest CTA's share of its
-        // norm (float bits order as integers)
+        // the size of that right-hand side per column: the largest CTA's share of its norm
         if (act)
             for (int j = 0; j < jobs; ++j) {
                 const int col = (j0 + j) % nch * nw + n;
@@ -641,16 +658,7 @@ struct BcgCta {
                 for (int r = rg; r < nc; r += rgs) s += full2(j, r, col);
                 add2(col_acc(0, col), s);
             }
-        epi_sync();
-        for (int i = t; i < np; i += kEpi) {
-            float s = 0.f;
-            for (int g = 0; g < rgs; ++g) {
-                Sum2& e = acc[(size_t)g * np + i];
-                s += e.h;
-                e = Sum2{0.f, 0.f};
-            }
-            atomicMax(a.mx + i, __float_as_uint(fabsf(s)));   // fabs: one sign for every NaN
-        }
+        publish_size(0, a.mx, true);
         if (!grid_barrier(false)) return;
         for (int i = t; i < np; i += kEpi) {
             const unsigned int m = __ldcg(a.mx + i);
@@ -728,6 +736,7 @@ struct BcgCta {
             write_tile(a.bts, X, c);
         }
         ++phase;
+        publish_size(1, a.mx + np, false);
         for (int it = 0;; ++it) {
             if (!grid_barrier(true)) return;
             // phase A: u = D_c s, its tile and norm
@@ -750,6 +759,16 @@ struct BcgCta {
                 write_tile(a.btu, X, c);
             }
             ++phase;
+            if (it == 0) {
+                // units of the first sums: |D^dag r|^2 and |D D^dag r|^2 of a right-hand side of
+                // low modes are many orders of magnitude below |r|^2
+                publish_size(0, a.mx + 2 * np, false);
+                if (!grid_barrier(false)) return;
+                for (int i = t; i < np; i += kEpi) {
+                    fx[i] = unit_of(__uint_as_float(__ldcg(a.mx + 2 * np + i)));
+                    fx[np + i] = unit_of(__uint_as_float(__ldcg(a.mx + np + i)));
+                }
+            }
             unsigned long long* sums = a.sums + (size_t)(it & 1) * 3 * np;
             publish(fx, sums);
             if (!grid_barrier(true)) return;
@@ -777,7 +796,7 @@ struct BcgCta {
                     } else {
                         rho0[i] = rho;
                     }
-                    if ((it > 0 && rho <= a.tol2 * rho0[i]) || it >= a.maxit || !(gamma > 0) || !(den > 0)) {
+                    if (__ldcg(a.bad + i) || (it > 0 && rho <= a.tol2 * rho0[i]) || it >= a.maxit || !(gamma > 0) || !(den > 0)) {
                         done[i] = 1;
                         al[i] = be[i] = 0.f;
                     } else {
@@ -953,7 +972,8 @@ size_t bcg_tile_bytes(int nc, int npad, long long Vc) { return (size_t)Vc * 4 * 
 cudaError_t bcg_launch(const BcgArgs& args, cudaStream_t st) {
     BcgArgs a = args;
     a.mx = a.bar + 4;
-    a.sums = reinterpret_cast<unsigned long long*>(a.bar + 4 + a.npad);
+    a.sums = reinterpret_cast<unsigned long long*>(a.bar + 4 + 3 * a.npad);
+    a.bad = reinterpret_cast<unsigned int*>(a.sums + 6 * (size_t)a.npad);
     if (!bcg_shape(a.nc, a.npad, a.ord ? a.g.Vc / 2 : a.g.Vc, &a.nw, &a.stages)) return cudaErrorInvalidValue;
     a.first_dag = a.mode == BCG_APPLY ? a.dag : 1;   // the CG starts with s = D_c^dag r
     if (!a.rc_full) a.rc_full = a.rc;

@@ -378,8 +378,9 @@ struct BcgArgs {
     const int* nbr;          // coarse neighbour table [Vc][9]
     unsigned int* bar;       // bcg_sync_bytes(npad), 8-byte aligned, cleared by the launcher: grid barrier
                              // counter, then (set by the launcher)
-    unsigned int* mx;        // [npad] sizes of the right-hand sides and
-    unsigned long long* sums;   // [2][3][npad] fixed-point grid sums
+    unsigned int* mx;        // [3][npad] sizes of the right-hand sides, of s and of u,
+    unsigned long long* sums;   // [2][3][npad] fixed-point grid sums and
+    unsigned int* bad;       // [npad] columns with a sum out of range
     int* err;                // set to 1 if a bounded wait gave up
     double* iters;           // [npad] CG iterations (BCG_SOLVE)
     double* scal;            // optional: solver scalars that receive column 0's iterations
@@ -394,7 +395,7 @@ struct BcgArgs {
     int third;               // one right-hand side: third part of its operand in column 1 (set by the launcher)
     uint32_t tmem_cols;      // (set by the launcher)
 };
-inline size_t bcg_sync_bytes(int npad) { return 16 + (size_t)npad * (4 + 2 * 3 * 8); }
+inline size_t bcg_sync_bytes(int npad) { return 16 + (size_t)npad * (3 * 4 + 2 * 3 * 8 + 4); }
 bool bcg_shape(int nc, int npad, int Vc, int* nw, int* stages);   // false: no shape for this panel
 size_t bcg_tile_bytes(int nc, int npad, long long Vc);
 cudaError_t bcg_launch(const BcgArgs& args, cudaStream_t st);

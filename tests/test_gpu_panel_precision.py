@@ -76,3 +76,24 @@ def test_operand_keeps_its_bits(nrhs, bits):
                 for part in (np.real, np.imag):
                     p, q = part(y[i, far][z]), part(ref[i, far][z])
                     assert np.all(np.abs(p - q) <= 2.0 ** -bits * np.abs(q)), (k, i)
+
+
+@pytest.mark.parametrize("prec,nrhs", [(wmg.MG_FP32, 1), (wmg.MG_FP32, 5), (wmg.MG_FP16, 3)])
+def test_sums_of_a_low_mode(prec, nrhs):
+    """The constant mode of the free periodic operator: D_c v = m v exactly, so the CG on
+    D_c^dag D_c solves it in one iteration with alpha = |s|^2 / |u|^2 = m^-2 to a few times
+    2^-24.  |u|^2 is 2^-40 of |r|^2; alpha off by more than the tolerance, 10^-3, takes a
+    second iteration.  81 aggregates (no red-black form)."""
+    L = (12, 12, 12, 12)
+    rng = np.random.default_rng(5)
+    V = np.zeros((4, 12 ** 4, 4, 3), complex)
+    for i in range(4):
+        V[i, :, i // 3, i % 3] = V[i, :, 2 + i // 3, i % 3] = 1.0
+    c = rng.standard_normal((nrhs, 4, 2)) @ np.array([1, 1j])
+    b = np.einsum("ni,ivsc->nvsc", c, V)
+    with context(L, (4, 4, 4, 4), 4, synth.unit_gauge(L), 2.0 ** -10, V, t_antiperiodic=0, prec_inner=prec,
+                 coarse_tol=1e-3, max_outer=1) as mg:
+        A = mg.coarse_op()
+        assert np.array_equal(A, A.real.astype(np.float16) + 1j * A.imag.astype(np.float16).astype(float))
+        infos = mg.solve_batched(b)[1]
+    assert [i["coarse_iters"] for i in infos] == [1] * nrhs
