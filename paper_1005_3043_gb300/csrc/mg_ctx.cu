@@ -33,8 +33,8 @@ struct CoarseLevel {
     double2* A64 = nullptr;   // [X][9][nc][nc] column-major blocks
     float2* A32 = nullptr;
     __half* At = nullptr;     // FP16 tensor-core tiles of A64 (batched path), built on demand
-    float* as = nullptr;      // and their scales [X]
-    bool at_valid = false;
+    float* as = nullptr;      // and their scales [X] (coarse_tiles)
+    bool at_valid = false, at_top = false;
     __half2* A16 = nullptr;   // FP16 copy with per-block scales s16 (FP16-storage mode), built on demand
     float* s16 = nullptr;
     bool a16_valid = false;
@@ -48,7 +48,7 @@ struct CoarseLevel {
     float* hs16 = nullptr;
     __half* Ht = nullptr;     // its FP16 tensor-core tiles (batched path) and their scales
     float* hts = nullptr;
-    bool ht_valid = false;
+    bool ht_valid = false, ht_top = false;
     void* Hu = nullptr;       // its CGLS units, as Au
     float* hsu = nullptr;
     size_t hu_bytes = 0;
@@ -605,13 +605,14 @@ int ensure_schur(mg_ctx* ctx, CoarseLevel& L, const Geom& g, bool h16, bool* ok)
 }
 
 // ---------------------------------------------------------------- coarse solve of a panel
-int ensure_tiles(mg_ctx* ctx, CoarseLevel& L, int Vc) {
-    if (L.at_valid) return MG_OK;
+int ensure_tiles(mg_ctx* ctx, CoarseLevel& L, int Vc, bool top) {
+    if (L.at_valid && L.at_top == top) return MG_OK;
     const size_t nc = (size_t)2 * L.cap;
     if (!L.At) TRY(dalloc_all(ctx, {{&L.At, sizeof(__half) * (size_t)Vc * 9 * 2 * nc * nc}, {&L.as, sizeof(float) * Vc}}));
-    coarse_tiles(L.At, L.as, L.A64, L.nc, Vc, ctx->st);
+    coarse_tiles(L.At, L.as, L.A64, L.nc, Vc, top, ctx->st);
     CKL();
     L.at_valid = true;
+    L.at_top = top;
     return MG_OK;
 }
 int ensure_panel(mg_ctx* ctx, PanelWork& w, int npad, int nc, int Vc) {
@@ -632,9 +633,10 @@ int ensure_panel(mg_ctx* ctx, PanelWork& w, int npad, int nc, int Vc) {
 // CG on the normal equations of the level's operator for nrhs columns of the panel
 // w.rc -> w.y, red-black where the lattice allows it (see coarse_solve).  *err is
 // raised on a timed-out wait; scal (optional) receives column 0's iterations.
-// MG_ERR_OOM before anything is launched.
+// top: the scales of the operator's tiles (coarse_tiles; a batch keeps powers of two, so
+// that its operator is D_c rounded to FP16).  MG_ERR_OOM before anything is launched.
 int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, const int* ord, PanelWork& w, int nrhs,
-                double tol, int maxit, int* err, double* scal) {
+                bool top, double tol, int maxit, int* err, double* scal) {
     BcgArgs c{};
     c.bts = w.bts; c.btu = w.btu; c.rc = w.rc;
     c.y = w.y; c.r = w.r; c.s = w.s; c.u = w.u; c.p = w.p; c.z = w.z; c.q = w.q;
@@ -650,10 +652,11 @@ int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, cons
         if (st != MG_OK) TRY(without_schur(ctx, L, st, &eo));
     }
     if (!eo) {
-        TRY(ensure_tiles(ctx, L, g.Vc));
-    } else if (!L.ht_valid) {
-        coarse_tiles(L.Ht, L.hts, L.H64, L.nc, g.Vc, ctx->st);
+        TRY(ensure_tiles(ctx, L, g.Vc, top));
+    } else if (!L.ht_valid || L.ht_top != top) {
+        coarse_tiles(L.Ht, L.hts, L.H64, L.nc, g.Vc, top, ctx->st);
         L.ht_valid = true;
+        L.ht_top = top;
     }
     c.At = eo ? L.Ht : L.At;
     c.as = eo ? L.hts : L.as;
@@ -765,7 +768,7 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         if (st == MG_OK) {
             panel_column(w.rc, (const float2*)rc, n, w.npad, ctx->st);
             CK(cudaMemsetAsync(ctx->bar, 0, sizeof(unsigned int) * 3, ctx->st));
-            st = panel_solve(ctx, Lm, sys.g, sys.nbr, sys.ord, w, 1, tol, maxit,
+            st = panel_solve(ctx, Lm, sys.g, sys.nbr, sys.ord, w, 1, true, tol, maxit,
                              (int*)(ctx->bar + 2), ctx->R.scal);
         }
         if (st == MG_OK) {
@@ -2884,7 +2887,7 @@ int ensure_batch(mg_ctx* ctx, int nrhs) {
 // iters_out[n] += coarse iterations of column n.
 int batched_coarse_solve(mg_ctx* ctx, int nrhs, double tol, int maxit, std::vector<double>& iters_out) {
     BatchWork& b = ctx->bw;
-    TRY(panel_solve(ctx, ctx->full, ctx->g, ctx->cnbr, ctx->cord, b.pw, nrhs, tol, maxit, b.pw.flags, nullptr));
+    TRY(panel_solve(ctx, ctx->full, ctx->g, ctx->cnbr, ctx->cord, b.pw, nrhs, false, tol, maxit, b.pw.flags, nullptr));
     CK(cudaMemcpyAsync(b.h_flags, b.pw.flags, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaMemcpyAsync(b.h_iters, b.pw.iters, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
@@ -3202,7 +3205,7 @@ int bcg_apply_args(mg_ctx* ctx, int npad, int nrhs, bool dag, BcgArgs* out, std:
     TRY(get(&a.bar, bcg_sync_bytes(npad)));
     TRY(get(&fl, sizeof(int) * 4));
     CK(cudaMemsetAsync(fl, 0, sizeof(int) * 4, ctx->st));
-    TRY(ensure_tiles(ctx, L, ctx->g.Vc));
+    TRY(ensure_tiles(ctx, L, ctx->g.Vc, false));
     a.At = L.At; a.as = L.as; a.rc = x; a.nbr = ctx->cnbr; a.err = fl;
     a.nc = L.nc; a.npad = npad; a.nrhs = nrhs; a.mode = BCG_APPLY; a.dag = dag ? 1 : 0; a.g = ctx->g;
     *out = a;

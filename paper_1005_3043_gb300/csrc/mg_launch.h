@@ -359,8 +359,8 @@ void coarse_pack16(__half2* A16, float* s16, const double2* A, int nc, int Vc, c
 // ---------------------------------------------------------------- batched (multi-RHS) coarse level
 // Panel layout xB[X][b][n], n < npad (multiple of 16), complex FP32.
 // At: per (X, d) the FP16 rows [Re A; Im A] of A[X][d] in tensor-core tiles (2 nc^2 halves
-// each), times 1 / as[X], a power of two
-void coarse_tiles(__half* At, float* as, const double2* A, int nc, int Vc, cudaStream_t st);
+// each), times 1 / as[X]: a power of two, or (top) what brings the largest entry to 2^15
+void coarse_tiles(__half* At, float* as, const double2* A, int nc, int Vc, bool top, cudaStream_t st);
 // SIMT reference of the same contraction with the FP64 operator
 template <typename T>
 void coarse_apply_batched_simt(v2<T>* y, const double2* A, const v2<T>* x, int nc, int npad, bool dag, const Geom& g,

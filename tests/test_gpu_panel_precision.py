@@ -97,3 +97,21 @@ def test_sums_of_a_low_mode(prec, nrhs):
         assert np.array_equal(A, A.real.astype(np.float16) + 1j * A.imag.astype(np.float16).astype(float))
         infos = mg.solve_batched(b)[1]
     assert [i["coarse_iters"] for i in infos] == [1] * nrhs
+
+
+@pytest.mark.parametrize("mass", [-0.3, 0.2])
+def test_one_source_is_as_near_to_64_bits_as_before(mass):
+    """A single FP16 source whose operator exceeds the chip: the correction of the panel
+    kernel (coarse_kernel 0) is as near to the FP64 one as the register-streaming kernel's
+    (coarse_kernel 1).  Both round the same entries to 11 bits under a scale of the largest
+    one (per aggregate, per block), so their errors are of one size; odd coarse extents: both
+    run on D_c."""
+    L, nv = (12, 16, 16, 10), 16
+    U, b, V = rough_gauge(L, seed=8), synth.gaussian_spinor(L, 98), synth.gaussian_vectors(L, nv, 97)
+    xs = []
+    for prec, kernel, tol in ((wmg.MG_FP64, 0, 1e-12), (wmg.MG_FP16, 1, 1e-5), (wmg.MG_FP16, 0, 1e-5)):
+        with context(L, (2, 2, 2, 2), nv, U, mass, V, prec_inner=prec, coarse_kernel=kernel, coarse_tol=tol, max_outer=1,
+                     smoother_fp16=2, max_coarse=20000) as mg:
+            xs.append(mg.solve(b)[0])
+    register, panel = (np.linalg.norm(x - xs[0]) for x in xs[1:])
+    assert panel <= 1.2 * register
