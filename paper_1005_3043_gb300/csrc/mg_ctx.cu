@@ -65,14 +65,15 @@ struct CoarseLevel {
     bool valid = false;
 };
 
-// Workspace of the panel coarse solver (kernels_batched.cu) for npad columns.
+// Workspace of the panel coarse solver (kernels_batched.cu): room for cap columns, the
+// call's panels npad columns wide.
 struct PanelWork {
-    int npad = 0, nc = 0, Vc = 0;
+    int cap = 0, npad = 0, nc = 0, Vc = 0;
     float2 *rc = nullptr, *y = nullptr, *r = nullptr, *s = nullptr, *p = nullptr, *q = nullptr, *u = nullptr, *z = nullptr;
     float2* e = nullptr;            // red-black form: rhat (even sites) and A_oo^-1 r (odd sites)
     __half *bts = nullptr, *btu = nullptr;   // operand tiles of the tensor-core stencil
     unsigned int* sync = nullptr;   // grid barrier and grid sums
-    double* iters = nullptr;        // npad
+    double* iters = nullptr;        // cap
     int* flags = nullptr;           // [0] error
 };
 
@@ -616,16 +617,17 @@ int ensure_tiles(mg_ctx* ctx, CoarseLevel& L, int Vc, bool top) {
     return MG_OK;
 }
 int ensure_panel(mg_ctx* ctx, PanelWork& w, int npad, int nc, int Vc) {
-    if (w.npad >= npad && w.nc == nc && w.Vc == Vc) return MG_OK;
-    if (w.npad) CK(cudaStreamSynchronize(ctx->st));   // grow: the smaller workspace goes first
-    w.npad = 0;
+    w.npad = npad;   // not the widest so far: the width sets the work and the order of the sums
+    if (w.cap >= npad && w.nc == nc && w.Vc == Vc) return MG_OK;
+    if (w.cap) CK(cudaStreamSynchronize(ctx->st));   // grow: the smaller workspace goes first
+    w.cap = 0;
     const size_t pe = sizeof(float2) * (size_t)Vc * nc * npad;
     TRY(dalloc_all(ctx, {{&w.rc, pe}, {&w.y, pe}, {&w.r, pe}, {&w.s, pe}, {&w.p, pe}, {&w.q, pe}, {&w.u, pe}, {&w.z, pe},
                          {&w.e, pe}, {&w.bts, bcg_tile_bytes(nc, npad, Vc)}, {&w.btu, bcg_tile_bytes(nc, npad, Vc)},
                          {&w.sync, bcg_sync_bytes(npad)}, {&w.iters, sizeof(double) * npad}, {&w.flags, sizeof(int) * 4}}));
     for (float2* q : {w.rc, w.y, w.r, w.s, w.p, w.q, w.u, w.z, w.e}) CK(cudaMemsetAsync(q, 0, pe, ctx->st));
     CK(cudaMemsetAsync(w.flags, 0, sizeof(int) * 4, ctx->st));
-    w.npad = npad;
+    w.cap = npad;
     w.nc = nc;
     w.Vc = Vc;
     return MG_OK;

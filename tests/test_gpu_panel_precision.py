@@ -115,3 +115,17 @@ def test_one_source_is_as_near_to_64_bits_as_before(mass):
             xs.append(mg.solve(b)[0])
     register, panel = (np.linalg.norm(x - xs[0]) for x in xs[1:])
     assert panel <= 1.2 * register
+
+
+@pytest.mark.parametrize("L,B", [((8, 8, 8, 16), (2, 2, 2, 2)), ((6, 8, 8, 16), (2, 2, 2, 2))])
+def test_a_batch_does_not_depend_on_earlier_ones(L, B):
+    """The same two sources before and after a batch of 40, bit for bit: the panels of a
+    call are as wide as its own sources need."""
+    U, b = rough_gauge(L, seed=8), np.stack([synth.gaussian_spinor(L, 98, stream=i) for i in range(40)])
+    with context(L, B, 8, U, 0.1, synth.gaussian_vectors(L, 8, 97), prec_inner=wmg.MG_FP32, tol=1e-8) as mg:
+        first = mg.solve_batched(b[:2])
+        mg.solve_batched(b)
+        again = mg.solve_batched(b[:2])
+    assert np.array_equal(first[0], again[0])
+    for i, k in zip(first[1], again[1]):
+        assert i["coarse_iters"] == k["coarse_iters"]
