@@ -461,18 +461,22 @@ int mg_profile_classes(mg_ctx* ctx, unsigned int mask);
  * measurement hook, no counterpart in the paper). */
 long long mg_kernel_launches(void);
 
-/* Which coarse CGNR kernel the last coarse solve of this context ran (a
- * diagnostic; no counterpart in the paper): MG_CK_REGISTER the kernel that reads
+/* Which coarse CGNR kernel the last coarse solve of this context ran, a batched
+ * solve's included (a diagnostic; no counterpart in the paper): MG_CK_REGISTER the kernel that reads
  * the operator from global memory (in FP64 once per launch where the SMs' shared
  * memory holds it), MG_CK_SMEM operator resident in shared
  * memory, MG_CK_STREAM operator streamed through a shared-memory ring,
  * MG_CK_TMEM operator resident in tensor memory, products on the CUDA cores,
  * MG_CK_TMEM_MMA operator resident in tensor memory, products on the tensor
- * cores; MG_CK_NONE before any. */
+ * cores, MG_CK_PANEL the kernel for panels of right-hand sides (batched solves, and
+ * FP16 operators larger than the chip); MG_CK_NONE before any. */
 enum mg_coarse_kernel_id {
-    MG_CK_NONE = -1, MG_CK_REGISTER = 0, MG_CK_SMEM = 1, MG_CK_STREAM = 2, MG_CK_TMEM = 3, MG_CK_TMEM_MMA = 4
+    MG_CK_NONE = -1, MG_CK_REGISTER = 0, MG_CK_SMEM = 1, MG_CK_STREAM = 2, MG_CK_TMEM = 3, MG_CK_TMEM_MMA = 4,
+    MG_CK_PANEL = 5
 };
 int mg_coarse_kernel(mg_ctx* ctx);
+/* Whether it ran on the red-black form of D_c: 1, or 0 on D_c itself (-1 before any). */
+int mg_coarse_red_black(mg_ctx* ctx);
 
 /* Check of the library's bounded device waits (the paper has no counterpart;
  * every spin-wait in these kernels gives up after a poll limit, raises the

@@ -115,6 +115,7 @@ _SIGS = {
     "mg_profile_classes": ([_P, ctypes.c_uint], _I),
     "mg_kernel_launches": ([], ctypes.c_longlong),
     "mg_coarse_kernel": ([ctypes.c_void_p], ctypes.c_int),
+    "mg_coarse_red_black": ([_P], _I),
     "mg_check_wait_timeout": ([_P, _I, ctypes.c_longlong], _I),
     "mg_fail_allocation": ([_P, _I], _I),
     "mg_status_string": ([_I], ctypes.c_char_p),
@@ -508,11 +509,16 @@ COARSE_KERNELS = {-1: "none", 0: "k_cgnr_persistent (operator from global memory
                   1: "k_cgls_onchip (operator resident in shared memory)",
                   2: "k_cgls_onchip (operator streamed through shared memory)",
                   3: "k_cgls_onchip (operator resident in tensor memory, products on the CUDA cores)",
-                  4: "k_cgls_onchip (operator resident in tensor memory, products on the tensor cores)"}
+                  4: "k_cgls_onchip (operator resident in tensor memory, products on the tensor cores)",
+                  5: "k_bcg (panels of right-hand sides, products on the tensor cores)"}
 
 
 def mg_coarse_kernel(ctx) -> int:
     return int(load().mg_coarse_kernel(ctx))
+
+
+def mg_coarse_red_black(ctx) -> int:
+    return int(load().mg_coarse_red_black(ctx))
 
 
 def mg_check_wait_timeout(ctx, kind: int, spin_limit: int = 20000) -> int:
@@ -713,3 +719,7 @@ class WilsonMG:
     def coarse_kernel(self) -> int:
         """MG_CK_* id of the coarse CGNR kernel the last coarse solve ran."""
         return mg_coarse_kernel(self.ctx)
+
+    def coarse_red_black(self) -> int:
+        """1: the last coarse solve ran on the red-black form of D_c, 0: on D_c (-1: none ran)."""
+        return mg_coarse_red_black(self.ctx)

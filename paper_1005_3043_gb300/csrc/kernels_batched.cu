@@ -673,12 +673,14 @@ struct BcgCta {
             fr[i] = finite ? __int_as_float((127 - e) << 23) : 1.f;
             done[i] = (i >= a.nrhs || zero || !finite || a.maxit <= 0) ? (finite ? 1 : 2) : 0;
             its[i] = 0;
+            rho0[i] = 0.0;
             sc_s[i] = sc_u[i] = col_scale(4.0, rows);
             iss[i] = isu[i] = 1.f / sc_s[i];
             fx[i] = fx[np + i] = fx[2 * np + i] = 0x1p42f;
         }
         epi_sync();
         int phase = 0;
+        double last = 0.0;   // thread 0: |r|^2 of column 0
         // the odd half of a red-black stencil: t = sum H x, straight into the operand's tiles
         // (the scale of x, so that both halves' operands add up in one accumulator)
         auto odd_half = [&](__half* bt, const float* inv, const float* sc) {
@@ -793,6 +795,7 @@ struct BcgCta {
                     }
                     const double delta = tot[0], gamma = tot[1], rho = tot[2];
                     its[i] = it;
+                    if (i == 0) last = rho;
                     double beta = 0.0, den = delta;
                     if (it > 0) {   // gam, alo: reciprocals of the last gamma and alpha
                         beta = gamma * gam[i];
@@ -889,7 +892,11 @@ struct BcgCta {
         if (blockIdx.x == 0)
             for (int i = t; i < np; i += kEpi) {
                 a.iters[i] = (double)its[i];
-                if (i == 0 && a.scal) {
+                if (i == 0 && a.scal) {   // rho0 and last in the units of rc
+                    const double f = 1.0 / ((double)fr[0] * fr[0]);
+                    a.scal[S_CG_RC2] = f * rho0[0];
+                    a.scal[S_CG_R2] = f * last;
+                    a.scal[S_CG_DONE] = 1.0;
                     a.scal[S_CG_ITERS] = (double)its[0];
                     a.scal[S_CG_TOTAL] += (double)its[0];
                 }

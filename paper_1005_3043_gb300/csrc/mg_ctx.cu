@@ -224,6 +224,7 @@ struct mg_ctx {
     unsigned int xch_epoch = 1;          // next free epoch
     double* scal_s = nullptr;            // scalars of the GMRES smoother (its Hessenberg matrix)
     int coarse_kernel_used = MG_CK_NONE;
+    int red_black_used = -1;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     std::vector<void*> allocs;
     // launch timer
@@ -672,6 +673,8 @@ int panel_solve(mg_ctx* ctx, CoarseLevel& L, const Geom& g, const int* nbr, cons
     if (eo) schur_rows<float>(w.y, w.e, L.H32, w.y, ord + half, half, nbr, L.nc, 1, 9, -1.0, nrhs, w.npad, ctx->st);
     PROF_END(MG_K_COARSE_SOLVE);
     CKL();
+    ctx->coarse_kernel_used = MG_CK_PANEL;
+    ctx->red_black_used = eo;
     return MG_OK;
 }
 
@@ -754,6 +757,7 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
             schur_rows<float>((v2<float>*)y, (v2<float>*)sys.eb, L.H32, (v2<float>*)y, sys.ord + half, half, sys.nbr, L.nc, 1, 9,
                               -1.0, 1, 1, ctx->st);
         PROF_END(MG_K_COARSE_SOLVE);
+        ctx->red_black_used = eo;
         ctx->coarse_kernel_used = c.sh.tm == 2 ? MG_CK_TMEM_MMA : c.sh.tm ? MG_CK_TMEM : c.sh.resident ? MG_CK_SMEM : MG_CK_STREAM;
     }
     int nw = 0, stages = 0;
@@ -776,7 +780,6 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         if (st == MG_OK) {
             column_of_panel((float2*)y, w.y, n, w.npad, ctx->st);
             CKL();
-            ctx->coarse_kernel_used = MG_CK_REGISTER;
         }
         if (st != MG_ERR_OOM) return st;
         ctx->panel_refused = true;   // no memory for its panels or tiles: the register-streaming kernel
@@ -813,6 +816,7 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         PROF_END(MG_K_COARSE_SOLVE);
         CKL();
         ctx->coarse_kernel_used = MG_CK_REGISTER;
+        ctx->red_black_used = eo;
     }
     if (iters) {
         TRY(read_scalars(ctx, S_CG_RC2, 3));
@@ -2552,6 +2556,7 @@ int mg_fail_allocation(mg_ctx* ctx, int nth) {
     return pending;
 }
 int mg_coarse_kernel(mg_ctx* ctx) { return ctx ? ctx->coarse_kernel_used : MG_CK_NONE; }
+int mg_coarse_red_black(mg_ctx* ctx) { return ctx ? ctx->red_black_used : -1; }
 
 const char* mg_status_string(int status) {
     int i = -status;

@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 
+import oracle
 import paper_1005_3043_gb300 as wmg
 import synth
 from tests._fields import rough_gauge
@@ -49,3 +50,42 @@ def test_a_solve_prepares_the_form_that_it_runs(shape, prec, kernel, launches):
             mg.solve(b)
             counts.append(wmg.mg_kernel_launches() - before)
     assert counts[0] - counts[1] == launches, counts
+
+
+# 8^4 with 2^4 aggregates, Nv = 24 in FP32: 42 MB, six 32-word chunks of a thread's share, four in
+# tensor memory and two in shared memory
+CHUNKS = ((8, 8, 8, 8), (2, 2, 2, 2), 24)
+REGISTER, TMEM, TMEM_MMA, PANEL = 0, 3, 4, 5
+
+
+@pytest.mark.parametrize("shape,prec,kernel,ran,red_black", [
+    (SMALL, wmg.MG_FP64, 0, REGISTER, 1), (SMALL, wmg.MG_FP32, 1, REGISTER, 1), (SMALL, wmg.MG_FP16, 1, REGISTER, 1),
+    (SMALL, wmg.MG_FP32, 0, TMEM, 1), (SMALL, wmg.MG_FP16, 4, TMEM, 1),
+    (SMALL, wmg.MG_FP16, 0, TMEM_MMA, 0),              # its iterations are too short for the halves' barriers
+    (((12, 8, 8, 8), (4, 4, 4, 4), 8), wmg.MG_FP32, 0, TMEM, 0), (((12, 8, 8, 8), (4, 4, 4, 4), 8), wmg.MG_FP64, 0, REGISTER, 0),
+    (CHUNKS, wmg.MG_FP32, 0, TMEM, 1), (BIG, wmg.MG_FP16, 0, PANEL, 1), (BIG_ODD, wmg.MG_FP16, 0, PANEL, 0),
+    (BIG, wmg.MG_FP16, 1, REGISTER, 1)])
+def test_kernel_and_form_of_a_solve(shape, prec, kernel, ran, red_black):
+    """The kernel and form that each route takes, and that its correction is that of D_c:
+    after one outer iteration x is <D z, b> / |D z|^2 z, z the V-cycle of b, which runs on
+    D_c (tolerances: test_gpu_red_black_coarse.py)."""
+    L = shape[0]
+    tol, eps = {wmg.MG_FP64: (1e-12, 1e-12), wmg.MG_FP32: (1e-5, 1e-5), wmg.MG_FP16: (1e-5, 2.0 ** -11)}[prec]
+    b = synth.gaussian_spinor(L, 98)
+    with context(shape, prec, kernel, coarse_tol=tol, max_outer=1) as mg:
+        assert (mg.coarse_kernel(), mg.coarse_red_black()) == (-1, -1)
+        x = mg.solve(b)[0]
+        assert (mg.coarse_kernel(), mg.coarse_red_black()) == (ran, red_black)
+        z = mg.vcycle(b, prec)
+        assert mg.coarse_red_black() == 0
+    q = oracle.dslash(rough_gauge(L, seed=8), z, MASS, L)
+    ref = np.vdot(q, b) / np.vdot(q, q) * z
+    assert np.linalg.norm(x - ref) < 20 * eps * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("shape,red_black", [(SMALL, 1), (((12, 8, 8, 8), (4, 4, 4, 4), 8), 0)])
+def test_kernel_and_form_of_a_batch(shape, red_black):
+    with context(shape, wmg.MG_FP32, 0) as mg:
+        b = np.stack([synth.gaussian_spinor(shape[0], 98, stream=i) for i in range(2)])
+        mg.solve_batched(b)
+        assert (mg.coarse_kernel(), mg.coarse_red_black()) == (PANEL, red_black)
