@@ -331,18 +331,35 @@ __device__ __forceinline__ void build_stage(const v2<TC>* __restrict__ P, const 
     }
 }
 
-// One CTA per (aggregate, direction).  TC: precision of the products (double, or
-// float with the sums over a chunk's sites added up in FP64).  Threads: chirality
+template <typename TC>
+__device__ __forceinline__ void build_stage_of(int h, const v2<TC>* __restrict__ P, const v2<TC>* __restrict__ U, int nv,
+                                               const Geom& g, int X, const int (&xcX)[4], int m0, int cs, v2<TC>* Wsh,
+                                               v2<TC>* Psh, int ws, int ps) {
+    switch (h) {
+        case 0: build_stage<TC, 0, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+        case 1: build_stage<TC, 0, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+        case 2: build_stage<TC, 1, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+        case 3: build_stage<TC, 1, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+        case 4: build_stage<TC, 2, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+        case 5: build_stage<TC, 2, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+        case 6: build_stage<TC, 3, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+        default: build_stage<TC, 3, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
+    }
+}
+
+// FP32: one CTA per (aggregate, direction), products in FP32 with the sums over a
+// chunk's sites added up in FP64.  Threads: chirality
 // of the row (2) x 8 x 16, each with NT x NT products, rows ta + 8 i, columns
 // tb + 16 j (NT = ceil(nv / 8), at most 4 for nv <= 25): an entry of shared memory
 // feeds NT products.  (With one product per two entries the shared-memory pipe, not
 // the FMA units, was at work: the six builds of a setup on 16^3x32, 4^4 aggregates,
-// 16 to 20 columns, FP32: 40 -> 22 ms; the products alone take 5, their sums and
+// 16 to 20 columns: 40 -> 22 ms; the products alone take 5, their sums and
 // conversions in FP64 another 6.)
-template <typename TC, int NT>
-__global__ void __launch_bounds__(256, sizeof(TC) == 4 && NT <= 3 ? 2 : 1)
-k_coarse_hop(double2* __restrict__ A, double2* __restrict__ Aself, const v2<TC>* __restrict__ P, const v2<TC>* __restrict__ U,
+template <int NT>
+__global__ void __launch_bounds__(256, NT <= 3 ? 2 : 1)
+k_coarse_hop(double2* __restrict__ A, double2* __restrict__ Aself, const float2* __restrict__ P, const float2* __restrict__ U,
              int nv, Geom g) {
+    using TC = float;
     extern __shared__ unsigned char smem_raw[];
     const int nc = 2 * nv, ws = build_stride<TC>(nc * kWStride), ps = build_stride<TC>(nc * 6);
     v2<TC>* Wsh = reinterpret_cast<v2<TC>*>(smem_raw);
@@ -366,16 +383,7 @@ k_coarse_hop(double2* __restrict__ A, double2* __restrict__ Aself, const v2<TC>*
             for (int j = 0; j < NT; ++j) acc[i][j] = cx<double>(0, 0);
         for (int m0 = set ? nface : 0; m0 < end; m0 += kBuildChunk) {
             const int cs = min(kBuildChunk, end - m0);
-            switch (h) {
-                case 0: build_stage<TC, 0, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-                case 1: build_stage<TC, 0, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-                case 2: build_stage<TC, 1, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-                case 3: build_stage<TC, 1, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-                case 4: build_stage<TC, 2, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-                case 5: build_stage<TC, 2, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-                case 6: build_stage<TC, 3, true>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-                default: build_stage<TC, 3, false>(P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps); break;
-            }
+            build_stage_of<TC>(h, P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps);
             __syncthreads();
             cx<TC> t[NT][NT];
 #pragma unroll
@@ -415,6 +423,63 @@ k_coarse_hop(double2* __restrict__ A, double2* __restrict__ Aself, const v2<TC>*
                     st<double>(out + (size_t)(tb + 16 * j) * nc + sa * nv + ta + 8 * i, acc[i][j]);
     }
 }
+// FP64: bound by the FP64 pipe, two operations a clock and SM, whatever feeds it.  So no
+// product is formed that is not stored: the pairs (a, b) are dealt out in order, Q per
+// thread, and warps past the last pair have nothing to do (the tiles above form 1.4 times
+// the products at nv = 20, 1.8 times at nv = 12).  Builds of one setup at 2 to 20 columns
+// on 16^3x32: 799 ms, in tiles about 1130, with two accumulators per pair 930; at 2 to 12
+// columns on 12^3x24 54, 100 and 71.
+template <int Q>
+__global__ void __launch_bounds__(256) k_coarse_hop_pairs(double2* __restrict__ A, double2* __restrict__ Aself,
+                                                          const double2* __restrict__ P, const double2* __restrict__ U,
+                                                          int nv, Geom g) {
+    extern __shared__ unsigned char smem_raw[];
+    const int nc = 2 * nv, npair = nc * nc, ws = build_stride<double>(nc * kWStride), ps = build_stride<double>(nc * 6);
+    double2* Wsh = reinterpret_cast<double2*>(smem_raw);
+    double2* Psh = Wsh + (size_t)kBuildChunk * ws;
+    const int X = blockIdx.x >> 3, h = blockIdx.x & 7;
+    int xcX[4], pa[Q], pb[Q];
+    coarse_coords(g, X, xcX);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int pr = threadIdx.x + q * 256, a = pr < npair ? pr / nc : 0, b = pr < npair ? pr - a * nc : 0;
+        pa[q] = a * 6;
+        pb[q] = b * kWStride + (a >= nv ? 6 : 0);
+    }
+    const int nface = g.Vb / (h < 2 ? g.B[0] : h < 4 ? g.B[1] : h < 6 ? g.B[2] : g.B[3]);
+    for (int set = 0; set < 2; ++set) {
+        const int end = set ? g.Vb : nface;
+        cx<double> acc[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[q] = cx<double>(0, 0);
+        for (int m0 = set ? nface : 0; m0 < end; m0 += kBuildChunk) {
+            const int cs = min(kBuildChunk, end - m0);
+            build_stage_of<double>(h, P, U, nv, g, X, xcX, m0, cs, Wsh, Psh, ws, ps);
+            __syncthreads();
+            cx<double> t[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) t[q] = cx<double>(0, 0);
+            for (int xi = 0; xi < cs; ++xi) {
+                const double2* wx = Wsh + (size_t)xi * ws;
+                const double2* px = Psh + xi * ps;
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if ((int)threadIdx.x + q * 256 < npair)
+#pragma unroll
+                        for (int kk = 0; kk < 6; ++kk) cmadc(t[q], ld<double>(px + pa[q] + kk), ld<double>(wx + pb[q] + kk));
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) acc[q] = acc[q] + t[q];
+            __syncthreads();
+        }
+        double2* out = set ? Aself + ((size_t)X * 8 + h) * npair : A + ((size_t)X * 9 + 1 + h) * npair;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int a = pa[q] / 6, b = pb[q] / kWStride;   // 6 < kWStride
+            if ((int)threadIdx.x + q * 256 < npair) st<double>(out + (size_t)b * nc + a, acc[q]);
+        }
+    }
+}
 // A[X][0] = (4+m) I + sum_h Aself[X][h] (fixed order)
 __global__ void k_coarse_diag(double2* A, const double2* __restrict__ Aself, int nc, double diag, Geom g) {
     long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -428,12 +493,12 @@ __global__ void k_coarse_diag(double2* A, const double2* __restrict__ Aself, int
     st<double>(A + (size_t)X * 9 * nc * nc + r, v);
 }
 
-template <typename TC>
-void coarse_build_t(double2* A, double2* Aself, const v2<TC>* P, const v2<TC>* U, int nv, double mass, const Geom& g,
-                    cudaStream_t st) {
-    int nc = 2 * nv;
-    const size_t sm = sizeof(v2<TC>) * kBuildChunk * (build_stride<TC>(nc * kWStride) + build_stride<TC>(nc * 6));
-    auto kern = nv <= 8 ? k_coarse_hop<TC, 1> : nv <= 16 ? k_coarse_hop<TC, 2> : nv <= 24 ? k_coarse_hop<TC, 3> : k_coarse_hop<TC, 4>;
+// T: precision of the products
+template <typename T>
+static void coarse_build_with(void (*kern)(double2*, double2*, const v2<T>*, const v2<T>*, int, Geom), double2* A, double2* Aself,
+                              const v2<T>* P, const v2<T>* U, int nv, double mass, const Geom& g, cudaStream_t st) {
+    const int nc = 2 * nv;
+    const size_t sm = sizeof(v2<T>) * kBuildChunk * (build_stride<T>(nc * kWStride) + build_stride<T>(nc * 6));
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     note_launch();
     kern<<<g.Vc * 8, kThreads, sm, st>>>(A, Aself, P, U, nv, g);
@@ -443,12 +508,14 @@ void coarse_build_t(double2* A, double2* Aself, const v2<TC>* P, const v2<TC>* U
 }
 void coarse_build_f32(double2* A, double2* Aself, const float2* P, const float2* U, int nv, double mass, const Geom& g,
                       cudaStream_t st) {
-    coarse_build_t<float>(A, Aself, P, U, nv, mass, g, st);
+    coarse_build_with<float>(nv <= 8 ? k_coarse_hop<1> : nv <= 16 ? k_coarse_hop<2> : nv <= 24 ? k_coarse_hop<3> : k_coarse_hop<4>,
+                             A, Aself, P, U, nv, mass, g, st);
 }
 
 void coarse_build(double2* A, double2* Aself, const double2* P, const double2* U, int nv, double mass, const Geom& g,
                   cudaStream_t st) {
-    coarse_build_t<double>(A, Aself, P, U, nv, mass, g, st);
+    coarse_build_with<double>(nv <= 8 ? k_coarse_hop_pairs<1> : nv <= 16 ? k_coarse_hop_pairs<4> : k_coarse_hop_pairs<10>, A,
+                              Aself, P, U, nv, mass, g, st);
 }
 
 __global__ void k_coarse_shift(double2* A, int nc, double dm, int Vc) {
