@@ -89,3 +89,21 @@ def test_kernel_and_form_of_a_batch(shape, red_black):
         b = np.stack([synth.gaussian_spinor(shape[0], 98, stream=i) for i in range(2)])
         mg.solve_batched(b)
         assert (mg.coarse_kernel(), mg.coarse_red_black()) == (PANEL, red_black)
+
+
+# rows that a CTA takes in two passes: 512 aggregates in four parts, 1280 in three
+@pytest.mark.parametrize("L,nv", [((8, 8, 8, 16), 16), ((8, 8, 10, 32), 6)])
+def test_fp64_iterations_in_several_passes(L, nv):
+    """Four CG iterations on D_c in FP64 against the oracle's (the bound and its derivation:
+    test_gpu_red_black_coarse.py)."""
+    B = (2, 2, 2, 2)
+    U, V0 = rough_gauge(L, seed=8), synth.gaussian_vectors(L, nv, 97)
+    P, st = oracle.block_orthonormalize(V0, L, B)
+    assert st == 0
+    A, Lc = oracle.coarse_build(U, P, MASS, L, B), oracle.coarse_dims(L, B)
+    rc = synth.gaussian(oracle.volume(Lc) * 2 * nv, 8, 0).reshape(-1, 2 * nv)
+    ref, _, _ = oracle.cgnr(A, rc, Lc, 0.0, 4)
+    with context((L, B, nv), wmg.MG_FP64, 0) as mg:
+        y, it, _ = mg.coarse_solve(rc, 0.0, 4, wmg.MG_FP64)
+    assert it == 4
+    assert np.abs(y - ref).max() <= 1e-10 * np.abs(ref).max()
