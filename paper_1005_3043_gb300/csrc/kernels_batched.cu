@@ -425,9 +425,12 @@ struct BcgCta {
     // entries staged in S2[row][n] (scaled) -> the four FP16 rows of the tile.  A single
     // right-hand side (a.third): what its hi and lo leave, times 2^22, goes into the hi
     // rows of the unused column 1, so that its operand has the 24 bits of an FP32 number.
-    __device__ void write_tile(__half* bt, int X, int c) {
+    __device__ __forceinline__ void write_tile(__half* bt, int X, int c) {
+        if (a.third && c == 0) write_parts<true>(bt, X, c);
+        else write_parts<false>(bt, X, c);
+    }
+    template <bool THIRD> __device__ void write_parts(__half* bt, int X, int c) {
         __half* base = bt + ((size_t)X * nch + c) * 4 * nc * nw;
-        const bool third = a.third && c == 0;
         for (int i = t; i < (nc >> 3) * nw; i += kEpi) {
             const int kc = i / nw, m = i - kc * nw;
             uint32_t w[4][4];
@@ -437,14 +440,14 @@ struct BcgCta {
                 float hr[2], hi[2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    v[q] = S2[(kc * 8 + 2 * e + q) * L.ts + (third && m == 1 ? 0 : m)];
+                    v[q] = S2[(kc * 8 + 2 * e + q) * L.ts + (THIRD && m == 1 ? 0 : m)];
                     v[q].x = fminf(fmaxf(v[q].x, -65504.f), 65504.f);
                     v[q].y = fminf(fmaxf(v[q].y, -65504.f), 65504.f);
                     hr[q] = __half2float(__float2half_rn(v[q].x));
                     hi[q] = __half2float(__float2half_rn(v[q].y));
                     v[q].x = 0x1p11f * (v[q].x - hr[q]);
                     v[q].y = 0x1p11f * (v[q].y - hi[q]);
-                    if (third && m == 1) {
+                    if (THIRD && m == 1) {
                         hr[q] = 0x1p11f * (v[q].x - __half2float(__float2half_rn(v[q].x)));
                         hi[q] = 0x1p11f * (v[q].y - __half2float(__float2half_rn(v[q].y)));
                         v[q] = make_float2(0.f, 0.f);
@@ -499,10 +502,10 @@ struct BcgCta {
         if (t == 0) next_phase();
     }
 
-    // products of the next job (at site X) into T, in the operator's units; false on
-    // failure (uniform over the warps)
-    __device__ bool take(uint32_t tmem, int X, int c) {
-        const float f = __ldg(a.as + X);
+    // products of the next job (column chunk c) into T, in units of the operator's scale
+    // (unit); false on failure (uniform over the warps)
+    __device__ float unit(int X) const { return __ldg(a.as + X); }
+    __device__ bool take(uint32_t tmem, int c) {
         const int buf = (int)(job_count & 1), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         const int quad = warp & 3, half = (warp - 4) >> 2, m = 32 * quad + lane;
         const bool ok = __all_sync(0xffffffffu, bcg_wait(acc_full + buf, (uint32_t)((job_count >> 1) & 1), fail, a.err));
@@ -525,8 +528,8 @@ struct BcgCta {
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
                         T[(size_t)m * L.ts + c0 + e] =
-                            make_float2(f * (__uint_as_float(rh[e]) + 0x1p-11f * __uint_as_float(rl[e])),
-                                        f * (__uint_as_float(ih[e]) + 0x1p-11f * __uint_as_float(il[e])));
+                            make_float2(__uint_as_float(rh[e]) + 0x1p-11f * __uint_as_float(rl[e]),
+                                        __uint_as_float(ih[e]) + 0x1p-11f * __uint_as_float(il[e]));
             }
         }
         tc_fence_before();
@@ -629,10 +632,11 @@ struct BcgCta {
             if (!grid_barrier(true)) return;
             for (int j = 0; j < jobs; ++j) {
                 const int X = (j0 + j) / nch, c = j0 + j - X * nch;
-                if (!take(tmem, X, c)) return;
+                const float f = unit(X);
+                if (!take(tmem, c)) return;
                 if (act)
                     for (int r = rg; r < nc; r += rgs)
-                        a.y[((size_t)X * nc + r) * np + c * nw + n] = product(r, 1.f, a.dag != 0);
+                        a.y[((size_t)X * nc + r) * np + c * nw + n] = product(r, f, a.dag != 0);
                 epi_sync();
             }
             if (t == 0) *stop = 1;
@@ -687,9 +691,12 @@ struct BcgCta {
             if (!eo) return true;
             for (int j = 0; j < jobs; ++j) {
                 const int X = site(phase, j0 + j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem, X, c)) return false;
-                if (act)
-                    for (int r = rg; r < nc; r += rgs) stage(r, product(r, inv[col], false), sc[col], false);
+                const float f = unit(X);
+                if (!take(tmem, c)) return false;
+                if (act) {
+                    const float p = f * inv[col];
+                    for (int r = rg; r < nc; r += rgs) stage(r, product(r, p, false), sc[col], false);
+                }
                 epi_sync();
                 write_tile(bt, X, c);
             }
@@ -726,10 +733,11 @@ struct BcgCta {
         if (!odd_half(a.btu, isu, sc_u)) return;
         for (int j = 0; j < jobs; ++j) {
             const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-            if (!take(tmem, X, c)) return;
+            const float f = unit(X);
+            if (!take(tmem, c)) return;
             if (act) {
                 float s = 0.f;
-                const float inv = isu[col], sc = sc_s[col];
+                const float inv = f * isu[col], sc = sc_s[col];
                 for (int r = rg; r < nc; r += rgs) {
                     const float2 v = product(r, inv, true);
                     a.s[((size_t)X * nc + r) * np + col] = v;
@@ -749,10 +757,11 @@ struct BcgCta {
             if (!odd_half(a.bts, iss, sc_s)) return;
             for (int j = 0; j < jobs; ++j) {
                 const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem, X, c)) return;
+                const float f = unit(X);
+                if (!take(tmem, c)) return;
                 if (act) {
                     float s = 0.f;
-                    const float inv = iss[col], sc = sc_u[col];
+                    const float inv = f * iss[col], sc = sc_u[col];
                     for (int r = rg; r < nc; r += rgs) {
                         const float2 v = product(r, inv, false);
                         a.u[((size_t)X * nc + r) * np + col] = v;
@@ -825,17 +834,18 @@ struct BcgCta {
                 if (!odd_half(a.btu, isu, sc_tu)) return;
             } else if (eo) {   // the odd half that was started; its even half never is
                 for (int j = 0; j < jobs; ++j)
-                    if (!take(tmem, site(phase, j0 + j), (j0 + j) % nch)) return;
+                    if (!take(tmem, (j0 + j) % nch)) return;
                 break;
             }
             for (int j = 0; j < jobs; ++j) {
                 const int X = at(j), c = (j0 + j) % nch, col = c * nw + n;
-                if (!take(tmem, X, c)) return;
+                const float f = unit(X);
+                if (!take(tmem, c)) return;
                 if (!running) continue;   // nothing left to do but to take what was started
                 if (act) {
                     float sg = 0.f, sr = 0.f;
                     const bool frozen = done[col] != 0;
-                    const float inv = isu[col], sc = sc_s[col], alpha = al[col], beta = be[col];
+                    const float inv = f * isu[col], sc = sc_s[col], alpha = al[col], beta = be[col];
 #pragma unroll 3
                     for (int r = rg; r < nc; r += rgs) {
                         const size_t o = ((size_t)X * nc + r) * np + col;
