@@ -31,7 +31,8 @@
 // the reductions and the updates (ten launches per iteration, replayed from a
 // graph) took 76 us per iteration on 16^3x32 with 12 sources (Nv = 16), 34 us of it
 // in each stencil, and 64 us on 8^3x16 with 21 sources, all latency; this kernel
-// takes 25 and 14 us (red-black, four barriers: 36 and 28 us for half the iterations).
+// takes 29 and 16 us (red-black, four barriers: 38 and 31 us for less than half the
+// iterations).
 // What is left: about 1.2 us per job (copies, 18 MMAs and the epilogue overlap), 2 to
 // 3 us per grid barrier.
 #include <cuda_fp16.h>

@@ -134,7 +134,7 @@ enum { OV_P = 0, OV_Z = 1, OV_Q = 2, OV_Y = 3, OV_R = 4, OV_S = 5, OV_U = 6, OV_
 // 128 TMEM columns, the rest in shared memory (64 KB per chunk).  FP32 at 16^3x32
 // (Nv = 20, six chunks, 394 KB per SM) stays on chip this way, 9.3 us per CG
 // iteration against 26.4 with the operator read from L2 twice an iteration (a solve
-// with 3943 iterations 113 -> 64 ms, although the latter ran red-black).
+// with 3943 iterations 113 -> 64 ms, although the former ran red-black).
 constexpr int kTmemChunks = 4;
 constexpr int kStageRegs = 4;   // staged operand entries per thread kept as precomputed offsets
 
@@ -1386,9 +1386,10 @@ size_t mma_smem(size_t off, CglsShape& s, int K, int smem_optin) {
 
 // Pick the rows per unit RU (a divisor of nc, a multiple of 4, with RU * element
 // bytes a multiple of 16, RU >= 8 when nc allows) that minimises the rows of
-// the busiest CTA.  mode CGLS_AUTO: the operator in tensor memory when every
-// thread's share fits its 128 columns, else in shared memory when a CTA's units
-// fit there (none: false, the caller uses the register-streaming kernel);
+// the busiest CTA.  mode CGLS_AUTO: the operator in tensor memory, what exceeds a
+// thread's 128 columns (up to as much again) in shared memory, else all of it in
+// shared memory when a CTA's units fit there (none: false, the caller uses the
+// register-streaming kernel);
 // CGLS_SMEM: shared memory only; CGLS_STREAM: streamed through two one-unit
 // slot groups by about a third as many CTAs as units (several waves per phase,
 // so the ring wraps within every phase), whatever the size.

@@ -749,8 +749,9 @@ namespace wmg {
 // upb consecutive units at a time, tpu = 9 * bs * (row groups of a part) threads
 // each: thread (unit, d, column part, row group).
 // FP32 and FP16 operators (bound by the operator's bytes): whole aggregates (rsp =
-// 1), as many as fit the CTA while every SM has two CTAs, then column parts.  FP64 (bound by the FP64 pipe, two FMAs
-// per clock and SM): every SM has to have an equal share of the rows.  With
+// 1), as many as fit the CTA while every SM has one, then column parts.  FP64 (bound by
+// the FP64 pipe, two FMAs per clock and SM): every SM has to have an equal share of the
+// rows.  With
 // whole aggregates an 8^4 lattice (16 aggregates) ran on 4 SMs and 12^3 x 24
 // (162 aggregates) on 54; cut into parts, one CTA per SM (its partial sums are
 // re-added in FP64 by every CTA, so no more CTAs than SMs).  Measured with the

@@ -216,7 +216,7 @@ struct mg_ctx {
     Reduce R{};
     double* h_scal = nullptr;        // pinned host copy of the scalars
     int* d_status = nullptr;
-    unsigned int* bar = nullptr;     // persistent-kernel barrier: count, generation, error flag
+    unsigned int* bar = nullptr;     // persistent kernels: [0] barrier count, [2] error flag
     int* cnbr = nullptr;             // coarse neighbour table [Vc][9]
     int* cord = nullptr;            // coarse sites by parity (even extents only)
     bool in_solve = false;          // inside a solve: its preconditioner may use the red-black form
@@ -634,7 +634,10 @@ int ensure_panel(mg_ctx* ctx, PanelWork& w, int npad, int nc, int Vc) {
     return MG_OK;
 }
 // CG on the normal equations of the level's operator for nrhs columns of the panel
-// w.rc -> w.y, red-black where the lattice allows it (see coarse_solve).  *err is
+// w.rc -> w.y, red-black where the lattice allows it: less than half the iterations, each
+// of four barriers instead of two.  Coarse solves of a call on D_c and red-black: 12
+// sources on 16^3x32 (Nv = 16) 210 and 126 ms, 21 on 8^3x16 (Nv = 8), where barriers weigh
+// most, 29 and 25, one on 24^3x32 (Nv = 24) 255 and 130.  *err is
 // raised on a timed-out wait; scal (optional) receives column 0's iterations.
 // top: the scales of the operator's tiles (coarse_tiles; a batch keeps powers of two, so
 // that its operator is D_c rounded to FP16).  MG_ERR_OOM before anything is launched.
@@ -766,8 +769,8 @@ int coarse_solve(mg_ctx* ctx, const CoarseLevel& L, const CgSys<T>& sys, const v
         bcg_shape(L.nc, 8, sys.g.Vc / 2, &nw, &stages)) {
         // FP16 operator larger than the chip: the panel solver with one column of eight in
         // use, its operator tiles streaming ahead across the grid barriers (24^3x32, Nv =
-        // 24: 249 -> 114 ms of coarse solves per solve against the
-        // register-streaming kernel on D_c, 177 with that kernel red-black)
+        // 24, per CG iteration: the register-streaming kernel 84 us on D_c and 124 red-black,
+        // this one 79 and 82, red-black half the iterations)
         PanelWork& w = ctx->pw1;
         int st = ensure_panel(ctx, w, 8, L.nc, sys.g.Vc);
         const long long n = (long long)sys.g.Vc * L.nc;
