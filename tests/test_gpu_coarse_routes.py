@@ -107,3 +107,29 @@ def test_fp64_iterations_in_several_passes(L, nv):
         y, it, _ = mg.coarse_solve(rc, 0.0, 4, wmg.MG_FP64)
     assert it == 4
     assert np.abs(y - ref).max() <= 1e-10 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("prec,kernel", [(wmg.MG_FP64, 0), (wmg.MG_FP32, 1), (wmg.MG_FP16, 1)])
+def test_red_black_form_of_the_widest_level(prec, kernel):
+    """Level 2 at Nv2 = 32, the widest operator there is (64 dof): the solve runs its
+    red-black form and reaches its tolerance."""
+    L = (8, 8, 8, 16)
+    b = synth.gaussian_spinor(L, 98)
+    kw = dict(levels=3, nvec2=32, smoother_steps1=2, tol=1e-8, delta=0.0 if prec == wmg.MG_FP64 else 1e-4)
+    p = wmg.mg_default_params()
+    for i in range(4):
+        p.block[i] = p.block2[i] = 2
+    p.nvec, p.setup_group, p.prec_inner, p.coarse_kernel = 16, 2, prec, kernel
+    for k, v in kw.items():
+        setattr(p, k, v)
+    U = rough_gauge(L, seed=8)
+    with wmg.WilsonMG(L, p) as mg:
+        mg.set_links(U)
+        mg.set_mass(MASS)
+        mg.set_null_vectors(synth.gaussian_vectors(L, 16, 97))
+        n1 = mg.Vc * mg.nc
+        mg.set_level2_vectors(synth.gaussian(32 * n1, 5, 0).reshape(32, mg.Vc, mg.nc))
+        x, info = mg.solve(b)
+        assert (mg.coarse_kernel(), mg.coarse_red_black()) == (REGISTER, 1)
+    assert info["status"] == wmg.MG_OK
+    assert np.linalg.norm(b - oracle.dslash(U, x, MASS, L)) <= 2e-8 * np.linalg.norm(b)
